@@ -10,10 +10,10 @@
 // S = 64 symbols starting at symbol k0 reads y[2 k0 - 12, 2 k0 + 140).
 // Parameter vector: W1[32][9][2] b1[32] W2[32][9][32] b2[32] W3[32][9][32] b3[32]
 //                   M1[64][32] c1[64] M2[2][64] c2[2].
-// Activations are channel-last, so the im2col row of output position p of a
-// 32-channel layer is the contiguous slice act[32 p, 32 p + 288): the
-// convolution is a plain GEMM A[p][k] = act[32 p + k], k = 9 x 32, against
-// W[o][k], computed with mma.sync m16n8k16 (BF16 in, FP32 accumulate).
+// Activations are channel-last, so the im2col row of output position p of a 32-channel
+// layer is 9 consecutive rows of 32 channels: the convolution is a plain GEMM of the rows
+// from p on against W[o][k], k = 9 x 32, computed with mma.sync m16n8k16 (BF16 in, FP32
+// accumulate); the receiver's inference kernel (tcgen05) is further below.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -31,12 +31,11 @@
 namespace rxk {
 
 constexpr int CC = 32, CK = 9, CH = 64, CS = 64;          // channels, kernel, hidden, symbols per segment
-constexpr int L0 = 2 * CS + 24, L1 = L0 - 8, L2 = L1 - 8, L3 = L2 - 8;
+constexpr int L0 = 2 * CS + 24, L1 = L0 - 8, L2 = L1 - 8;
 constexpr int KW = CK * CC;                               // 288
 constexpr int OW1 = 0, OB1 = OW1 + CC * CK * 2, OW2 = OB1 + CC, OB2 = OW2 + CC * KW, OW3 = OB2 + CC,
               OB3 = OW3 + CC * KW, OM1 = OB3 + CC, OC1 = OM1 + CH * CC, OM2 = OC1 + CH, OC2 = OM2 + 2 * CH,
               NPRM = OC2 + 2;
-constexpr int kCnnThreads = 128;
 
 __device__ __forceinline__ float gelu_f(float u) { return 0.5f * u * (1.0f + erff(u * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_df(float u)
@@ -52,497 +51,728 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// saved forward state of one segment (training)
-struct CnnSave {
-    float *u1, *u2, *u3;          // pre-activations, [seg][L][32]
-    __nv_bfloat16 *h1, *h2, *h3;  // activations, [seg][L][32]
-    float *v;                     // MLP pre-activation, [seg][S][64]
-    float *out;                   // outputs, [seg][S][2]
-};
+// ------------------------------------------------- shared-memory operand tiles
+// Activations are rows of 32 channels (64 bytes, four 16-byte chunks), read by
+// ldmatrix.  Eight consecutive rows at a 64-byte pitch would fall on two groups of four
+// banks; the chunk index is therefore exclusive-ored with bits 1-2 of the row, which
+// spreads the eight rows of every 8 x 8 matrix over all 32 banks, for any row offset
+// (a tap moves the rows) and for plain and transposed loads.  Weight rows (288 values,
+// 36 chunks) have the same pitch modulo 128 bytes and take the same rule.
+__device__ __forceinline__ uint32_t row_off(int row, int chunk) { return row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4); }
+__device__ __forceinline__ uint32_t w_off(int o, int chunk) { return o * (KW * 2) + ((chunk ^ ((o >> 1) & 3)) << 4); }
+// rows of 64 values (128 bytes, eight chunks)
+__device__ __forceinline__ uint32_t row128_off(int row, int chunk) { return row * 128 + ((chunk ^ (row & 7)) << 4); }
 
-// 32-channel valid convolution layer on the tensor cores:
-// dst[p][o] = GELU(b[o] + sum_k src[32 p + k] W[o][k]) for p < Lout; src has at
-// least 16 * ceil(Lout / 16) + 8 rows (extra rows zero).
-template <int LOUT>
-__device__ __forceinline__ void conv32_mma(const __nv_bfloat16 *src, const __nv_bfloat16 *W, const float *b,
-                                           __nv_bfloat16 *dst, float *u_save, int warp, int lane)
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr)
 {
-    constexpr int TILES = (LOUT + 15) / 16;
-    const int g = lane >> 2, tq = lane & 3;
-    for (int tile = warp; tile < TILES; tile += kCnnThreads / 32) {
-        const int r0 = 16 * tile;
-        float acc[4][4];
-#pragma unroll
-        for (int n = 0; n < 4; n++)
-#pragma unroll
-            for (int i = 0; i < 4; i++) acc[n][i] = 0.f;
-#pragma unroll 2
-        for (int k0 = 0; k0 < KW; k0 += 16) {
-            uint32_t a[4];
-            const __nv_bfloat16 *ar = src + 32 * (r0 + g) + k0 + 2 * tq;
-            a[0] = *reinterpret_cast<const uint32_t *>(ar);
-            a[1] = *reinterpret_cast<const uint32_t *>(ar + 32 * 8);
-            a[2] = *reinterpret_cast<const uint32_t *>(ar + 8);
-            a[3] = *reinterpret_cast<const uint32_t *>(ar + 32 * 8 + 8);
-#pragma unroll
-            for (int n = 0; n < 4; n++) {
-                const __nv_bfloat16 *br = W + KW * (8 * n + g) + k0 + 2 * tq;
-                mma_bf16(acc[n], a, *reinterpret_cast<const uint32_t *>(br),
-                         *reinterpret_cast<const uint32_t *>(br + 8));
-            }
-        }
-#pragma unroll
-        for (int n = 0; n < 4; n++)
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                int r = r0 + g + 8 * (i >> 1), o = 8 * n + 2 * tq + (i & 1);
-                if (r < LOUT) {
-                    float u = acc[n][i] + b[o];
-                    dst[32 * r + o] = __float2bfloat16(gelu_f(u));
-                    if (u_save) u_save[32 * r + o] = u;
-                }
-            }
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ uint32_t bf2(float a, float b)
+{
+    __nv_bfloat162 h = __halves2bfloat162(__float2bfloat16(a), __float2bfloat16(b));
+    return *reinterpret_cast<uint32_t *>(&h);
+}
+
+// BF16 weights of a 32-channel layer, global [32][288] -> shared rows with swizzled chunks
+template <int NTH>
+__device__ __forceinline__ void stage_w(unsigned char *dst, const __nv_bfloat16 *src, int tid)
+{
+    for (int i = tid; i < CC * (KW / 8); i += NTH) {
+        const int o = i / (KW / 8), ch = i - o * (KW / 8);
+        cp_async16(dst + w_off(o, ch), src + o * KW + 8 * ch);
     }
 }
 
-// shared-memory layout of the forward kernel (bytes)
-struct FwdSmem {
-    static constexpr int X = 0;                                     // float [L0][2]
-    static constexpr int W1 = X + L0 * 2 * 4;                       // float [32][18]
-    static constexpr int B = W1 + CC * 18 * 4;                      // float b1, b2, b3 [96]
-    static constexpr int M1 = B + 3 * CC * 4;                       // float [64][32]
-    static constexpr int C1 = M1 + CH * CC * 4;                     // float [64]
-    static constexpr int M2 = C1 + CH * 4;                          // float [2][64] + c2 [2]
-    static constexpr int WB2 = ((M2 + (2 * CH + 2) * 4) + 15) & ~15; // bf16 [32][288]
-    static constexpr int WB3 = WB2 + CC * KW * 2;
-    static constexpr int H1 = WB3 + CC * KW * 2;                    // bf16 [L1 + 16][32]
-    static constexpr int H2 = H1 + (L1 + 16) * CC * 2;              // bf16 [L2 + 16][32]
-    static constexpr int H3 = H2 + (L2 + 16) * CC * 2;              // bf16 [L3][32]
-    static constexpr int OUT = H3 + L3 * CC * 2;                    // float [S][2]
-    static constexpr int TOTAL = OUT + CS * 2 * 4;
+// Layer 1 (2 -> 32, K = 18) in FP32, a channel pair per lane (2 cp, 2 cp + 1) as one
+// packed FP32 pair, RPH consecutive rows per half-warp.  xs holds every input value
+// twice, (re, re, im, im), so that one 16-byte load feeds both channels.  Products are
+// accumulated from the bias on in tap order, re before im.
+struct L1Weights {
+    f2x b, w[18];
 };
+// shared copy of the weights and biases as channel pairs: [k][pair], row 18 the biases
+constexpr int kW1Floats = 19 * CC;
+template <int NTH>
+__device__ __forceinline__ void stage_l1(float *w1, const float *__restrict__ prm, int tid)
+{
+    for (int i = tid; i < kW1Floats; i += NTH) {
+        const int k = i / CC, o = i % CC;
+        w1[i] = k < 18 ? prm[OW1 + o * 18 + k] : prm[OB1 + o];
+    }
+}
+__device__ __forceinline__ void load_l1(L1Weights &W, const float *w1, int cp)
+{
+    const f2x *p = reinterpret_cast<const f2x *>(w1) + cp;
+#pragma unroll
+    for (int k = 0; k < 18; k++) W.w[k] = p[k * (CC / 2)];
+    W.b = p[18 * (CC / 2)];
+}
+template <int RPH, typename Emit>
+__device__ __forceinline__ void layer1_rows(const L1Weights &W, const float4 *xs, int p0, Emit emit)
+{
+    ulonglong2 x[RPH + 8];
+#pragma unroll
+    for (int i = 0; i < RPH + 8; i++) x[i] = reinterpret_cast<const ulonglong2 *>(xs)[p0 + i];
+#pragma unroll
+    for (int i = 0; i < RPH; i++) {
+        f2x a = W.b;
+#pragma unroll
+        for (int t = 0; t < CK; t++) {
+            a = f2_fma(W.w[2 * t], x[i + t].x, a);
+            a = f2_fma(W.w[2 * t + 1], x[i + t].y, a);
+        }
+        emit(p0 + i, f2_unpack(a));
+    }
+}
 
-// Forward pass of nseg segments, one CTA each.  y: complex 2-sps input; seg_start[s]:
-// index in y of the segment's first input sample (2 k0 - 12).  Writes out[s][j][2]
-// and, when sv.u1 is set, the activations for the backward pass.  In receiver mode
-// (dec non-null) it decides the symbols instead and scores them (window records).
-__global__ void __launch_bounds__(kCnnThreads)
+// One 16-row tile of a 32-channel, 9-tap convolution: acc[n] += A B over K = 288 in steps
+// of 16 (tap ks / 2, channels 16 (ks % 2) ..), 2 NP blocks of 8 output channels from n0.
+// a_addr(tap, chunk) is this lane's row address (row lane % 16 of the tile).
+template <int NP, typename Addr>
+__device__ __forceinline__ void conv_tile(float (&acc)[2 * NP][4], uint32_t w, int n0, int lane, Addr a_addr)
+{
+    uint32_t wa[2][NP];
+#pragma unroll
+    for (int p = 0; p < NP; p++) {
+        const int n = n0 + 16 * p + (lane & 7) + ((lane >> 4) << 3);
+        wa[0][p] = w + w_off(n, (lane >> 3) & 1);
+        wa[1][p] = w + w_off(n, 2 + ((lane >> 3) & 1));
+    }
+#pragma unroll
+    for (int n = 0; n < 2 * NP; n++)
+#pragma unroll
+        for (int i = 0; i < 4; i++) acc[n][i] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < KW / 16; ks++) {
+        uint32_t a[4], b[NP][4];
+        ldsm4(a, a_addr(ks >> 1, 2 * (ks & 1) + (lane >> 4)));
+#pragma unroll
+        for (int p = 0; p < NP; p++) ldsm4(b[p], wa[ks & 1][p] + 64 * (ks >> 1));
+#pragma unroll
+        for (int p = 0; p < NP; p++) {
+            mma_bf16(acc[2 * p], a, b[p][0], b[p][1]);
+            mma_bf16(acc[2 * p + 1], a, b[p][2], b[p][3]);
+        }
+    }
+}
+
+// ------------------------------------------------------------------- inference
+// rx_cnn_forward: persistent CTAs of nine warps, three per SM, each looping over
+// segments with the weights staged once.  Nine warps because layer 2 has nine row tiles
+// of 16 (144 computed positions) and layer 1 144 rows: every warp does one tile with all
+// 32 channels.  Layer 3 runs at the symbol (even) positions only, the ones the MLP reads:
+// layer 2 stores even and odd positions in two row sets, tap t reads set t & 1.
+// The MLP's first layer takes its FP32 weights as three BF16 terms (8 + 8 + 8 bits, the
+// sum exact), so its products with the BF16 activations are those of the FP32 weights,
+// accumulated in FP32 on the tensor cores.
+// Bound: FP32 issue of the erf GELU (472 warp-wide evaluations a segment).  4096 segments:
+// 128 us; 457 us with one 128-thread CTA per segment that staged all weights for it, layer
+// 3 at every position, 4-byte operand loads and the MLP on the CUDA cores.
+constexpr int kFwThreads = 288, kFwPerSm = 3;
+constexpr int kH1Rows = L1 + 8;              // rows L1 .. are zero (read by the last tile's taps)
+constexpr int kH2Half = L2 / 2;              // rows of each of layer 2's even / odd sets
+struct FwdSmem {
+    static constexpr int W2 = 0;
+    static constexpr int W3 = W2 + CC * KW * 2;
+    static constexpr int M1 = W3 + CC * KW * 2;            // bf16 [3 terms][64][32]
+    static constexpr int H1 = M1 + 3 * CH * CC * 2;        // bf16 [kH1Rows][32]; then h3 [64][32]
+    static constexpr int H2 = H1 + kH1Rows * CC * 2;       // bf16 [2][kH2Half][32]
+    static constexpr int XD = H2;                          // float4 [L0]: the input, every value twice (layer 1 only)
+    static constexpr int X = H2 + 2 * kH2Half * CC * 2;    // float2 [2][L0]: this and the next segment's input
+    static constexpr int W1 = X + 2 * L0 * 8;              // float [19][32]
+    static constexpr int B = W1 + kW1Floats * 4;           // float b2, b3 [64], c1 [64], M2 [128], c2 [2] (+ 2)
+    static constexpr int OUT = B + (64 + CH + 2 * CH + 4) * 4;   // float [2 halves][64][2]
+    static constexpr int TOTAL = OUT + 2 * CS * 2 * 4;
+};
+static_assert(kFwPerSm * (FwdSmem::TOTAL + 1024) <= 228 * 1024, "three CTAs per SM");
+static_assert(FwdSmem::H1 % 16 == 0 && FwdSmem::X % 16 == 0 && FwdSmem::XD % 16 == 0, "16-byte rows");
+static_assert(L0 * 16 <= 2 * kH2Half * CC * 2, "the doubled input fits the layer-2 rows");
+
+__global__ void __launch_bounds__(kFwThreads, kFwPerSm)
     k_cnn_fwd(const float *__restrict__ prm, const __nv_bfloat16 *__restrict__ prm_bf, const float2 *__restrict__ y,
-              const long long *__restrict__ seg_start, long long seg_base, long long seg_step, float *__restrict__ out,
-              CnnSave sv, uint8_t *__restrict__ dec, uint8_t *__restrict__ winb, uint4 *__restrict__ winrec,
-              const uint32_t *__restrict__ prbs_bits, long long k_first, float scale, int mq)
+              const long long *__restrict__ seg_start, int nseg, float *__restrict__ out)
 {
     extern __shared__ __align__(16) unsigned char sm[];
-    float *xs = reinterpret_cast<float *>(sm + FwdSmem::X);
-    float *w1 = reinterpret_cast<float *>(sm + FwdSmem::W1);
-    float *bb = reinterpret_cast<float *>(sm + FwdSmem::B);
-    float *m1 = reinterpret_cast<float *>(sm + FwdSmem::M1);
-    float *c1 = reinterpret_cast<float *>(sm + FwdSmem::C1);
-    float *m2 = reinterpret_cast<float *>(sm + FwdSmem::M2);
-    __nv_bfloat16 *wb2 = reinterpret_cast<__nv_bfloat16 *>(sm + FwdSmem::WB2);
-    __nv_bfloat16 *wb3 = reinterpret_cast<__nv_bfloat16 *>(sm + FwdSmem::WB3);
-    __nv_bfloat16 *h1 = reinterpret_cast<__nv_bfloat16 *>(sm + FwdSmem::H1);
-    __nv_bfloat16 *h2 = reinterpret_cast<__nv_bfloat16 *>(sm + FwdSmem::H2);
-    __nv_bfloat16 *h3 = reinterpret_cast<__nv_bfloat16 *>(sm + FwdSmem::H3);
+    float2 *x2 = reinterpret_cast<float2 *>(sm + FwdSmem::X);
+    float4 *xd = reinterpret_cast<float4 *>(sm + FwdSmem::XD);
+    float *b2 = reinterpret_cast<float *>(sm + FwdSmem::B), *b3 = b2 + CC, *c1 = b3 + CC, *m2 = c1 + CH;
     float *os = reinterpret_cast<float *>(sm + FwdSmem::OUT);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int s = blockIdx.x;
-    const long long st = seg_start ? seg_start[s] : seg_base + seg_step * s;
-    // stage inputs and parameters
-    for (int i = tid; i < L0; i += kCnnThreads) {
-        float2 v = y[st + i];
-        xs[2 * i] = v.x;
-        xs[2 * i + 1] = v.y;
-    }
-    for (int i = tid; i < CC * 18; i += kCnnThreads) w1[i] = prm[OW1 + i];
-    for (int i = tid; i < CC; i += kCnnThreads) {
-        bb[i] = prm[OB1 + i];
-        bb[CC + i] = prm[OB2 + i];
-        bb[2 * CC + i] = prm[OB3 + i];
-    }
-    for (int i = tid; i < CH * CC; i += kCnnThreads) m1[i] = prm[OM1 + i];
-    for (int i = tid; i < CH; i += kCnnThreads) c1[i] = prm[OC1 + i];
-    for (int i = tid; i < 2 * CH + 2; i += kCnnThreads) m2[i] = prm[OM2 + i];
-    for (int i = tid; i < CC * KW / 8; i += kCnnThreads) {
-        reinterpret_cast<uint4 *>(wb2)[i] = reinterpret_cast<const uint4 *>(prm_bf + OW2)[i];
-        reinterpret_cast<uint4 *>(wb3)[i] = reinterpret_cast<const uint4 *>(prm_bf + OW3)[i];
-    }
-    // zero the padding rows read by the last (partial) row tiles
-    for (int i = tid; i < 16 * CC; i += kCnnThreads) {
-        h1[L1 * CC + i] = __float2bfloat16(0.f);
-        h2[L2 * CC + i] = __float2bfloat16(0.f);
-    }
-    __syncthreads();
-    // layer 1 (2 input channels, K = 18) on the CUDA cores
-    float *u1s = sv.u1 ? sv.u1 + (size_t)s * L1 * CC : nullptr;
-    for (int i = tid; i < L1 * CC; i += kCnnThreads) {
-        int p = i >> 5, o = i & 31;
-        float a = bb[o];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, tq = lane & 3;
+    const uint32_t sW2 = smem_u32(sm + FwdSmem::W2), sW3 = smem_u32(sm + FwdSmem::W3), sM1 = smem_u32(sm + FwdSmem::M1);
+    const uint32_t sH1 = smem_u32(sm + FwdSmem::H1), sH2 = smem_u32(sm + FwdSmem::H2);
+    auto prefetch = [&](int s, int buf) {
+        const float2 *src = y + seg_start[s];
+        for (int i = tid; i < L0; i += kFwThreads) cp_async8(x2 + buf * L0 + i, src + i, true);
+        cp_async_commit();
+    };
+    int s = blockIdx.x;
+    if (s < nseg) prefetch(s, 0);
+    stage_w<kFwThreads>(sm + FwdSmem::W2, prm_bf + OW2, tid);
+    stage_w<kFwThreads>(sm + FwdSmem::W3, prm_bf + OW3, tid);
+    cp_async_commit();
+    for (int i = tid; i < CH * CC; i += kFwThreads) {   // w = t0 + t1 + t2, every remainder exact in FP32
+        const int m = i >> 5, c = i & 31;
+        float w = prm[OM1 + i];
 #pragma unroll
-        for (int k = 0; k < 18; k++) a = fmaf(w1[o * 18 + k], xs[2 * p + k], a);
-        h1[i] = __float2bfloat16(gelu_f(a));
-        if (u1s) u1s[i] = a;
+        for (int t = 0; t < 3; t++) {
+            const __nv_bfloat16 h = __float2bfloat16(w);
+            w -= __bfloat162float(h);
+            *reinterpret_cast<__nv_bfloat16 *>(sm + FwdSmem::M1 + t * CH * CC * 2 + row_off(m, c >> 3) + 2 * (c & 7)) = h;
+        }
     }
-    __syncthreads();
-    conv32_mma<L2>(h1, wb2, bb + CC, h2, sv.u2 ? sv.u2 + (size_t)s * L2 * CC : nullptr, warp, lane);
-    __syncthreads();
-    conv32_mma<L3>(h2, wb3, bb + 2 * CC, h3, sv.u3 ? sv.u3 + (size_t)s * L3 * CC : nullptr, warp, lane);
-    __syncthreads();
-    if (sv.h1) {
-        for (int i = tid; i < L1 * CC / 8; i += kCnnThreads)
-            reinterpret_cast<uint4 *>(sv.h1 + (size_t)s * L1 * CC)[i] = reinterpret_cast<const uint4 *>(h1)[i];
-        for (int i = tid; i < L2 * CC / 8; i += kCnnThreads)
-            reinterpret_cast<uint4 *>(sv.h2 + (size_t)s * L2 * CC)[i] = reinterpret_cast<const uint4 *>(h2)[i];
-        for (int i = tid; i < L3 * CC / 8; i += kCnnThreads)
-            reinterpret_cast<uint4 *>(sv.h3 + (size_t)s * L3 * CC)[i] = reinterpret_cast<const uint4 *>(h3)[i];
+    if (tid < CC) {
+        b2[tid] = prm[OB2 + tid];
+        b3[tid] = prm[OB3 + tid];
+        reinterpret_cast<uint4 *>(sm + FwdSmem::H1 + L1 * 64)[tid] = make_uint4(0, 0, 0, 0);   // 8 rows of 64 bytes
     }
-    // MLP head at the symbol positions: two threads per symbol, 32 hidden units each
+    for (int i = tid; i < CH; i += kFwThreads) c1[i] = prm[OC1 + i];
+    for (int i = tid; i < 2 * CH + 2; i += kFwThreads) m2[i] = prm[OM2 + i];
+    float *w1 = reinterpret_cast<float *>(sm + FwdSmem::W1);
+    stage_l1<kFwThreads>(w1, prm, tid);
+    for (int buf = 0; s < nseg; s += gridDim.x, buf ^= 1) {
+        cp_async_wait_all();
+        __syncthreads();   // this segment's input (and, the first time, the weights)
+        if (s + (int)gridDim.x < nseg) prefetch(s + gridDim.x, buf ^ 1);
+        for (int i = tid; i < L0; i += kFwThreads) {
+            const float2 v = x2[buf * L0 + i];
+            xd[i] = make_float4(v.x, v.x, v.y, v.y);
+        }
+        __syncthreads();
+        L1Weights W1;
+        load_l1(W1, w1, lane & 15);
+        layer1_rows<8>(W1, xd, 16 * warp + 8 * (lane >> 4), [&](int p, float2 u) {
+            const int cp = lane & 15;
+            *reinterpret_cast<uint32_t *>(sm + FwdSmem::H1 + row_off(p, cp >> 2) + 4 * (cp & 3)) =
+                bf2(gelu_f(u.x), gelu_f(u.y));
+        });
+        __syncthreads();
+        {   // layer 2: rows 16 warp ..
+            float acc[4][4];
+            conv_tile<2>(acc, sW2, 0, lane, [&](int t, int ch) { return sH1 + row_off(16 * warp + (lane & 15) + t, ch); });
+#pragma unroll
+            for (int n = 0; n < 4; n++) {
+                const float2 b = *reinterpret_cast<const float2 *>(b2 + 8 * n + 2 * tq);
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int r = 16 * warp + g + 8 * h;
+                    if (r < L2)
+                        *reinterpret_cast<uint32_t *>(sm + FwdSmem::H2 + (r & 1) * kH2Half * 64 + row_off(r >> 1, n) + 4 * tq) =
+                            bf2(gelu_f(acc[n][2 * h] + b.x), gelu_f(acc[n][2 * h + 1] + b.y));
+                }
+            }
+        }
+        __syncthreads();
+        if (warp < 8) {   // layer 3 at the symbols 16 tile ..: channels 16 half ..
+            const int tile = warp >> 1, half = warp & 1;
+            float acc[2][4];
+            conv_tile<1>(acc, sW3, 16 * half, lane, [&](int t, int ch) {
+                return sH2 + (t & 1) * kH2Half * 64 + row_off(16 * tile + (lane & 15) + (t >> 1), ch);
+            });
+#pragma unroll
+            for (int n = 0; n < 2; n++) {
+                const float2 b = *reinterpret_cast<const float2 *>(b3 + 16 * half + 8 * n + 2 * tq);
+#pragma unroll
+                for (int h = 0; h < 2; h++)
+                    *reinterpret_cast<uint32_t *>(sm + FwdSmem::H1 + row_off(16 * tile + g + 8 * h, 2 * half + n) + 4 * tq) =
+                        bf2(gelu_f(acc[n][2 * h] + b.x), gelu_f(acc[n][2 * h + 1] + b.y));
+            }
+        }
+        __syncthreads();
+        if (warp < 8) {   // MLP: symbols 16 tile .., hidden units 32 half ..
+            const int tile = warp >> 1, half = warp & 1;
+            float acc[4][4];
+#pragma unroll
+            for (int n = 0; n < 4; n++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) acc[n][i] = 0.f;
+            uint32_t a[2][4];
+#pragma unroll
+            for (int ks = 0; ks < 2; ks++) ldsm4(a[ks], sH1 + row_off(16 * tile + (lane & 15), 2 * ks + (lane >> 4)));
+#pragma unroll
+            for (int t = 2; t >= 0; t--)   // smallest terms first
+#pragma unroll
+                for (int ks = 0; ks < 2; ks++)
+#pragma unroll
+                    for (int p = 0; p < 2; p++) {
+                        uint32_t b[4];
+                        ldsm4(b, sM1 + t * CH * CC * 2 +
+                                     row_off(32 * half + 16 * p + (lane & 7) + ((lane >> 4) << 3), 2 * ks + ((lane >> 3) & 1)));
+                        mma_bf16(acc[2 * p], a[ks], b[0], b[1]);
+                        mma_bf16(acc[2 * p + 1], a[ks], b[2], b[3]);
+                    }
+            float o[2][2] = {{0.f, 0.f}, {0.f, 0.f}};   // [row g, g + 8][output]
+#pragma unroll
+            for (int n = 0; n < 4; n++)
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    const int m = 32 * half + 8 * n + 2 * tq + i;
+                    const float c = c1[m], ma = m2[m], mb = m2[CH + m];
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const float z = gelu_f(acc[n][2 * h + i] + c);
+                        o[h][0] = fmaf(ma, z, o[h][0]);
+                        o[h][1] = fmaf(mb, z, o[h][1]);
+                    }
+                }
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+#pragma unroll
+                for (int q = 0; q < 2; q++) {
+                    o[h][q] += __shfl_xor_sync(0xffffffffu, o[h][q], 1);
+                    o[h][q] += __shfl_xor_sync(0xffffffffu, o[h][q], 2);
+                }
+            if (tq == 0)
+#pragma unroll
+                for (int h = 0; h < 2; h++)
+                    *reinterpret_cast<float2 *>(os + 2 * (CS * half + 16 * tile + g + 8 * h)) = make_float2(o[h][0], o[h][1]);
+        }
+        __syncthreads();
+        if (tid < 2 * CS) out[(size_t)s * 2 * CS + tid] = os[tid] + os[2 * CS + tid] + m2[2 * CH + (tid & 1)];
+    }
+    cp_async_wait_all();
+}
+
+// --------------------------------------------------------------------- training
+// Forward and backward pass of one segment per CTA, everything between them in shared
+// memory: 18 warps, since layer 2 has 9 row tiles x 2 channel halves, its input gradient
+// the same, and a weight gradient 2 x 9 (output-channel half, tap) units.  The GELU
+// derivative is taken with the GELU (they share the erf) and kept in FP32 in place of the
+// pre-activation.  The transposed operands of the backward products (du and the layer
+// inputs with the positions along K, the weights with the output channels along K) are
+// read with transposing ldmatrix from the forward's own tiles, so nothing is rearranged.
+// A step of 64 segments (this kernel, the reduction and Adam): 34 us; 146 us with a forward
+// and a backward kernel that passed activations through global memory and rearranged their
+// operands in shared memory.  Bound: the chain of eleven phases, each a few hundred cycles
+// of one CTA per SM.
+// BF16 operands, FP32 accumulation over the positions in order (mma.sync m16n8k16: the
+// contractions of a segment are 32 wide, below a tcgen05 tile); GELU derivatives, dM2,
+// biases and the 2-channel layer 1 in FP32.
+constexpr int kTrThreads = 576, kTrWarps = kTrThreads / 32;
+constexpr int kZP = CH + 1;                                  // padded row of the hidden units
+struct TrainSmem {
+    static constexpr int W2 = 0;
+    static constexpr int W3 = W2 + CC * KW * 2;
+    static constexpr int M1B = W3 + CC * KW * 2;             // bf16 [64][32]
+    static constexpr int M1 = M1B + CH * CC * 2;             // float [64][32]
+    static constexpr int H1 = M1 + CH * CC * 4;              // bf16 [kH1Rows][32]
+    static constexpr int H2 = H1 + kH1Rows * CC * 2;         // bf16 [L2][32]
+    static constexpr int H3 = H2 + L2 * CC * 2;              // bf16 [64][32] (symbols)
+    static constexpr int DVB = H3 + CS * CC * 2;             // bf16 [64 symbols][64 units] dv
+    static constexpr int DU3 = DVB + CS * CH * 2;            // bf16 [160][32]: du3 from row 8 on
+    static constexpr int DU2 = DU3 + 160 * CC * 2;           // bf16 [160][32]: du2 from row 8 on
+    static constexpr int D1 = DU2 + 160 * CC * 2;            // float [L1][32]: gelu'(u1), then du1
+    static constexpr int D2 = D1 + L1 * CC * 4;              // float [L2][32]: gelu'(u2)
+    static constexpr int D3 = D2 + L2 * CC * 4;              // float [64][32]: gelu'(u3)
+    static constexpr int Z = D3 + CS * CC * 4;               // float [64][kZP] hidden units
+    static constexpr int DZ = Z + CS * kZP * 4;              // float [64][kZP] gelu'(v), then dv
+    static constexpr int XD = DZ + CS * kZP * 4;             // float4 [L0]
+    static constexpr int W1 = XD + L0 * 16;                  // float [19][32]
+    static constexpr int B = W1 + kW1Floats * 4;             // float b2, b3 [64], c1 [64], M2 [128] c2 [2] (+ 2)
+    static constexpr int DO = B + (64 + CH + 2 * CH + 4) * 4;   // float [64][2] gradient at the outputs
+    static constexpr int RED = DO + CS * 2 * 4;              // float [18][32] bias partials, [4] loss
+    static constexpr int TOTAL = RED + (kTrWarps * CC + 4) * 4;
+    static constexpr int P1 = D2;                            // float [18][576] layer-1 partials (D2, D3, Z are free)
+};
+static_assert(TrainSmem::TOTAL <= 227 * 1024, "one training CTA per SM");
+static_assert(TrainSmem::P1 + kTrWarps * CC * 18 * 4 <= TrainSmem::DZ, "layer-1 partials fit");
+static_assert(TrainSmem::M1 % 16 == 0 && TrainSmem::H1 % 16 == 0 && TrainSmem::DU3 % 16 == 0 && TrainSmem::XD % 16 == 0,
+              "16-byte rows");
+
+__global__ void __launch_bounds__(kTrThreads, 1)
+    k_cnn_train(const float *__restrict__ prm, const __nv_bfloat16 *__restrict__ prm_bf, const float2 *__restrict__ y,
+                const long long *__restrict__ seg_start, const float *__restrict__ tgt, float norm,
+                float *__restrict__ gpart, float *__restrict__ lpart)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    float4 *xd = reinterpret_cast<float4 *>(sm + TrainSmem::XD);
+    float *b2 = reinterpret_cast<float *>(sm + TrainSmem::B), *b3 = b2 + CC, *c1 = b3 + CC, *m2 = c1 + CH;
+    float *m1 = reinterpret_cast<float *>(sm + TrainSmem::M1);
+    float *d1 = reinterpret_cast<float *>(sm + TrainSmem::D1), *d2 = reinterpret_cast<float *>(sm + TrainSmem::D2);
+    float *d3 = reinterpret_cast<float *>(sm + TrainSmem::D3);
+    float *zs = reinterpret_cast<float *>(sm + TrainSmem::Z), *dz = reinterpret_cast<float *>(sm + TrainSmem::DZ);
+    float *dout = reinterpret_cast<float *>(sm + TrainSmem::DO), *red = reinterpret_cast<float *>(sm + TrainSmem::RED);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, tq = lane & 3;
+    const uint32_t sW2 = smem_u32(sm + TrainSmem::W2), sW3 = smem_u32(sm + TrainSmem::W3);
+    const uint32_t sH1 = smem_u32(sm + TrainSmem::H1), sH2 = smem_u32(sm + TrainSmem::H2), sH3 = smem_u32(sm + TrainSmem::H3);
+    const uint32_t sDV = smem_u32(sm + TrainSmem::DVB), sM1B = smem_u32(sm + TrainSmem::M1B);
+    const int s = blockIdx.x;
+    float *G = gpart + (size_t)s * NPRM;
+
+    // ---- stage: the input and what layer 1 needs first, the weights behind it
+    stage_w<kTrThreads>(sm + TrainSmem::W2, prm_bf + OW2, tid);
+    stage_w<kTrThreads>(sm + TrainSmem::W3, prm_bf + OW3, tid);
+    for (int i = tid; i < CH * 4; i += kTrThreads)
+        cp_async16(sm + TrainSmem::M1B + row_off(i >> 2, i & 3), prm_bf + OM1 + 8 * i);
+    for (int i = tid; i < CH * CC / 4; i += kTrThreads) cp_async16(m1 + 4 * i, prm + OM1 + 4 * i);
+    cp_async_commit();
     {
-        int j = tid >> 1, half = tid & 1;
+        const float2 *src = y + seg_start[s];
+        for (int i = tid; i < L0; i += kTrThreads) {
+            const float2 v = src[i];
+            xd[i] = make_float4(v.x, v.x, v.y, v.y);
+        }
+    }
+    if (tid < CC) {
+        b2[tid] = prm[OB2 + tid];
+        b3[tid] = prm[OB3 + tid];
+        reinterpret_cast<uint4 *>(sm + TrainSmem::H1 + L1 * 64)[tid] = make_uint4(0, 0, 0, 0);
+    }
+    for (int i = tid; i < CH; i += kTrThreads) c1[i] = prm[OC1 + i];
+    for (int i = tid; i < 2 * CH + 2; i += kTrThreads) m2[i] = prm[OM2 + i];
+    // du3 is zero at the odd positions and both du in the rows around them
+    for (int i = tid; i < 160 * 4; i += kTrThreads) {
+        reinterpret_cast<uint4 *>(sm + TrainSmem::DU3)[i] = make_uint4(0, 0, 0, 0);
+        if (i < 8 * 4 || i >= (8 + L2) * 4) reinterpret_cast<uint4 *>(sm + TrainSmem::DU2)[i] = make_uint4(0, 0, 0, 0);
+    }
+    float *w1 = reinterpret_cast<float *>(sm + TrainSmem::W1);
+    stage_l1<kTrThreads>(w1, prm, tid);
+    __syncthreads();
+    // ---- layer 1
+    L1Weights W1;
+    load_l1(W1, w1, lane & 15);
+    layer1_rows<4>(W1, xd, 8 * warp + 4 * (lane >> 4), [&](int p, float2 u) {
+        const int cp = lane & 15;
+        *reinterpret_cast<uint32_t *>(sm + TrainSmem::H1 + row_off(p, cp >> 2) + 4 * (cp & 3)) =
+            bf2(gelu_f(u.x), gelu_f(u.y));
+        *reinterpret_cast<float2 *>(d1 + p * CC + 2 * cp) = make_float2(gelu_df(u.x), gelu_df(u.y));
+    });
+    cp_async_wait_all();
+    __syncthreads();
+    const int tile9 = warp % 9, half2 = warp / 9;   // a row tile and a half of the channels
+    {   // ---- layer 2
+        float acc[2][4];
+        conv_tile<1>(acc, sW2, 16 * half2, lane, [&](int t, int ch) { return sH1 + row_off(16 * tile9 + (lane & 15) + t, ch); });
+#pragma unroll
+        for (int n = 0; n < 2; n++) {
+            const int o = 16 * half2 + 8 * n + 2 * tq;
+            const float2 b = *reinterpret_cast<const float2 *>(b2 + o);
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int r = 16 * tile9 + g + 8 * h;
+                if (r < L2) {
+                    const float u0 = acc[n][2 * h] + b.x, u1 = acc[n][2 * h + 1] + b.y;
+                    *reinterpret_cast<uint32_t *>(sm + TrainSmem::H2 + row_off(r, 2 * half2 + n) + 4 * tq) =
+                        bf2(gelu_f(u0), gelu_f(u1));
+                    *reinterpret_cast<float2 *>(d2 + r * CC + o) = make_float2(gelu_df(u0), gelu_df(u1));
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (warp < 8) {   // ---- layer 3 at the symbol (even) positions
+        const int tile = warp >> 1, half = warp & 1;
+        float acc[2][4];
+        conv_tile<1>(acc, sW3, 16 * half, lane,
+                     [&](int t, int ch) { return sH2 + row_off(2 * (16 * tile + (lane & 15)) + t, ch); });
+#pragma unroll
+        for (int n = 0; n < 2; n++) {
+            const int o = 16 * half + 8 * n + 2 * tq;
+            const float2 b = *reinterpret_cast<const float2 *>(b3 + o);
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int r = 16 * tile + g + 8 * h;
+                const float u0 = acc[n][2 * h] + b.x, u1 = acc[n][2 * h + 1] + b.y;
+                *reinterpret_cast<uint32_t *>(sm + TrainSmem::H3 + row_off(r, 2 * half + n) + 4 * tq) =
+                    bf2(gelu_f(u0), gelu_f(u1));
+                *reinterpret_cast<float2 *>(d3 + r * CC + o) = make_float2(gelu_df(u0), gelu_df(u1));
+            }
+        }
+    }
+    __syncthreads();
+    if (warp < 16) {   // ---- MLP hidden layer in FP32: 8 units per warp, a symbol per lane
+        const int j = 32 * (warp & 1) + lane, m0 = 8 * (warp >> 1);
         float hv[CC];
 #pragma unroll
-        for (int c = 0; c < CC; c++) hv[c] = __bfloat162float(h3[(2 * j) * CC + c]);
-        float o0 = 0.f, o1 = 0.f;
-        for (int mm = 0; mm < CH / 2; mm++) {
-            int m = half * (CH / 2) + mm;
-            float a = c1[m];
+        for (int q = 0; q < 4; q++) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(sm + TrainSmem::H3 + row_off(j, q));
+            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int c = 0; c < CC; c++) a = fmaf(m1[m * CC + c], hv[c], a);
-            if (sv.v) sv.v[((size_t)s * CS + j) * CH + m] = a;
-            float z = gelu_f(a);
+            for (int i = 0; i < 4; i++) {
+                hv[8 * q + 2 * i] = __uint_as_float(u[i] << 16);
+                hv[8 * q + 2 * i + 1] = __uint_as_float(u[i] & 0xFFFF0000u);
+            }
+        }
+#pragma unroll 2
+        for (int mm = 0; mm < 8; mm++) {
+            const int m = m0 + mm;
+            float a = c1[m];
+            const float4 *w4 = reinterpret_cast<const float4 *>(m1 + m * CC);
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const float4 w = w4[q];
+                a = fmaf(w.x, hv[4 * q], a);
+                a = fmaf(w.y, hv[4 * q + 1], a);
+                a = fmaf(w.z, hv[4 * q + 2], a);
+                a = fmaf(w.w, hv[4 * q + 3], a);
+            }
+            zs[j * kZP + m] = gelu_f(a);
+            dz[j * kZP + m] = gelu_df(a);
+        }
+    }
+    __syncthreads();
+    if (tid < 2 * CS) {   // ---- outputs, loss, gradient at the outputs: two threads per symbol, 32 units each
+        const int j = tid >> 1, half = tid & 1;
+        float o0 = 0.f, o1 = 0.f;
+#pragma unroll 8
+        for (int mm = 0; mm < CH / 2; mm++) {
+            const int m = half * (CH / 2) + mm;
+            const float z = zs[j * kZP + m];
             o0 = fmaf(m2[m], z, o0);
             o1 = fmaf(m2[CH + m], z, o1);
         }
         o0 += __shfl_xor_sync(0xffffffffu, o0, 1);
         o1 += __shfl_xor_sync(0xffffffffu, o1, 1);
-        if (!half) {
-            o0 += m2[2 * CH];
-            o1 += m2[2 * CH + 1];
-            os[2 * j] = o0;
-            os[2 * j + 1] = o1;
-            if (out) {
-                out[((size_t)s * CS + j) * 2] = o0;
-                out[((size_t)s * CS + j) * 2 + 1] = o1;
-            }
-            if (sv.out) {
-                sv.out[((size_t)s * CS + j) * 2] = o0;
-                sv.out[((size_t)s * CS + j) * 2 + 1] = o1;
-            }
-        }
+        const float o = (half ? o1 : o0) + m2[2 * CH + half];
+        const float e = o - tgt[(size_t)s * 2 * CS + tid];
+        dout[tid] = 2.f * e * norm;
+        const float l = warp_sum_f(e * e);
+        if (lane == 0) red[kTrWarps * CC + warp] = l;
     }
-    if (!dec) return;
     __syncthreads();
-    // receiver mode: decisions, decision bytes and the window record (one warp)
-    if (warp == 0) {
-        const int NB = mq == 2 ? 1 : 2, BPS = 2 * NB;
-        long long k0 = k_first + (long long)s * CS;
-        int pwin = (int)(((long long)BPS * k0) % 32767);
-        unsigned eA = 0, eB = 0, se = 0, nn = 0;
-        for (int h = 0; h < 2; h++) {
-            int q = lane + 32 * h;
-            float vr = scale * os[2 * q], vi = scale * os[2 * q + 1];
-            int LI = 0, LQ = 0;
-            bool nr = false;
-            for (int jj = 0; jj < mq - 1; jj++) {
-                float th = (float)(2 * jj - (mq - 2));
-                LI += vr >= th;
-                LQ += vi >= th;
-                nr |= fabsf(vr - th) < 1e-4f || fabsf(vi - th) < 1e-4f;
-            }
-            dec[(size_t)s * CS + q] = (uint8_t)(LI | (LQ << 3) | (nr ? 64 : 0));
-            int pos = pwin + BPS * q;
-            uint32_t w0 = prbs_bits[pos >> 5], w1 = prbs_bits[(pos >> 5) + 1];
-            int ref = (int)(__funnelshift_l(w1, w0, pos & 31) >> (32 - BPS));
-            for (int rq = 0; rq < 4; rq++) {
-                int a = LI, bq = LQ;
-                if (rq & 2) { a = mq - 1 - a; bq = mq - 1 - bq; }
-                if (rq & 1) { int t = a; a = bq; bq = mq - 1 - t; }
-                unsigned ne = __popc((((a ^ (a >> 1)) << NB) | (bq ^ (bq >> 1))) ^ ref);
-                if (rq < 2) eA += ne << (16 * rq);
-                else eB += ne << (16 * (rq - 2));
-                se += (ne > 0) << (8 * rq);
-            }
-            nn += nr;
-        }
-        eA = warp_sum_i(eA);
-        eB = warp_sum_i(eB);
-        se = warp_sum_i(se);
-        nn = warp_sum_i(nn);
-        if (lane == 0) {
-            winb[s] = 0;
-            winrec[s] = make_uint4(eA, eB, se, nn << 8);
-        }
+    if (tid == 0) {
+        const float *l = red + kTrWarps * CC;
+        lpart[s] = (l[0] + l[1]) + (l[2] + l[3]);
     }
-}
-
-// shared-memory layout of the backward kernel (bytes)
-struct BwdSmem {
-    static constexpr int LDV = CH + 8;                           // padded rows of the MLP tiles (bf16)
-    static constexpr int LDT = 152;                              // positions of duT (>= 144 + 8)
-    static constexpr int LDH = 160;                              // positions of the transposed layer input
-    static constexpr int NDU = 160;                              // rows of the padded du (8 zero rows first)
-    static constexpr int X = 0;                                  // float [L0][2]
-    static constexpr int DV = 1280;                              // float [S][64]
-    static constexpr int DVB = DV + CS * CH * 4;                 // bf16 [S][LDV]   dv, rows j
-    static constexpr int DVT = DVB + CS * LDV * 2;               // bf16 [64][LDV]  dv transposed, rows m
-    static constexpr int H3T = DVT + CH * LDV * 2;               // bf16 [32][LDV]  h3 at the symbols, rows c
-    static constexpr int M1T = H3T + CC * LDV * 2;               // bf16 [32][LDV]  M1 transposed, rows c
-    static constexpr int DH = M1T + CC * LDV * 2;                // float [L1][32]  gradient of the layer output
-    static constexpr int DUP = DH + L1 * CC * 4;                 // bf16 [NDU][32]  du from row 8 on
-    static constexpr int DUT = DUP + NDU * CC * 2;               // bf16 [32][LDT]  du transposed
-    static constexpr int HT0 = DUT + CC * LDT * 2;               // bf16 [32][LDH]  layer input transposed
-    static constexpr int HT1 = HT0 + CC * LDH * 2;               // bf16 [32][LDH]  the same from position 1 on
-    static constexpr int RED = HT1 + CC * LDH * 2;               // float [8][32]   bias partials
-    static constexpr int TOTAL = RED + 8 * CC * 4;
-};
-static_assert(BwdSmem::TOTAL <= 113 * 1024, "two backward CTAs per SM");
-static_assert(L1 + 8 <= BwdSmem::LDT && L1 + 16 <= BwdSmem::NDU && L0 <= BwdSmem::LDH,
-              "padded tiles cover the largest layer");
-
-// one m16n8k16 BF16 product: D += A * B with A row-major (row stride lda elements,
-// even) and B given by its transpose Bt, row-major (row stride ldb, even)
-__device__ __forceinline__ void mma_tile(float (&d)[4], const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *Bt,
-                                         int ldb, int g, int tq)
-{
-    uint32_t a[4];
-    a[0] = *reinterpret_cast<const uint32_t *>(A + lda * g + 2 * tq);
-    a[1] = *reinterpret_cast<const uint32_t *>(A + lda * (g + 8) + 2 * tq);
-    a[2] = *reinterpret_cast<const uint32_t *>(A + lda * g + 2 * tq + 8);
-    a[3] = *reinterpret_cast<const uint32_t *>(A + lda * (g + 8) + 2 * tq + 8);
-    mma_bf16(d, a, *reinterpret_cast<const uint32_t *>(Bt + ldb * g + 2 * tq),
-             *reinterpret_cast<const uint32_t *>(Bt + ldb * g + 2 * tq + 8));
-}
-
-// Backward pass of one segment per CTA (256 threads): per-segment partial gradient
-// gpart[s][NPRM].  The contractions run on the tensor cores with BF16 operands and
-// FP32 accumulation (mma.sync m16n8k16): the MLP's dM1 and the gradient at the
-// layer-3 output; per convolution layer 3 and 2 the weight gradient (K = the
-// positions) and the input gradient (the forward's convolution over the zero-padded
-// du with the tap-flipped, transposed weights wdT).  Elementwise steps (GELU
-// derivatives, dM2, biases) and the 2-channel layer 1 stay in FP32.
-__global__ void __launch_bounds__(256)
-    k_cnn_bwd(const float *__restrict__ prm, const __nv_bfloat16 *__restrict__ wdT, const float2 *__restrict__ y,
-              const long long *__restrict__ seg_start, const float *__restrict__ tgt, CnnSave sv, float norm,
-              float *__restrict__ gpart)
-{
-    extern __shared__ __align__(16) unsigned char sm[];
-    float *xs = reinterpret_cast<float *>(sm + BwdSmem::X);
-    float *dv = reinterpret_cast<float *>(sm + BwdSmem::DV);
-    __nv_bfloat16 *dvb = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::DVB);
-    __nv_bfloat16 *dvt = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::DVT);
-    __nv_bfloat16 *h3t = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::H3T);
-    __nv_bfloat16 *m1t = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::M1T);
-    float *dh = reinterpret_cast<float *>(sm + BwdSmem::DH);
-    __nv_bfloat16 *dup = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::DUP);
-    __nv_bfloat16 *dut = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::DUT);
-    __nv_bfloat16 *ht0 = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::HT0);
-    __nv_bfloat16 *ht1 = reinterpret_cast<__nv_bfloat16 *>(sm + BwdSmem::HT1);
-    float *red = reinterpret_cast<float *>(sm + BwdSmem::RED);
-    constexpr int LDV = BwdSmem::LDV, LDT = BwdSmem::LDT, LDH = BwdSmem::LDH, NDU = BwdSmem::NDU;
-    const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, tq = lane & 3;
-    const int s = blockIdx.x;
-    const __nv_bfloat16 bz = __float2bfloat16(0.f);
-    float *G = gpart + (size_t)s * NPRM;
-    const long long st = seg_start[s];
-    for (int i = tid; i < L0; i += nth) {
-        float2 v = y[st + i];
-        xs[2 * i] = v.x;
-        xs[2 * i + 1] = v.y;
-    }
-    const __nv_bfloat16 *h3 = sv.h3 + (size_t)s * L3 * CC;
-    // ---- MLP head: dv = (dout . M2) gelu'(v) in FP32, bf16 copies for the products
-    for (int i = tid; i < CS * CH; i += nth) {
-        int j = i / CH, m = i - CH * j;
-        float o0 = sv.out[((size_t)s * CS + j) * 2], o1 = sv.out[((size_t)s * CS + j) * 2 + 1];
-        float d0 = 2.f * (o0 - tgt[((size_t)s * CS + j) * 2]) * norm;
-        float d1 = 2.f * (o1 - tgt[((size_t)s * CS + j) * 2 + 1]) * norm;
-        float vv = sv.v[((size_t)s * CS + j) * CH + m];
-        float dz = d0 * prm[OM2 + m] + d1 * prm[OM2 + CH + m];
-        float d = dz * gelu_df(vv);
-        dv[i] = d;
-        dvb[j * LDV + m] = __float2bfloat16(d);
-        dvt[m * LDV + j] = __float2bfloat16(d);
-    }
-    for (int i = tid; i < CC * CS; i += nth) {   // h3 at the symbol positions, transposed
-        int c = i / CS, j = i - CS * c;
-        h3t[c * LDV + j] = h3[(2 * j) * CC + c];
-    }
-    for (int i = tid; i < CC * CH; i += nth) {   // M1 transposed, bf16
-        int c = i / CH, m = i - CH * c;
-        m1t[c * LDV + m] = __float2bfloat16(prm[OM1 + m * CC + c]);
-    }
-    for (int i = tid; i < L3 * CC; i += nth)     // odd positions of h3 feed nothing
-        if ((i >> 5) & 1) dh[i] = 0.f;
-    __syncthreads();
-    // dM2, dc2 (z recomputed from v) and dc1 in FP32
-    for (int i = tid; i < 2 * CH + 2 + CH; i += nth) {
-        float a = 0.f;
-        if (i < 2 * CH + 2) {
-            const int oc = i < 2 * CH ? i / CH : i - 2 * CH;
-            for (int j = 0; j < CS; j++) {
-                float o = sv.out[((size_t)s * CS + j) * 2 + oc];
-                float d = 2.f * (o - tgt[((size_t)s * CS + j) * 2 + oc]) * norm;
-                a += (i < 2 * CH) ? d * gelu_f(sv.v[((size_t)s * CS + j) * CH + (i % CH)]) : d;
-            }
-            G[OM2 + i] = a;   // OC2 follows OM2 contiguously
-        } else {
-            const int m = i - (2 * CH + 2);
-            for (int j = 0; j < CS; j++) a += dv[j * CH + m];
-            G[OC1 + m] = a;
-        }
-    }
-    // tiles 0..15: dM1[m][c] = sum_j dv[j][m] h3[2j][c]   (M = 64 m, N = 32 c, K = 64 j)
-    // tiles 16..31: dh3[2j][c] = sum_m M1[m][c] dv[j][m]   (M = 64 j, N = 32 c, K = 64 m)
-    for (int tile = warp; tile < 32; tile += 8) {
-        const bool second = tile >= 16;
-        const int mt = (tile & 15) >> 2, nt = tile & 3;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        const __nv_bfloat16 *A = (second ? dvb : dvt) + LDV * 16 * mt;
-        const __nv_bfloat16 *Bt = (second ? m1t : h3t) + LDV * 8 * nt;
+    for (int i = tid; i < CS * CH / 2; i += kTrThreads) {   // ---- dv = (dout . M2) gelu'(v)
+        const int j = i >> 5, m = 2 * (i & 31);
+        const float g0 = dout[2 * j], g1 = dout[2 * j + 1];
+        float d[2];
 #pragma unroll
-        for (int k0 = 0; k0 < 64; k0 += 16) mma_tile(acc, A + k0, LDV, Bt + k0, LDV, g, tq);
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const int r = 16 * mt + g + 8 * (i >> 1), c = 8 * nt + 2 * tq + (i & 1);
-            if (second) dh[(2 * r) * CC + c] = acc[i];
-            else G[OM1 + r * CC + c] = acc[i];
+        for (int q = 0; q < 2; q++) {
+            const float dzv = g0 * m2[m + q] + g1 * m2[CH + m + q];
+            d[q] = dzv * dz[j * kZP + m + q];
+            dz[j * kZP + m + q] = d[q];
         }
+        *reinterpret_cast<uint32_t *>(sm + TrainSmem::DVB + row128_off(j, m >> 3) + 2 * (m & 7)) = bf2(d[0], d[1]);
     }
     __syncthreads();
-    // ---- convolution layers 3 and 2 on the tensor cores, layer 1 in FP32
-    for (int l = 3; l >= 1; l--) {
-        const int Lout = (l == 3) ? L3 : (l == 2) ? L2 : L1;
-        const int Lin = Lout + 8;
-        const float *U = (l == 3) ? sv.u3 + (size_t)s * L3 * CC : (l == 2) ? sv.u2 + (size_t)s * L2 * CC
-                                                                          : sv.u1 + (size_t)s * L1 * CC;
-        const int OW = (l == 3) ? OW3 : (l == 2) ? OW2 : OW1, OB = (l == 3) ? OB3 : (l == 2) ? OB2 : OB1;
-        // du = dh gelu'(u) for positions p < Lout (zero beyond): bias partials in FP32,
-        // bf16 copies padded (dup: row p + 8) and transposed (dut); layer 1 in place
-        float bsum = 0.f;
-        for (int i = tid; i < LDT * CC; i += nth) {   // thread tid always holds channel tid & 31
-            const int p = i >> 5, o = i & 31;
-            const float d = p < Lout ? dh[p * CC + o] * gelu_df(U[p * CC + o]) : 0.f;
-            bsum += d;
-            if (l > 1) {
-                dut[o * LDT + p] = __float2bfloat16(d);
-                if (p + 8 < NDU) dup[(p + 8) * CC + o] = __float2bfloat16(d);
-            } else if (p < Lout) {
-                dh[p * CC + o] = d;
-            }
-        }
-        red[warp * CC + lane] = bsum;
-        if (l > 1) {
-            for (int i = tid; i < 8 * CC; i += nth) dup[i] = bz;
-            // layer input (h2 for layer 3, h1 for layer 2) transposed, zero beyond Lin
-            const __nv_bfloat16 *src = (l == 3) ? sv.h2 + (size_t)s * L2 * CC : sv.h1 + (size_t)s * L1 * CC;
-            for (int i = tid; i < CC * LDH; i += nth) {
-                const int c = i / LDH, q = i - LDH * c;
-                ht0[i] = q < Lin ? src[q * CC + c] : bz;
-                ht1[i] = q + 1 < Lin ? src[(q + 1) * CC + c] : bz;
-            }
-        }
-        __syncthreads();
-        if (tid < CC) {
+    // ---- tasks 0..6: dM2, dc2, dc1 in FP32 (one sum over the symbols per lane);
+    // 7..22: du3[j][c] = gelu'(u3) sum_m dv[j][m] M1[m][c] (16 symbols x 8 channels);
+    // 23..38: dM1[m][c] = sum_j dv[j][m] h3[j][c] (16 units x 8 channels)
+    for (int task = warp; task < 39; task += kTrWarps) {
+        if (task < 7) {
+            const int i = 32 * task + lane;   // dM2 [2][64], dc2 [2] (contiguous in G), then dc1 from 160 on
             float a = 0.f;
-            for (int w = 0; w < 8; w++) a += red[w * CC + tid];
-            G[OB + tid] = a;
+            if (i < 2 * CH) {
+                const int oc = i >> 6, m = i & 63;
+#pragma unroll 8
+                for (int j = 0; j < CS; j++) a = fmaf(dout[2 * j + oc], zs[j * kZP + m], a);
+                G[OM2 + i] = a;
+            } else if (i < 2 * CH + 2) {
+                for (int j = 0; j < CS; j++) a += dout[2 * j + i - 2 * CH];
+                G[OM2 + i] = a;
+            } else if (i >= 160) {
+#pragma unroll 8
+                for (int j = 0; j < CS; j++) a += dz[j * kZP + i - 160];
+                G[OC1 + i - 160] = a;
+            }
+            continue;
         }
-        if (l > 1) {
-            // weight gradient dW[o][t][c] = sum_p du[p][o] h_in[p + t][c]: M = 32 (o),
-            // N = 288 (t, c), K = 144 (p; du is zero from Lout on)
-            for (int tile = warp; tile < 2 * 36; tile += 8) {
-                const int mt = tile / 36, nt = tile - 36 * mt, t = nt >> 2, c0 = 8 * (nt & 3);
-                // 32-bit loads need an even start: odd taps read the copy shifted by one
-                const __nv_bfloat16 *Bt = ((t & 1) ? ht1 + (t - 1) : ht0 + t) + LDH * c0;
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 3
-                for (int k0 = 0; k0 < 144; k0 += 16) mma_tile(acc, dut + LDT * 16 * mt + k0, LDT, Bt + k0, LDH, g, tq);
+        const bool in = task < 23;
+        const int mt = (in ? task - 7 : task - 23) >> 2, nt = (in ? task - 7 : task - 23) & 3;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    const int o = 16 * mt + g + 8 * (i >> 1), n = 8 * nt + 2 * tq + (i & 1);
-                    G[OW + o * KW + n] = acc[i];
-                }
+        for (int ks = 0; ks < 4; ks++) {
+            uint32_t a[4], b[4];
+            if (in) {   // A: dv rows (symbols); B: M1 with the units along K
+                ldsm4(a, sDV + row128_off(16 * mt + (lane & 15), 2 * ks + (lane >> 4)));
+                ldsm4_t(b, sM1B + row_off(16 * ks + (lane & 15), nt));
+            } else {    // A: dv with the symbols along K; B: h3 with the symbols along K
+                ldsm4_t(a, sDV + row128_off(16 * ks + (lane & 7) + ((lane >> 4) << 3), 2 * mt + ((lane >> 3) & 1)));
+                ldsm4_t(b, sH3 + row_off(16 * ks + (lane & 15), nt));
             }
-            // input gradient dh_in[q][c] = sum_t sum_o W[o][t][c] du[q - t][o]: row q of the
-            // A operand is the padded du from row q on (tap t' = 8 - t at row q + t'); dh
-            // (this layer's output gradient) was consumed above, so it takes dh_in
-            const __nv_bfloat16 *Wt = wdT + (size_t)(l == 3 ? 1 : 0) * CC * KW;
-            for (int tile = warp; tile < 9 * 4; tile += 8) {
-                const int mt = tile >> 2, nt = tile & 3;
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-                for (int k0 = 0; k0 < KW; k0 += 16) {
-                    uint32_t a[4];
-                    const __nv_bfloat16 *ar = dup + CC * (16 * mt + g) + k0 + 2 * tq;
-                    a[0] = *reinterpret_cast<const uint32_t *>(ar);
-                    a[1] = *reinterpret_cast<const uint32_t *>(ar + CC * 8);
-                    a[2] = *reinterpret_cast<const uint32_t *>(ar + 8);
-                    a[3] = *reinterpret_cast<const uint32_t *>(ar + CC * 8 + 8);
-                    const __nv_bfloat16 *br = Wt + KW * (8 * nt + g) + k0 + 2 * tq;
-                    mma_bf16(acc, a, __ldg(reinterpret_cast<const unsigned int *>(br)),
-                             __ldg(reinterpret_cast<const unsigned int *>(br + 8)));
-                }
+            mma_bf16(acc, a, b[0], b[1]);
+        }
+        if (in) {
+            float cs[2] = {0.f, 0.f};
 #pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    const int q = 16 * mt + g + 8 * (i >> 1), c = 8 * nt + 2 * tq + (i & 1);
-                    if (q < Lin) dh[q * CC + c] = acc[i];
-                }
+            for (int h = 0; h < 2; h++) {
+                const int j = 16 * mt + g + 8 * h, c = 8 * nt + 2 * tq;
+                const float2 f = *reinterpret_cast<const float2 *>(d3 + j * CC + c);
+                const float v0 = acc[2 * h] * f.x, v1 = acc[2 * h + 1] * f.y;
+                *reinterpret_cast<uint32_t *>(sm + TrainSmem::DU3 + row_off(8 + 2 * j, nt) + 4 * tq) = bf2(v0, v1);
+                cs[0] += v0;
+                cs[1] += v1;
             }
+#pragma unroll
+            for (int q = 0; q < 2; q++)
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) cs[q] += __shfl_xor_sync(0xffffffffu, cs[q], o);
+            if (g == 0) *reinterpret_cast<float2 *>(red + mt * CC + 8 * nt + 2 * tq) = make_float2(cs[0], cs[1]);
         } else {
-            // layer 1 (2 input channels) in FP32: dW1[o][t][c] = sum_p du1[p][o] x[p + t][c]
-            for (int i = tid; i < CC * CK * 2; i += nth) {
-                int o = i / (CK * 2), r = i - o * CK * 2, t = r / 2, c = r - 2 * t;
-                float a = 0.f;
-                for (int p = 0; p < Lout; p++) a = fmaf(dh[p * CC + o], xs[(p + t) * 2 + c], a);
-                G[OW + i] = a;
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+                *reinterpret_cast<float2 *>(G + OM1 + (16 * mt + g + 8 * h) * CC + 8 * nt + 2 * tq) =
+                    make_float2(acc[2 * h], acc[2 * h + 1]);
+        }
+    }
+    __syncthreads();
+    // ---- convolution layers 3 and 2: per warp one unit of the weight gradient
+    // dW[o][t][c] = sum_p du[p][o] h_in[p + t][c] (16 output channels, one tap, 32 input
+    // channels) and one of the input gradient dh_in[q][c] = sum_{t, o} W[o][t][c] du[q - t][o]
+    // (16 positions, 16 channels; row q of the padded du from row q on, tap 8 - t at row
+    // q + 8 - t), which times gelu' is the du of the layer below
+#pragma unroll
+    for (int l = 3; l >= 2; l--) {
+        const uint32_t sDU = smem_u32(sm + (l == 3 ? TrainSmem::DU3 : TrainSmem::DU2));
+        const uint32_t sHin = l == 3 ? sH2 : sH1, sW = l == 3 ? sW3 : sW2;
+        const int OW = l == 3 ? OW3 : OW2, OB = l == 3 ? OB3 : OB2;
+        const int nred = l == 3 ? 4 : 9;   // bias partials left by the step before
+        if (warp == kTrWarps - 1) {
+            float a = 0.f;
+            for (int w = 0; w < nred; w++) a += red[w * CC + lane];
+            G[OB + lane] = a;
+        }
+        {
+            const int t = tile9;
+            float acc[4][4];
+#pragma unroll
+            for (int n = 0; n < 4; n++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) acc[n][i] = 0.f;
+            // positions 16 ks ..; layer 3's du is zero from position 128 on
+#pragma unroll
+            for (int ks = 0; ks < (l == 3 ? 8 : 9); ks++) {
+                uint32_t a[4], b[2][4];
+                ldsm4_t(a, sDU + row_off(8 + 16 * ks + (lane & 7) + ((lane >> 4) << 3), 2 * half2 + ((lane >> 3) & 1)));
+#pragma unroll
+                for (int p = 0; p < 2; p++) ldsm4_t(b[p], sHin + row_off(16 * ks + (lane & 15) + t, 2 * p + (lane >> 4)));
+#pragma unroll
+                for (int p = 0; p < 2; p++) {
+                    mma_bf16(acc[2 * p], a, b[p][0], b[p][1]);
+                    mma_bf16(acc[2 * p + 1], a, b[p][2], b[p][3]);
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < 4; n++)
+#pragma unroll
+                for (int h = 0; h < 2; h++)
+                    *reinterpret_cast<float2 *>(G + OW + (16 * half2 + g + 8 * h) * KW + t * CC + 8 * n + 2 * tq) =
+                        make_float2(acc[n][2 * h], acc[n][2 * h + 1]);
+        }
+        float acc[2][4];
+#pragma unroll
+        for (int n = 0; n < 2; n++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) acc[n][i] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KW / 16; ks++) {
+            uint32_t a[4], b[4];
+            ldsm4(a, sDU + row_off(16 * tile9 + (lane & 15) + (ks >> 1), 2 * (ks & 1) + (lane >> 4)));
+            ldsm4_t(b, sW + w_off(16 * (ks & 1) + (lane & 15), 4 * (CK - 1 - (ks >> 1)) + 2 * half2 + (lane >> 4)));
+            mma_bf16(acc[0], a, b[0], b[1]);
+            mma_bf16(acc[1], a, b[2], b[3]);
+        }
+        __syncthreads();   // the partials in red are read
+        const int Lin = l == 3 ? L2 : L1;
+        float cs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int n = 0; n < 2; n++)
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int q = 16 * tile9 + g + 8 * h, c = 16 * half2 + 8 * n + 2 * tq;
+                if (q >= Lin) continue;
+                float2 *f = reinterpret_cast<float2 *>((l == 3 ? d2 : d1) + q * CC + c);
+                const float v0 = acc[n][2 * h] * f->x, v1 = acc[n][2 * h + 1] * f->y;
+                if (l == 3)
+                    *reinterpret_cast<uint32_t *>(sm + TrainSmem::DU2 + row_off(8 + q, 2 * half2 + n) + 4 * tq) = bf2(v0, v1);
+                else
+                    *f = make_float2(v0, v1);
+                cs[2 * n] += v0;
+                cs[2 * n + 1] += v1;
+            }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) cs[q] += __shfl_xor_sync(0xffffffffu, cs[q], o);
+        if (g == 0)
+#pragma unroll
+            for (int n = 0; n < 2; n++)
+                *reinterpret_cast<float2 *>(red + tile9 * CC + 16 * half2 + 8 * n + 2 * tq) =
+                    make_float2(cs[2 * n], cs[2 * n + 1]);
+        __syncthreads();
+    }
+    // ---- layer 1 in FP32: dW1[o][t][c] = sum_p du1[p][o] x[p + t][c], eight positions per
+    // warp with an output channel per lane, then the 18 partials of each weight
+    {
+        float a[18], du[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) du[i] = d1[(8 * warp + i) * CC + lane];
+#pragma unroll
+        for (int k = 0; k < 18; k++) a[k] = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            const float4 x = xd[8 * warp + i];
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const int t = i - q;
+                if (t < 0 || t >= CK) continue;
+                a[2 * t] = fmaf(du[q], x.x, a[2 * t]);
+                a[2 * t + 1] = fmaf(du[q], x.z, a[2 * t + 1]);
             }
         }
+        float *part = reinterpret_cast<float *>(sm + TrainSmem::P1);
+#pragma unroll
+        for (int k = 0; k < 18; k++) part[warp * (18 * CC) + k * CC + lane] = a[k];
         __syncthreads();
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < kTrWarps; w++) v += part[w * (18 * CC) + tid];
+        G[OW1 + (tid & 31) * 18 + (tid >> 5)] = v;
+        if (warp == 0) {
+            float b = 0.f;
+            for (int w = 0; w < 9; w++) b += red[w * CC + lane];
+            G[OB1 + lane] = b;
+        }
     }
 }
 
-// grad[i] = sum_s gpart[s][i] (fixed order)
-__global__ void k_cnn_reduce(const float *__restrict__ gpart, int nseg, float *__restrict__ grad)
+// grad[i] = sum_s gpart[s][i] in segment order, copied to the caller's buffer (or null);
+// the last CTA sums the segments' loss parts
+constexpr int kRedThreads = 128;
+__global__ void __launch_bounds__(kRedThreads)
+    k_cnn_reduce(const float *__restrict__ gpart, const float *__restrict__ lpart, int nseg, float norm,
+                 float *__restrict__ grad, float *grad_out, float *__restrict__ loss, float *loss_out)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ float part[kRedThreads / 32];
+        float a = 0.f;
+        for (int s = threadIdx.x; s < nseg; s += kRedThreads) a += lpart[s];
+        a = warp_sum_f(a);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = a;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const float v = ((part[0] + part[1]) + (part[2] + part[3])) * norm;
+            *loss = v;
+            if (loss_out) *loss_out = v;
+        }
+        return;
+    }
+    const int i = blockIdx.x * kRedThreads + threadIdx.x;
     if (i >= NPRM) return;
     float a = 0.f;
+#pragma unroll 16
     for (int s = 0; s < nseg; s++) a += gpart[(size_t)s * NPRM + i];
     grad[i] = a;
+    if (grad_out) grad_out[i] = a;
 }
 
-// sum of the per-symbol squared errors (loss), fixed order within one CTA
-__global__ void k_cnn_loss(const float *__restrict__ out, const float *__restrict__ tgt, long long n, float norm,
-                           float *__restrict__ loss)
-{
-    __shared__ float red[256];
-    float a = 0.f;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-        float d = out[i] - tgt[i];
-        a = fmaf(d, d, a);
-    }
-    red[threadIdx.x] = a;
-    __syncthreads();
-    for (int s2 = 128; s2 > 0; s2 >>= 1) {
-        if ((int)threadIdx.x < s2) red[threadIdx.x] += red[threadIdx.x + s2];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = red[0] * norm;
-}
-
-// BF16 copy of a weight of layer 2 or 3 in the layout the backward input gradient
-// reads: wdT[layer - 2][c][(8 - t) 32 + o] = W[o][t][c]
-__device__ __forceinline__ void put_wdt(__nv_bfloat16 *wdT, int i, float w)
-{
-    const int lay = (i >= OW2 && i < OW2 + CC * KW) ? 0 : (i >= OW3 && i < OW3 + CC * KW) ? 1 : -1;
-    if (lay < 0) return;
-    const int rel = i - (lay ? OW3 : OW2), o = rel / KW, t = (rel % KW) / CC, c = rel % CC;
-    wdT[(size_t)lay * CC * KW + c * KW + (CK - 1 - t) * CC + o] = __float2bfloat16(w);
-}
-
-// Adam on the FP32 master weights; refreshes the BF16 copies
-__global__ void k_cnn_adam(float *__restrict__ prm, __nv_bfloat16 *__restrict__ prm_bf, __nv_bfloat16 *__restrict__ wdT,
+// Adam on the FP32 master weights; refreshes the BF16 copy
+__global__ void k_cnn_adam(float *__restrict__ prm, __nv_bfloat16 *__restrict__ prm_bf,
                            float *__restrict__ m, float *__restrict__ v, const float *__restrict__ grad, float lr,
                            float b1t, float b2t)
 {
@@ -557,17 +787,12 @@ __global__ void k_cnn_adam(float *__restrict__ prm, __nv_bfloat16 *__restrict__ 
     float w = prm[i] - lr * mh / (sqrtf(vh) + eps);
     prm[i] = w;
     prm_bf[i] = __float2bfloat16(w);
-    put_wdt(wdT, i, w);
 }
 
-__global__ void k_cnn_tobf(const float *__restrict__ prm, __nv_bfloat16 *__restrict__ prm_bf,
-                           __nv_bfloat16 *__restrict__ wdT)
+__global__ void k_cnn_tobf(const float *__restrict__ prm, __nv_bfloat16 *__restrict__ prm_bf)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < NPRM) {
-        prm_bf[i] = __float2bfloat16(prm[i]);
-        put_wdt(wdT, i, prm[i]);
-    }
+    if (i < NPRM) prm_bf[i] = __float2bfloat16(prm[i]);
 }
 
 // ====================================================================
@@ -1046,11 +1271,9 @@ cudaError_t launch_cnn_decide(const float *prm, const float2 *y, long long seg_b
 using namespace rxk;
 
 struct rx_cnn {
-    int max_seg;
-    float *prm, *grad, *m, *v, *gpart, *loss;
+    int max_seg, nsm;
+    float *prm, *grad, *m, *v, *gpart, *lpart, *loss;   // gpart, lpart: gradient and loss of each segment
     __nv_bfloat16 *prm_bf;
-    __nv_bfloat16 *wdT;   // layer 2 and 3 weights for the backward input gradient
-    CnnSave sv;
     long long step;
 };
 
@@ -1061,8 +1284,7 @@ int rx_cnn_nparams(void) { return NPRM; }
 void rx_cnn_destroy(rx_cnn *c)
 {
     if (!c) return;
-    void *p[] = {c->prm, c->grad, c->m, c->v, c->gpart, c->loss, c->prm_bf, c->wdT, c->sv.u1, c->sv.u2, c->sv.u3,
-                 c->sv.h1, c->sv.h2, c->sv.h3, c->sv.v, c->sv.out};
+    void *p[] = {c->prm, c->grad, c->m, c->v, c->gpart, c->lpart, c->loss, c->prm_bf};
     for (void *q : p)
         if (q) cudaFree(q);
     free(c);
@@ -1084,17 +1306,9 @@ rx_status rx_cnn_create(int max_seg, rx_cnn **out)
               {(void **)&c->m, NPRM * 4},
               {(void **)&c->v, NPRM * 4},
               {(void **)&c->gpart, S * NPRM * 4},
+              {(void **)&c->lpart, S * 4},
               {(void **)&c->loss, 16},
-              {(void **)&c->prm_bf, NPRM * 2 + 64},
-              {(void **)&c->wdT, 2 * CC * KW * 2},
-              {(void **)&c->sv.u1, S * L1 * CC * 4},
-              {(void **)&c->sv.u2, S * L2 * CC * 4},
-              {(void **)&c->sv.u3, S * L3 * CC * 4},
-              {(void **)&c->sv.h1, S * L1 * CC * 2},
-              {(void **)&c->sv.h2, S * L2 * CC * 2},
-              {(void **)&c->sv.h3, S * L3 * CC * 2},
-              {(void **)&c->sv.v, S * CS * CH * 4},
-              {(void **)&c->sv.out, S * CS * 2 * 4}};
+              {(void **)&c->prm_bf, NPRM * 2 + 64}};
     for (auto &a : al) {
         if (cudaMalloc(a.p, a.b) != cudaSuccess || cudaMemset(*a.p, 0, a.b) != cudaSuccess) {
             cudaGetLastError();
@@ -1102,8 +1316,15 @@ rx_status rx_cnn_create(int max_seg, rx_cnn **out)
             return RX_ENOMEM;
         }
     }
-    cudaFuncSetAttribute(k_cnn_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem::TOTAL);
-    cudaFuncSetAttribute(k_cnn_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem::TOTAL);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(k_cnn_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem::TOTAL) != cudaSuccess ||
+        cudaFuncSetAttribute(k_cnn_train, cudaFuncAttributeMaxDynamicSharedMemorySize, TrainSmem::TOTAL) != cudaSuccess) {
+        cudaGetLastError();
+        rx_cnn_destroy(c);
+        return RX_ECUDA;
+    }
     *out = c;
     return RX_OK;
 }
@@ -1115,7 +1336,7 @@ rx_status rx_cnn_set_params(rx_cnn *c, const float *host, int n)
     cudaMemset(c->m, 0, NPRM * 4);
     cudaMemset(c->v, 0, NPRM * 4);
     c->step = 0;
-    k_cnn_tobf<<<(NPRM + 255) / 256, 256>>>(c->prm, c->prm_bf, c->wdT);
+    k_cnn_tobf<<<(NPRM + 255) / 256, 256>>>(c->prm, c->prm_bf);
     if (cudaDeviceSynchronize() != cudaSuccess) return RX_ECUDA;
     return RX_OK;
 }
@@ -1130,11 +1351,9 @@ rx_status rx_cnn_get_params(rx_cnn *c, float *host, int n)
 rx_status rx_cnn_forward(rx_cnn *c, const float *y, const int64_t *seg_start, int nseg, float *out, void *stream)
 {
     if (!c || !y || !seg_start || !out || nseg <= 0) return RX_EINVAL;
-    CnnSave sv;
-    memset(&sv, 0, sizeof sv);
-    k_cnn_fwd<<<nseg, kCnnThreads, FwdSmem::TOTAL, (cudaStream_t)stream>>>(
-        c->prm, c->prm_bf, (const float2 *)y, (const long long *)seg_start, 0, 0, out, sv, nullptr, nullptr, nullptr,
-        nullptr, 0, 1.f, 4);
+    const int grid = nseg < kFwPerSm * c->nsm ? nseg : kFwPerSm * c->nsm;   // persistent CTAs
+    k_cnn_fwd<<<grid, kFwThreads, FwdSmem::TOTAL, (cudaStream_t)stream>>>(c->prm, c->prm_bf, (const float2 *)y,
+                                                                          (const long long *)seg_start, nseg, out);
     return cudaGetLastError() == cudaSuccess ? RX_OK : RX_ECUDA;
 }
 
@@ -1144,15 +1363,14 @@ rx_status rx_cnn_grad(rx_cnn *c, const float *y, const int64_t *seg_start, const
     if (!c || !y || !seg_start || !tgt || nseg <= 0 || nseg > c->max_seg) return RX_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     float norm = 1.f / ((float)nseg * CS);
-    k_cnn_fwd<<<nseg, kCnnThreads, FwdSmem::TOTAL, st>>>(c->prm, c->prm_bf, (const float2 *)y,
-                                                         (const long long *)seg_start, 0, 0, nullptr, c->sv, nullptr,
-                                                         nullptr, nullptr, nullptr, 0, 1.f, 4);
-    k_cnn_bwd<<<nseg, 256, BwdSmem::TOTAL, st>>>(c->prm, c->wdT, (const float2 *)y, (const long long *)seg_start,
-                                                 tgt, c->sv, norm, c->gpart);
-    k_cnn_reduce<<<(NPRM + 255) / 256, 256, 0, st>>>(c->gpart, nseg, c->grad);
-    k_cnn_loss<<<1, 256, 0, st>>>(c->sv.out, tgt, (long long)nseg * CS * 2, norm, c->loss);
-    if (grad_out) cudaMemcpyAsync(grad_out, c->grad, NPRM * 4, cudaMemcpyDeviceToDevice, st);
-    if (loss_out) cudaMemcpyAsync(loss_out, c->loss, 4, cudaMemcpyDeviceToDevice, st);
+    k_cnn_train<<<nseg, kTrThreads, TrainSmem::TOTAL, st>>>(c->prm, c->prm_bf, (const float2 *)y,
+                                                           (const long long *)seg_start, tgt, norm, c->gpart, c->lpart);
+    // the caller's buffers are written by the reduction itself where they are aligned
+    float *go = ((uintptr_t)grad_out & 3) ? nullptr : grad_out, *lo = ((uintptr_t)loss_out & 3) ? nullptr : loss_out;
+    k_cnn_reduce<<<(NPRM + kRedThreads - 1) / kRedThreads + 1, kRedThreads, 0, st>>>(c->gpart, c->lpart, nseg, norm,
+                                                                                   c->grad, go, c->loss, lo);
+    if (grad_out && !go) cudaMemcpyAsync(grad_out, c->grad, NPRM * 4, cudaMemcpyDeviceToDevice, st);
+    if (loss_out && !lo) cudaMemcpyAsync(loss_out, c->loss, 4, cudaMemcpyDeviceToDevice, st);
     return cudaGetLastError() == cudaSuccess ? RX_OK : RX_ECUDA;
 }
 
@@ -1161,7 +1379,7 @@ rx_status rx_cnn_adam_step(rx_cnn *c, float lr, void *stream)
     if (!c || !(lr > 0)) return RX_EINVAL;
     c->step++;
     float b1t = powf(0.9f, (float)c->step), b2t = powf(0.999f, (float)c->step);
-    k_cnn_adam<<<(NPRM + 255) / 256, 256, 0, (cudaStream_t)stream>>>(c->prm, c->prm_bf, c->wdT, c->m, c->v, c->grad,
+    k_cnn_adam<<<(NPRM + 255) / 256, 256, 0, (cudaStream_t)stream>>>(c->prm, c->prm_bf, c->m, c->v, c->grad,
                                                                      lr, b1t, b2t);
     return cudaGetLastError() == cudaSuccess ? RX_OK : RX_ECUDA;
 }
