@@ -7,22 +7,18 @@
 // a Hankel matrix), times a K x 32 real Toeplitz matrix of the taps (complex
 // split to real: re / im output of each symbol).  Tiles of 128 rows (2048
 // symbols) run through M = 128, N = 32 tcgen05.mma in BF16, FP16 or FP8-E4M3
-// with FP32 accumulation in tensor memory.  Persistent CTAs (two per SM), per
-// tile:
-//   - a bulk copy (cp.async.bulk) stages the next tile's 4.1 k complex FP32
-//     inputs while this tile is processed (two stage buffers, one mbarrier each);
-//   - the threads convert the staged inputs into the K-major no-swizzle operand
-//     layout (core matrices of 8 rows x 16 bytes), lanes spread over 8 rows x 4
-//     K-columns with a rotated read order so that neither the shared-memory reads
-//     nor the 16-byte stores conflict; FP8 first takes a power-of-two scale per
-//     block of rows_per_scale rows from the block's largest input;
-//   - one thread issues the MMAs and commits them to an mbarrier;
-//   - each warp reads its 32 accumulator lanes (tcgen05.ld 32x32b), rescales,
-//     transposes through shared memory and stores 512 contiguous bytes per
-//     instruction.
+// with FP32 accumulation in tensor memory.  Persistent CTAs, per tile:
+//   - the threads load the tile's 4.1 k complex FP32 inputs into registers, coalesced and
+//     once, convert them and store them into the K-major no-swizzle operand layout (core
+//     matrices of 8 rows x 16 bytes); FP8 first takes a power-of-two scale per block of
+//     rows_per_scale rows from the block's largest input;
+//   - one thread issues the MMAs and commits them to an mbarrier, while the next tile's
+//     loads are in flight;
+//   - each warp reads its 32 accumulator lanes (tcgen05.ld 32x32b), rescales and stores
+//     them.
 // The taps' Toeplitz operand is built once per CTA.  Every wait is bounded: on
-// time-out the kernel records RX_ETIMEOUT, waits (bounded) for its own copies and
-// MMAs, frees its tensor memory and returns.
+// time-out the kernel records RX_ETIMEOUT, waits (bounded) for its own MMAs, frees its
+// tensor memory and returns.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -36,43 +32,20 @@ namespace {
 constexpr int kRowSyms = 16;                       // symbols per GEMM row
 constexpr int kTileRows = 128;                     // M of one MMA
 constexpr int kN = 2 * kRowSyms;                   // real outputs per row
-constexpr int kKP = 128;                           // padded K (2 * (30 + NT) <= 122)
-constexpr int kThreads = 256;            // 8 warps: (row quarter, K / column half)
-constexpr int kStage = 2 * kRowSyms * kTileRows + 64;   // staged complex inputs per tile
-constexpr int kOutPitch = kN + 4;                  // floats per row of the output transpose
 constexpr uint32_t kTmemCols = 32;
-// dynamic shared memory: A | B | stage[2] | barriers and scratch
-constexpr int kOffA = 0;
-constexpr int kOffB = kOffA + kTileRows * kKP * 2;   // 32 KB (16-bit A; FP8 uses half)
-constexpr int kOffStage = kOffB + kN * kKP * 2;      // + 8 KB
-constexpr int kStageBytes = kStage * 8;
-constexpr int kOffMisc = kOffStage + 2 * kStageBytes;
-// misc: 3 mbarriers + TMEM slot (64 B) | per-row maxima (128 floats) | scale exponents (128 ints)
-constexpr int kOffRmax = kOffMisc + 64;                 // float [2 halves][128 rows]
-constexpr int kOffExp = kOffRmax + 2 * kTileRows * 4;
-constexpr int kSmem = kOffExp + kTileRows * 4;
-static_assert(kTileRows * kOutPitch * 4 <= kStageBytes, "output transpose fits a stage buffer");
-static_assert(kSmem <= 113 * 1024, "two CTAs per SM");
 
 template <int PREC> struct Fmt;
 template <> struct Fmt<RX_FIR_BF16> {
-    static constexpr int esize = 2;
     static constexpr uint32_t code = 1;   // kind::f16, BF16
 };
 template <> struct Fmt<RX_FIR_FP16> {
-    static constexpr int esize = 2;
     static constexpr uint32_t code = 0;   // kind::f16, F16
 };
-template <> struct Fmt<RX_FIR_FP8> {
-    static constexpr int esize = 1;
-    static constexpr uint32_t code = 0;   // kind::f8f6f4, E4M3
-};
-
-// 8 (16-bit) or 16 (FP8) consecutive K elements -> one 16-byte core-matrix row
+// 8 consecutive K elements -> one 16-byte core-matrix row
 template <int PREC>
-__device__ __forceinline__ uint4 pack16(const float *v, float s);
+__device__ __forceinline__ uint4 pack16(const float *v);
 template <>
-__device__ __forceinline__ uint4 pack16<RX_FIR_BF16>(const float *v, float)
+__device__ __forceinline__ uint4 pack16<RX_FIR_BF16>(const float *v)
 {
     uint32_t w[4];
 #pragma unroll
@@ -83,7 +56,7 @@ __device__ __forceinline__ uint4 pack16<RX_FIR_BF16>(const float *v, float)
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 template <>
-__device__ __forceinline__ uint4 pack16<RX_FIR_FP16>(const float *v, float)
+__device__ __forceinline__ uint4 pack16<RX_FIR_FP16>(const float *v)
 {
     uint32_t w[4];
 #pragma unroll
@@ -93,20 +66,6 @@ __device__ __forceinline__ uint4 pack16<RX_FIR_FP16>(const float *v, float)
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
-template <>
-__device__ __forceinline__ uint4 pack16<RX_FIR_FP8>(const float *v, float s)
-{
-    uint32_t w[4];
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(v[4 * i] * s, v[4 * i + 1] * s), __NV_SATFINITE, __NV_E4M3);
-        uint32_t hi =
-            __nv_cvt_float2_to_fp8x2(make_float2(v[4 * i + 2] * s, v[4 * i + 3] * s), __NV_SATFINITE, __NV_E4M3);
-        w[i] = (lo & 0xFFFFu) | (hi << 16);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 // power-of-two scale that brings the largest magnitude m to at most 448 (E4M3 max)
 __device__ __forceinline__ int fp8_exp(float m)
 {
@@ -116,225 +75,180 @@ __device__ __forceinline__ int fp8_exp(float m)
     return min(max(e - 1, -60), 60);
 }
 
-template <int PREC>
-__global__ void __launch_bounds__(kThreads, 2)
-    k_fir_tc(const float2 *__restrict__ Y, long long ybase, long long k_lo, int nrows,
-             const float2 *__restrict__ taps, int ntaps, int rows_per_scale, float2 *__restrict__ z, int *err)
+// FP8 form.  Output row r (symbols k = k_lo + 16 (r0 + r) + j, j < 16) reads the samples
+// 32 r .. 32 r + 30 + NT - 1 of the tile, counted from stream sample 2 (k_lo + 16 r0) - TH:
+// K elements 0..63 are block row r (32 samples), 64..127 the start of block row r + 1, zero
+// from sample 30 + NT on.  A scale belongs to rows_per_scale consecutive rows and follows
+// from the largest input any of them reads (the first samples of the next block's first row
+// included), so the two halves of a row are stored apart: a sample is converted with its own
+// block's scale into the first half of row r and with row r - 1's scale into the second half
+// of that row; the two conversions differ at the first row of a block only.  Lanes hold
+// consecutive samples of a block row: loads are coalesced, a row's maximum is one warp
+// reduction of the magnitudes' bit patterns, and planes 16 bytes apart modulo 128 take the
+// 2-byte stores without conflicts.  Every input is read once, into registers; the next
+// tile's loads are in flight while this tile's MMAs and stores run.
+// 777 x 1024 symbols, scale block 1024: @F8US@ us; 28.7 us when each row gathered its 122
+// K elements from a staged copy twice (once for the maxima) through a rotated read order.
+// Three CTAs per SM: the tile's chain (maxima, scales, conversion, MMA, store) is latency
+// bound.
+constexpr int kT8Planes = 8;                         // 128 K elements, 16 per 16-byte core row
+constexpr int kT8Plane = kTileRows * 16 + 16;        // plane pitch
+constexpr int kT8BPlane = kN * 16;
+constexpr int kT8OffB = kT8Planes * kT8Plane;
+constexpr int kT8OffW = kT8OffB + kT8Planes * kT8BPlane;      // the taps (32 complex)
+constexpr int kT8OffMax = kT8OffW + 32 * 8;                   // row maxima [129], halo maxima [129] (bit patterns)
+constexpr int kT8OffExp = kT8OffMax + 2 * (kTileRows + 1) * 4;   // scale exponents [<= 128]
+constexpr int kT8OffBar = (kT8OffExp + kTileRows * 4 + 7) & ~7;
+constexpr int kT8Smem = kT8OffBar + 16;
+constexpr int kT8Threads = 256, kT8Warps = kT8Threads / 32, kT8PerSm = 3;
+constexpr int kT8Iter = (kTileRows + 1 + kT8Warps - 1) / kT8Warps;   // block rows per warp
+static_assert(kT8Plane % 16 == 0 && kT8OffB % 16 == 0 && kT8OffW % 8 == 0, "16-byte aligned operands");
+static_assert(kT8Smem <= 48 * 1024, "no shared-memory attribute needed");
+
+// two scaled values as E4M3 (round to nearest even, saturating)
+__device__ __forceinline__ uint16_t fp8_pair(float2 v, float s)
 {
-    constexpr int ES = Fmt<PREC>::esize;
-    constexpr int EPP = 16 / ES;                    // K elements per 16-byte core row
-    constexpr int PLANES = kKP / EPP;               // K core-matrix columns (16 or 8)
-    constexpr int PLANE_A = kTileRows * 16, PLANE_B = kN * 16;
-    constexpr int NMMA = PLANES / 2;                // each MMA consumes two K core matrices
-    constexpr int F2 = EPP / 2;                     // float2 reads per (row, plane)
+    return __nv_cvt_float2_to_fp8x2(make_float2(v.x * s, v.y * s), __NV_SATFINITE, __NV_E4M3);
+}
+
+__global__ void __launch_bounds__(kT8Threads, kT8PerSm)
+    k_fir_tc8(const float2 *__restrict__ Y, long long ybase, long long k_lo, int nrows,
+              const float2 *__restrict__ taps, int ntaps, int rows_per_scale, float2 *__restrict__ z, int *err)
+{
     extern __shared__ __align__(1024) unsigned char sm[];
-    unsigned char *sA = sm + kOffA, *sB = sm + kOffB;
-    uint64_t *bar_ld = reinterpret_cast<uint64_t *>(sm + kOffMisc);   // [2]
-    uint64_t *bar_mma = bar_ld + 2;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar_ld + 3);
-    float *s_rmax = reinterpret_cast<float *>(sm + kOffRmax);          // [2][128]
-    int *s_exp = reinterpret_cast<int *>(sm + kOffExp);                // [<= 128]
+    unsigned char *sA = sm, *sB = sm + kT8OffB;
+    float2 *s_w = reinterpret_cast<float2 *>(sm + kT8OffW);
+    unsigned *s_max = reinterpret_cast<unsigned *>(sm + kT8OffMax), *s_halo = s_max + kTileRows + 1;
+    int *s_exp = reinterpret_cast<int *>(sm + kT8OffExp);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kT8OffBar);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, quarter = warp & 3, half = warp >> 2;
-    const int th = (ntaps - 1) / 2;
-    const int ns = 2 * kRowSyms - 2 + ntaps;       // complex inputs per row
-    const int ntiles = (nrows + kTileRows - 1) / kTileRows;
-
-    // staged range of tile t: from an even element offset, so the copy starts on 16 bytes
-    auto tile_src = [&](int t, long long &es, int &shift, int &nst) {
-        int r0 = t * kTileRows, rows = min(kTileRows, nrows - r0);
-        long long e0 = 2 * (k_lo + (long long)r0 * kRowSyms) - th - ybase;
-        es = e0 & ~1LL;
-        shift = (int)(e0 - es);
-        nst = ((shift + 2 * kRowSyms * (rows - 1) + ns) + 1) & ~1;
+    const int th = (ntaps - 1) / 2, ns = 2 * kRowSyms - 2 + ntaps;   // complex inputs per row
+    const int nhalo = ns - 32;                                       // of them in the next block row (may be <= 0)
+    const int ntiles = (nrows + kTileRows - 1) / kTileRows, rshift = 31 - __clz(rows_per_scale);
+    float2 v[kT8Iter];
+    auto load_tile = [&](int t) {   // lane = sample of block row warp + 8 i; zero outside what the rows read
+        const int r0 = t * kTileRows, n = 32 * (min(kTileRows, nrows - r0) - 1) + ns;
+        const float2 *Yb = Y + (2 * (k_lo + (long long)r0 * kRowSyms) - th - ybase);
+#pragma unroll
+        for (int i = 0; i < kT8Iter; i++) {
+            const int j = tid + i * kT8Threads;
+            v[i] = j < n ? __ldg(Yb + j) : make_float2(0.f, 0.f);
+        }
     };
-    auto issue = [&](int t, int buf) {
-        long long es;
-        int shift, nst;
-        tile_src(t, es, shift, nst);
-        fence_async_smem();   // earlier generic writes to this buffer precede the copy
-        mbar_expect_tx(bar_ld + buf, (unsigned)(nst * 8));
-        bulk_g2s(sm + kOffStage + buf * kStageBytes, Y + es, (unsigned)(nst * 8), bar_ld + buf);
-    };
-    if (tid == 0) {
-        mbar_init(bar_ld, 1);
-        mbar_init(bar_ld + 1, 1);
-        mbar_init(bar_mma, 1);
-        if ((int)blockIdx.x < ntiles) issue(blockIdx.x, 0);
-    }
-    __syncwarp();
+    int t = blockIdx.x;
+    if (tid < 32) s_w[tid] = tid < ntaps ? __ldg(taps + tid) : make_float2(0.f, 0.f);
+    if (t < ntiles) load_tile(t);
+    if (tid == 0) mbar_init(bar, 1);
     if (warp == 0) tmem_alloc(tslot, kTmemCols);
-
-    // B: Toeplitz matrix of the taps, rows n = 2j + c (c: re / im output of
-    // symbol j), K index 2s + d (d: re / im of input s); tap i = 2j + 2TH - s
-    float wmax = 0.f;
-    for (int i = 0; i < ntaps; i++) wmax = fmaxf(wmax, fmaxf(fabsf(taps[i].x), fabsf(taps[i].y)));
-    const int eB = PREC == RX_FIR_FP8 ? fp8_exp(wmax) : 0;
+    __syncthreads();   // the taps in shared memory
+    // B: Toeplitz matrix of the taps, rows n = 2 j + c (c: re / im output of symbol j), K
+    // index 2 s + d (d: re / im of input s); tap i = 2 j + 2 TH - s
+    const float2 wl = s_w[lane];
+    const int eB = fp8_exp(__uint_as_float(
+        __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fmaxf(0.f, fabsf(wl.x)), fabsf(wl.y))))));
     const float sBv = ldexpf(1.f, eB);
-    for (int u = tid; u < kN * PLANES; u += kThreads) {
-        int n = u % kN, pl = u / kN;
-        int j = n >> 1, c = n & 1;
-        float v[16];
+    {
+        const int n = tid % kN, pl = tid / kN, j = n >> 1, c = n & 1;
+        uint16_t h[8];
 #pragma unroll
-        for (int t = 0; t < EPP; t++) {
-            int k = pl * EPP + t, s = k >> 1, d = k & 1;
-            int i = 2 * j + 2 * th - s;
-            float val = 0.f;
+        for (int q = 0; q < 8; q++) {
+            const int s = 8 * pl + q, i = 2 * j + 2 * th - s;
+            float2 a = make_float2(0.f, 0.f);
             if (s < ns && i >= 0 && i < ntaps) {
-                float2 w = taps[i];
+                const float2 w = s_w[i];
                 // conj(w) y: re = a yr + b yi, im = a yi - b yr
-                val = c == 0 ? (d == 0 ? w.x : w.y) : (d == 0 ? -w.y : w.x);
+                a = c == 0 ? w : make_float2(-w.y, w.x);
             }
-            v[t] = val;
+            h[q] = fp8_pair(a, sBv);
         }
-        *reinterpret_cast<uint4 *>(sB + pl * PLANE_B + n * 16) = pack16<PREC>(v, sBv);
+        *reinterpret_cast<uint4 *>(sB + pl * kT8BPlane + n * 16) =
+            make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
+                       h[6] | (uint32_t)h[7] << 16);
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tslot;
-    const uint32_t idesc = umma_idesc(Fmt<PREC>::code, kTileRows, kN);
-
-    // lane -> (row r_lo, K column p_lo) of an 8 x 4 group; a warp's groups cover
-    // the 32 rows of its lane quarter and half of the K columns
-    const int r_lo = lane & 7, p_lo = lane >> 3, rot = r_lo % F2;
+    static_assert(kN * kT8Planes == kT8Threads, "one core row of B per thread");
+    const uint32_t idesc = umma_idesc(0, kTileRows, kN);   // kind::f8f6f4, E4M3
     bool ok = true;
-    int it = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
-        const int buf = it & 1;
+    for (int it = 0; t < ntiles; t += gridDim.x, it++) {
         const int r0 = t * kTileRows, rows = min(kTileRows, nrows - r0);
-        long long es;
-        int shift, nst;
-        tile_src(t, es, shift, nst);
-        if (tid == 0 && t + (int)gridDim.x < ntiles) issue(t + gridDim.x, buf ^ 1);   // prefetch
-        bool got = mbar_wait(bar_ld + buf, (unsigned)((it >> 1) & 1));
-        if (!got) {
-            atomicExch(err, (int)RX_ETIMEOUT);
-            mbar_wait(bar_ld + buf, (unsigned)((it >> 1) & 1));
+        // largest magnitude of each block row and, where it starts a scale block, of the
+        // part of it that the last row of the block before reads
+#pragma unroll
+        for (int i = 0; i < kT8Iter; i++) {
+            const int q = warp + kT8Warps * i;
+            if (q > kTileRows) break;
+            const unsigned m = __float_as_uint(fmaxf(fmaxf(0.f, fabsf(v[i].x)), fabsf(v[i].y)));
+            const unsigned mr = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) s_max[q] = mr;
+            if ((q & (rows_per_scale - 1)) == 0) {
+                const unsigned mh = __reduce_max_sync(0xffffffffu, lane < nhalo ? m : 0u);
+                if (lane == 0) s_halo[q] = mh;
+            }
         }
-        ok = __syncthreads_and(got) != 0;
-        if (!ok) break;
-        const float *stf = reinterpret_cast<const float *>(sm + kOffStage + buf * kStageBytes) + 2 * shift;
-
-        // (row, K column) -> the 16 bytes of K elements it holds, read in a rotated
-        // order; returns the EPP floats in natural order
-        auto load_unit = [&](int r, int pl, float (&v)[16]) {
-            const float *base = stf + 4 * kRowSyms * r + pl * EPP;   // rows start 2 kRowSyms complex apart
-            float2 tmp[F2];
-#pragma unroll
-            for (int q = 0; q < F2; q++) {
-                int qq = (q + rot) % F2;
-                tmp[q] = *reinterpret_cast<const float2 *>(base + 2 * qq);
-            }
-#pragma unroll
-            for (int q = 0; q < F2; q++) {
-                // undo the rotation: element qq came in slot (qq - rot) mod F2
-                float2 e = tmp[0];
-#pragma unroll
-                for (int u = 1; u < F2; u++)
-                    if (((q - rot + F2) % F2) == u) e = tmp[u];
-                v[2 * q] = e.x;
-                v[2 * q + 1] = e.y;
-            }
-#pragma unroll
-            for (int u = 0; u < EPP; u++)
-                if (r >= rows || pl * EPP + u >= 2 * ns) v[u] = 0.f;
-        };
-
-        if (PREC == RX_FIR_FP8) {
-            // per-row largest input magnitude, then per scale block
-#pragma unroll 1
-            for (int rh = 0; rh < 4; rh++) {
-                int r = 32 * quarter + 8 * rh + r_lo;
-                float m = 0.f;
-#pragma unroll 1
-                for (int ph = half * (PLANES / 8); ph < (half + 1) * (PLANES / 8); ph++) {
-                    float v[16];
-                    load_unit(r, 4 * ph + p_lo, v);
-#pragma unroll
-                    for (int u = 0; u < EPP; u++) m = fmaxf(m, fabsf(v[u]));
-                }
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-                if (p_lo == 0) s_rmax[half * kTileRows + r] = m;
-            }
-            __syncthreads();
-            if (tid < kTileRows / rows_per_scale) {
-                float bm = 0.f;
-                for (int r = tid * rows_per_scale; r < (tid + 1) * rows_per_scale; r++)
-                    bm = fmaxf(bm, fmaxf(s_rmax[r], s_rmax[kTileRows + r]));
-                s_exp[tid] = fp8_exp(bm);
-            }
-            __syncthreads();
+        __syncthreads();
+        for (int b = warp; b < (kTileRows >> rshift); b += kT8Warps) {
+            unsigned m = lane == 0 ? s_halo[(b + 1) << rshift] : 0u;
+            for (int r = lane; r < rows_per_scale; r += 32) m = max(m, s_max[(b << rshift) + r]);
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) s_exp[b] = fp8_exp(__uint_as_float(m));
         }
-        // A: row r, K index k -> staged float 2 (shift + 32 r) + k for k < 2 ns, else 0
-#pragma unroll 1
-        for (int rh = 0; rh < 4; rh++) {
-            int r = 32 * quarter + 8 * rh + r_lo;
-            float sAv = PREC == RX_FIR_FP8 ? ldexpf(1.f, s_exp[r / rows_per_scale]) : 1.f;
-#pragma unroll 2
-            for (int ph = half * (PLANES / 8); ph < (half + 1) * (PLANES / 8); ph++) {
-                int pl = 4 * ph + p_lo;
-                float v[16];
-                load_unit(r, pl, v);
-                *reinterpret_cast<uint4 *>(sA + pl * PLANE_A + r * 16) = pack16<PREC>(v, sAv);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kT8Iter; i++) {
+            const int q = warp + kT8Warps * i;
+            if (q > kTileRows) break;
+            unsigned char *dst = sA + (lane >> 3) * kT8Plane + (lane & 7) * 2;
+            const int e0 = q < kTileRows ? s_exp[q >> rshift] : 0;
+            const uint16_t h = fp8_pair(v[i], ldexpf(1.f, e0));
+            if (q < kTileRows) *reinterpret_cast<uint16_t *>(dst + q * 16) = lane < ns ? h : 0;
+            if (q > 0) {
+                uint16_t h1 = h;
+                if ((q & (rows_per_scale - 1)) == 0) h1 = fp8_pair(v[i], ldexpf(1.f, s_exp[(q - 1) >> rshift]));
+                *reinterpret_cast<uint16_t *>(dst + (kT8Planes / 2) * kT8Plane + (q - 1) * 16) = lane < nhalo ? h1 : 0;
             }
         }
         fence_async_smem();
+        tc_fence_before();
         __syncthreads();
+        tc_fence_after();
+        const uint32_t tmem = *tslot;
+        if (t + (int)gridDim.x < ntiles) load_tile(t + gridDim.x);
         if (tid == 0) {
-            tc_fence_after();
             const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
 #pragma unroll
-            for (int q = 0; q < NMMA; q++) {
-                uint64_t ad = umma_sdesc(a0 + q * 2 * PLANE_A, PLANE_A, 128);
-                uint64_t bd = umma_sdesc(b0 + q * 2 * PLANE_B, PLANE_B, 128);
-                if (PREC == RX_FIR_FP8) umma_f8(tmem, ad, bd, idesc, q > 0);
-                else umma_f16(tmem, ad, bd, idesc, q > 0);
-            }
-            umma_commit(bar_mma);
+            for (int q = 0; q < kT8Planes / 2; q++)
+                umma_f8(tmem, umma_sdesc(a0 + q * 2 * kT8Plane, kT8Plane, 128),
+                        umma_sdesc(b0 + q * 2 * kT8BPlane, kT8BPlane, 128), idesc, q > 0);
+            umma_commit(bar);
         }
-        bool done = mbar_wait(bar_mma, (unsigned)(it & 1));
+        bool done = mbar_wait(bar, (unsigned)(it & 1));
         if (!done) {
             atomicExch(err, (int)RX_ETIMEOUT);
-            mbar_wait(bar_mma, (unsigned)(it & 1));
+            mbar_wait(bar, (unsigned)(it & 1));
         }
         ok = __syncthreads_and(done) != 0;
-        if (!ok) break;
         tc_fence_after();
-        // epilogue: warp (quarter, half) owns accumulator lanes 32 quarter .. + 31 (rows)
-        // and columns 16 half .. + 15; rows go through the consumed stage buffer to
-        // leave as contiguous 512-byte stores
-        {
-            uint32_t acc[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * quarter) << 16) + 16 * half, acc);
-            const int r = 32 * quarter + lane;
-            float inv = 1.f;
-            if (PREC == RX_FIR_FP8) inv = ldexpf(1.f, -(eB + s_exp[r / rows_per_scale]));
-            float *ot = reinterpret_cast<float *>(sm + kOffStage + buf * kStageBytes);
+        if (!ok) break;
+        // warp (quarter, half): accumulator lanes (rows) 32 quarter .. + 31, columns
+        // 16 half .. + 15 = symbols 8 half .. + 7 of the row, unscaled exactly
+        uint32_t acc[16];
+        tmem_ld16(tmem + ((uint32_t)(32 * quarter) << 16) + 16 * half, acc);
+        const int r = 32 * quarter + lane;
+        if (r < rows) {
+            const float inv = ldexpf(1.f, -(eB + s_exp[r >> rshift]));
+            float4 *zr = reinterpret_cast<float4 *>(z + ((long long)(r0 + r) * kRowSyms + 8 * half));
 #pragma unroll
             for (int q = 0; q < 4; q++)
-                *reinterpret_cast<float4 *>(ot + r * kOutPitch + 16 * half + 4 * q) =
-                    make_float4(__uint_as_float(acc[4 * q]) * inv, __uint_as_float(acc[4 * q + 1]) * inv,
-                                __uint_as_float(acc[4 * q + 2]) * inv, __uint_as_float(acc[4 * q + 3]) * inv);
-            __syncthreads();
-            float4 *zt = reinterpret_cast<float4 *>(z + (long long)r0 * kRowSyms);
-            for (int i = tid; i < kTileRows * 8; i += kThreads) {
-                int rr = i >> 3, ch = i & 7;
-                if (rr < rows) zt[rr * 8 + ch] = *reinterpret_cast<const float4 *>(ot + rr * kOutPitch + 4 * ch);
-            }
+                zr[q] = make_float4(__uint_as_float(acc[4 * q]) * inv, __uint_as_float(acc[4 * q + 1]) * inv,
+                                    __uint_as_float(acc[4 * q + 2]) * inv, __uint_as_float(acc[4 * q + 3]) * inv);
         }
         tc_fence_before();
-        __syncthreads();   // A, the accumulator and this stage buffer are free again
-    }
-    if (!ok && tid == 0) {
-        // a prefetch may still be in flight: wait for it (bounded) before leaving
-        mbar_wait(bar_ld + ((it + 1) & 1), (unsigned)(((it + 1) >> 1) & 1));
+        __syncthreads();   // A, the scales and the accumulator are free again
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+    if (warp == 0) tmem_dealloc(*tslot, kTmemCols);
 }
-
 
 // ---------------------------------------------------------------------------
 // 16-bit forms (BF16, FP16): each input sample is converted once.  Block row q of
@@ -355,7 +269,7 @@ constexpr int kT2OffB = kT2Planes * kT2Plane;
 constexpr int kT2OffW = kT2OffB + 2 * kT2Planes * kT2BPlane;   // the taps (32 complex)
 constexpr int kT2OffBar = kT2OffW + 32 * 8;
 constexpr int kT2Smem = kT2OffBar + 16;
-constexpr int kT2Threads = 256;
+constexpr int kT2Threads = 256, kT2PerSm = 3;
 constexpr int kT2Samples = (kTileRows + 1) * 2 * kRowSyms;   // complex samples a tile converts
 constexpr int kT2Iter = (kT2Samples + kT2Threads - 1) / kT2Threads;
 static_assert(kT2Plane % 16 == 0 && kT2OffB % 16 == 0 && kT2OffBar % 8 == 0, "16-byte aligned operands");
@@ -374,7 +288,7 @@ __device__ __forceinline__ uint32_t pack2(float a, float b)
 }
 
 template <int PREC>
-__global__ void __launch_bounds__(kT2Threads, 2)
+__global__ void __launch_bounds__(kT2Threads, kT2PerSm)
     k_fir_tc2(const float2 *__restrict__ Y, long long ybase, long long k_lo, int nrows,
               const float2 *__restrict__ taps, int ntaps, float2 *__restrict__ z, int *err)
 {
@@ -426,7 +340,7 @@ __global__ void __launch_bounds__(kT2Threads, 2)
             }
             vb[q] = val;
         }
-        *reinterpret_cast<uint4 *>(sB + pl * kT2BPlane + n * 16) = pack16<PREC>(vb, 1.f);
+        *reinterpret_cast<uint4 *>(sB + pl * kT2BPlane + n * 16) = pack16<PREC>(vb);
     }
     const uint32_t idesc = umma_idesc(Fmt<PREC>::code, kTileRows, kN);
     bool ok = true;
@@ -492,12 +406,8 @@ __global__ void __launch_bounds__(kT2Threads, 2)
 
 cudaError_t prepare_fir_tc(int prec)
 {
-    switch (prec) {
-    case RX_FIR_BF16:
-    case RX_FIR_FP16: return cudaSuccess;   // the 16-bit kernel's shared memory is under the default limit
-    case RX_FIR_FP8: return cudaFuncSetAttribute(k_fir_tc<RX_FIR_FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    default: return cudaErrorInvalidValue;
-    }
+    // every form's shared memory is under the default limit
+    return prec == RX_FIR_BF16 || prec == RX_FIR_FP16 || prec == RX_FIR_FP8 ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_fir_tc(int prec, const float2 *Y, long long ybase, long long k_lo, long long nsym,
@@ -512,18 +422,16 @@ cudaError_t launch_fir_tc(int prec, const float2 *Y, long long ybase, long long 
     int rps = scale_block / kRowSyms;
     int ntiles = (nrows + kTileRows - 1) / kTileRows;
     if (prec == RX_FIR_BF16 || prec == RX_FIR_FP16) {
-        const unsigned g2 = (unsigned)min(ntiles, 2 * nsm);   // two persistent CTAs per SM
+        const unsigned g2 = (unsigned)min(ntiles, kT2PerSm * nsm);   // persistent CTAs
         if (prec == RX_FIR_BF16)
             k_fir_tc2<RX_FIR_BF16><<<g2, kT2Threads, kT2Smem, st>>>(Y, ybase, k_lo, nrows, taps, ntaps, z, err);
         else
             k_fir_tc2<RX_FIR_FP16><<<g2, kT2Threads, kT2Smem, st>>>(Y, ybase, k_lo, nrows, taps, ntaps, z, err);
         return cudaGetLastError();
     }
-    unsigned grid = (unsigned)min(ntiles, 2 * nsm);   // two persistent CTAs per SM
-#define RX_FIR_LAUNCH(P) k_fir_tc<P><<<grid, kThreads, kSmem, st>>>(Y, ybase, k_lo, nrows, taps, ntaps, rps, z, err)
     if (prec != RX_FIR_FP8) return cudaErrorInvalidValue;
-    RX_FIR_LAUNCH(RX_FIR_FP8);
-#undef RX_FIR_LAUNCH
+    const unsigned g8 = (unsigned)min(ntiles, kT8PerSm * nsm);   // persistent CTAs
+    k_fir_tc8<<<g8, kT8Threads, kT8Smem, st>>>(Y, ybase, k_lo, nrows, taps, ntaps, rps, z, err);
     return cudaGetLastError();
 }
 
