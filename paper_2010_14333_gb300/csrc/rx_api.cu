@@ -737,7 +737,8 @@ rx_status rx_create(rx_format f, double baud, double fs, int64_t buf_len, const 
     if (kk) {
         for (int i = 0; i < kSlots; i++) RX_ALLOC(h->E[i], (kEHist + nb) * sizeof(float2));
         for (int i = 0; i < 3; i++) RX_ALLOC(h->phist[i], (size_t)h->nhist * 3 / 2 + 16);
-        for (int i = 0; i < 2; i++) RX_ALLOC(h->fftws[i], (size_t)h->npairs_max * h->N * sizeof(float2));
+        for (int i = 0; i < 2 && h->N == 65536; i++)   // 4096-point blocks stay in shared memory
+            RX_ALLOC(h->fftws[i], (size_t)h->npairs_max * h->N * sizeof(float2));
         RX_ALLOC(h->twN, kk_tw_entries(h->N) * sizeof(float2));
         RX_ALLOC(h->twN2, kk_tw_entries(h->N2) * sizeof(float2));
         RX_ALLOC(h->lnt, kLutCodes * sizeof(float));

@@ -270,12 +270,46 @@ __device__ __forceinline__ uint32_t col_code(const uint32_t *rw, const ColPos &c
     return v & 0xFFFu;
 }
 
+// (dst may be null on a stream's first call)
 __device__ __forceinline__ uint32_t first_code(const KkPacked &pk, const DevState *dst)
 {
     if (!pk.first_call) return (uint32_t)dst->first_code;
     uint32_t a, b;
     decode_pair(pk.in[0], pk.in[1], pk.in[2], pk.order, a, b);
     return a;
+}
+
+// u = ln(I)/2 of both blocks of a pair at window positions n1 + N2T q, q < 16
+template <int ORD, int N2T>
+__device__ __forceinline__ void load_columns(const KkGeom &g, int pair, int n1, bool hb, const uint32_t (*raw)[kRawWords],
+                                             const ColPos &cp, uint32_t c_first, const float *s_ln, float2 (&x)[16])
+{
+    const long long wa = ols_ws(g, 2 * pair) + n1, wb = hb ? ols_ws(g, 2 * pair + 1) + n1 : 0;
+    // rows q below qa (qb) hold stream indices before the stream: the first code
+    const int qa = wa < 0 ? (int)min((-wa + N2T - 1) / N2T, 16LL) : 0;
+    const int qb = wb < 0 ? (int)min((-wb + N2T - 1) / N2T, 16LL) : 0;
+#pragma unroll
+    for (int q = 0; q < 16; q++) {
+        uint32_t ca = q < qa ? c_first : col_code<ORD>(raw[q], cp);
+        float ua = s_ln[ca], ub = 0.f;
+        if (hb) {
+            uint32_t cb = q < qb ? c_first : col_code<ORD>(raw[16 + q], cp);
+            ub = s_ln[cb];
+        }
+        x[q] = make_float2(ua, ub);
+    }
+}
+
+// packed history of the next call, samples [avail - nhist, avail) = virtual bytes
+// [in_bytes, in_bytes + hist_bytes), copied by CTAs 0 .. ncta - 1 (this one is cta)
+__device__ __forceinline__ void copy_hist(const KkPacked &pk, int cta, int ncta)
+{
+    const long long nch = pk.hist_bytes / 16;
+    for (long long c = (long long)cta * blockDim.x + threadIdx.x; c < nch; c += (long long)ncta * blockDim.x) {
+        long long vb = pk.in_bytes + 16 * c;
+        const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
+        reinterpret_cast<uint4 *>(pk.hist_next)[c] = __ldg(reinterpret_cast<const uint4 *>(src));
+    }
 }
 
 // K1a: unpack, u = ln(I)/2 by table, radix-16 pass over the stride-N2 index of two
@@ -292,14 +326,7 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2
     int pair = blockIdx.y;
     if (pk.lat && blockIdx.x == 0 && pair == 0 && threadIdx.x == 0) lat_start(pk.lat, pk.lat_slot);
     if (pair == g.npairs) {
-        // history of the next call: samples [avail - nhist, avail) = virtual bytes
-        // [in_bytes, in_bytes + hist_bytes)
-        long long nch = pk.hist_bytes / 16;
-        for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < nch; c += (long long)gridDim.x * blockDim.x) {
-            long long vb = pk.in_bytes + 16 * c;
-            const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
-            reinterpret_cast<uint4 *>(pk.hist_next)[c] = __ldg(reinterpret_cast<const uint4 *>(src));
-        }
+        copy_hist(pk, blockIdx.x, gridDim.x);
         return;
     }
     const TwSmem tw = stage_tw(tb.twN, g.N, s_tw);
@@ -308,29 +335,15 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2
     for (int i = threadIdx.x; i < kLutCodes / 4; i += blockDim.x)
         reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
     const int c0 = blockIdx.x * blockDim.x;
-    const int jb = 2 * pair + 1;
-    const bool hb = jb < g.J;
+    const bool hb = 2 * pair + 1 < g.J;
     stage_rows<N2T>(g, pk, pair, c0, raw, hb);
     const uint32_t c_first = first_code(pk, dst);
-    if (pk.first_call && blockIdx.x == 0 && pair == 0 && threadIdx.x == 0) dst->first_code = (int)c_first;
+    if (pk.first_call && dst && blockIdx.x == 0 && pair == 0 && threadIdx.x == 0) dst->first_code = (int)c_first;
     __syncthreads();
     const int t = threadIdx.x, n1 = c0 + t;
-    const long long wa = ols_ws(g, 2 * pair) + c0 + t, wb = hb ? ols_ws(g, jb) + c0 + t : 0;
-    // rows q below qa (qb) hold stream indices before the stream: the first code
-    const int qa = wa < 0 ? (int)min((-wa + N2T - 1) / N2T, 16LL) : 0;
-    const int qb = wb < 0 ? (int)min((-wb + N2T - 1) / N2T, 16LL) : 0;
     const ColPos cp = col_pos<ORD>(t);
     float2 x[16];
-#pragma unroll
-    for (int q = 0; q < 16; q++) {
-        uint32_t ca = q < qa ? c_first : col_code<ORD>(raw[q], cp);
-        float ua = s_ln[ca], ub = 0.f;
-        if (hb) {
-            uint32_t cb = q < qb ? c_first : col_code<ORD>(raw[16 + q], cp);
-            ub = s_ln[cb];
-        }
-        x[q] = make_float2(ua, ub);
-    }
+    load_columns<ORD, N2T>(g, pair, n1, hb, raw, cp, c_first, s_ln, x);
     dft16<false>(x);
     twiddle16<false>(x, tw, n1);
     float2 *out = fftws + (size_t)pair * g.N + n1;
@@ -355,42 +368,27 @@ __device__ __forceinline__ float2 hilbert_mul(float2 v, int k, int N)
     return (2 * k < N) ? make_float2(v.y, -v.x) : make_float2(-v.y, v.x);
 }
 
-// K1b: per row k2 of a block pair, N2-point FFT (radix-16 decimation in
-// frequency, digit-reversed output), Hilbert multiplier on the bins k = k2 + 16 k1,
-// inverse FFT (radix-16 decimation in time back to natural order).  In place.
-template <int P>
+// K1b: per row k2 of a block pair of 2^16-point blocks, 4096-point FFT (radix-16
+// decimation in frequency, digit-reversed output), Hilbert multiplier on the bins
+// k = k2 + 16 k1, inverse FFT (radix-16 decimation in time back to natural order).  In
+// place, one row per CTA.
+constexpr int kRowN2 = 4096, kRowPad = kRowN2 + kRowN2 / 16;   // row and padded row
 __global__ void __launch_bounds__(256, 3) k_kk_rows(KkGeom g, float2 *__restrict__ fftws,
                                                    const float2 *__restrict__ twN2g)
 {
-    constexpr int N2 = 1 << (4 * P);
-    constexpr int TPR = N2 / 16;                  // threads per row
-    constexpr int RPC = 256 / TPR;                // rows per CTA
-    constexpr int SROW = N2 + N2 / 16;            // padded row in shared memory
-    extern __shared__ float2 sm[];
+    constexpr int P = 3, N2 = kRowN2, TPR = N2 / 16;
+    extern __shared__ float2 s[];                 // the padded row
     __shared__ float2 s_tw[128];
     const TwSmem tw2 = stage_tw(twN2g, N2, s_tw);
     __syncthreads();
-    int lr = threadIdx.x / TPR, t = threadIdx.x % TPR;
-    int row = blockIdx.x * RPC + lr;
-    bool active = row < g.npairs * 16;
-    int k2 = row & 15;
-    float2 *s = sm + lr * SROW;
-    float2 *d = fftws + (size_t)(active ? row : 0) * N2;
+    const int t = threadIdx.x, row = blockIdx.x, k2 = row & 15;
+    float2 *d = fftws + (size_t)row * N2;
     float2 x[16];
     // forward pass 0 (sub-transform size N2) straight from global memory
 #pragma unroll
-    for (int r = 0; r < 16; r++) x[r] = active ? d[t + r * TPR] : make_float2(0.f, 0.f);
+    for (int r = 0; r < 16; r++) x[r] = d[t + r * TPR];
     dft16<false>(x);
     twiddle16<false>(x, tw2, t);
-    if (P == 1) {
-#pragma unroll
-        for (int r = 0; r < 16; r++) x[r] = hilbert_mul(x[r], k2 + 16 * drev16<P>(r), g.N);
-        dft16<true>(x);
-        if (active)
-#pragma unroll
-            for (int r = 0; r < 16; r++) d[r] = x[r];
-        return;
-    }
     // a pass's 16 elements base + r stride sit at pad16(base) + r (stride + stride / 16)
     // when stride is a multiple of 16, or base is one and stride is 1: one pointer per
     // pass and compile-time offsets
@@ -443,9 +441,8 @@ __global__ void __launch_bounds__(256, 3) k_kk_rows(KkGeom g, float2 *__restrict
     for (int r = 0; r < 16; r++) x[r] = s0[r * STR0];
     twiddle16<true>(x, tw2, t);
     dft16<true>(x);
-    if (active)
 #pragma unroll
-        for (int r = 0; r < 16; r++) d[t + r * TPR] = x[r];
+    for (int r = 0; r < 16; r++) d[t + r * TPR] = x[r];
 }
 
 // Carrier and intensity sums of a call, from which its carrier and gain follow.
@@ -461,6 +458,7 @@ constexpr double kCarrierUnit = 16777216.0;   // 2^24
 __device__ __forceinline__ void carrier_sums(const KkGeom &g, DevState *dst, float sre, float sim, int si2,
                                              int ncta)
 {
+    if (!dst) return;   // field only
     __shared__ long long s_q[3][32];
     sre = warp_sum_f(sre);
     sim = warp_sum_f(sim);
@@ -498,42 +496,25 @@ __device__ __forceinline__ void carrier_sums(const KkGeom &g, DevState *dst, flo
     dst->ticket[g.slot] = 0u;
 }
 
-// K1c: inverse radix-16 pass, then for every kept output
-// E = sqrt(I) * exp(j phi) (Fig. 1d), written at its stream position, and the
-// per-call carrier / intensity sums (exact integer totals, carrier_sums).  The
-// codes for sqrt(I) come from the same staged rows.  ORD: the pack order; N2T: the
-// row length N / 16.
-template <int ORD, int N2T>
-__global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const float2 *__restrict__ fftws,
-                                                  const KkTables tb, float2 *__restrict__ E,
-                                                  const float2 *__restrict__ E_prev, DevState *dst)
+// field history for the matched filter: E[n], n in [e_prev - kEHist, e_prev) (E_prev null:
+// the caller keeps none)
+__device__ __forceinline__ void carry_field(const KkGeom &g, float2 *__restrict__ E, const float2 *__restrict__ E_prev)
 {
-    __shared__ float2 s_tw[512];
-    __shared__ __align__(16) uint32_t raw[32][kRawWords];
-    const TwSmem tw = stage_tw(tb.twN, g.N, s_tw);
-    int pair = blockIdx.y;
-    const int c0 = blockIdx.x * blockDim.x;
-    const bool hb = 2 * pair + 1 < g.J;
-    stage_rows<N2T>(g, pk, pair, c0, raw, hb);
-    const uint32_t c_first = first_code(pk, dst);
-    float sre = 0.f, sim = 0.f;
-    int si2 = 0;
-    if (blockIdx.x == 0 && blockIdx.y == 0) {
-        // field history for the matched filter: E[n], n in [e_prev - kEHist, e_prev)
-        for (int i = threadIdx.x; i < kEHist; i += blockDim.x) {
-            long long n = g.e_prev - kEHist + i;
-            E[i] = (n < 0) ? make_float2(0.f, 0.f) : E_prev[n - g.ebase_prev];
-        }
+    if (!E_prev) return;
+    for (int i = threadIdx.x; i < kEHist; i += blockDim.x) {
+        long long n = g.e_prev - kEHist + i;
+        E[i] = (n < 0) ? make_float2(0.f, 0.f) : E_prev[n - g.ebase_prev];
     }
-    const int t = threadIdx.x, n1 = c0 + t;
-    const ColPos cp = col_pos<ORD>(t);
-    float2 x[16];
-    const float2 *in = fftws + (size_t)pair * g.N + n1;
-#pragma unroll
-    for (int k2 = 0; k2 < 16; k2++) x[k2] = in[k2 * N2T];
-    __syncthreads();   // staged twiddles and rows
-    twiddle16<true>(x, tw, n1);
-    dft16<true>(x);
+}
+
+// E = sqrt(I) exp(j phi) (Fig. 1d) of the kept outputs of a column of a block pair: x[q]
+// holds N times the phase of both blocks at window position n1 + N2T q; the codes come from
+// the staged rows.  Adds to the carrier / intensity sums.
+template <int ORD, int N2T>
+__device__ __forceinline__ void emit_field(const KkGeom &g, int pair, int n1, const float2 (&x)[16],
+                                           const uint32_t (*raw)[kRawWords], const ColPos &cp, uint32_t c_first,
+                                           float2 *__restrict__ E, float &sre, float &sim, int &si2)
+{
     const float invN = 1.0f / (float)g.N;
 #pragma unroll
     for (int half = 0; half < 2; half++) {
@@ -565,7 +546,132 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const 
             si2 += code ? 2 * (int)code : 1;
         }
     }
+}
+
+// K1c: inverse radix-16 pass, then the field of every kept output, written at its stream
+// position, and the per-call carrier / intensity sums (exact integer totals,
+// carrier_sums).  ORD: the pack order; N2T: the row length N / 16.
+template <int ORD, int N2T>
+__global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const float2 *__restrict__ fftws,
+                                                  const KkTables tb, float2 *__restrict__ E,
+                                                  const float2 *__restrict__ E_prev, DevState *dst)
+{
+    __shared__ float2 s_tw[512];
+    __shared__ __align__(16) uint32_t raw[32][kRawWords];
+    const TwSmem tw = stage_tw(tb.twN, g.N, s_tw);
+    int pair = blockIdx.y;
+    const int c0 = blockIdx.x * blockDim.x;
+    const bool hb = 2 * pair + 1 < g.J;
+    stage_rows<N2T>(g, pk, pair, c0, raw, hb);
+    const uint32_t c_first = first_code(pk, dst);
+    float sre = 0.f, sim = 0.f;
+    int si2 = 0;
+    if (blockIdx.x == 0 && blockIdx.y == 0) carry_field(g, E, E_prev);
+    const int t = threadIdx.x, n1 = c0 + t;
+    const ColPos cp = col_pos<ORD>(t);
+    float2 x[16];
+    const float2 *in = fftws + (size_t)pair * g.N + n1;
+#pragma unroll
+    for (int k2 = 0; k2 < 16; k2++) x[k2] = in[k2 * N2T];
+    __syncthreads();   // staged twiddles and rows
+    twiddle16<true>(x, tw, n1);
+    dft16<true>(x);
+    emit_field<ORD, N2T>(g, pair, n1, x, raw, cp, c_first, E, sre, sim, si2);
     carrier_sums(g, dst, sre, sim, si2, gridDim.x * gridDim.y);
+}
+
+// ============================================== KK front end, 4096-point blocks
+// A pair of 4096-point blocks (32 KB of complex spectrum) fits one CTA, so the whole
+// Hilbert transform of the pair runs in one kernel: thread t takes column t of the 16 x 256
+// four-step layout (codes, u = ln(I)/2, radix-16 DFT, twiddle), then a sixteenth of row
+// t / 16 (256-point FFT in two radix-16 passes, multiplier, inverse; a row belongs to half a
+// warp), then column t again (inverse DFT, field, carrier sums).  The arithmetic is that of
+// the three-kernel form of the 2^16-point blocks, pass by pass.  CTAs from npairs on copy
+// the next call's history.
+// Bound by latency: a chain of six passes at three CTAs per SM.  41,984 samples with V = 512
+// (six CTAs): 10.2 us per call of rx_kk_field_noalloc; 28.7 us as three kernels (column DFT, rows,
+// column DFT and field, the spectrum through global memory twice), a clear and a copy.
+constexpr int kBkN2 = 256, kBkRow = kBkN2 + kBkN2 / 16;   // row length and padded row
+struct BkSmem {
+    static constexpr int FFT = 0;                                    // float2 [16][kBkRow]; before it the ln table
+    static constexpr int RAW = FFT + 16 * kBkRow * 8;                // staged packed rows
+    static constexpr int TW = RAW + 32 * kRawWords * 4;              // factored W_4096 (128), W_256 (32)
+    static constexpr int TOTAL = TW + (128 + 32) * 8;
+};
+static_assert(kLutCodes * 4 <= BkSmem::RAW, "the ln table fits the spectrum's place");
+
+template <int ORD>
+__global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, const KkTables tb,
+                                                       float2 *__restrict__ E, const float2 *__restrict__ E_prev,
+                                                       DevState *dst)
+{
+    extern __shared__ __align__(16) unsigned char bksm[];
+    float2 *fft = reinterpret_cast<float2 *>(bksm + BkSmem::FFT);
+    float *s_ln = reinterpret_cast<float *>(bksm + BkSmem::FFT);
+    uint32_t(*raw)[kRawWords] = reinterpret_cast<uint32_t(*)[kRawWords]>(bksm + BkSmem::RAW);
+    float2 *s_tw = reinterpret_cast<float2 *>(bksm + BkSmem::TW);
+    const int pair = blockIdx.x, t = threadIdx.x;
+    if (pk.lat && pair == 0 && t == 0) lat_start(pk.lat, pk.lat_slot);
+    if (pair >= g.npairs) {
+        copy_hist(pk, pair - g.npairs, gridDim.x - g.npairs);
+        return;
+    }
+    const TwSmem tw = stage_tw(tb.twN, 16 * kBkN2, s_tw);
+    const TwSmem tw2 = stage_tw(tb.twN2, kBkN2, s_tw + 128);
+    for (int i = t; i < kLutCodes / 4; i += kCtaK1)
+        reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
+    const bool hb = 2 * pair + 1 < g.J;
+    stage_rows<kBkN2>(g, pk, pair, 0, raw, hb);
+    const uint32_t c_first = first_code(pk, dst);
+    if (pk.first_call && dst && pair == 0 && t == 0) dst->first_code = (int)c_first;
+    if (pair == 0) carry_field(g, E, E_prev);
+    __syncthreads();
+    const ColPos cp = col_pos<ORD>(t);
+    float2 x[16];
+    load_columns<ORD, kBkN2>(g, pair, t, hb, raw, cp, c_first, s_ln, x);
+    __syncthreads();   // the ln table has been read: the spectrum takes its place
+    dft16<false>(x);
+    twiddle16<false>(x, tw, t);
+    float2 *const col = fft + pad16(t);
+#pragma unroll
+    for (int k2 = 0; k2 < 16; k2++) col[k2 * kBkRow] = x[k2];
+    __syncthreads();
+    {
+        const int k2 = t >> 4, tt = t & 15;
+        float2 *const r0 = fft + k2 * kBkRow + tt;             // positions tt + 16 r: pad16 = tt + 17 r
+        float2 *const r1 = fft + k2 * kBkRow + pad16(16 * tt);   // positions 16 tt + r
+#pragma unroll
+        for (int r = 0; r < 16; r++) x[r] = r0[17 * r];
+        dft16<false>(x);
+        twiddle16<false>(x, tw2, tt);
+#pragma unroll
+        for (int r = 0; r < 16; r++) r0[17 * r] = x[r];
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 16; r++) x[r] = r1[r];
+        dft16<false>(x);
+#pragma unroll
+        for (int r = 0; r < 16; r++) x[r] = hilbert_mul(x[r], k2 + 16 * drev16<2>(16 * tt + r), 16 * kBkN2);
+        dft16<true>(x);
+#pragma unroll
+        for (int r = 0; r < 16; r++) r1[r] = x[r];
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 16; r++) x[r] = r0[17 * r];
+        twiddle16<true>(x, tw2, tt);
+        dft16<true>(x);
+#pragma unroll
+        for (int r = 0; r < 16; r++) r0[17 * r] = x[r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k2 = 0; k2 < 16; k2++) x[k2] = col[k2 * kBkRow];
+    twiddle16<true>(x, tw, t);
+    dft16<true>(x);
+    float sre = 0.f, sim = 0.f;
+    int si2 = 0;
+    emit_field<ORD, kBkN2>(g, pair, t, x, raw, cp, c_first, E, sre, sim, si2);
+    carrier_sums(g, dst, sre, sim, si2, g.npairs);
 }
 
 // ====================================================== KK front end, fused
@@ -629,19 +735,8 @@ __global__ void __cluster_dims__(kClC, 1, 1) __launch_bounds__(kClThreads, 3)
     if (pk.first_call && blockIdx.x == 0 && t == 0) dst->first_code = (int)c_first;
     // history of the next call (packed bytes [in_bytes, in_bytes + hist_bytes) of
     // the virtual buffer), spread over the grid
-    if (pk.hist_next) {
-        long long nch = pk.hist_bytes / 16;
-        for (long long ch = (long long)blockIdx.x * blockDim.x + t; ch < nch; ch += (long long)gridDim.x * blockDim.x) {
-            long long vb = pk.in_bytes + 16 * ch;
-            const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
-            reinterpret_cast<uint4 *>(pk.hist_next)[ch] = __ldg(reinterpret_cast<const uint4 *>(src));
-        }
-    }
-    if (blockIdx.x == 0)   // field history for the matched filter
-        for (int i = t; i < kEHist; i += blockDim.x) {
-            long long n = g.e_prev - kEHist + i;
-            E[i] = (n < 0) ? make_float2(0.f, 0.f) : E_prev[n - g.ebase_prev];
-        }
+    if (pk.hist_next) copy_hist(pk, blockIdx.x, gridDim.x);
+    if (blockIdx.x == 0) carry_field(g, E, E_prev);
     __syncthreads();   // staged twiddles
 
     // ---- A: forward column DFTs, scattered to the row owners
@@ -787,12 +882,7 @@ __global__ void __cluster_dims__(kClC, 1, 1) __launch_bounds__(kClThreads, 3)
 __global__ void k_kk_hist(KkPacked pk)
 {
     if (pk.lat && blockIdx.x == 0 && threadIdx.x == 0) lat_start(pk.lat, pk.lat_slot);
-    long long nch = pk.hist_bytes / 16;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < nch; c += (long long)gridDim.x * blockDim.x) {
-        long long vb = pk.in_bytes + 16 * c;
-        const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
-        reinterpret_cast<uint4 *>(pk.hist_next)[c] = __ldg(reinterpret_cast<const uint4 *>(src));
-    }
+    copy_hist(pk, blockIdx.x, gridDim.x);
 }
 
 cudaError_t launch_kk_hist(const KkInput &inp, cudaStream_t st, const KkSync &sync)
@@ -815,7 +905,12 @@ cudaError_t launch_kk_hist(const KkInput &inp, cudaStream_t st, const KkSync &sy
 
 cudaError_t prepare_kk_front()
 {
-    return cudaFuncSetAttribute(k_kk_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_kk_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_kk_block<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, BkSmem::TOTAL);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_kk_block<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, BkSmem::TOTAL);
+    return e;
 }
 
 cudaError_t launch_kk_front(const KkGeom &g, const KkInput &inp, float2 *fftws, const KkTables &tb,
@@ -844,40 +939,34 @@ cudaError_t launch_kk_front(const KkGeom &g, const KkInput &inp, float2 *fftws, 
         prof_stage(prof, -4, st);
         return cudaGetLastError();
     }
-    dim3 grid(g.N2 / kCtaK1, g.npairs);
-    dim3 grid_a(g.N2 / kCtaK1, g.npairs + (inp.hist_next ? 1 : 0));
+    if (g.N2 == kBkN2) {
+        // 4096-point blocks: one kernel (profiled as the K1a stage)
+        if (sync.wait_fwd) cudaStreamWaitEvent(st, sync.wait_fwd, 0);
+        if (sync.wait_inv) cudaStreamWaitEvent(st, sync.wait_inv, 0);
+        prof_stage(prof, 1, st);
+        const unsigned grid = g.npairs + (inp.hist_next ? 1 : 0);
+        if (pk.order) k_kk_block<1><<<grid, kCtaK1, BkSmem::TOTAL, st>>>(g, pk, tb, E, E_prev, dst);
+        else k_kk_block<0><<<grid, kCtaK1, BkSmem::TOTAL, st>>>(g, pk, tb, E, E_prev, dst);
+        if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
+        prof_stage(prof, -2, st);
+        prof_stage(prof, -3, st);
+        prof_stage(prof, -4, st);
+        return cudaGetLastError();
+    }
+    if (g.N2 != kRowN2) return cudaErrorInvalidValue;   // N is 65536 or 4096
+    dim3 grid(kRowN2 / kCtaK1, g.npairs);
+    dim3 grid_a(kRowN2 / kCtaK1, g.npairs + (inp.hist_next ? 1 : 0));
     if (sync.wait_fwd) cudaStreamWaitEvent(st, sync.wait_fwd, 0);
     prof_stage(prof, 1, st);
-    if (g.N2 != 4096 && g.N2 != 256) return cudaErrorInvalidValue;   // N is 65536 or 4096
-    const bool long_rows = g.N2 == 4096;
-    if (pk.order) {
-        if (long_rows) k_kk_fwd<1, 4096><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
-        else k_kk_fwd<1, 256><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
-    } else {
-        if (long_rows) k_kk_fwd<0, 4096><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
-        else k_kk_fwd<0, 256><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
-    }
+    if (pk.order) k_kk_fwd<1, kRowN2><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
+    else k_kk_fwd<0, kRowN2><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
     if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
     prof_stage(prof, -2, st);
-    int rows = g.npairs * 16;
-    if (g.N2 == 4096) {
-        size_t smem = (size_t)(4096 + 256) * sizeof(float2);
-        k_kk_rows<3><<<rows, 256, smem, st>>>(g, fftws, tb.twN2);
-    } else if (g.N2 == 256) {
-        size_t smem = (size_t)16 * (256 + 16) * sizeof(float2);
-        k_kk_rows<2><<<(rows + 15) / 16, 256, smem, st>>>(g, fftws, tb.twN2);
-    } else {
-        k_kk_rows<1><<<(rows + 255) / 256, 256, 0, st>>>(g, fftws, tb.twN2);
-    }
+    k_kk_rows<<<g.npairs * 16, 256, kRowPad * sizeof(float2), st>>>(g, fftws, tb.twN2);
     if (sync.wait_inv) cudaStreamWaitEvent(st, sync.wait_inv, 0);
     prof_stage(prof, -3, st);
-    if (pk.order) {
-        if (long_rows) k_kk_inv<1, 4096><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
-        else k_kk_inv<1, 256><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
-    } else {
-        if (long_rows) k_kk_inv<0, 4096><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
-        else k_kk_inv<0, 256><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
-    }
+    if (pk.order) k_kk_inv<1, kRowN2><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
+    else k_kk_inv<0, kRowN2><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
     prof_stage(prof, -4, st);
     return cudaGetLastError();
 }

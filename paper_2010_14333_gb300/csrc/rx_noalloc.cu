@@ -25,9 +25,9 @@ constexpr size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 //   hist     the packed history the front end is handed; on a stream's first buffer it
 //            is never read for values (samples before the stream are the first sample
 //            replicated), so it only has to be a valid region of ols_n * 3 / 2 bytes
-//   fft      the two-block complex FFT rows, at most 2^19 complex values
-//   E        the field [kEHist history | buffer]
-//   state    the front end's reduction state (carrier sums and their ticket)
+//   fft      the two-block complex FFT rows of 2^16-point blocks, at most 2^19 complex values
+// The field goes straight to the caller's buffer: no field history is kept and no carrier
+// sums are taken.
 constexpr int kNaSizes = 2;
 constexpr size_t kTabBytes = 4096 * sizeof(float) + 1024 * sizeof(float2);   // >= one block
 constexpr size_t kOffTw = 0;
@@ -35,10 +35,7 @@ constexpr size_t kOffHist = align_up(kOffTw + kNaSizes * kTabBytes);
 constexpr size_t kHistBytes = (size_t)65536 * 3 / 2;
 constexpr size_t kOffFft = align_up(kOffHist + kHistBytes);
 constexpr size_t kFftBytes = 4u << 20;                   // two-block complex FFT rows
-constexpr size_t kOffE = align_up(kOffFft + kFftBytes);
-constexpr size_t kEBytes = (size_t)(kEHist + kNaMaxSamples) * sizeof(float2);
-constexpr size_t kOffState = align_up(kOffE + kEBytes);
-constexpr size_t kScratchBytes = align_up(kOffState + sizeof(DevState));
+constexpr size_t kScratchBytes = align_up(kOffFft + kFftBytes);
 
 // One scratch region per GPU that loads the library (held until the process exits).
 // Every call uses it, so calls that overlap on the GPU race with each other.
@@ -80,19 +77,14 @@ cudaError_t setup_device(int dev, cudaStream_t st, unsigned char **out)
         float2 *t1 = (float2 *)(ln + 4096), *t2 = t1 + kk_tw_entries(sizes[i]);
         kk_host_tables(sizes[i], ln, t1, t2);
     }
-    e = cudaMemcpyAsync((unsigned char *)p + kOffTw, blk, sizeof blk, cudaMemcpyHostToDevice, st);
+    e = prepare_kk_front();
+    if (e == cudaSuccess) e = cudaMemcpyAsync((unsigned char *)p + kOffTw, blk, sizeof blk, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
     g_dev_ptr[dev] = (unsigned char *)p;
     g_ready[dev].store(true, std::memory_order_release);
     *out = (unsigned char *)p;
     return cudaSuccess;
-}
-
-__global__ void k_na_copy_field(const float2 *__restrict__ src, float2 *__restrict__ dst, long long n)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = src[i];
 }
 
 }  // namespace
@@ -118,8 +110,7 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
     g.e_k = e_k;
     g.avail = nsamp;
     g.cbase = -(long long)ols_n;        // stream index of the packed history's first sample
-    g.ebase = -kEHist;                  // field: [kEHist history | buffer]
-    g.ebase_prev = -kEHist;
+    g.ebase = 0;                        // the field starts with stream sample 0
     g.sps = 4;
     g.slot = 0;
     size_t need_fft = (size_t)g.npairs * ols_n * sizeof(float2);
@@ -137,10 +128,6 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
     tb.twN2 = tb.twN + kk_tw_entries(ols_n);
     const uint8_t *hist = base + kOffHist;
     float2 *fftws = (float2 *)(base + kOffFft);
-    float2 *E = (float2 *)(base + kOffE);
-    DevState *ds = (DevState *)(base + kOffState);
-    // the carrier sums and the last-CTA ticket of their reduction must start at zero
-    if (cudaMemsetAsync(ds, 0, sizeof(DevState), st) != cudaSuccess) return RX_ECUDA;
     KkInput kin;
     kin.hist = hist;                        // never read for values: the first call fills the pre-stream
     kin.in = packed12_in;
@@ -152,9 +139,8 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
     kin.lat = nullptr;
     kin.lat_slot = 0;
     const KkSync none = {nullptr, nullptr, nullptr};
-    if (launch_kk_front(g, kin, fftws, tb, E, E, ds, st, nullptr, none) != cudaSuccess) return RX_ECUDA;
-    unsigned grid = (unsigned)((e_k + 255) / 256);
-    k_na_copy_field<<<grid, 256, 0, st>>>(E + kEHist, reinterpret_cast<float2 *>(field_out), e_k);
-    if (cudaGetLastError() != cudaSuccess) return RX_ECUDA;
+    if (launch_kk_front(g, kin, fftws, tb, reinterpret_cast<float2 *>(field_out), nullptr, nullptr, st, nullptr, none) !=
+        cudaSuccess)
+        return RX_ECUDA;
     return RX_OK;
 }
