@@ -946,6 +946,9 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     cudaError_t stale = cudaGetLastError();
     if (stale != cudaSuccess) traced(stale, "an earlier CUDA call (cleared)");
     const bool two = sf != sb;
+    // one stream: kernel follows kernel, so each may start while the one before it drains
+    // (not in the pipeline, whose stages are ordered by events, nor between stage events)
+    const bool pdl = !two && !h->in_group && h->prof_on <= 0;
     // in the pipeline the filter runs on a third stream between the front end (KK field,
     // PAM unpack) and the equaliser (back); field and codes slots wait for it to be done
     const bool three = two && smid;
@@ -963,7 +966,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     // and a second field in flight holds SMs it waits for.
     const bool alt = three && h->kk && h->front2 && !h->cnn;
     if (alt && par) sf = h->front2;
-    const KkSync ksync = {alt ? h->ev_hist : nullptr, alt ? h->ev_hist : nullptr, alt ? h->ev_front : nullptr};
+    const KkSync ksync = {alt ? h->ev_hist : nullptr, alt ? h->ev_hist : nullptr, alt ? h->ev_front : nullptr, pdl};
     if (host_in) {
         in = h->in_stage[isl];
         if (sc != sf) cudaStreamWaitEvent(sc, h->ev_infree[isl], 0);   // the front end kInSlots calls back is done
@@ -989,7 +992,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
         const bool sums = !h->kk && !h->flush_mode;
         e = launch_unpack(in, h->codes[cw_new], h->codes[h->cw], h->nb, h->nhist, h->nb, h->calls == 0,
                           c.pack_order, sums ? &h->st->pam_s1[spar] : nullptr,
-                          sums ? &h->st->pam_s2[spar] : nullptr, sf, lat_first, lat_slot);
+                          sums ? &h->st->pam_s2[spar] : nullptr, sf, lat_first, lat_slot, pdl);
         lat_first = nullptr;   // stamped: the KK front end (debug view) comes after
         h->cw = cw_new;
         prof_end(h, 0, sf);
@@ -1070,21 +1073,21 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
         if (h->kk && h->fd)
             e = launch_kk_fdmf(Ef, efbase, h->f_prev, s.f_k, c.fd_n, h->fd_H, h->fd_tw, h->ds_tab,
                                c.ds_num, c.ds_den, cgp, (float2 *)h->Y[yw_new], yb,
-                               (const float2 *)h->Y[h->yw], h->ybase_cur, sm, h->clk, h->clk_w);
+                               (const float2 *)h->Y[h->yw], h->ybase_cur, sm, h->clk, h->clk_w, pdl);
         else if (h->kk)
             e = launch_kk_mf(Ef, efbase, s.r_k, h->f_prev, s.f_k, h->rrc, h->hmf, h->ds_tab, c.ds_num,
                              c.ds_den, cgp, (float2 *)h->Y[yw_new], yb, (const float2 *)h->Y[h->yw],
-                             h->ybase_cur, sm, h->rrc_host);
+                             h->ybase_cur, sm, h->rrc_host, pdl);
         else if (h->rs)
             e = launch_pam_mf_r(h->R[h->rw], h->rbase_cur, h->f_prev, s.f_k, h->rrc, h->hmf, (float *)h->Y[yw_new], yb,
                                 (const float *)h->Y[h->yw], h->ybase_cur, sm);
         else if (h->fd)
             e = launch_pam_fd1024(h->codes[h->cw], cbase, h->nb, s.avail, h->f_prev, s.f_k, h->fd_H, h->fd_tw, h->st,
                                   ppar, (float *)h->Y[yw_new], yb, (const float *)h->Y[h->yw], h->ybase_cur, sm,
-                                  h->clk, h->clk_w);
+                                  h->clk, h->clk_w, pdl);
         else
             e = launch_pam_mf(h->codes[h->cw], cbase, h->nb, s.avail, h->f_prev, s.f_k, h->rrc, h->hmf, h->st, ppar,
-                              (float *)h->Y[yw_new], yb, (const float *)h->Y[h->yw], h->ybase_cur, sm);
+                              (float *)h->Y[yw_new], yb, (const float *)h->Y[h->yw], h->ybase_cur, sm, pdl);
         if (e == cudaSuccess && h->fd && c.clk_track) {
             // blocks of this call: outputs at 2 samples/symbol per block N/4 (KK) or N/2 (PAM)
             const long long per = h->kk ? c.fd_n / 4 : c.fd_n / 2;
@@ -1128,7 +1131,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     prof_begin(h, 5, sb);
     if (e == cudaSuccess && do_train) {
         e = launch_eq(h->ep, g, 1, h->Y[h->yw], nullptr, h->taps[h->tw], nullptr, h->dec[ds], h->winb[ds], h->winrec[ds],
-                      nullptr, h->dbg_z, h->prbs, h->prbs_bits, h->st, sb);
+                      nullptr, h->dbg_z, h->prbs, h->prbs_bits, h->st, sb, pdl);
         h->trained = 1;
     }
     if (e == cudaSuccess && g.nblk > 0) {
@@ -1138,18 +1141,18 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
             e = launch_cnn_decide(rx_cnn_dev_params(h->cnn), (const float2 *)h->Y[h->yw], seg_base, s.f_k - h->ybase_cur, g.nwin, h->dec[ds],
                                   h->winb[ds], h->winrec[ds], h->prbs_bits, pay_lo, h->ep.scale, h->mq,
                                   h->dbg_z ? h->dbg_z + (pay_lo - sym_lo) : nullptr, &h->st->err, h->nsm, sb,
-                                  c.cnn_bf16);
+                                  c.cnn_bf16, pdl);
         } else {
             const float2 *zin = nullptr;
             if (c.fir_prec >= RX_FIR_BF16) {
                 // frozen taps: the whole payload's filter as one tensor-core GEMM
                 e = launch_fir_tc(c.fir_prec, (const float2 *)h->Y[h->yw], h->ybase_cur, pay_lo, npay,
-                                  h->taps[h->tw], c.ntaps, c.eq_block, h->zbuf, &h->st->err, h->nsm, sb);
+                                  h->taps[h->tw], c.ntaps, c.eq_block, h->zbuf, &h->st->err, h->nsm, sb, pdl);
                 zin = h->zbuf;
             }
             if (e == cudaSuccess)
                 e = launch_eq(h->ep, g, 0, h->Y[h->yw], zin, h->taps[h->tw], h->taps[h->tw ^ 1], h->dec[ds],
-                              h->winb[ds], h->winrec[ds], h->dbg_win, h->dbg_z, h->prbs, h->prbs_bits, h->st, sb);
+                              h->winb[ds], h->winrec[ds], h->dbg_win, h->dbg_z, h->prbs, h->prbs_bits, h->st, sb, pdl);
             h->tw ^= 1;
         }
     }
@@ -1161,7 +1164,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
         prof_begin(h, 6, st4);
         int resolve = h->kk && !h->amb_done;
         e = launch_demap(h->ep, g, resolve, h->uw, h->dec[ds], h->winb[ds], h->winrec[ds], h->dbg_win, bits_out,
-                         h->prbs_bits, h->st, st4);
+                         h->prbs_bits, h->st, st4, pdl);
         if (h->kk) h->uw ^= 1;
         h->amb_done = 1;
         prof_end(h, 6, st4);
@@ -1738,7 +1741,7 @@ rx_status rx_fir_block(const float *y, int64_t ny, const float *w, int ntaps, in
         return RX_ECUDA;
     cudaError_t e = launch_fir_tc(prec, (const float2 *)y, -(long long)((ntaps - 1) / 2), 0, nsym,
                                   (const float2 *)w, ntaps, scale_block, (float2 *)z_out, (int *)status, nsm,
-                                  (cudaStream_t)stream);
+                                  (cudaStream_t)stream, true);
     return e == cudaSuccess ? RX_OK : RX_ECUDA;
 }
 

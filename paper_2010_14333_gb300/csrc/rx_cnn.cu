@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(kFwThreads, kFwPerSm)
         cp_async_commit();
     };
     int s = blockIdx.x;
+    pdl_wait();
     if (s < nseg) prefetch(s, 0);
     stage_w<kFwThreads>(sm + FwdSmem::W2, prm_bf + OW2, tid);
     stage_w<kFwThreads>(sm + FwdSmem::W3, prm_bf + OW3, tid);
@@ -413,6 +414,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
     float *G = gpart + (size_t)s * NPRM;
 
     // ---- stage: the input and what layer 1 needs first, the weights behind it
+    pdl_wait();
     stage_w<kTrThreads>(sm + TrainSmem::W2, prm_bf + OW2, tid);
     stage_w<kTrThreads>(sm + TrainSmem::W3, prm_bf + OW3, tid);
     for (int i = tid; i < CH * 4; i += kTrThreads)
@@ -748,6 +750,7 @@ __global__ void __launch_bounds__(kRedThreads)
     k_cnn_reduce(const float *__restrict__ gpart, const float *__restrict__ lpart, int nseg, float norm,
                  float *__restrict__ grad, float *grad_out, float *__restrict__ loss, float *loss_out)
 {
+    pdl_wait();
     if (blockIdx.x == gridDim.x - 1) {
         __shared__ float part[kRedThreads / 32];
         float a = 0.f;
@@ -776,6 +779,7 @@ __global__ void k_cnn_adam(float *__restrict__ prm, __nv_bfloat16 *__restrict__ 
                            float *__restrict__ m, float *__restrict__ v, const float *__restrict__ grad, float lr,
                            float b1t, float b2t)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NPRM) return;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -960,6 +964,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
     if (gtid == 0) mbar_init(bar, 1);
     __syncwarp();
     if (warp == 0) tmem_alloc(tslot, kRxTmem);
+    pdl_wait();
     // weights: B operands as K-major planes (chunk (row n, K column kk) at kk * rows * 16 + n * 16)
     // 8 FP32 weights of a layer that reads GELU outputs -> 16 bytes of FP16 / BF16,
     // halved (the epilogues store 2 GELU(u))
@@ -1252,18 +1257,13 @@ cudaError_t prepare_cnn_rx()
 cudaError_t launch_cnn_decide(const float *prm, const float2 *y, long long seg_base, long long y_end,
                               int nwin, uint8_t *dec, uint8_t *winb, uint4 *winrec, const uint32_t *prbs_bits,
                               long long k_first, float scale, int mq, float2 *soft, int *err, int nsm, cudaStream_t st,
-                              int bf16)
+                              int bf16, bool pdl)
 {
     if (nwin <= 0) return cudaSuccess;
     int ntiles = (nwin + kWinT - 1) / kWinT, nctas = (ntiles + kRxGroups - 1) / kRxGroups;
     unsigned grid = (unsigned)(nctas < nsm ? nctas : nsm);   // one persistent CTA per SM
-    if (bf16)
-        k_cnn_rx_tc<true><<<grid, kRxThreads, RxSmem::TOTAL, st>>>(prm, y, seg_base, y_end, nwin, dec, winb, winrec,
-                                                                  prbs_bits, k_first, scale, mq, soft, err);
-    else
-        k_cnn_rx_tc<false><<<grid, kRxThreads, RxSmem::TOTAL, st>>>(prm, y, seg_base, y_end, nwin, dec, winb, winrec,
-                                                                   prbs_bits, k_first, scale, mq, soft, err);
-    return cudaGetLastError();
+    return launch_k(bf16 ? k_cnn_rx_tc<true> : k_cnn_rx_tc<false>, grid, kRxThreads, RxSmem::TOTAL, st, pdl, prm, y, seg_base,
+                    y_end, nwin, dec, winb, winrec, prbs_bits, k_first, scale, mq, soft, err);
 }
 
 }  // namespace rxk
@@ -1352,9 +1352,10 @@ rx_status rx_cnn_forward(rx_cnn *c, const float *y, const int64_t *seg_start, in
 {
     if (!c || !y || !seg_start || !out || nseg <= 0) return RX_EINVAL;
     const int grid = nseg < kFwPerSm * c->nsm ? nseg : kFwPerSm * c->nsm;   // persistent CTAs
-    k_cnn_fwd<<<grid, kFwThreads, FwdSmem::TOTAL, (cudaStream_t)stream>>>(c->prm, c->prm_bf, (const float2 *)y,
-                                                                          (const long long *)seg_start, nseg, out);
-    return cudaGetLastError() == cudaSuccess ? RX_OK : RX_ECUDA;
+    return launch_k(k_cnn_fwd, grid, kFwThreads, FwdSmem::TOTAL, (cudaStream_t)stream, true, c->prm, c->prm_bf, (const float2 *)y,
+                    (const long long *)seg_start, nseg, out) == cudaSuccess
+               ? RX_OK
+               : RX_ECUDA;
 }
 
 rx_status rx_cnn_grad(rx_cnn *c, const float *y, const int64_t *seg_start, const float *tgt, int nseg, float *grad_out,
@@ -1363,15 +1364,17 @@ rx_status rx_cnn_grad(rx_cnn *c, const float *y, const int64_t *seg_start, const
     if (!c || !y || !seg_start || !tgt || nseg <= 0 || nseg > c->max_seg) return RX_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     float norm = 1.f / ((float)nseg * CS);
-    k_cnn_train<<<nseg, kTrThreads, TrainSmem::TOTAL, st>>>(c->prm, c->prm_bf, (const float2 *)y,
-                                                           (const long long *)seg_start, tgt, norm, c->gpart, c->lpart);
+    cudaError_t e = launch_k(k_cnn_train, nseg, kTrThreads, TrainSmem::TOTAL, st, true, c->prm, c->prm_bf, (const float2 *)y,
+                             (const long long *)seg_start, tgt, norm, c->gpart, c->lpart);
     // the caller's buffers are written by the reduction itself where they are aligned
     float *go = ((uintptr_t)grad_out & 3) ? nullptr : grad_out, *lo = ((uintptr_t)loss_out & 3) ? nullptr : loss_out;
-    k_cnn_reduce<<<(NPRM + kRedThreads - 1) / kRedThreads + 1, kRedThreads, 0, st>>>(c->gpart, c->lpart, nseg, norm,
-                                                                                   c->grad, go, c->loss, lo);
-    if (grad_out && !go) cudaMemcpyAsync(grad_out, c->grad, NPRM * 4, cudaMemcpyDeviceToDevice, st);
-    if (loss_out && !lo) cudaMemcpyAsync(loss_out, c->loss, 4, cudaMemcpyDeviceToDevice, st);
-    return cudaGetLastError() == cudaSuccess ? RX_OK : RX_ECUDA;
+    if (e == cudaSuccess)
+        e = launch_k(k_cnn_reduce, (NPRM + kRedThreads - 1) / kRedThreads + 1, kRedThreads, 0, st, true, c->gpart, c->lpart,
+                     nseg, norm, c->grad, go, c->loss, lo);
+    if (e == cudaSuccess && grad_out && !go)
+        e = cudaMemcpyAsync(grad_out, c->grad, NPRM * 4, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess && loss_out && !lo) e = cudaMemcpyAsync(loss_out, c->loss, 4, cudaMemcpyDeviceToDevice, st);
+    return e == cudaSuccess ? RX_OK : RX_ECUDA;
 }
 
 rx_status rx_cnn_adam_step(rx_cnn *c, float lr, void *stream)
@@ -1379,9 +1382,10 @@ rx_status rx_cnn_adam_step(rx_cnn *c, float lr, void *stream)
     if (!c || !(lr > 0)) return RX_EINVAL;
     c->step++;
     float b1t = powf(0.9f, (float)c->step), b2t = powf(0.999f, (float)c->step);
-    k_cnn_adam<<<(NPRM + 255) / 256, 256, 0, (cudaStream_t)stream>>>(c->prm, c->prm_bf, c->m, c->v, c->grad,
-                                                                     lr, b1t, b2t);
-    return cudaGetLastError() == cudaSuccess ? RX_OK : RX_ECUDA;
+    return launch_k(k_cnn_adam, (NPRM + 255) / 256, 256, 0, (cudaStream_t)stream, true, c->prm, c->prm_bf, c->m, c->v, c->grad,
+                    lr, b1t, b2t) == cudaSuccess
+               ? RX_OK
+               : RX_ECUDA;
 }
 
 // device pointers of the parameters (for the receiver's CNN path)

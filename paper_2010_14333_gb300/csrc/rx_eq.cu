@@ -361,6 +361,7 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
          const uint32_t *__restrict__ prbs_bits, DevState *dst)
 {
     typedef typename std::conditional<QAM, float2, float>::type T;
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     const T *Y = reinterpret_cast<const T *>(Yv);
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -473,6 +474,7 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
                 uint8_t *__restrict__ winb, uint4 *__restrict__ winrec, float4 *__restrict__ dbg_win,
                 float2 *__restrict__ dbg_z, const uint32_t *__restrict__ prbs_bits, DevState *dst)
 {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int ylen = 2 * kWin + 2 * kYHist;
@@ -557,13 +559,12 @@ template <bool QAM, int NT, int MQ>
 static cudaError_t launch_eq_t(const EqParams &p, const EqGeom &g, int train, const void *Y, const float2 *zin,
                                float2 *taps_in, float2 *taps_out, uint8_t *dec, uint8_t *winb, uint4 *winrec,
                                float4 *dbg_win, float2 *dbg_z, const uint8_t *prbs, const uint32_t *prbs_bits,
-                               DevState *dst, cudaStream_t st)
+                               DevState *dst, cudaStream_t st, bool pdl)
 {
     if (train) {
         size_t smem = eq_smem_per_warp(QAM, kWin);
-        k_eq<QAM, NT, MQ><<<1, 32, smem, st>>>(p, g, 1, Y, taps_in, taps_out, dec, winb, winrec, dbg_win, dbg_z,
-                                               prbs, prbs_bits, dst);
-        return cudaGetLastError();
+        return launch_k(k_eq<QAM, NT, MQ>, 1, 32, smem, st, pdl, p, g, 1, Y, taps_in, taps_out, dec, winb, winrec, dbg_win,
+                        dbg_z, prbs, prbs_bits, dst);
     }
     if constexpr (QAM) {
         if (p.frozen) {
@@ -573,16 +574,14 @@ static cudaError_t launch_eq_t(const EqParams &p, const EqGeom &g, int train, co
             cudaError_t e = cudaMemsetAsync(&dst->eq_ticket, 0, sizeof(unsigned), st);
             if (e != cudaSuccess) return e;
             unsigned grid = (unsigned)((g.nwin + p.warps - 1) / p.warps);
-            k_eq_frozen<NT, MQ><<<grid, 32 * p.warps, eq_smem_frozen_per_warp() * p.warps, st>>>(
-                p, g, (const float2 *)Y, zin, taps_in, taps_out, dec, winb, winrec, dbg_win, dbg_z, prbs_bits, dst);
-            return cudaGetLastError();
+            return launch_k(k_eq_frozen<NT, MQ>, grid, 32 * p.warps, eq_smem_frozen_per_warp() * p.warps, st, pdl, p, g,
+                            (const float2 *)Y, zin, taps_in, taps_out, dec, winb, winrec, dbg_win, dbg_z, prbs_bits, dst);
         }
     }
     size_t smem = eq_smem_per_warp(QAM, p.eq_block) * p.warps;
     unsigned grid = (unsigned)((g.nblk + p.warps - 1) / p.warps);
-    k_eq<QAM, NT, MQ><<<grid, 32 * p.warps, smem, st>>>(p, g, 0, Y, taps_in, taps_out, dec, winb, winrec, dbg_win,
-                                                          dbg_z, prbs, prbs_bits, dst);
-    return cudaGetLastError();
+    return launch_k(k_eq<QAM, NT, MQ>, grid, 32 * p.warps, smem, st, pdl, p, g, 0, Y, taps_in, taps_out, dec, winb, winrec,
+                    dbg_win, dbg_z, prbs, prbs_bits, dst);
 }
 
 // shared-memory attribute of the payload kernel, set to the largest CTA any
@@ -770,7 +769,8 @@ cudaError_t prepare_eq(const EqParams &p)
 
 cudaError_t launch_eq(const EqParams &p, const EqGeom &g, int train, const void *Y, const float2 *zin,
                       float2 *taps_in, float2 *taps_out, uint8_t *dec, uint8_t *winb, uint4 *winrec, float4 *dbg_win,
-                      float2 *dbg_z, const uint8_t *prbs, const uint32_t *prbs_bits, DevState *dst, cudaStream_t st)
+                      float2 *dbg_z, const uint8_t *prbs, const uint32_t *prbs_bits, DevState *dst, cudaStream_t st,
+                      bool pdl)
 {
     if (p.dd) {
         const float2 *Yc = (const float2 *)Y;
@@ -788,15 +788,15 @@ cudaError_t launch_eq(const EqParams &p, const EqGeom &g, int train, const void 
 #define RX_CASE(NTV)                                                                                           \
     if (p.ntaps == NTV) {                                                                                      \
         if (p.kk && p.mq == 2) return launch_eq_t<true, NTV, 2>(p, g, train, Y, zin, taps_in, taps_out, dec, winb,  \
-                                                                winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st);                \
+                                                                winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st, pdl);                \
         if (p.kk && p.mq == 4) return launch_eq_t<true, NTV, 4>(p, g, train, Y, zin, taps_in, taps_out, dec, winb,  \
-                                                                winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st);                \
+                                                                winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st, pdl);                \
         if (!p.kk && p.mq == 2) return launch_eq_t<false, NTV, 2>(p, g, train, Y, zin, taps_in, taps_out, dec,      \
-                                                                  winb, winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st);        \
+                                                                  winb, winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st, pdl);        \
         if (!p.kk && p.mq == 4) return launch_eq_t<false, NTV, 4>(p, g, train, Y, zin, taps_in, taps_out, dec,      \
-                                                                  winb, winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st);        \
+                                                                  winb, winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st, pdl);        \
         if (!p.kk && p.mq == 8) return launch_eq_t<false, NTV, 8>(p, g, train, Y, zin, taps_in, taps_out, dec,      \
-                                                                  winb, winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st);        \
+                                                                  winb, winrec, dbg_win, dbg_z, prbs, prbs_bits, dst, st, pdl);        \
     }
     RX_EQ_TAPS(RX_CASE)
 #undef RX_CASE
@@ -860,6 +860,7 @@ __global__ void __launch_bounds__(kDemapThreads)
     __shared__ int s_red[NW];
     __shared__ int s_r;
     __shared__ unsigned s_cnt[C_NCNT];
+    pdl_wait();
     int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     int w0 = blockIdx.x * kDemapWin;
     int wend = min(w0 + kDemapWin, g.nwin);
@@ -1107,19 +1108,20 @@ __global__ void __launch_bounds__(kDemapThreads)
 
 cudaError_t launch_demap(const EqParams &p, const EqGeom &g, int resolve_amb, int uw_in, const uint8_t *dec,
                          const uint8_t *winb, const uint4 *winrec, float4 *dbg_win, uint8_t *bits_out,
-                         const uint32_t *prbs_bits, DevState *dst, cudaStream_t st)
+                         const uint32_t *prbs_bits, DevState *dst, cudaStream_t st, bool pdl)
 {
+    cudaError_t e;
     unsigned grid = (unsigned)((g.nwin + kDemapWin - 1) / kDemapWin);
 #define RX_DEMAP(Q, B, M)                                                                                   \
-    k_demap<Q, B, M><<<grid, kDemapThreads, 0, st>>>(p, g, resolve_amb, uw_in, dec, winb, winrec, dbg_win,  \
-                                                     bits_out, prbs_bits, dst)
+    e = launch_k(k_demap<Q, B, M>, grid, kDemapThreads, 0, st, pdl, p, g, resolve_amb, uw_in, dec, winb, winrec,  \
+                 dbg_win, bits_out, prbs_bits, dst)
     if (p.kk && p.mq == 4) RX_DEMAP(true, 4, 4);
     else if (p.kk) RX_DEMAP(true, 2, 2);
     else if (p.mq == 2) RX_DEMAP(false, 1, 2);
     else if (p.mq == 4) RX_DEMAP(false, 2, 4);
     else RX_DEMAP(false, 3, 8);
 #undef RX_DEMAP
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace rxk

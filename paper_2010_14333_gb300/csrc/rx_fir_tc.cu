@@ -137,10 +137,11 @@ __global__ void __launch_bounds__(kT8Threads, kT8PerSm)
         }
     };
     int t = blockIdx.x;
-    if (tid < 32) s_w[tid] = tid < ntaps ? __ldg(taps + tid) : make_float2(0.f, 0.f);
-    if (t < ntiles) load_tile(t);
     if (tid == 0) mbar_init(bar, 1);
     if (warp == 0) tmem_alloc(tslot, kTmemCols);
+    pdl_wait();
+    if (tid < 32) s_w[tid] = tid < ntaps ? __ldg(taps + tid) : make_float2(0.f, 0.f);
+    if (t < ntiles) load_tile(t);
     __syncthreads();   // the taps in shared memory
     // B: Toeplitz matrix of the taps, rows n = 2 j + c (c: re / im output of symbol j), K
     // index 2 s + d (d: re / im of input s); tap i = 2 j + 2 TH - s
@@ -316,10 +317,11 @@ __global__ void __launch_bounds__(kT2Threads, kT2PerSm)
         }
     };
     int t = blockIdx.x;
-    if (tid < 32) s_w[tid] = tid < ntaps ? __ldg(taps + tid) : make_float2(0.f, 0.f);
-    if (t < ntiles) load_tile(t);
     if (tid == 0) mbar_init(bar, 1);
     if (warp == 0) tmem_alloc(tslot, kTmemCols);
+    pdl_wait();
+    if (tid < 32) s_w[tid] = tid < ntaps ? __ldg(taps + tid) : make_float2(0.f, 0.f);
+    if (t < ntiles) load_tile(t);
     __syncthreads();   // the taps in shared memory
     // B: rows n = 2 j + c (c: re / im output of symbol j), K index k = 64 h + 2 s + d
     // (block row r + h, sample s, d: re / im); sample 32 h + s of the pair is stream
@@ -412,7 +414,7 @@ cudaError_t prepare_fir_tc(int prec)
 
 cudaError_t launch_fir_tc(int prec, const float2 *Y, long long ybase, long long k_lo, long long nsym,
                           const float2 *taps, int ntaps, int scale_block, float2 *z, int *err, int nsm,
-                          cudaStream_t st)
+                          cudaStream_t st, bool pdl)
 {
     if (nsym <= 0) return cudaSuccess;
     if (nsym % kRowSyms || ntaps < 1 || ntaps > 31 || !(ntaps & 1) || scale_block % kRowSyms ||
@@ -423,16 +425,12 @@ cudaError_t launch_fir_tc(int prec, const float2 *Y, long long ybase, long long 
     int ntiles = (nrows + kTileRows - 1) / kTileRows;
     if (prec == RX_FIR_BF16 || prec == RX_FIR_FP16) {
         const unsigned g2 = (unsigned)min(ntiles, kT2PerSm * nsm);   // persistent CTAs
-        if (prec == RX_FIR_BF16)
-            k_fir_tc2<RX_FIR_BF16><<<g2, kT2Threads, kT2Smem, st>>>(Y, ybase, k_lo, nrows, taps, ntaps, z, err);
-        else
-            k_fir_tc2<RX_FIR_FP16><<<g2, kT2Threads, kT2Smem, st>>>(Y, ybase, k_lo, nrows, taps, ntaps, z, err);
-        return cudaGetLastError();
+        return launch_k(prec == RX_FIR_BF16 ? k_fir_tc2<RX_FIR_BF16> : k_fir_tc2<RX_FIR_FP16>, g2, kT2Threads, kT2Smem, st,
+                        pdl, Y, ybase, k_lo, nrows, taps, ntaps, z, err);
     }
     if (prec != RX_FIR_FP8) return cudaErrorInvalidValue;
     const unsigned g8 = (unsigned)min(ntiles, kT8PerSm * nsm);   // persistent CTAs
-    k_fir_tc8<<<g8, kT8Threads, kT8Smem, st>>>(Y, ybase, k_lo, nrows, taps, ntaps, rps, z, err);
-    return cudaGetLastError();
+    return launch_k(k_fir_tc8, g8, kT8Threads, kT8Smem, st, pdl, Y, ybase, k_lo, nrows, taps, ntaps, rps, z, err);
 }
 
 }  // namespace rxk

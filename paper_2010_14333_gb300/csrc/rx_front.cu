@@ -41,6 +41,7 @@ __global__ void k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ 
                          long long prev_off, int first_call, int order, long long *s1,
                          long long *s2, LatRecord *lat, int lat_slot)
 {
+    pdl_wait();
     long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (lat && g == 0) lat_start(lat, lat_slot);
     long long ngroups = nb / 8;
@@ -102,14 +103,13 @@ __global__ void k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ 
 cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *codes_prev,
                           long long nb, int nhist, long long prev_off, int first_call,
                           int pack_order, long long *s1, long long *s2, cudaStream_t st, LatRecord *lat,
-                          int lat_slot)
+                          int lat_slot, bool pdl)
 {
     long long items = nb / 8 + nhist;
     int tpb = 256;
     unsigned grid = (unsigned)((items + tpb - 1) / tpb);
-    k_unpack<<<grid, tpb, 0, st>>>(in, codes, codes_prev, nb, nhist, prev_off, first_call,
-                                   pack_order, s1, s2, lat, lat_slot);
-    return cudaGetLastError();
+    return launch_k(k_unpack, grid, tpb, 0, st, pdl, in, codes, codes_prev, nb, nhist, prev_off, first_call, pack_order, s1,
+                    s2, lat, lat_slot);
 }
 
 // ============================================================= KK Hilbert
@@ -324,16 +324,18 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2
     __shared__ __align__(16) uint32_t raw[32][kRawWords];
     __shared__ __align__(16) float s_ln[kLutCodes];
     int pair = blockIdx.y;
+    const TwSmem tw = stage_tw(tb.twN, g.N, s_tw);
+    // the ln table in shared memory: a gather over 32 random codes costs a few bank
+    // conflicts there instead of one L1 wavefront per distinct cache line
+    if (pair < g.npairs)
+        for (int i = threadIdx.x; i < kLutCodes / 4; i += blockDim.x)
+            reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
+    pdl_wait();
     if (pk.lat && blockIdx.x == 0 && pair == 0 && threadIdx.x == 0) lat_start(pk.lat, pk.lat_slot);
     if (pair == g.npairs) {
         copy_hist(pk, blockIdx.x, gridDim.x);
         return;
     }
-    const TwSmem tw = stage_tw(tb.twN, g.N, s_tw);
-    // the ln table in shared memory: a gather over 32 random codes costs a few bank
-    // conflicts there instead of one L1 wavefront per distinct cache line
-    for (int i = threadIdx.x; i < kLutCodes / 4; i += blockDim.x)
-        reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
     const int c0 = blockIdx.x * blockDim.x;
     const bool hb = 2 * pair + 1 < g.J;
     stage_rows<N2T>(g, pk, pair, c0, raw, hb);
@@ -380,6 +382,7 @@ __global__ void __launch_bounds__(256, 3) k_kk_rows(KkGeom g, float2 *__restrict
     extern __shared__ float2 s[];                 // the padded row
     __shared__ float2 s_tw[128];
     const TwSmem tw2 = stage_tw(twN2g, N2, s_tw);
+    pdl_wait();
     __syncthreads();
     const int t = threadIdx.x, row = blockIdx.x, k2 = row & 15;
     float2 *d = fftws + (size_t)row * N2;
@@ -559,6 +562,7 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const 
     __shared__ float2 s_tw[512];
     __shared__ __align__(16) uint32_t raw[32][kRawWords];
     const TwSmem tw = stage_tw(tb.twN, g.N, s_tw);
+    pdl_wait();
     int pair = blockIdx.y;
     const int c0 = blockIdx.x * blockDim.x;
     const bool hb = 2 * pair + 1 < g.J;
@@ -611,15 +615,16 @@ __global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, c
     uint32_t(*raw)[kRawWords] = reinterpret_cast<uint32_t(*)[kRawWords]>(bksm + BkSmem::RAW);
     float2 *s_tw = reinterpret_cast<float2 *>(bksm + BkSmem::TW);
     const int pair = blockIdx.x, t = threadIdx.x;
+    const TwSmem tw = stage_tw(tb.twN, 16 * kBkN2, s_tw);
+    const TwSmem tw2 = stage_tw(tb.twN2, kBkN2, s_tw + 128);
+    for (int i = t; i < kLutCodes / 4; i += kCtaK1)
+        reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
+    pdl_wait();
     if (pk.lat && pair == 0 && t == 0) lat_start(pk.lat, pk.lat_slot);
     if (pair >= g.npairs) {
         copy_hist(pk, pair - g.npairs, gridDim.x - g.npairs);
         return;
     }
-    const TwSmem tw = stage_tw(tb.twN, 16 * kBkN2, s_tw);
-    const TwSmem tw2 = stage_tw(tb.twN2, kBkN2, s_tw + 128);
-    for (int i = t; i < kLutCodes / 4; i += kCtaK1)
-        reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
     const bool hb = 2 * pair + 1 < g.J;
     stage_rows<kBkN2>(g, pk, pair, 0, raw, hb);
     const uint32_t c_first = first_code(pk, dst);
@@ -726,6 +731,7 @@ __global__ void __cluster_dims__(kClC, 1, 1) __launch_bounds__(kClThreads, 3)
     float2 *rows = smc;                         // [2][kClRow]
     const TwSmem tw = stage_tw(tb.twN, g.N, smc + 2 * kClRow);
     const TwSmem tw2 = stage_tw(tb.twN2, kClN2, smc + 2 * kClRow + 512);
+    pdl_wait();
     const int c = (int)cl.block_rank();
     const int pair = blockIdx.x / kClC;
     const int t = threadIdx.x;
@@ -881,6 +887,7 @@ __global__ void __cluster_dims__(kClC, 1, 1) __launch_bounds__(kClThreads, 3)
 
 __global__ void k_kk_hist(KkPacked pk)
 {
+    pdl_wait();
     if (pk.lat && blockIdx.x == 0 && threadIdx.x == 0) lat_start(pk.lat, pk.lat_slot);
     copy_hist(pk, blockIdx.x, gridDim.x);
 }
@@ -898,9 +905,9 @@ cudaError_t launch_kk_hist(const KkInput &inp, cudaStream_t st, const KkSync &sy
     pk.first_call = inp.first_call;
     pk.lat = inp.lat;
     pk.lat_slot = inp.lat_slot;
-    k_kk_hist<<<32, 256, 0, st>>>(pk);
+    const cudaError_t e = launch_k(k_kk_hist, 32, 256, 0, st, sync.pdl, pk);
     if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t prepare_kk_front()
@@ -927,48 +934,41 @@ cudaError_t launch_kk_front(const KkGeom &g, const KkInput &inp, float2 *fftws, 
     pk.first_call = inp.first_call;
     pk.lat = inp.lat;
     pk.lat_slot = inp.lat_slot;
-    if (g.N2 == kClN2 && g.fused) {
-        // 2^16-point blocks: the fused cluster kernel (profiled as the K1a stage)
-        if (sync.wait_fwd) cudaStreamWaitEvent(st, sync.wait_fwd, 0);
+    cudaError_t e = cudaSuccess;
+    if (sync.wait_fwd) cudaStreamWaitEvent(st, sync.wait_fwd, 0);
+    if ((g.N2 == kClN2 && g.fused) || g.N2 == kBkN2) {
+        // one kernel: the cluster form of 2^16-point blocks or the one-CTA form of
+        // 4096-point blocks (profiled as the K1a stage)
         if (sync.wait_inv) cudaStreamWaitEvent(st, sync.wait_inv, 0);
         prof_stage(prof, 1, st);
-        k_kk_cluster<<<g.npairs * kClC, kClThreads, kClSmem, st>>>(g, pk, tb, E, E_prev, dst);
+        if (g.N2 == kClN2)
+            e = launch_k(k_kk_cluster, g.npairs * kClC, kClThreads, kClSmem, st, sync.pdl, g, pk, tb, E, E_prev, dst);
+        else
+            e = launch_k(pk.order ? k_kk_block<1> : k_kk_block<0>, g.npairs + (inp.hist_next ? 1 : 0), kCtaK1,
+                         BkSmem::TOTAL, st, sync.pdl, g, pk, tb, E, E_prev, dst);
         if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
         prof_stage(prof, -2, st);
         prof_stage(prof, -3, st);
         prof_stage(prof, -4, st);
-        return cudaGetLastError();
-    }
-    if (g.N2 == kBkN2) {
-        // 4096-point blocks: one kernel (profiled as the K1a stage)
-        if (sync.wait_fwd) cudaStreamWaitEvent(st, sync.wait_fwd, 0);
-        if (sync.wait_inv) cudaStreamWaitEvent(st, sync.wait_inv, 0);
-        prof_stage(prof, 1, st);
-        const unsigned grid = g.npairs + (inp.hist_next ? 1 : 0);
-        if (pk.order) k_kk_block<1><<<grid, kCtaK1, BkSmem::TOTAL, st>>>(g, pk, tb, E, E_prev, dst);
-        else k_kk_block<0><<<grid, kCtaK1, BkSmem::TOTAL, st>>>(g, pk, tb, E, E_prev, dst);
-        if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
-        prof_stage(prof, -2, st);
-        prof_stage(prof, -3, st);
-        prof_stage(prof, -4, st);
-        return cudaGetLastError();
+        return e;
     }
     if (g.N2 != kRowN2) return cudaErrorInvalidValue;   // N is 65536 or 4096
     dim3 grid(kRowN2 / kCtaK1, g.npairs);
     dim3 grid_a(kRowN2 / kCtaK1, g.npairs + (inp.hist_next ? 1 : 0));
-    if (sync.wait_fwd) cudaStreamWaitEvent(st, sync.wait_fwd, 0);
     prof_stage(prof, 1, st);
-    if (pk.order) k_kk_fwd<1, kRowN2><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
-    else k_kk_fwd<0, kRowN2><<<grid_a, kCtaK1, 0, st>>>(g, pk, fftws, tb, dst);
+    e = launch_k(pk.order ? k_kk_fwd<1, kRowN2> : k_kk_fwd<0, kRowN2>, grid_a, kCtaK1, 0, st, sync.pdl, g, pk, fftws, tb,
+                 dst);
     if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
     prof_stage(prof, -2, st);
-    k_kk_rows<<<g.npairs * 16, 256, kRowPad * sizeof(float2), st>>>(g, fftws, tb.twN2);
+    if (e == cudaSuccess)
+        e = launch_k(k_kk_rows, g.npairs * 16, 256, kRowPad * sizeof(float2), st, sync.pdl, g, fftws, tb.twN2);
     if (sync.wait_inv) cudaStreamWaitEvent(st, sync.wait_inv, 0);
     prof_stage(prof, -3, st);
-    if (pk.order) k_kk_inv<1, kRowN2><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
-    else k_kk_inv<0, kRowN2><<<grid, kCtaK1, 0, st>>>(g, pk, fftws, tb, E, E_prev, dst);
+    if (e == cudaSuccess)
+        e = launch_k(pk.order ? k_kk_inv<1, kRowN2> : k_kk_inv<0, kRowN2>, grid, kCtaK1, 0, st, sync.pdl, g, pk, fftws, tb,
+                     E, E_prev, dst);
     prof_stage(prof, -4, st);
-    return cudaGetLastError();
+    return e;
 }
 
 // ============================================================ KK matched filter
@@ -985,6 +985,7 @@ __global__ void __launch_bounds__(kMfOut) k_kk_mf(const float2 *__restrict__ E, 
                                                  const float2 *__restrict__ Y_prev, long long ybase_prev)
 {
     extern __shared__ float2 xs[];
+    pdl_wait();
     long long m0 = f_prev + (long long)blockIdx.x * kMfOut;
     int L = 2 * kMfOut + 2 * hmf;
     float2 c = make_float2((float)cg[0], (float)cg[1]);
@@ -1050,12 +1051,13 @@ __global__ void __launch_bounds__(kMfThreads) k_kk_mf_t(const float2 *__restrict
     __shared__ float4 s_tp[HMF + 1];   // (ge, ge, go, go) per tap index u (go[HMF] = 0)
     long long m0 = f_prev + (long long)blockIdx.x * kMfTileOut;
     long long n0 = 2 * m0 - HMF;
-    const float2 c = make_float2((float)cg[0], (float)cg[1]);
-    const float gn = (float)cg[2];
     for (int u = threadIdx.x; u <= HMF; u += kMfThreads) {
         const float ho = u < HMF ? taps.go[u] : 0.f;
         s_tp[u] = make_float4(taps.ge[u], taps.ge[u], ho, ho);
     }
+    pdl_wait();
+    const float2 c = make_float2((float)cg[0], (float)cg[1]);
+    const float gn = (float)cg[2];
     // integer phase index of the downshift, advanced incrementally
     int idx = (int)((((n0 % ds_den) + ds_den) % ds_den + 2LL * threadIdx.x) % ds_den);
     idx = (int)(((long long)idx * ds_num) % ds_den);
@@ -1128,7 +1130,7 @@ cudaError_t launch_kk_mf(const float2 *E, long long ebase, long long e_k, long l
                          long long f_k, const float *rrc, int hmf, const float2 *ds_tab,
                          int ds_num, int ds_den, const double *cg, float2 *Y, long long ybase,
                          const float2 *Y_prev, long long ybase_prev, cudaStream_t st,
-                         const float *rrc_host)
+                         const float *rrc_host, bool pdl)
 {
     long long n = f_k - f_prev;
     if (hmf == 32 && rrc_host) {
@@ -1137,15 +1139,13 @@ cudaError_t launch_kk_mf(const float2 *E, long long ebase, long long e_k, long l
         for (int u = 0; u < 32; u++) t.go[u] = rrc_host[32 + (32 - 2 * u - 1)];
         unsigned grid = (unsigned)((n + kMfTileOut - 1) / kMfTileOut);
         size_t smem = (size_t)pad8(kMfTileOut + 32 + kMfR) * sizeof(float4) + 16;
-        k_kk_mf_t<32><<<grid, kMfThreads, smem, st>>>(E, ebase, e_k, f_prev, f_k, t, ds_tab, ds_num, ds_den, cg,
-                                                      Y, ybase, Y_prev, ybase_prev);
-        return cudaGetLastError();
+        return launch_k(k_kk_mf_t<32>, grid, kMfThreads, smem, st, pdl, E, ebase, e_k, f_prev, f_k, t, ds_tab, ds_num, ds_den,
+                        cg, Y, ybase, Y_prev, ybase_prev);
     }
     unsigned grid = (unsigned)((n + kMfOut - 1) / kMfOut);
     size_t smem = (size_t)(2 * kMfOut + 2 * hmf) * sizeof(float2);
-    k_kk_mf<<<grid, kMfOut, smem, st>>>(E, ebase, e_k, f_prev, f_k, rrc, hmf, ds_tab, ds_num,
-                                        ds_den, cg, Y, ybase, Y_prev, ybase_prev);
-    return cudaGetLastError();
+    return launch_k(k_kk_mf, grid, kMfOut, smem, st, pdl, E, ebase, e_k, f_prev, f_k, rrc, hmf, ds_tab, ds_num, ds_den, cg, Y,
+                    ybase, Y_prev, ybase_prev);
 }
 
 // ================================================ resampler to the transmitter's grid
@@ -1302,6 +1302,7 @@ __global__ void __launch_bounds__(kFdThreads) k_kk_fdmf(const float2 *__restrict
 {
     extern __shared__ float2 fbuf[];   // [2][N]
     float2 *a = fbuf, *b = fbuf + N;
+    pdl_wait();
     const long long blk = b_first + blockIdx.x;
     const long long n0 = (N / 2) * blk - N / 4;   // stream index of the block's first input
     const float2 c = make_float2((float)cg[0], (float)cg[1]);
@@ -1413,6 +1414,7 @@ __global__ void __launch_bounds__(32 * kFdWarps, 4)
     __shared__ float2 s_t[kFdWarps][32 * kFdPitch];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < 1024; i += blockDim.x) s_tw[i] = tw[i];
+    pdl_wait();
     if (blockIdx.x == 0)
         for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
             Y[m - ybase] = (m < 0) ? make_float2(0.f, 0.f) : Y_prev[m - ybase_prev];
@@ -1488,7 +1490,7 @@ __global__ void __launch_bounds__(32 * kFdWarps, 4)
 cudaError_t launch_kk_fdmf(const float2 *E, long long ebase, long long f_prev, long long f_k, int N,
                            const float2 *H, const float2 *tw, const float2 *ds_tab, int ds_num, int ds_den,
                            const double *cg, float2 *Y, long long ybase, const float2 *Y_prev,
-                           long long ybase_prev, cudaStream_t st, float2 *clk, int wbin)
+                           long long ybase_prev, cudaStream_t st, float2 *clk, int wbin, bool pdl)
 {
     const int per = N / 4;   // outputs per block
     if (N < 16 || (N & (N - 1)) || f_prev % per || f_k % per || wbin < 0 || wbin >= N / 8 || (N == 1024 && wbin > 31))
@@ -1496,14 +1498,12 @@ cudaError_t launch_kk_fdmf(const float2 *E, long long ebase, long long f_prev, l
     const long long nblk = (f_k - f_prev) / per;
     if (nblk <= 0) return cudaSuccess;
     if (N == 1024) {
-        k_kk_fd1024<<<(unsigned)((nblk + kFdWarps - 1) / kFdWarps), 32 * kFdWarps, 0, st>>>(
-            E, ebase, f_prev / per, nblk, H, tw, ds_tab, ds_num, ds_den, cg, Y, ybase, f_prev, Y_prev, ybase_prev,
-            clk, wbin);
-        return cudaGetLastError();
+        return launch_k(k_kk_fd1024, (unsigned)((nblk + kFdWarps - 1) / kFdWarps), 32 * kFdWarps, 0, st, pdl, E, ebase,
+                        f_prev / per, nblk, H, tw, ds_tab, ds_num, ds_den, cg, Y, ybase, f_prev, Y_prev, ybase_prev, clk,
+                        wbin);
     }
-    k_kk_fdmf<<<(unsigned)nblk, kFdThreads, 2 * N * sizeof(float2), st>>>(
-        E, ebase, f_prev / per, N, H, tw, ds_tab, ds_num, ds_den, cg, Y, ybase, f_prev, Y_prev, ybase_prev, clk, wbin);
-    return cudaGetLastError();
+    return launch_k(k_kk_fdmf, (unsigned)nblk, kFdThreads, 2 * N * sizeof(float2), st, pdl, E, ebase, f_prev / per, N, H, tw,
+                    ds_tab, ds_num, ds_den, cg, Y, ybase, f_prev, Y_prev, ybase_prev, clk, wbin);
 }
 
 // =========================================================== PAM matched filter
@@ -1517,6 +1517,7 @@ __global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *__restrict__ 
 {
     extern __shared__ float xf[];
     __shared__ float s_mu, s_inv;
+    pdl_wait();
     if (threadIdx.x == 0) {
         double mu = (double)dst->pam_s1[parity] / (double)nb;
         double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
@@ -1648,6 +1649,7 @@ __global__ void __launch_bounds__(32 * kFdWarps, 4)
     __shared__ float s_mu, s_inv;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < 1024; i += blockDim.x) s_tw[i] = tw[i];
+    pdl_wait();
     if (threadIdx.x == 0) {
         double mu = (double)dst->pam_s1[parity] / (double)nb;
         double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
@@ -1721,15 +1723,13 @@ __global__ void __launch_bounds__(32 * kFdWarps, 4)
 cudaError_t launch_pam_fd1024(const uint16_t *codes, long long cbase, long long nb, long long n_end,
                               long long f_prev, long long f_k, const float2 *H, const float2 *tw, DevState *dst,
                               int parity, float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
-                              cudaStream_t st, float2 *clk, int wbin)
+                              cudaStream_t st, float2 *clk, int wbin, bool pdl)
 {
     if (f_prev % 512 || f_k % 512 || wbin < 0 || wbin > 31) return cudaErrorInvalidValue;
     const long long nblk = (f_k - f_prev) / 512;
     if (nblk <= 0) return cudaSuccess;
-    k_pam_fd1024<<<(unsigned)((nblk + kFdWarps - 1) / kFdWarps), 32 * kFdWarps, 0, st>>>(
-        codes, cbase, nb, n_end, f_prev / 512, nblk, H, tw, dst, parity, Y, ybase, f_prev, Y_prev, ybase_prev, clk,
-        wbin);
-    return cudaGetLastError();
+    return launch_k(k_pam_fd1024, (unsigned)((nblk + kFdWarps - 1) / kFdWarps), 32 * kFdWarps, 0, st, pdl, codes, cbase, nb,
+                    n_end, f_prev / 512, nblk, H, tw, dst, parity, Y, ybase, f_prev, Y_prev, ybase_prev, clk, wbin);
 }
 
 // Register-tiled PAM matched filter for a compile-time half length HMF: each thread
@@ -1749,6 +1749,8 @@ __global__ void __launch_bounds__(kPmThreads) k_pam_mf_t(const uint16_t *__restr
     __shared__ float xf[kPmTile + 2 * HMF];
     __shared__ float s_h[2 * HMF + 1];
     __shared__ float s_mu, s_inv;
+    for (int i = threadIdx.x; i <= 2 * HMF; i += kPmThreads) s_h[i] = __ldg(rrc + i);
+    pdl_wait();
     if (threadIdx.x == 0) {
         double mu = (double)dst->pam_s1[parity] / (double)nb;
         double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
@@ -1760,7 +1762,6 @@ __global__ void __launch_bounds__(kPmThreads) k_pam_mf_t(const uint16_t *__restr
             dst->pam_inv_sd = inv;
         }
     }
-    for (int i = threadIdx.x; i <= 2 * HMF; i += kPmThreads) s_h[i] = __ldg(rrc + i);
     __syncthreads();
     const long long m0 = f_prev + (long long)blockIdx.x * kPmTile;
     const long long n0 = m0 - HMF;
@@ -1807,20 +1808,18 @@ __global__ void __launch_bounds__(kPmThreads) k_pam_mf_t(const uint16_t *__restr
 cudaError_t launch_pam_mf(const uint16_t *codes, long long cbase, long long nb, long long n_end, long long f_prev,
                           long long f_k, const float *rrc, int hmf, DevState *dst, int parity,
                           float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
-                          cudaStream_t st)
+                          cudaStream_t st, bool pdl)
 {
     long long n = f_k - f_prev;
     if (hmf == 16) {   // the default span (16 symbols at 2 samples/symbol)
         unsigned grid = (unsigned)((n + kPmTile - 1) / kPmTile);
-        k_pam_mf_t<16><<<grid, kPmThreads, 0, st>>>(codes, cbase, nb, n_end, f_prev, f_k, rrc, dst, parity, Y, ybase,
-                                                    Y_prev, ybase_prev);
-        return cudaGetLastError();
+        return launch_k(k_pam_mf_t<16>, grid, kPmThreads, 0, st, pdl, codes, cbase, nb, n_end, f_prev, f_k, rrc, dst, parity,
+                        Y, ybase, Y_prev, ybase_prev);
     }
     unsigned grid = (unsigned)((n + kMfOut - 1) / kMfOut);
     size_t smem = (size_t)(kMfOut + 2 * hmf) * sizeof(float);
-    k_pam_mf<<<grid, kMfOut, smem, st>>>(codes, cbase, nb, n_end, f_prev, f_k, rrc, hmf, dst, parity, Y,
-                                         ybase, Y_prev, ybase_prev);
-    return cudaGetLastError();
+    return launch_k(k_pam_mf, grid, kMfOut, smem, st, pdl, codes, cbase, nb, n_end, f_prev, f_k, rrc, hmf, dst, parity, Y,
+                    ybase, Y_prev, ybase_prev);
 }
 
 // bin and clear every latency slot still holding a record (rx_stats)

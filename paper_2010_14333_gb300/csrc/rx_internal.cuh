@@ -168,12 +168,43 @@ struct EqParams {
     int dd;       // KK: the short decision-directed LMS updated symbol by symbol, no phase search
 };
 
+// ------------------------------------------------- programmatic dependent launch
+// Kernels of one call follow each other on one stream, most of them a few microseconds
+// long, so the drain of one grid and the start of the next are a sizeable part of a call.
+// A kernel launched with `pdl` may start while the grid before it on the stream drains:
+// up to pdl_wait() it touches only its own shared memory and constant tables written when
+// the handle was made; pdl_wait() returns once every earlier grid has completed and its
+// writes are visible (a grid completes after its own pdl_wait, so this holds for the whole
+// chain), and then lets the next grid start likewise.  Every thread calls it before its
+// first access to memory another kernel of the stream reads or writes.  Without the launch
+// attribute the call does nothing.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, A... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
 // ------------------------------------------------------------------ launchers
 // (each returns cudaGetLastError() after enqueuing)
 cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *codes_prev,
                           long long nb, int nhist, long long prev_off, int first_call,
                           int pack_order, long long *s1, long long *s2, cudaStream_t st,
-                          LatRecord *lat = nullptr, int lat_slot = 0);
+                          LatRecord *lat, int lat_slot, bool pdl);
 
 // copy of the next call's packed history only (calls that emit no field)
 // Cross-stream order of the front end when consecutive calls run on different
@@ -183,6 +214,7 @@ cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *co
 // carries as history).
 struct KkSync {
     cudaEvent_t wait_fwd, rec_fwd, wait_inv;
+    bool pdl;   // one stream: launch every kernel as a programmatic dependent
 };
 cudaError_t launch_kk_hist(const KkInput &inp, cudaStream_t st, const KkSync &sync);
 
@@ -196,7 +228,7 @@ cudaError_t launch_kk_mf(const float2 *E, long long ebase, long long e_k, long l
                          long long f_k, const float *rrc, int hmf, const float2 *ds_tab,
                          int ds_num, int ds_den, const double *cg, float2 *Y, long long ybase,
                          const float2 *Y_prev, long long ybase_prev, cudaStream_t st,
-                         const float *rrc_host);
+                         const float *rrc_host, bool pdl);
 
 // resampler of the KK field to the transmitter's grid: outputs [r_prev, r_k) at ADC
 // positions (i0 2^32 + f0 + (m - r_prev) step) / 2^32; tab: 1024 x 16 taps
@@ -210,14 +242,14 @@ cudaError_t launch_kk_resample(const float2 *E, long long ebase, long long r_pre
 cudaError_t launch_kk_fdmf(const float2 *E, long long ebase, long long f_prev, long long f_k, int N,
                            const float2 *H, const float2 *tw, const float2 *ds_tab, int ds_num, int ds_den,
                            const double *cg, float2 *Y, long long ybase, const float2 *Y_prev,
-                           long long ybase_prev, cudaStream_t st, float2 *clk, int w);
+                           long long ybase_prev, cudaStream_t st, float2 *clk, int w, bool pdl);
 
 // PAM frequency-domain form, 1024-point blocks (hop 512) at the input rate;
 // f_prev and f_k are multiples of 512
 cudaError_t launch_pam_fd1024(const uint16_t *codes, long long cbase, long long nb, long long n_end,
                               long long f_prev, long long f_k, const float2 *H, const float2 *tw, DevState *dst,
                               int parity, float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
-                              cudaStream_t st, float2 *clk, int wbin);
+                              cudaStream_t st, float2 *clk, int wbin, bool pdl);
 
 // PAM with the resampler: the call's normalised codes for [cbase, n_end) as a complex
 // series (imaginary 0), then the matched filter on the resampled series
@@ -229,20 +261,20 @@ cudaError_t launch_pam_mf_r(const float2 *R, long long rbase, long long f_prev, 
 cudaError_t launch_pam_mf(const uint16_t *codes, long long cbase, long long nb, long long n_end, long long f_prev,
                           long long f_k, const float *rrc, int hmf, DevState *dst, int parity,
                           float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
-                          cudaStream_t st);
+                          cudaStream_t st, bool pdl);
 
 // zin: soft symbols of the payload from the block-Toeplitz tensor-core FIR
 // (frozen form), or null to filter in FP32 inside the equaliser
 cudaError_t launch_eq(const EqParams &p, const EqGeom &g, int train, const void *Y, const float2 *zin,
                       float2 *taps_in, float2 *taps_out, uint8_t *dec, uint8_t *winb, uint4 *winrec,
                       float4 *dbg_win, float2 *dbg_z, const uint8_t *prbs, const uint32_t *prbs_bits,
-                      DevState *dst, cudaStream_t st);
+                      DevState *dst, cudaStream_t st, bool pdl);
 
 // block-Toeplitz FIR on the tensor cores (frozen taps): z[k - k_lo] for
 // k in [k_lo, k_lo + nsym), z_k = sum_i conj(w_i) Y[2k + TH - i - ybase]
 cudaError_t launch_fir_tc(int prec, const float2 *Y, long long ybase, long long k_lo, long long nsym,
                           const float2 *taps, int ntaps, int scale_block, float2 *z, int *err, int nsm,
-                          cudaStream_t st);
+                          cudaStream_t st, bool pdl);
 
 // one-time kernel attributes (dynamic shared memory above 48 KB) of what a handle
 // launches, set at creation so that launches and graph captures make no such calls
@@ -254,7 +286,7 @@ cudaError_t prepare_kk_front();
 
 cudaError_t launch_demap(const EqParams &p, const EqGeom &g, int resolve_amb, int uw_in,
                          const uint8_t *dec, const uint8_t *winb, const uint4 *winrec, float4 *dbg_win,
-                         uint8_t *bits_out, const uint32_t *prbs_bits, DevState *dst, cudaStream_t st);
+                         uint8_t *bits_out, const uint32_t *prbs_bits, DevState *dst, cudaStream_t st, bool pdl);
 
 // CNN decisions for nseg consecutive payload windows (receiver mode)
 // CNN receiver on the tensor cores: soft symbols and decisions of nwin 64-symbol
@@ -262,7 +294,7 @@ cudaError_t launch_demap(const EqParams &p, const EqGeom &g, int resolve_amb, in
 cudaError_t launch_cnn_decide(const float *prm, const float2 *y, long long seg_base, long long y_end,
                               int nwin, uint8_t *dec, uint8_t *winb, uint4 *winrec, const uint32_t *prbs_bits,
                               long long k_first, float scale, int mq, float2 *soft, int *err, int nsm, cudaStream_t st,
-                              int bf16);
+                              int bf16, bool pdl);
 cudaError_t prepare_cnn_rx();
 
 }  // namespace rxk
