@@ -1121,6 +1121,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     g.pay_lo = pay_lo;
     g.q_k = s.q_k;
     g.ybase = h->ybase_cur;
+    g.pos0 = (int)((long long)h->bps * pay_lo % 32767);
     g.nblk = npay > 0 ? (int)(npay / c.eq_block) : 0;
     g.nwin = npay > 0 ? (int)(npay / kWin) : 0;
     g.gpart = h->gpart;

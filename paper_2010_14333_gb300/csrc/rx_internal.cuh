@@ -151,6 +151,7 @@ struct EqGeom {
     long long pay_lo;          // first payload symbol
     long long q_k;             // symbols processed up to (exclusive)
     long long ybase;           // stream index (2-sps) of Y workspace [0]
+    int pos0;                  // PRBS position of the first payload symbol's bits
     int nblk;                  // payload blocks in this call
     int nwin;                  // payload windows in this call
     float2 *gpart;             // frozen form: per-window tap-gradient partials of the last block
