@@ -833,16 +833,25 @@ cudaError_t launch_eq(const EqParams &p, const EqGeom &g, int train, const void 
 }
 
 // ------------------------------------------------------------------ demap / BER
-// kDemapWin windows per CTA, kDemapWin / 8 per warp.  The pi/2 unwrap
-// counter of window w is the carried value plus a prefix sum of integer
-// increments; each CTA sums the increments of all earlier windows itself
-// (16-byte loads of the window phase indices), then scans its own.  The
-// equaliser has already scored every window against the PRBS under the four
-// absolute rotations of its decisions (window records), so the bit-error
-// statistics here are selections: the decoded rotation q = m + r gives the raw
-// count, and the slip-tolerant count takes the best rotation, ties to q.
-constexpr int kDemapWin = 32;
+// The pi/2 unwrap counter of window w is the carried value plus a prefix sum of integer
+// increments; each CTA sums the increments of all earlier windows itself (16-byte loads of
+// the window phase indices, four windows per 32-bit word), then ranks its own with two
+// ballots.  The equaliser has already scored every window against the PRBS under the four
+// absolute rotations of its decisions (window records), so the bit-error statistics here
+// are selections: the decoded rotation q = m + r gives the raw count, and the slip-tolerant
+// count takes the best rotation, ties to q.
+//
+// k_demap (plain Gray mapping): a thread turns 16 consecutive decisions (one 16-byte load,
+// four symbols per 32-bit word) into 2 BPS bytes of output, four threads per window, 64
+// windows per CTA.  Gray(MQ-1-L) = Gray(L) ^ cm, so a rotation of the decisions is a swap
+// and exclusive-ors of the two Gray codes, the same for the whole window.  Bound by latency
+// (one dependent chain: phase indices, prefix, output); 6.4 us for a 2^22-sample 16QAM
+// buffer, 8.2 us with one symbol pair per lane, shuffled output bytes and 32 windows per CTA.
+// k_demap_diff (differential coding): quadrant differences need each symbol's predecessor;
+// 32 windows per CTA, four per warp, two symbols per lane.
 constexpr int kDemapThreads = 256;
+constexpr int kDemapWpc = kDemapThreads / 4;   // windows per CTA of k_demap
+constexpr int kDemapWin = 32;                  // of k_demap_diff
 
 __device__ __forceinline__ int unwrap_inc(int b_prev, int b, int B)
 {
@@ -872,15 +881,244 @@ __device__ __forceinline__ int quad_t(int LI, int LQ, int &lb)
     return q;
 }
 
+// sum of this thread's share of the unwrap increments of windows [0, w0), w0 a multiple of
+// 16; blast: phase index of the window before the call (have: there is one).  Indices are
+// below 32, so with bit 7 of every byte set, subtracting the other index and B/2 + 1 leaves
+// bit 7 where the difference exceeds B/2: four windows per subtraction.
+__device__ __forceinline__ int unwrap_prefix(const uint8_t *__restrict__ winb, int w0, int tid, int B, int have, int blast)
+{
+    const uint32_t H = (uint32_t)(B / 2 + 1) * 0x01010101u, top = 0x80808080u;
+    const int nch = w0 / 16;
+    int part = 0;
+    for (int cb = tid; cb < nch; cb += 4 * kDemapThreads) {
+        uint4 v[4];
+        uint32_t pv[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {   // four loads in flight per thread
+            const int c = cb + k * kDemapThreads;
+            if (c >= nch) break;
+            v[k] = *reinterpret_cast<const uint4 *>(winb + 16 * c);
+            // before the stream's first window there is no step: its own index
+            pv[k] = c ? winb[16 * c - 1] : have ? (uint32_t)blast : v[k].x & 0xFFu;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (cb + k * kDemapThreads >= nch) break;
+            const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+            uint32_t before = pv[k] << 24;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint32_t prev = __funnelshift_l(before, w[i], 8);   // the window before each of the four
+                part += __popc(((prev | top) - w[i] - H) & top) - __popc(((w[i] | top) - prev - H) & top);
+                before = w[i];
+            }
+        }
+    }
+    return part;
+}
+
+// stream-start pi/2 ambiguity from the first amb_syms payload symbols (windows 0.. of this,
+// the first payload call): the rotation r whose decoded symbols (rotation m_w + r) match the
+// transmitted ones best, ties to the lowest r; one warp
+__device__ __forceinline__ int find_rotation(const EqParams &p, const uint8_t *__restrict__ winb,
+                                             const uint4 *__restrict__ winrec, int lane)
+{
+    const int nw = p.amb_syms / kWin;
+    int acc = 0;
+    unsigned cnt[4] = {0, 0, 0, 0};
+    for (int h = 0; h < 2; h++) {
+        int w = lane + 32 * h;
+        int v = (w < nw && w > 0) ? unwrap_inc(winb[w - 1], winb[w], p.bps_b) : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            int t = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += t;
+        }
+        int m = acc + v;
+        acc += __shfl_sync(0xffffffffu, v, 31);
+        if (w < nw) {
+            uint4 rw = winrec[w];
+#pragma unroll
+            for (int r = 0; r < 4; r++) cnt[r] += rec_serr(rw, (m + r) & 3);
+        }
+    }
+    int best = 0;
+    unsigned bc = 0;
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        unsigned c = warp_sum_i(cnt[r]);
+        if (r == 0 || c < bc) { bc = c; best = r; }
+    }
+    return best;
+}
+
 template <bool QAM, int BPS, int MQ>
 __global__ void __launch_bounds__(kDemapThreads)
     k_demap(EqParams p, EqGeom g, int resolve_amb, int uw_in, const uint8_t *__restrict__ dec,
+            const uint8_t *__restrict__ winb, const uint4 *__restrict__ winrec, float4 *__restrict__ dbg_win,
+            uint8_t *__restrict__ bits_out, DevState *dst)
+{
+    constexpr int NW = kDemapThreads / 32, WPC = kDemapWpc;
+    constexpr int NB = QAM ? BPS / 2 : BPS;
+    static_assert(WPC == 64, "two warps rank the CTA's windows");
+    __shared__ int s_q[WPC];                 // rotation of each window, before r
+    __shared__ int s_red[NW], s_half, s_r;
+    __shared__ unsigned s_cnt[2][C_NCNT];
+    pdl_wait();
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int w0 = blockIdx.x * WPC, wi = w0 + (tid >> 2);
+    // every load that does not depend on the unwrap counter first
+    uint4 dv = make_uint4(0u, 0u, 0u, 0u), rc = dv;
+    if (wi < g.nwin) dv = *reinterpret_cast<const uint4 *>(dec + (size_t)w0 * kWin + 16 * tid);
+    const int ws = w0 + tid;                 // the window ranked and scored by thread tid < WPC
+    const bool own = tid < WPC && ws < g.nwin;
+    if (own) rc = winrec[ws];
+    long long m = 0;                         // unwrap count of window ws
+    int sb = 0;
+    if (QAM) {
+        const int have = dst->unwrap_have[uw_in], blast = dst->unwrap_b[uw_in];
+        const long long mstart = have ? dst->unwrap_m[uw_in] : 0;
+        int inc = 0;
+        if (own) {
+            sb = winb[ws];
+            if (ws > 0 || have) inc = unwrap_inc(ws ? winb[ws - 1] : blast, sb, p.bps_b);
+        }
+        const int part = (int)__reduce_add_sync(0xffffffffu, (unsigned)unwrap_prefix(winb, w0, tid, p.bps_b, have, blast));
+        if (lane == 0) s_red[wid] = part;
+        const unsigned le = 0xffffffffu >> (31 - lane);
+        const unsigned up = __ballot_sync(0xffffffffu, inc > 0), dn = __ballot_sync(0xffffffffu, inc < 0);
+        const int rank = __popc(up & le) - __popc(dn & le);
+        if (wid == 0) {
+            if (lane == 31) s_half = rank;
+            if (resolve_amb) {
+                const int r = find_rotation(p, winb, winrec, lane);
+                if (lane == 0) {
+                    s_r = r;
+                    if (blockIdx.x == 0) dst->amb_r = r;
+                }
+            } else if (lane == 0) {
+                s_r = dst->amb_r;
+            }
+        }
+        __syncthreads();
+        if (tid < WPC) {
+            long long pre = 0;
+#pragma unroll
+            for (int i = 0; i < NW; i++) pre += s_red[i];
+            m = mstart + pre + rank + (wid ? s_half : 0);
+            s_q[tid] = (int)(m & 3);
+        }
+        __syncthreads();
+    }
+    const int r = QAM ? s_r : 0;
+    if (tid < WPC) {   // statistics of window ws, summed over the warp
+        unsigned c[C_NCNT];
+#pragma unroll
+        for (int i = 0; i < C_NCNT; i++) c[i] = 0;
+        if (own) {
+            const long long k0 = g.pay_lo + (long long)ws * kWin, amb_end = QAM ? (long long)p.ntrain + p.amb_syms : 0;
+            const int qd = QAM ? (int)((m + r) & 3) : 0;
+            if (!(QAM && k0 < amb_end) && k0 + kWin <= g.score_end) {
+                int best = 0;
+                unsigned be = rec_err(rc, qd);
+#pragma unroll
+                for (int rho = 1; rho < (QAM ? 4 : 1); rho++) {
+                    unsigned e = rec_err(rc, (qd + rho) & 3);
+                    if (e < be) { be = e; best = rho; }
+                }
+                c[C_BITERR] = be;
+                c[C_RAWERR] = rec_err(rc, qd);
+                c[C_SYMERR] = rec_serr(rc, (qd + best) & 3);
+                c[C_SLIP] = best != 0;
+                c[C_NEAR] = rc.w >> 8;
+                c[C_BITS] = BPS * kWin;
+                c[C_SYMBOLS] = kWin;
+            }
+            c[C_WINDOWS] = 1;
+            if (QAM && dbg_win) dbg_win[ws].y = (float)m;
+            if (QAM && ws == g.nwin - 1) {   // carry the unwrap state to the next call
+                const int o = uw_in ^ 1;
+                dst->unwrap_have[o] = 1;
+                dst->unwrap_b[o] = sb;
+                dst->unwrap_m[o] = m;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < C_NCNT; i++)
+            if (i != C_AMBIG) {
+                const unsigned v = __reduce_add_sync(0xffffffffu, c[i]);
+                if (lane == 0) s_cnt[wid][i] = v;
+            }
+    }
+    if (wi < g.nwin) {   // output bits, MSB first within a symbol and packed MSB first
+        const int qd = QAM ? (s_q[tid >> 2] + r) & 3 : 0;
+        constexpr uint32_t cm = (MQ == 2 ? 1u : 2u) * 0x01010101u, lm = (uint32_t)(MQ - 1) * 0x01010101u;
+        const uint32_t xh = qd >= 2 ? cm : 0u, xl = (qd == 1 || qd == 2) ? cm : 0u;
+        const uint32_t dw[4] = {dv.x, dv.y, dv.z, dv.w};
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            uint32_t gI = dw[i] & lm, x;
+            gI ^= (gI >> 1) & (lm >> 1 & 0x03030303u);
+            if (QAM) {
+                uint32_t gQ = (dw[i] >> 3) & lm;
+                gQ ^= (gQ >> 1) & (lm >> 1 & 0x03030303u);
+                const uint32_t hi = ((qd & 1) ? gQ : gI) ^ xh, lo = ((qd & 1) ? gI : gQ) ^ xl;
+                x = (hi << NB) | lo;
+            } else {
+                x = gI;
+            }
+            // the four symbols' words side by side, the first one highest
+            if (BPS == 4) {
+                const uint32_t y = (x << 4) | (x >> 8);
+                o[i] = ((y & 0xFFu) << 8) | ((y >> 16) & 0xFFu);
+            } else if (BPS == 2) {
+                o[i] = (x * 0x40100401u) >> 24;
+            } else if (BPS == 1) {
+                o[i] = ((x * 0x08040201u) >> 24) & 0xFu;
+            } else {
+                o[i] = ((x & 7u) << 9) | ((x >> 2) & 0x1C0u) | ((x >> 13) & 0x38u) | (x >> 24);
+            }
+        }
+        uint8_t *out = bits_out + (size_t)w0 * (8 * BPS) + 2 * BPS * tid;
+        unsigned long long w;    // the 16 symbols' 16 BPS bits, first bit highest
+        if (BPS == 4)
+            w = ((unsigned long long)(o[0] << 16 | o[1]) << 32) | (o[2] << 16 | o[3]);
+        else
+            w = ((unsigned long long)((o[0] << 4 * BPS) | o[1]) << 8 * BPS) | ((o[2] << 4 * BPS) | o[3]);
+        // as bytes in memory order; wide stores where the caller's pointer allows them
+        if ((((uintptr_t)bits_out) & 7) == 0) {
+            if (BPS == 4) {
+                *reinterpret_cast<uint2 *>(out) =
+                    make_uint2(__byte_perm((uint32_t)(w >> 32), 0, 0x0123), __byte_perm((uint32_t)w, 0, 0x0123));
+            } else if (BPS == 2) {
+                *reinterpret_cast<uint32_t *>(out) = __byte_perm((uint32_t)w, 0, 0x0123);
+            } else {
+#pragma unroll
+                for (int i = 0; i < BPS; i++) {
+                    const uint32_t h = (uint32_t)(w >> (16 * (BPS - 1 - i))) & 0xFFFFu;
+                    reinterpret_cast<uint16_t *>(out)[i] = (uint16_t)((h >> 8) | (h << 8));
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 2 * BPS; i++) out[i] = (uint8_t)(w >> (8 * (2 * BPS - 1 - i)));
+        }
+    }
+    __syncthreads();
+    if (tid < C_NCNT && tid != C_AMBIG && s_cnt[0][tid] + s_cnt[1][tid])
+        atomicAdd(&dst->cnt[tid], (unsigned long long)(s_cnt[0][tid] + s_cnt[1][tid]));
+    if (g.lat && tid == 0) lat_end(g.lat, g.lat_slot);
+}
+
+template <int BPS, int MQ>
+__global__ void __launch_bounds__(kDemapThreads)
+    k_demap_diff(EqParams p, EqGeom g, int resolve_amb, int uw_in, const uint8_t *__restrict__ dec,
             const uint8_t *__restrict__ winb, const uint4 *__restrict__ winrec, float4 *__restrict__ dbg_win,
             uint8_t *__restrict__ bits_out, const uint32_t *__restrict__ prbs_bits, DevState *dst)
 {
     constexpr int NW = kDemapThreads / 32;
     constexpr int WPW = kDemapWin / NW;                            // windows per warp
-    constexpr int NB = QAM ? BPS / 2 : BPS;
     constexpr int NBYTES = 8 * BPS;                                // 64 symbols * BPS bits / 8
     constexpr int NS = (8 % BPS == 0) ? 8 / BPS : 8 / BPS + 2;     // symbols one output byte touches
     static_assert(kDemapWin == 32 && WPW <= 32, "one scan lane per window of the CTA");
@@ -911,7 +1149,7 @@ __global__ void __launch_bounds__(kDemapThreads)
     const int wr = w0 + wid + NW * lane;
     uint4 rc = make_uint4(0u, 0u, 0u, 0u);
     if (lane < WPW && wr < wend) rc = winrec[wr];
-    if (QAM) {
+    {
         int have = dst->unwrap_have[uw_in];
         int blast = dst->unwrap_b[uw_in];
         long long mstart = have ? dst->unwrap_m[uw_in] : 0;
@@ -921,36 +1159,7 @@ __global__ void __launch_bounds__(kDemapThreads)
             sb = winb[ws];
             sbp = ws > 0 ? winb[ws - 1] : 0;
         }
-        // prefix of increments over windows [0, w0): 16 windows per 16-byte load,
-        // four loads in flight per thread
-        const int nch = w0 / 16;
-        int part = 0;
-        for (int cb = tid; cb < nch; cb += 4 * kDemapThreads) {
-            uint4 v[4];
-            int pv[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                int c = cb + k * kDemapThreads;
-                if (c < nch) {
-                    v[k] = *reinterpret_cast<const uint4 *>(winb + 16 * c);
-                    pv[k] = c ? winb[16 * c - 1] : 0;
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                int c = cb + k * kDemapThreads;
-                if (c >= nch) break;
-                uint32_t wd[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-                int prev = c ? pv[k] : blast;
-                bool use_first = (c > 0) || have;
-#pragma unroll
-                for (int i = 0; i < 16; i++) {
-                    int b = (wd[i >> 2] >> (8 * (i & 3))) & 0xFF;
-                    if (i > 0 || use_first) part += unwrap_inc(prev, b, p.bps_b);
-                    prev = b;
-                }
-            }
-        }
+        int part = unwrap_prefix(winb, w0, tid, p.bps_b, have, blast);
         part = warp_sum_i(part);
         if (lane == 0) s_red[wid] = part;
         __syncthreads();
@@ -969,36 +1178,8 @@ __global__ void __launch_bounds__(kDemapThreads)
             if (tid == 0) s_mbase = mstart + pre;
         }
         if (resolve_amb) {
-            // stream-start pi/2 ambiguity from the first amb_syms payload symbols:
-            // the rotation r whose decoded symbols (rotation m_w + r) match the
-            // transmitted ones best, ties to the lowest r; every CTA finds it alike
-            if (tid < 32) {
-                int nw = p.amb_syms / kWin;   // windows 0..nw-1 of this call (first payload call)
-                int acc = 0;
-                unsigned cnt[4] = {0, 0, 0, 0};
-                for (int h = 0; h < 2; h++) {
-                    int w = lane + 32 * h;
-                    int v = (w < nw && w > 0) ? unwrap_inc(winb[w - 1], winb[w], p.bps_b) : 0;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        int t = __shfl_up_sync(0xffffffffu, v, o);
-                        if (lane >= o) v += t;
-                    }
-                    int m = acc + v;
-                    acc += __shfl_sync(0xffffffffu, v, 31);
-                    if (w < nw) {
-                        uint4 rw = winrec[w];
-#pragma unroll
-                        for (int r = 0; r < 4; r++) cnt[r] += rec_serr(rw, (m + r) & 3);
-                    }
-                }
-                int best = 0;
-                unsigned bc = 0;
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    unsigned c = warp_sum_i(cnt[r]);
-                    if (r == 0 || c < bc) { bc = c; best = r; }
-                }
+            if (tid < 32) {   // every CTA finds it alike
+                const int best = find_rotation(p, winb, winrec, lane);
                 if (tid == 0) {
                     s_r = best;
                     if (blockIdx.x == 0) dst->amb_r = best;
@@ -1009,36 +1190,17 @@ __global__ void __launch_bounds__(kDemapThreads)
         }
     }
     __syncthreads();
-    const int r = QAM ? s_r : 0;
-    const long long amb_end = QAM ? (long long)p.ntrain + p.amb_syms : 0;
-    // statistics: lane i < WPW selects from the record of the warp's window i
+    const int r = s_r;
+    const long long amb_end = (long long)p.ntrain + p.amb_syms;
+    // near-threshold and window counts of the warp's window i by lane i < WPW; the errors are
+    // counted on the decoded bits below
     if (lane < WPW && wr < wend) {
-        long long k0 = g.pay_lo + (long long)wr * kWin;
-        int qd = QAM ? (int)((s_m[wr - w0] + r) & 3) : 0;
-        if (QAM && p.diff) {   // differential coding: errors are counted on the decoded bits below
-            if (!(k0 < amb_end) && k0 + kWin <= g.score_end) atomicAdd(&s_cnt[C_NEAR], rc.w >> 8);
-        } else if (!(QAM && k0 < amb_end) && k0 + kWin <= g.score_end) {
-            int best = 0;
-            unsigned be = rec_err(rc, qd);
-#pragma unroll
-            for (int rho = 1; rho < (QAM ? 4 : 1); rho++) {
-                unsigned e = rec_err(rc, (qd + rho) & 3);
-                if (e < be) { be = e; best = rho; }
-            }
-            int qb = (qd + best) & 3;
-            atomicAdd(&s_cnt[C_BITERR], be);
-            atomicAdd(&s_cnt[C_RAWERR], rec_err(rc, qd));
-            atomicAdd(&s_cnt[C_SYMERR], rec_serr(rc, qb));
-            atomicAdd(&s_cnt[C_SLIP], (unsigned)(best != 0));
-            atomicAdd(&s_cnt[C_NEAR], rc.w >> 8);
-            atomicAdd(&s_cnt[C_BITS], (unsigned)(BPS * kWin));
-            atomicAdd(&s_cnt[C_SYMBOLS], (unsigned)kWin);
-        }
+        const long long k0 = g.pay_lo + (long long)wr * kWin;
+        if (!(k0 < amb_end) && k0 + kWin <= g.score_end) atomicAdd(&s_cnt[C_NEAR], rc.w >> 8);
         atomicAdd(&s_cnt[C_WINDOWS], 1u);
     }
-    // output bits: Gray codes of the rotated decisions, byte b of a window holding
-    // its bits [8b, 8b+8) MSB first, gathered from the owning lanes by shuffle.
-    // Differential coding: the word of a symbol is the Gray code of its quadrant step
+    // output bits: byte b of a window holds its bits [8b, 8b+8) MSB first, gathered from the
+    // owning lanes by shuffle.  The word of a symbol is the Gray code of its quadrant step
     // from the previous symbol, then (16QAM) its point's bits in the quadrant; the
     // previous symbol of a window's first one is the last of the window before it
     // (or the last of the previous call), and the decoded bits are scored here.
@@ -1048,14 +1210,11 @@ __global__ void __launch_bounds__(kDemapThreads)
     for (int i = 0; i < WPW; i++) {
         int wi = w0 + wid + NW * i;
         if (wi >= wend) break;   // warp-uniform
-        int qd = 0;
-        if (QAM) {
-            long long mw = s_m[wi - w0];
-            qd = (int)((mw + r) & 3);
-            if (dbg_win && lane == 0) dbg_win[wi].y = (float)mw;
-        }
+        const long long mw = s_m[wi - w0];
+        const int qd = (int)((mw + r) & 3);
+        if (dbg_win && lane == 0) dbg_win[wi].y = (float)mw;
         uint32_t grp2 = 0;
-        if (QAM && p.diff) {
+        {
             int qu[2], lb[2];
 #pragma unroll
             for (int h = 0; h < 2; h++) {
@@ -1105,14 +1264,6 @@ __global__ void __launch_bounds__(kDemapThreads)
                 dst->diff_q[uw_in ^ 1] = qu[1];
                 dst->diff_have[uw_in ^ 1] = 1;
             }
-        } else {
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                int dvb = (dv[i] >> (8 * h)) & 0xFF;
-                int LI = dvb & 7, LQ = QAM ? ((dvb >> 3) & 7) : 0;
-                if (QAM) rot_t<MQ>(LI, LQ, qd);
-                grp2 |= (uint32_t)(QAM ? ((gray(LI) << NB) | gray(LQ)) : gray(LI)) << (8 * h);
-            }
         }
         uint32_t acc = 0;
 #pragma unroll
@@ -1126,7 +1277,7 @@ __global__ void __launch_bounds__(kDemapThreads)
     __syncthreads();
     if (tid < C_NCNT && s_cnt[tid]) atomicAdd(&dst->cnt[tid], (unsigned long long)s_cnt[tid]);
     // carry the unwrap state to the next call
-    if (QAM && wend == g.nwin && w0 < wend && tid == 0) {
+    if (wend == g.nwin && w0 < wend && tid == 0) {
         int o = uw_in ^ 1;
         dst->unwrap_have[o] = 1;
         dst->unwrap_b[o] = winb[g.nwin - 1];
@@ -1139,18 +1290,15 @@ cudaError_t launch_demap(const EqParams &p, const EqGeom &g, int resolve_amb, in
                          const uint8_t *winb, const uint4 *winrec, float4 *dbg_win, uint8_t *bits_out,
                          const uint32_t *prbs_bits, DevState *dst, cudaStream_t st, bool pdl)
 {
-    cudaError_t e;
-    unsigned grid = (unsigned)((g.nwin + kDemapWin - 1) / kDemapWin);
-#define RX_DEMAP(Q, B, M)                                                                                   \
-    e = launch_k(k_demap<Q, B, M>, grid, kDemapThreads, 0, st, pdl, p, g, resolve_amb, uw_in, dec, winb, winrec,  \
-                 dbg_win, bits_out, prbs_bits, dst)
-    if (p.kk && p.mq == 4) RX_DEMAP(true, 4, 4);
-    else if (p.kk) RX_DEMAP(true, 2, 2);
-    else if (p.mq == 2) RX_DEMAP(false, 1, 2);
-    else if (p.mq == 4) RX_DEMAP(false, 2, 4);
-    else RX_DEMAP(false, 3, 8);
-#undef RX_DEMAP
-    return e;
+    if (p.diff) {
+        const unsigned grid = (unsigned)((g.nwin + kDemapWin - 1) / kDemapWin);
+        return launch_k(p.mq == 4 ? k_demap_diff<4, 4> : k_demap_diff<2, 2>, grid, kDemapThreads, 0, st, pdl, p, g, resolve_amb,
+                        uw_in, dec, winb, winrec, dbg_win, bits_out, prbs_bits, dst);
+    }
+    const unsigned grid = (unsigned)((g.nwin + kDemapWpc - 1) / kDemapWpc);
+    auto k = p.kk ? (p.mq == 4 ? k_demap<true, 4, 4> : k_demap<true, 2, 2>)
+                  : (p.mq == 2 ? k_demap<false, 1, 2> : p.mq == 4 ? k_demap<false, 2, 4> : k_demap<false, 3, 8>);
+    return launch_k(k, grid, kDemapThreads, 0, st, pdl, p, g, resolve_amb, uw_in, dec, winb, winrec, dbg_win, bits_out, dst);
 }
 
 }  // namespace rxk

@@ -223,21 +223,52 @@ struct KkPacked {
 };
 constexpr int kRawWords = 100;   // 384 bytes of a row + spare word, 16-byte multiple
 
+// 16 bytes of the packed stream of one code repeated, from byte vb (the pairs start at the
+// multiples of three)
+__device__ __forceinline__ uint4 code_bytes(uint32_t c, int order, unsigned vb)
+{
+    // the pair's three bytes, least significant first
+    const uint32_t pat = order == 0 ? c | (c << 12) : (c >> 4) | ((((c & 0xFu) << 4) | (c >> 8)) << 8) | ((c & 0xFFu) << 16);
+    const unsigned long long rep = (unsigned long long)pat * 0x1000001ull;   // six bytes
+    const unsigned s = vb % 3;
+    const uint32_t w0 = (uint32_t)(rep >> (8 * s)), w1 = (uint32_t)(rep >> (8 * ((s + 1) % 3))),
+                   w2 = (uint32_t)(rep >> (8 * ((s + 2) % 3)));
+    return make_uint4(w0, w1, w2, w0);
+}
+
+// Whether a block of the pair starts before the stream, whose samples read as the stream's
+// first code (uniform in a CTA).
+__device__ __forceinline__ bool before_stream(const KkGeom &g, int pair, bool hb)
+{
+    return ols_ws(g, 2 * pair) < 0 || (hb && ols_ws(g, 2 * pair + 1) < 0);
+}
+
 // (CTAs of kCtaK1 threads; the loop is unrolled so that every load issues before the
-// first one is used)
+// first one is used).  Samples before the stream are staged as c_first.  Byte offsets fit
+// 32 bits: a buffer is at most 2^30 samples.
 template <int N2T>
 __device__ __forceinline__ void stage_rows(const KkGeom &g, const KkPacked &pk, int pair, int c0,
-                                           uint32_t (*raw)[kRawWords], bool hb)
+                                           uint32_t (*raw)[kRawWords], bool hb, uint32_t c_first)
 {
     static_assert((32 * 24) % kCtaK1 == 0, "whole iterations");
+    // virtual-buffer byte of the first sample of this CTA's row 0, per block (>= 0 for every
+    // window of the call), and of stream sample 0 (a multiple of 16: buffers and histories
+    // are multiples of 32 samples)
+    const unsigned v0 = (unsigned)((ols_ws(g, 2 * pair) + c0 - g.cbase) * 3 / 2);
+    const unsigned v1 = hb ? (unsigned)((ols_ws(g, 2 * pair + 1) + c0 - g.cbase) * 3 / 2) : 0u;
+    const unsigned vs = g.cbase < 0 ? (unsigned)(-g.cbase * 3 / 2) : 0u;
+    const unsigned hbytes = (unsigned)pk.hist_bytes;
+    const uint8_t *in0 = pk.in - hbytes;
 #pragma unroll
-    for (int i = threadIdx.x; i < 32 * 24; i += kCtaK1) {
-        int row = i / 24, ch = i - 24 * (i / 24), blk = row >> 4, q = row & 15;
-        if (blk && !hb) continue;
-        long long n = ols_ws(g, 2 * pair + blk) + c0 + (long long)N2T * q;
-        long long vb = (n - g.cbase) * 3 / 2 + 16 * ch;   // >= 0 for every window of the call
-        const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
-        *reinterpret_cast<uint4 *>(&raw[row][4 * ch]) = __ldg(reinterpret_cast<const uint4 *>(src));
+    for (int k = 0; k < 32 * 24 / kCtaK1; k++) {
+        const int i = threadIdx.x + k * kCtaK1;
+        const int row = i / 24, ch = i - 24 * row;
+        if (row >= 16 && !hb) continue;
+        const unsigned vb = (row < 16 ? v0 : v1) + (unsigned)(row & 15) * (N2T * 3 / 2) + 16 * ch;
+        uint4 w;
+        if (vb < vs) w = code_bytes(c_first, pk.order, vb);
+        else w = __ldg(reinterpret_cast<const uint4 *>((vb < hbytes ? pk.hist : in0) + vb));
+        *reinterpret_cast<uint4 *>(&raw[row][4 * ch]) = w;
     }
 }
 
@@ -279,23 +310,15 @@ __device__ __forceinline__ uint32_t first_code(const KkPacked &pk, const DevStat
     return a;
 }
 
-// u = ln(I)/2 of both blocks of a pair at window positions n1 + N2T q, q < 16
-template <int ORD, int N2T>
-__device__ __forceinline__ void load_columns(const KkGeom &g, int pair, int n1, bool hb, const uint32_t (*raw)[kRawWords],
-                                             const ColPos &cp, uint32_t c_first, const float *s_ln, float2 (&x)[16])
+// u = ln(I)/2 of both blocks of a pair at this column's 16 window positions
+template <int ORD>
+__device__ __forceinline__ void load_columns(bool hb, const uint32_t (*raw)[kRawWords], const ColPos &cp, const float *s_ln,
+                                             float2 (&x)[16])
 {
-    const long long wa = ols_ws(g, 2 * pair) + n1, wb = hb ? ols_ws(g, 2 * pair + 1) + n1 : 0;
-    // rows q below qa (qb) hold stream indices before the stream: the first code
-    const int qa = wa < 0 ? (int)min((-wa + N2T - 1) / N2T, 16LL) : 0;
-    const int qb = wb < 0 ? (int)min((-wb + N2T - 1) / N2T, 16LL) : 0;
 #pragma unroll
     for (int q = 0; q < 16; q++) {
-        uint32_t ca = q < qa ? c_first : col_code<ORD>(raw[q], cp);
-        float ua = s_ln[ca], ub = 0.f;
-        if (hb) {
-            uint32_t cb = q < qb ? c_first : col_code<ORD>(raw[16 + q], cp);
-            ub = s_ln[cb];
-        }
+        const float ua = s_ln[col_code<ORD>(raw[q], cp)];
+        const float ub = hb ? s_ln[col_code<ORD>(raw[16 + q], cp)] : 0.f;
         x[q] = make_float2(ua, ub);
     }
 }
@@ -338,14 +361,14 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2
     }
     const int c0 = blockIdx.x * blockDim.x;
     const bool hb = 2 * pair + 1 < g.J;
-    stage_rows<N2T>(g, pk, pair, c0, raw, hb);
-    const uint32_t c_first = first_code(pk, dst);
+    const uint32_t c_first = before_stream(g, pair, hb) || pk.first_call ? first_code(pk, dst) : 0u;
+    stage_rows<N2T>(g, pk, pair, c0, raw, hb, c_first);
     if (pk.first_call && dst && blockIdx.x == 0 && pair == 0 && threadIdx.x == 0) dst->first_code = (int)c_first;
     __syncthreads();
     const int t = threadIdx.x, n1 = c0 + t;
     const ColPos cp = col_pos<ORD>(t);
     float2 x[16];
-    load_columns<ORD, N2T>(g, pair, n1, hb, raw, cp, c_first, s_ln, x);
+    load_columns<ORD>(hb, raw, cp, s_ln, x);
     dft16<false>(x);
     twiddle16<false>(x, tw, n1);
     float2 *out = fftws + (size_t)pair * g.N + n1;
@@ -465,13 +488,12 @@ __device__ __forceinline__ void carrier_sums(const KkGeom &g, DevState *dst, flo
     __shared__ long long s_q[3][32];
     sre = warp_sum_f(sre);
     sim = warp_sum_f(sim);
-    si2 = warp_sum_i(si2);
+    si2 = (int)__reduce_add_sync(0xffffffffu, (unsigned)si2);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        s_q[0][wid] = __double2ll_rn((double)sre * kCarrierUnit);
-        s_q[1][wid] = __double2ll_rn((double)sim * kCarrierUnit);
-        s_q[2][wid] = si2;
-    }
+    // the power-of-two scaling is exact in FP32 (a warp's sum is far from overflow), so this
+    // rounds once, to the nearest integer
+    if (lane < 2) s_q[lane][wid] = __float2ll_rn((lane ? sim : sre) * (float)kCarrierUnit);
+    if (lane == 2) s_q[2][wid] = si2;
     __syncthreads();
     if (threadIdx.x != 0) return;
     long long a = 0, b = 0, c = 0;
@@ -512,41 +534,41 @@ __device__ __forceinline__ void carry_field(const KkGeom &g, float2 *__restrict_
 
 // E = sqrt(I) exp(j phi) (Fig. 1d) of the kept outputs of a column of a block pair: x[q]
 // holds N times the phase of both blocks at window position n1 + N2T q; the codes come from
-// the staged rows.  Adds to the carrier / intensity sums.
+// the staged rows.  Adds to the carrier sums and to the sum of the intensities (halves and
+// integers below 2^24: exact in FP32).
 template <int ORD, int N2T>
 __device__ __forceinline__ void emit_field(const KkGeom &g, int pair, int n1, const float2 (&x)[16],
-                                           const uint32_t (*raw)[kRawWords], const ColPos &cp, uint32_t c_first,
-                                           float2 *__restrict__ E, float &sre, float &sim, int &si2)
+                                           const uint32_t (*raw)[kRawWords], const ColPos &cp, float2 *__restrict__ E,
+                                           float &sre, float &sim, float &sint)
 {
     const float invN = 1.0f / (float)g.N;
 #pragma unroll
     for (int half = 0; half < 2; half++) {
         int j = 2 * pair + half;
         if (j >= g.J) break;
-        long long ws = ols_ws(g, j);
         int tlo, thi;
         ols_kept(g, j, tlo, thi);
-        // 32-bit offsets from the block's first stream index: E row base, and the
-        // local index below which the stream index is negative (before the stream)
-        float2 *Eb = E + (ws - g.ebase);
-        const int tneg = ws < 0 ? (int)(-ws) : 0;
+        float2 *Eb = E + (ols_ws(g, j) - g.ebase) + n1;
+        // rows q whose position n1 + N2T q lies in [tlo, thi), as a bit mask
+        const int qlo = max((tlo - n1 + N2T - 1) / N2T, 0), qhi = min((thi - n1 + N2T - 1) / N2T, 16);
+        const unsigned keep = qhi > qlo ? ((1u << qhi) - 1u) & ~((1u << qlo) - 1u) : 0u;
 #pragma unroll
         for (int q = 0; q < 16; q++) {
-            int tt = n1 + N2T * q;
-            if (tt < tlo || tt >= thi) continue;
-            uint32_t code = tt < tneg ? c_first : col_code<ORD>(raw[16 * half + q], cp);
+            if (!(keep & (1u << q))) continue;
+            const uint32_t code = col_code<ORD>(raw[16 * half + q], cp);
             float phi = (half ? x[q].y : x[q].x) * invN;
             float sn, cs;
             __sincosf(phi, &sn, &cs);   // |phi| < pi: absolute error <= 2^-21.41
             // the hardware square-root approximation (sqrt.approx.f32) in place of the
             // correctly rounded sequence; the field is held to the FP64 reference
             // within 1e-5 relative RMS
-            float A = sqrt_approx(code ? (float)code : 0.5f);
+            const float in = fmaxf((float)code, 0.5f);
+            const float A = sqrt_approx(in);
             float2 e = make_float2(A * cs, A * sn);
-            Eb[tt] = e;
+            Eb[N2T * q] = e;
             sre += e.x;
             sim += e.y;
-            si2 += code ? 2 * (int)code : 1;
+            sint += in;
         }
     }
 }
@@ -566,10 +588,8 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const 
     int pair = blockIdx.y;
     const int c0 = blockIdx.x * blockDim.x;
     const bool hb = 2 * pair + 1 < g.J;
-    stage_rows<N2T>(g, pk, pair, c0, raw, hb);
-    const uint32_t c_first = first_code(pk, dst);
-    float sre = 0.f, sim = 0.f;
-    int si2 = 0;
+    stage_rows<N2T>(g, pk, pair, c0, raw, hb, before_stream(g, pair, hb) ? first_code(pk, dst) : 0u);
+    float sre = 0.f, sim = 0.f, sint = 0.f;
     if (blockIdx.x == 0 && blockIdx.y == 0) carry_field(g, E, E_prev);
     const int t = threadIdx.x, n1 = c0 + t;
     const ColPos cp = col_pos<ORD>(t);
@@ -580,8 +600,8 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const 
     __syncthreads();   // staged twiddles and rows
     twiddle16<true>(x, tw, n1);
     dft16<true>(x);
-    emit_field<ORD, N2T>(g, pair, n1, x, raw, cp, c_first, E, sre, sim, si2);
-    carrier_sums(g, dst, sre, sim, si2, gridDim.x * gridDim.y);
+    emit_field<ORD, N2T>(g, pair, n1, x, raw, cp, E, sre, sim, sint);
+    carrier_sums(g, dst, sre, sim, (int)(2.f * sint), gridDim.x * gridDim.y);
 }
 
 // ============================================== KK front end, 4096-point blocks
@@ -626,14 +646,14 @@ __global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, c
         return;
     }
     const bool hb = 2 * pair + 1 < g.J;
-    stage_rows<kBkN2>(g, pk, pair, 0, raw, hb);
-    const uint32_t c_first = first_code(pk, dst);
+    const uint32_t c_first = before_stream(g, pair, hb) || pk.first_call ? first_code(pk, dst) : 0u;
+    stage_rows<kBkN2>(g, pk, pair, 0, raw, hb, c_first);
     if (pk.first_call && dst && pair == 0 && t == 0) dst->first_code = (int)c_first;
     if (pair == 0) carry_field(g, E, E_prev);
     __syncthreads();
     const ColPos cp = col_pos<ORD>(t);
     float2 x[16];
-    load_columns<ORD, kBkN2>(g, pair, t, hb, raw, cp, c_first, s_ln, x);
+    load_columns<ORD>(hb, raw, cp, s_ln, x);
     __syncthreads();   // the ln table has been read: the spectrum takes its place
     dft16<false>(x);
     twiddle16<false>(x, tw, t);
@@ -673,10 +693,9 @@ __global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, c
     for (int k2 = 0; k2 < 16; k2++) x[k2] = col[k2 * kBkRow];
     twiddle16<true>(x, tw, t);
     dft16<true>(x);
-    float sre = 0.f, sim = 0.f;
-    int si2 = 0;
-    emit_field<ORD, kBkN2>(g, pair, t, x, raw, cp, c_first, E, sre, sim, si2);
-    carrier_sums(g, dst, sre, sim, si2, g.npairs);
+    float sre = 0.f, sim = 0.f, sint = 0.f;
+    emit_field<ORD, kBkN2>(g, pair, t, x, raw, cp, E, sre, sim, sint);
+    carrier_sums(g, dst, sre, sim, (int)(2.f * sint), g.npairs);
 }
 
 // ====================================================== KK front end, fused
@@ -1029,6 +1048,14 @@ __global__ void __launch_bounds__(kMfOut) k_kk_mf(const float2 *__restrict__ E, 
 // and imaginary parts of an output accumulate as one packed FP32 pair (one
 // fma.rn.f32x2 per tap and output, the same roundings as two scalar FMAs in the
 // same order); the taps sit in shared memory as (ge, ge, go, go).
+// (ph0 + n step) mod den with ph0, step < den: the 64-bit remainder only where the product
+// needs it
+__device__ __forceinline__ unsigned phase_at(unsigned ph0, unsigned step, unsigned long long n, unsigned den)
+{
+    const unsigned long long v = ph0 + n * step;
+    return (v >> 32) ? (unsigned)(v % den) : (unsigned)v % den;
+}
+
 template <int HMF>
 struct MfTaps {
     float ge[HMF + 1];
@@ -1042,7 +1069,8 @@ template <int HMF>
 __global__ void __launch_bounds__(kMfThreads) k_kk_mf_t(const float2 *__restrict__ E, long long ebase,
                                                        long long e_k, long long f_prev, long long f_k,
                                                        const MfTaps<HMF> taps, const float2 *__restrict__ ds_tab,
-                                                       int ds_num, int ds_den, const double *__restrict__ cg,
+                                                       int ds_num, int ds_den, unsigned ph0,
+                                                       const double *__restrict__ cg,
                                                        float2 *__restrict__ Y, long long ybase,
                                                        const float2 *__restrict__ Y_prev, long long ybase_prev)
 {
@@ -1055,26 +1083,31 @@ __global__ void __launch_bounds__(kMfThreads) k_kk_mf_t(const float2 *__restrict
         const float ho = u < HMF ? taps.go[u] : 0.f;
         s_tp[u] = make_float4(taps.ge[u], taps.ge[u], ho, ho);
     }
+    // integer phase index of the downshift: ph0 + 2 pp ds_num (mod ds_den) at pair pp of the
+    // call's first tile, advanced incrementally
+    const unsigned den = (unsigned)ds_den, two = 2u * (unsigned)ds_num % den;
+    unsigned idx = phase_at(ph0, two, (unsigned long long)blockIdx.x * kMfTileOut + threadIdx.x, den);
+    const unsigned step = phase_at(0u, two, kMfThreads, den), odd = (unsigned)ds_num % den;
+    // tile samples [lo, hi) lie inside the stream and the field
+    const int lo = n0 < 0 ? (int)-n0 : 0, hi = (int)min(e_k - n0, (long long)(2 * NPAIR));
+    const float2 *Et = E + (n0 - ebase);
     pdl_wait();
     const float2 c = make_float2((float)cg[0], (float)cg[1]);
     const float gn = (float)cg[2];
-    // integer phase index of the downshift, advanced incrementally
-    int idx = (int)((((n0 % ds_den) + ds_den) % ds_den + 2LL * threadIdx.x) % ds_den);
-    idx = (int)(((long long)idx * ds_num) % ds_den);
-    const int step = (int)((2LL * kMfThreads * ds_num) % ds_den), odd = ds_num % ds_den;
     // unrolled (a compile-time trip count): every iteration's loads can issue before
     // the first one is used
 #pragma unroll
-    for (int pp = threadIdx.x; pp < NPAIR; pp += kMfThreads) {
-        long long n = n0 + 2 * pp;
+    for (int k = 0; k < (NPAIR + kMfThreads - 1) / kMfThreads; k++) {
+        const int pp = threadIdx.x + k * kMfThreads;
+        if (pp >= NPAIR) break;
         float2 a = make_float2(0.f, 0.f), b = a;
-        if (n >= 0 && n < e_k) a = cmul(csub(E[n - ebase], c), __ldg(ds_tab + idx));
-        int idx1 = idx + odd;
-        idx1 = idx1 >= ds_den ? idx1 - ds_den : idx1;
-        if (n + 1 >= 0 && n + 1 < e_k) b = cmul(csub(E[n + 1 - ebase], c), __ldg(ds_tab + idx1));
+        unsigned idx1 = idx + odd;
+        idx1 = idx1 >= den ? idx1 - den : idx1;
+        if (2 * pp >= lo && 2 * pp < hi) a = cmul(csub(Et[2 * pp], c), __ldg(ds_tab + idx));
+        if (2 * pp + 1 >= lo && 2 * pp + 1 < hi) b = cmul(csub(Et[2 * pp + 1], c), __ldg(ds_tab + idx1));
         pr[pad8(pp)] = make_float4(a.x, a.y, b.x, b.y);
         idx += step;
-        idx = idx >= ds_den ? idx - ds_den : idx;
+        idx = idx >= den ? idx - den : idx;
     }
     if (blockIdx.x == 0) {
         for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
@@ -1139,8 +1172,10 @@ cudaError_t launch_kk_mf(const float2 *E, long long ebase, long long e_k, long l
         for (int u = 0; u < 32; u++) t.go[u] = rrc_host[32 + (32 - 2 * u - 1)];
         unsigned grid = (unsigned)((n + kMfTileOut - 1) / kMfTileOut);
         size_t smem = (size_t)pad8(kMfTileOut + 32 + kMfR) * sizeof(float4) + 16;
+        const long long n0 = 2 * f_prev - hmf, r0 = (n0 % ds_den + ds_den) % ds_den;
+        const unsigned ph0 = (unsigned)(r0 * ds_num % ds_den);   // downshift phase of the call's first input
         return launch_k(k_kk_mf_t<32>, grid, kMfThreads, smem, st, pdl, E, ebase, e_k, f_prev, f_k, t, ds_tab, ds_num, ds_den,
-                        cg, Y, ybase, Y_prev, ybase_prev);
+                        ph0, cg, Y, ybase, Y_prev, ybase_prev);
     }
     unsigned grid = (unsigned)((n + kMfOut - 1) / kMfOut);
     size_t smem = (size_t)(2 * kMfOut + 2 * hmf) * sizeof(float2);
