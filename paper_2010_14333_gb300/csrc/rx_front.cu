@@ -14,6 +14,10 @@
 // style into a radix-16 pass over the stride-N2 index (K1a, registers only), an
 // N2-point FFT per row with the multiplier and the inverse in shared memory (K1b),
 // and the inverse radix-16 pass fused with sqrt/exp/field assembly (K1c).
+#include <string.h>
+
+#include <numeric>
+
 #include <cooperative_groups.h>
 
 #include "rx_common.cuh"
@@ -1047,7 +1051,22 @@ __global__ void __launch_bounds__(kMfOut) k_kk_mf(const float2 *__restrict__ E, 
 // which makes the stride-8-pair loads of a warp free of bank conflicts.  The real
 // and imaginary parts of an output accumulate as one packed FP32 pair (one
 // fma.rn.f32x2 per tap and output, the same roundings as two scalar FMAs in the
-// same order); the taps sit in shared memory as (ge, ge, go, go).
+// same order); the taps are kernel parameters, read from the constant bank as (g, g).
+// A thread stages the pairs t, t + STRIDE, ..: where STRIDE is a multiple of the downshift's
+// period in pairs (FIXED), they all turn by the same two phases, looked up once; otherwise
+// the phases are looked up pair by pair.  STRIDE 120 serves every period that divides it
+// (the default 11/80 cycles per sample: 40) and covers a tile in as many steps as 128.
+// Bound by the shared-memory pipe and the packed FMAs (two issue cycles each: 7 us of the
+// FMA pipe for 2^21 outputs) in 1.2 waves of CTAs.  2^22-sample buffer: 17.4 us on warm caches and
+// 7.7 M warp instructions; 19.5 us and 10.1 M with taps in shared memory, phases per
+// sample and 64-bit phase and range arithmetic.  Persistent CTAs that load the next tile
+// into registers during the FIR took 16.5 us alone on warm caches against 17.4 but 1 to 3 us
+// more in the receiver, where their 95 to 116 registers leave no room for other kernels.
+template <int HMF>
+struct MfTaps {
+    f2x ge[HMF + 1];   // (ge, ge)
+    f2x go[HMF];       // (go, go)
+};
 // (ph0 + n step) mod den with ph0, step < den: the 64-bit remainder only where the product
 // needs it
 __device__ __forceinline__ unsigned phase_at(unsigned ph0, unsigned step, unsigned long long n, unsigned den)
@@ -1056,58 +1075,75 @@ __device__ __forceinline__ unsigned phase_at(unsigned ph0, unsigned step, unsign
     return (v >> 32) ? (unsigned)(v % den) : (unsigned)v % den;
 }
 
-template <int HMF>
-struct MfTaps {
-    float ge[HMF + 1];
-    float go[HMF];
-};
-
 constexpr int kMfThreads = 128, kMfR = 8, kMfTileOut = kMfThreads * kMfR;
 __host__ __device__ __forceinline__ int pad8(int p) { return p + (p >> 3); }
 
-template <int HMF>
-__global__ void __launch_bounds__(kMfThreads) k_kk_mf_t(const float2 *__restrict__ E, long long ebase,
-                                                       long long e_k, long long f_prev, long long f_k,
-                                                       const MfTaps<HMF> taps, const float2 *__restrict__ ds_tab,
-                                                       int ds_num, int ds_den, unsigned ph0,
-                                                       const double *__restrict__ cg,
-                                                       float2 *__restrict__ Y, long long ybase,
-                                                       const float2 *__restrict__ Y_prev, long long ybase_prev)
+template <int HMF, int STRIDE, bool FIXED>
+__global__ void __launch_bounds__(kMfThreads)
+    k_kk_mf_t(const float2 *__restrict__ E, long long ebase, long long e_k, long long f_prev, long long f_k,
+              const __grid_constant__ MfTaps<HMF> taps, const float2 *__restrict__ ds_tab, int ds_num, int ds_den,
+              unsigned ph0, const double *__restrict__ cg, float2 *__restrict__ Y, long long ybase,
+              const float2 *__restrict__ Y_prev, long long ybase_prev)
 {
-    constexpr int NPAIR = kMfTileOut + HMF + kMfR;
+    constexpr int NPAIR = kMfTileOut + HMF + kMfR, NIT = (NPAIR + STRIDE - 1) / STRIDE;
+    static_assert(STRIDE <= kMfThreads && STRIDE % 8 == 0, "one padded slot per 8 pairs");
     extern __shared__ float4 pr[];     // padded pair tile
-    __shared__ float4 s_tp[HMF + 1];   // (ge, ge, go, go) per tap index u (go[HMF] = 0)
-    long long m0 = f_prev + (long long)blockIdx.x * kMfTileOut;
-    long long n0 = 2 * m0 - HMF;
-    for (int u = threadIdx.x; u <= HMF; u += kMfThreads) {
-        const float ho = u < HMF ? taps.go[u] : 0.f;
-        s_tp[u] = make_float4(taps.ge[u], taps.ge[u], ho, ho);
-    }
-    // integer phase index of the downshift: ph0 + 2 pp ds_num (mod ds_den) at pair pp of the
-    // call's first tile, advanced incrementally
-    const unsigned den = (unsigned)ds_den, two = 2u * (unsigned)ds_num % den;
+    const long long m0 = f_prev + (long long)blockIdx.x * kMfTileOut;
+    const long long n0 = 2 * m0 - HMF;
+    // integer phase index of the downshift: ph0 + 2 ds_num pp (mod ds_den) at pair pp from the
+    // call's first one on
+    const unsigned den = (unsigned)ds_den, two = 2u * (unsigned)ds_num % den, odd = (unsigned)ds_num % den;
     unsigned idx = phase_at(ph0, two, (unsigned long long)blockIdx.x * kMfTileOut + threadIdx.x, den);
-    const unsigned step = phase_at(0u, two, kMfThreads, den), odd = (unsigned)ds_num % den;
-    // tile samples [lo, hi) lie inside the stream and the field
+    const unsigned step = FIXED ? 0u : phase_at(0u, two, STRIDE, den);
+    auto phases = [&](unsigned i) {    // e^{-2 pi j i / den} and the next sample's
+        unsigned j = i + odd;
+        j = j >= den ? j - den : j;
+        const float2 a = __ldg(ds_tab + i), b = __ldg(ds_tab + j);
+        return make_float4(a.x, a.y, b.x, b.y);
+    };
+    float4 w = phases(idx);
+    // tile samples [lo, hi) lie inside the stream and the field; inner tiles load 16-byte
+    // pairs where the field's origin allows it
     const int lo = n0 < 0 ? (int)-n0 : 0, hi = (int)min(e_k - n0, (long long)(2 * NPAIR));
     const float2 *Et = E + (n0 - ebase);
+    const bool inner = lo == 0 && hi == 2 * NPAIR && ((uintptr_t)Et & 15) == 0;
+    const bool act = STRIDE == kMfThreads || threadIdx.x < STRIDE;
+    float4 *const ps = pr + pad8(threadIdx.x);
     pdl_wait();
     const float2 c = make_float2((float)cg[0], (float)cg[1]);
     const float gn = (float)cg[2];
-    // unrolled (a compile-time trip count): every iteration's loads can issue before
-    // the first one is used
+    if (inner) {
+        float4 v[NIT];   // every load issues before the first one is used
 #pragma unroll
-    for (int k = 0; k < (NPAIR + kMfThreads - 1) / kMfThreads; k++) {
-        const int pp = threadIdx.x + k * kMfThreads;
-        if (pp >= NPAIR) break;
-        float2 a = make_float2(0.f, 0.f), b = a;
-        unsigned idx1 = idx + odd;
-        idx1 = idx1 >= den ? idx1 - den : idx1;
-        if (2 * pp >= lo && 2 * pp < hi) a = cmul(csub(Et[2 * pp], c), __ldg(ds_tab + idx));
-        if (2 * pp + 1 >= lo && 2 * pp + 1 < hi) b = cmul(csub(Et[2 * pp + 1], c), __ldg(ds_tab + idx1));
-        pr[pad8(pp)] = make_float4(a.x, a.y, b.x, b.y);
-        idx += step;
-        idx = idx >= den ? idx - den : idx;
+        for (int k = 0; k < NIT; k++)
+            if (act && threadIdx.x + k * STRIDE < NPAIR)
+                v[k] = reinterpret_cast<const float4 *>(Et)[threadIdx.x + k * STRIDE];
+#pragma unroll
+        for (int k = 0; k < NIT; k++) {
+            if (!FIXED && k) {
+                idx += step;
+                idx = idx >= den ? idx - den : idx;
+                w = phases(idx);
+            }
+            const float2 a = cmul(csub(make_float2(v[k].x, v[k].y), c), make_float2(w.x, w.y));
+            const float2 b = cmul(csub(make_float2(v[k].z, v[k].w), c), make_float2(w.z, w.w));
+            if (act && threadIdx.x + k * STRIDE < NPAIR) ps[k * pad8(STRIDE)] = make_float4(a.x, a.y, b.x, b.y);
+        }
+    } else if (act) {
+#pragma unroll 1
+        for (int k = 0; k < NIT; k++) {
+            const int pp = threadIdx.x + k * STRIDE, n = 2 * pp;
+            if (pp >= NPAIR) break;
+            float2 a = make_float2(0.f, 0.f), b = a;
+            if (n >= lo && n < hi) a = cmul(csub(Et[n], c), make_float2(w.x, w.y));
+            if (n + 1 >= lo && n + 1 < hi) b = cmul(csub(Et[n + 1], c), make_float2(w.z, w.w));
+            ps[k * pad8(STRIDE)] = make_float4(a.x, a.y, b.x, b.y);
+            if (!FIXED) {
+                idx += step;
+                idx = idx >= den ? idx - den : idx;
+                w = phases(idx);
+            }
+        }
     }
     if (blockIdx.x == 0) {
         for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
@@ -1115,7 +1151,6 @@ __global__ void __launch_bounds__(kMfThreads) k_kk_mf_t(const float2 *__restrict
     }
     __syncthreads();
     const ulonglong2 *prp = reinterpret_cast<const ulonglong2 *>(pr);
-    const ulonglong2 *tpp = reinterpret_cast<const ulonglong2 *>(s_tp);
     const int j0 = kMfR * threadIdx.x;
     ulonglong2 win[kMfR];
 #pragma unroll
@@ -1125,12 +1160,11 @@ __global__ void __launch_bounds__(kMfThreads) k_kk_mf_t(const float2 *__restrict
     for (int r = 0; r < kMfR; r++) acc[r] = 0ull;   // (+0, +0)
 #pragma unroll
     for (int u = 0; u <= HMF; u++) {
-        const ulonglong2 T = tpp[u];
 #pragma unroll
-        for (int r = 0; r < kMfR; r++) acc[r] = f2_fma(T.x, win[r].x, acc[r]);
+        for (int r = 0; r < kMfR; r++) acc[r] = f2_fma(taps.ge[u], win[r].x, acc[r]);
         if (u < HMF) {
 #pragma unroll
-            for (int r = 0; r < kMfR; r++) acc[r] = f2_fma(T.y, win[r].y, acc[r]);
+            for (int r = 0; r < kMfR; r++) acc[r] = f2_fma(taps.go[u], win[r].y, acc[r]);
 #pragma unroll
             for (int r = 0; r < kMfR - 1; r++) win[r] = win[r + 1];
             win[kMfR - 1] = prp[pad8(j0 + u + kMfR)];
@@ -1168,14 +1202,21 @@ cudaError_t launch_kk_mf(const float2 *E, long long ebase, long long e_k, long l
     long long n = f_k - f_prev;
     if (hmf == 32 && rrc_host) {
         MfTaps<32> t;
-        for (int u = 0; u <= 32; u++) t.ge[u] = rrc_host[32 + (32 - 2 * u)];
-        for (int u = 0; u < 32; u++) t.go[u] = rrc_host[32 + (32 - 2 * u - 1)];
+        auto twice = [](float h) {
+            uint32_t b;
+            memcpy(&b, &h, 4);
+            return (f2x)b << 32 | b;
+        };
+        for (int u = 0; u <= 32; u++) t.ge[u] = twice(rrc_host[32 + (32 - 2 * u)]);
+        for (int u = 0; u < 32; u++) t.go[u] = twice(rrc_host[32 + (32 - 2 * u - 1)]);
         unsigned grid = (unsigned)((n + kMfTileOut - 1) / kMfTileOut);
         size_t smem = (size_t)pad8(kMfTileOut + 32 + kMfR) * sizeof(float4) + 16;
         const long long n0 = 2 * f_prev - hmf, r0 = (n0 % ds_den + ds_den) % ds_den;
         const unsigned ph0 = (unsigned)(r0 * ds_num % ds_den);   // downshift phase of the call's first input
-        return launch_k(k_kk_mf_t<32>, grid, kMfThreads, smem, st, pdl, E, ebase, e_k, f_prev, f_k, t, ds_tab, ds_num, ds_den,
-                        ph0, cg, Y, ybase, Y_prev, ybase_prev);
+        const long long period = ds_den / std::gcd(2LL * ds_num % ds_den, (long long)ds_den);   // in pairs
+        return launch_k(120 % period == 0 ? k_kk_mf_t<32, 120, true> : k_kk_mf_t<32, kMfThreads, false>, grid, kMfThreads,
+                        smem, st, pdl, E, ebase, e_k, f_prev, f_k, t, ds_tab, ds_num, ds_den, ph0, cg, Y, ybase, Y_prev,
+                        ybase_prev);
     }
     unsigned grid = (unsigned)((n + kMfOut - 1) / kMfOut);
     size_t smem = (size_t)(2 * kMfOut + 2 * hmf) * sizeof(float2);
