@@ -110,7 +110,7 @@ struct rx_handle {
     // end of stream (rx_flush)
     int flushed;               // rx_flush ran: no more buffers
     int flush_mode;            // the call being enqueued is a pad call of rx_flush
-    int flush_par;             // PAM: sums slot (call index mod 3) of the last real call (its mean and deviation)
+    int flush_par;             // PAM: slot (call index mod 3) of the last real call's mean and deviation
     long long flush_score_end; // windows reaching this symbol are not scored
     long long flush_bits;      // bound of the bits rx_flush emits
     long long pad_calls;       // pad calls run by rx_flush (not counted as input)
@@ -959,7 +959,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     cudaError_t e = cudaSuccess;
     int par = (int)(h->calls & 1);
     const int isl = (int)(h->calls % kInSlots);   // input staging slot of a host-buffer call
-    const int spar = (int)(h->calls % 3);   // PAM sums slot: the filter of call i clears call i+2's
+    const int spar = (int)(h->calls % 3);   // PAM slot of the call's mean and deviation
     int ds = (int)(h->calls % kSlots);   // decision slot of this call
     // KK in the pipeline: the field of odd calls on the second front-end stream.
     // Not with the CNN receiver: its decision kernel is persistent (one CTA per SM),
@@ -986,13 +986,12 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
         prof_begin(h, 0, sf);
         int cw_new = h->cw ^ 1;
         // PAM in the pipeline: the filter two calls back (on its own stream) is done with
-        // this codes slot, and has cleared this call's sums
+        // this codes slot
         if (three && !h->kk) cudaStreamWaitEvent(sf, h->ev_cfree[cw_new], 0);
         // a flush pad adds nothing to the PAM sums: its filter uses the last real buffer's
         const bool sums = !h->kk && !h->flush_mode;
         e = launch_unpack(in, h->codes[cw_new], h->codes[h->cw], h->nb, h->nhist, h->nb, h->calls == 0,
-                          c.pack_order, sums ? &h->st->pam_s1[spar] : nullptr,
-                          sums ? &h->st->pam_s2[spar] : nullptr, sf, lat_first, lat_slot, pdl);
+                          c.pack_order, sums ? h->st : nullptr, spar, sf, lat_first, lat_slot, pdl);
         lat_first = nullptr;   // stamped: the KK front end (debug view) comes after
         h->cw = cw_new;
         prof_end(h, 0, sf);
@@ -1052,7 +1051,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
         const long long rb = h->r_prev - kEHist;
         const int ppar_rs = h->flush_mode ? h->flush_par : spar;
         // the resampler reads the reconstructed field (KK) or the call's normalised codes (PAM)
-        if (!h->kk) e = launch_pam_norm(h->codes[h->cw], cbase, h->nb, s.avail, h->st, ppar_rs, h->E[0], sm);
+        if (!h->kk) e = launch_pam_norm(h->codes[h->cw], cbase, s.avail, h->st, ppar_rs, h->E[0], sm);
         if (e == cudaSuccess)
             e = launch_kk_resample(h->kk ? h->E[h->ew] : h->E[0], h->kk ? h->ebase_cur : cbase, h->r_prev, s.r_k,
                                    (long long)(psi >> 32), (unsigned)(psi & 0xFFFFFFFF), c.rs_step, h->rs_tab,
@@ -1082,11 +1081,11 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
             e = launch_pam_mf_r(h->R[h->rw], h->rbase_cur, h->f_prev, s.f_k, h->rrc, h->hmf, (float *)h->Y[yw_new], yb,
                                 (const float *)h->Y[h->yw], h->ybase_cur, sm);
         else if (h->fd)
-            e = launch_pam_fd1024(h->codes[h->cw], cbase, h->nb, s.avail, h->f_prev, s.f_k, h->fd_H, h->fd_tw, h->st,
+            e = launch_pam_fd1024(h->codes[h->cw], cbase, s.avail, h->f_prev, s.f_k, h->fd_H, h->fd_tw, h->st,
                                   ppar, (float *)h->Y[yw_new], yb, (const float *)h->Y[h->yw], h->ybase_cur, sm,
                                   h->clk, h->clk_w, pdl);
         else
-            e = launch_pam_mf(h->codes[h->cw], cbase, h->nb, s.avail, h->f_prev, s.f_k, h->rrc, h->hmf, h->st, ppar,
+            e = launch_pam_mf(h->codes[h->cw], cbase, s.avail, h->f_prev, s.f_k, h->rrc, h->rrc_host, h->hmf, h->st, ppar,
                               (float *)h->Y[yw_new], yb, (const float *)h->Y[h->yw], h->ybase_cur, sm, pdl);
         if (e == cudaSuccess && h->fd && c.clk_track) {
             // blocks of this call: outputs at 2 samples/symbol per block N/4 (KK) or N/2 (PAM)

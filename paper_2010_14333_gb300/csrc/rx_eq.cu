@@ -120,13 +120,16 @@ __device__ __forceinline__ PhaseTab phase_tab(const EqParams &p, int lane)
 // 16 of their 17 input pairs, their reference bits one fetch, their decisions and errors
 // one store.  Counts are reduced with redux (one instruction each).  zs holds the window's
 // outputs as 64 real parts, then 64 imaginary parts, so that the phase search rotates two
-// symbols per packed FP32 FMA.  Every output is bit for bit that of one symbol per lane and
+// symbols per packed FP32 FMA.  ref2: the reference bits of the lane's two symbols (loaded
+// a window ahead by the caller; score: count errors against them); update: the window's
+// tap step is wanted (the last window of a block but the call's last one feeds nothing).
+// Every output is bit for bit that of one symbol per lane and
 // half a window (products and sums in the same order); 25.6 instead of 28.7 M warp
 // instructions and 33.4 instead of 35.5 us for a 2^22-sample 16QAM buffer (issue bound).
 template <int NT, int MQ, bool FRZ = false>
 __device__ __forceinline__ WinOut qam_window(const EqParams &p, const float2 *ys, int c0, float *zs, float2 *es,
                                              float2 *ws, int mode, float mu, int lane, uint8_t *dec_out,
-                                             float2 *dbg_z, const uint32_t *prbs_bits, int pwin,
+                                             float2 *dbg_z, bool score, int ref2, bool update,
                                              const PhaseTab &ph, float inv_s, const float2 *zin = nullptr,
                                              float2 *G = nullptr)
 {
@@ -218,7 +221,6 @@ __device__ __forceinline__ WinOut qam_window(const EqParams &p, const float2 *ys
     // decisions and errors
     constexpr int NB = MQ == 2 ? 1 : 2, BPS = 2 * NB;
     unsigned eA = 0, eB = 0, se = 0, nn = 0, db = 0;
-    const int ref2 = prbs_bits ? ref_bits<2 * BPS>(prbs_bits, pwin + 2 * BPS * lane) : 0;
     float2 e[2];
 #pragma unroll
     for (int h = 0; h < 2; h++) {
@@ -227,7 +229,7 @@ __device__ __forceinline__ WinOut qam_window(const EqParams &p, const float2 *ys
         int LI = decide_t<MQ>(vr), LQ = decide_t<MQ>(vi);
         bool nr = near_t<MQ>(vr) || near_t<MQ>(vi);
         db |= (unsigned)(LI | (LQ << 3) | (nr ? 64 : 0)) << (8 * h);
-        if (prbs_bits) {
+        if (score) {
             // bit errors of this symbol under each absolute pi/2 rotation of the decision
             // with gray(MQ-1-L) = gray(L) ^ cm, rotation q of (LI, LQ) has the code
             // q0: (gI, gQ), q1: (gQ, gI^cm), q2: (gI^cm, gQ^cm), q3: (gQ^cm, gI)
@@ -254,7 +256,7 @@ __device__ __forceinline__ WinOut qam_window(const EqParams &p, const float2 *ys
     if (dec_out) *reinterpret_cast<uint16_t *>(dec_out + 2 * lane) = (uint16_t)db;
     reinterpret_cast<float4 *>(es)[lane] = make_float4(e[0].x, e[0].y, e[1].x, e[1].y);
     __syncwarp();
-    if (prbs_bits) {
+    if (score) {
         R.errA = __reduce_add_sync(0xffffffffu, eA);
         R.errB = __reduce_add_sync(0xffffffffu, eB);
         R.serr = __reduce_add_sync(0xffffffffu, se);
@@ -262,7 +264,7 @@ __device__ __forceinline__ WinOut qam_window(const EqParams &p, const float2 *ys
     }
     // block-LMS update after the window: w_i += mu sum_k y[2k + TH - i] conj(e_k);
     // frozen form: the sum only, accumulated in G (last block), taps unchanged
-    if (lane < NT && (!FRZ || G)) {
+    if (lane < NT && (FRZ ? G != nullptr : update)) {
         float gr = 0.f, gi = 0.f;
         const float2 *yb = ys + (c0 + TH - lane);
         const float4 *e4 = reinterpret_cast<const float4 *>(es);
@@ -291,8 +293,8 @@ __device__ __forceinline__ WinOut qam_window(const EqParams &p, const float2 *ys
 template <int NT, int MQ>
 __device__ __forceinline__ WinOut pam_window(const EqParams &p, const float *ys, int c0, long long k0, float *es,
                                              float *ws, int mode, float mu, int lane, uint8_t *dec_out,
-                                             float2 *dbg_z, const uint8_t *prbs_ext, const uint32_t *prbs_bits,
-                                             int pwin)
+                                             float2 *dbg_z, const uint8_t *prbs_ext, bool score, int ref2,
+                                             bool update)
 {
     WinOut R;
     R.b = 0;
@@ -325,7 +327,6 @@ __device__ __forceinline__ WinOut pam_window(const EqParams &p, const float *ys,
         }
         Y0 = Y1;
     }
-    const int ref2 = prbs_bits ? ref_bits<2 * nb>(prbs_bits, pwin + 2 * nb * lane) : 0;
 #pragma unroll
     for (int h = 0; h < 2; h++) {
         const int q = 2 * lane + h;
@@ -334,7 +335,7 @@ __device__ __forceinline__ WinOut pam_window(const EqParams &p, const float *ys,
         int L = decide_t<MQ>(a);
         bool nr = near_t<MQ>(a);
         db |= (unsigned)(L | (nr ? 64 : 0)) << (8 * h);
-        if (prbs_bits) {
+        if (score) {
             unsigned ne = __popc(gray(L) ^ (h ? ref2 & ((1 << nb) - 1) : ref2 >> nb));
             e0 += ne;
             s0 += ne > 0;
@@ -355,12 +356,12 @@ __device__ __forceinline__ WinOut pam_window(const EqParams &p, const float *ys,
     if (dec_out) *reinterpret_cast<uint16_t *>(dec_out + 2 * lane) = (uint16_t)db;
     reinterpret_cast<float2 *>(es)[lane] = make_float2(e[0], e[1]);
     __syncwarp();
-    if (prbs_bits) {
+    if (score) {
         R.errA = __reduce_add_sync(0xffffffffu, e0);
         R.serr = __reduce_add_sync(0xffffffffu, s0);
         R.nnear = __reduce_add_sync(0xffffffffu, nn);
     }
-    if (lane < NT) {
+    if (update && lane < NT) {
         const float *yb = ys + (c0 + TH - lane);
         const float4 *e4 = reinterpret_cast<const float4 *>(es);
         float g = 0.f;
@@ -407,6 +408,19 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
     T *ws = es + kWin;
     const int blk = blockIdx.x * (blockDim.x >> 5) + wid;
     if (!train && blk >= g.nblk) return;
+    constexpr int BPS = QAM ? (MQ == 2 ? 2 : 4) : (MQ == 2 ? 1 : MQ == 4 ? 2 : 3);
+    const int sb = blk * B;   // the block's first symbol, from pay_lo
+    // PRBS position of the block's first bit: fewer than 2^30 bits follow the call's first
+    int pwin = (int)(((unsigned)g.pos0 + (unsigned)(BPS * sb)) % 32767u), ref2 = 0;
+    if (!train) {   // the block's input, the taps and the first window's reference bits together
+        if (lane == 0) {
+            mbar_init(bar, 1);
+            unsigned bytes = (unsigned)(ylen * sizeof(T));
+            mbar_expect_tx(bar, bytes);
+            bulk_g2s(ys, Y + (2 * (g.pay_lo + sb) - kYHist - g.ybase), bytes, bar);
+        }
+        ref2 = ref_bits<2 * BPS>(prbs_bits, pwin + 2 * BPS * lane);
+    }
     // start taps; the slot past the last tap stays zero for the paired loads
     if (QAM) reinterpret_cast<float2 *>(ws)[lane] = lane < NT ? taps_in[lane] : make_float2(0.f, 0.f);
     else reinterpret_cast<float *>(ws)[lane] = lane < NT ? taps_in[lane].x : 0.f;
@@ -429,10 +443,10 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
                 float mu = mode == 0 ? p.mu_cma : p.mu;
                 qam_window<NT, MQ>(p, reinterpret_cast<float2 *>(ys), kYHist, reinterpret_cast<float *>(zs),
                                    reinterpret_cast<float2 *>(es), reinterpret_cast<float2 *>(ws), mode, mu, lane,
-                                   nullptr, dz, nullptr, 0, ph, inv_s);
+                                   nullptr, dz, false, 0, true, ph, inv_s);
             } else {
                 pam_window<NT, MQ>(p, reinterpret_cast<float *>(ys), kYHist, k0, reinterpret_cast<float *>(es),
-                                   reinterpret_cast<float *>(ws), 1, p.mu_train, lane, nullptr, dz, prbs_ext, nullptr, 0);
+                                   reinterpret_cast<float *>(ws), 1, p.mu_train, lane, nullptr, dz, prbs_ext, false, 0, true);
             }
         }
         if (lane < NT)
@@ -440,29 +454,26 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
                                 : make_float2(reinterpret_cast<float *>(ws)[lane], 0.f);
         return;
     }
-    const int sb = blk * B;   // the block's first symbol, from pay_lo
-    if (lane == 0) {
-        mbar_init(bar, 1);
-        unsigned bytes = (unsigned)(ylen * sizeof(T));
-        mbar_expect_tx(bar, bytes);
-        bulk_g2s(ys, Y + (2 * (g.pay_lo + sb) - kYHist - g.ybase), bytes, bar);
-    }
-    __syncwarp();
     if (!mbar_wait(bar, 0)) {
         if (lane == 0) atomicExch(&dst->err, (int)RX_ETIMEOUT);
         mbar_wait(bar, 0);
         return;
     }
-    // PRBS position of the block's first bit: fewer than 2^30 bits follow the call's first
-    int pwin = (int)(((unsigned)g.pos0 + (unsigned)p.bps * (unsigned)sb) % 32767u);
-    for (int w = 0; w < B / kWin; w++) {
+    const int nw = B / kWin;
+    for (int w = 0; w < nw; w++) {
+        // the next window's reference bits, before this window's work
+        pwin += BPS * kWin;
+        pwin = pwin >= 32767 ? pwin - 32767 : pwin;
+        const int ref = ref2;
+        if (w + 1 < nw) ref2 = ref_bits<2 * BPS>(prbs_bits, pwin + 2 * BPS * lane);
+        const bool update = w + 1 < nw || blk == g.nblk - 1;
         const int c0 = kYHist + 2 * w * kWin, wi = sb / kWin + w;
         uint8_t *dq = dec + wi * kWin;
         float2 *dz = dbg_z ? dbg_z + (g.pay_lo - g.sym_lo) + wi * kWin : nullptr;
         if (QAM) {
             WinOut R = qam_window<NT, MQ>(p, reinterpret_cast<float2 *>(ys), c0, reinterpret_cast<float *>(zs),
                                           reinterpret_cast<float2 *>(es), reinterpret_cast<float2 *>(ws), 2, p.mu,
-                                          lane, dq, dz, prbs_bits, pwin, ph, inv_s);
+                                          lane, dq, dz, true, ref, update, ph, inv_s);
             if (lane == 0) {
                 winb[wi] = (uint8_t)R.b;
                 winrec[wi] = make_uint4(R.errA, R.errB, R.serr, (unsigned)R.b | (R.nnear << 8));
@@ -471,14 +482,12 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
             }
         } else {
             WinOut R = pam_window<NT, MQ>(p, reinterpret_cast<float *>(ys), c0, 0, reinterpret_cast<float *>(es),
-                                          reinterpret_cast<float *>(ws), 2, p.mu, lane, dq, dz, prbs_ext, prbs_bits, pwin);
+                                          reinterpret_cast<float *>(ws), 2, p.mu, lane, dq, dz, prbs_ext, true, ref, update);
             if (lane == 0) {
                 winb[wi] = 0;
                 winrec[wi] = make_uint4(R.errA, 0u, R.serr, R.nnear << 8);
             }
         }
-        pwin += p.bps * kWin;
-        pwin = pwin >= 32767 ? pwin - 32767 : pwin;
     }
     if (blk == g.nblk - 1 && lane < NT) {
         taps_out[lane] = QAM ? reinterpret_cast<float2 *>(ws)[lane]
@@ -538,7 +547,8 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
     float2 G = make_float2(0.f, 0.f);
     WinOut R = qam_window<NT, MQ, true>(p, ys, kYHist, reinterpret_cast<float *>(zs), es, ws, 2, p.mu, lane,
                                         dec + (k0 - g.pay_lo),
-                                        dbg_z ? dbg_z + (k0 - g.sym_lo) : nullptr, prbs_bits, pwin,
+                                        dbg_z ? dbg_z + (k0 - g.sym_lo) : nullptr, true,
+                                        ref_bits<2 * (MQ == 2 ? 2 : 4)>(prbs_bits, pwin + 2 * p.bps * lane), false,
                                         phase_tab(p, lane), 1.0f / p.scale, zin ? zin + (k0 - g.pay_lo) : nullptr,
                                         last ? &G : nullptr);
     const long long wq = (k0 - g.pay_lo) / kWin;

@@ -40,16 +40,21 @@ __device__ __forceinline__ void decode_pair(uint32_t b0, uint32_t b1, uint32_t b
     }
 }
 
-__global__ void k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ codes,
-                         const uint16_t *__restrict__ codes_prev, long long nb, int nhist,
-                         long long prev_off, int first_call, int order, long long *s1,
-                         long long *s2, LatRecord *lat, int lat_slot)
+// With `sums` (PAM) also the buffer's integer sums; the CTA that takes the last ticket turns
+// them into the call's mean and 1 / deviation (slot) and clears them: the division and the
+// square root in FP64 (a few thousand cycles on this part) run once per call instead of at
+// the start of every CTA of the filter.
+constexpr int kUnpackThreads = 256;
+__global__ void __launch_bounds__(kUnpackThreads)
+    k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ codes, const uint16_t *__restrict__ codes_prev,
+             long long nb, int nhist, long long prev_off, int first_call, int order, DevState *sums, int slot,
+             LatRecord *lat, int lat_slot)
 {
     pdl_wait();
     long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (lat && g == 0) lat_start(lat, lat_slot);
     long long ngroups = nb / 8;
-    long long lsum = 0, lsq = 0;
+    unsigned lsum = 0, lsq = 0;   // 8 samples: below 2^28; a warp's 256: below 2^32
     if (g < ngroups) {
         const uint32_t *w = reinterpret_cast<const uint32_t *>(in + 12 * g);
         uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2);
@@ -69,10 +74,8 @@ __global__ void k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ 
         o.z = s[4] | (s[5] << 16);
         o.w = s[6] | (s[7] << 16);
         *reinterpret_cast<uint4 *>(codes + nhist + 8 * g) = o;
-        if (s1) {
 #pragma unroll
-            for (int i = 0; i < 8; i++) { lsum += s[i]; lsq += (long long)s[i] * s[i]; }
-        }
+        for (int i = 0; i < 8; i++) { lsum += s[i]; lsq += s[i] * s[i]; }
     } else if (g < ngroups + nhist) {
         long long j = g - ngroups;   // history sample j
         uint16_t v;
@@ -85,35 +88,47 @@ __global__ void k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ 
         }
         codes[j] = v;
     }
-    if (s1) {
-        // block reduction then one atomic per CTA (integer: exact and order free)
-        __shared__ long long r1[32], r2[32];
-        for (int o = 16; o; o >>= 1) {
-            lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-            lsq += __shfl_xor_sync(0xffffffffu, lsq, o);
-        }
-        int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (sums) {
+        // one atomic per CTA and sum (integer: exact and order free)
+        __shared__ unsigned r1[kUnpackThreads / 32], r2[kUnpackThreads / 32];
+        lsum = __reduce_add_sync(0xffffffffu, lsum);
+        lsq = __reduce_add_sync(0xffffffffu, lsq);
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         if (lane == 0) { r1[wid] = lsum; r2[wid] = lsq; }
         __syncthreads();
         if (threadIdx.x == 0) {
-            long long a = 0, b = 0;
-            for (int i = 0; i < (int)(blockDim.x >> 5); i++) { a += r1[i]; b += r2[i]; }
-            if (a) atomicAdd(reinterpret_cast<unsigned long long *>(s1), (unsigned long long)a);
-            if (b) atomicAdd(reinterpret_cast<unsigned long long *>(s2), (unsigned long long)b);
+            unsigned long long a = 0, b = 0;
+#pragma unroll
+            for (int i = 0; i < kUnpackThreads / 32; i++) { a += r1[i]; b += r2[i]; }
+            unsigned long long *S1 = reinterpret_cast<unsigned long long *>(&sums->pam_s1),
+                               *S2 = reinterpret_cast<unsigned long long *>(&sums->pam_s2);
+            if (a) atomicAdd(S1, a);
+            if (b) atomicAdd(S2, b);
+            __threadfence();
+            if (atomicAdd(&sums->pam_ticket, 1u) == gridDim.x - 1) {
+                __threadfence();
+                const double mu = (double)(long long)atomicExch(S1, 0ull) / (double)nb;
+                const double var = (double)(long long)atomicExch(S2, 0ull) / (double)nb - mu * mu;
+                const double inv = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
+                sums->pam_nd[slot][0] = mu;
+                sums->pam_nd[slot][1] = inv;
+                sums->pam_nf[slot][0] = (float)mu;
+                sums->pam_nf[slot][1] = (float)inv;
+                sums->pam_ticket = 0u;
+            }
         }
     }
 }
 
 cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *codes_prev,
                           long long nb, int nhist, long long prev_off, int first_call,
-                          int pack_order, long long *s1, long long *s2, cudaStream_t st, LatRecord *lat,
+                          int pack_order, DevState *sums, int slot, cudaStream_t st, LatRecord *lat,
                           int lat_slot, bool pdl)
 {
     long long items = nb / 8 + nhist;
-    int tpb = 256;
-    unsigned grid = (unsigned)((items + tpb - 1) / tpb);
-    return launch_k(k_unpack, grid, tpb, 0, st, pdl, in, codes, codes_prev, nb, nhist, prev_off, first_call, pack_order, s1,
-                    s2, lat, lat_slot);
+    unsigned grid = (unsigned)((items + kUnpackThreads - 1) / kUnpackThreads);
+    return launch_k(k_unpack, grid, kUnpackThreads, 0, st, pdl, in, codes, codes_prev, nb, nhist, prev_off, first_call,
+                    pack_order, sums, slot, lat, lat_slot);
 }
 
 // ============================================================= KK Hilbert
@@ -1585,27 +1600,29 @@ cudaError_t launch_kk_fdmf(const float2 *E, long long ebase, long long f_prev, l
 // =========================================================== PAM matched filter
 // x[n] = (code[n] - mu) / sd with the buffer's exact integer moments, x[n < 0] = 0;
 // y[m] = sum_i h_i x[m - i] at 2 samples/symbol.
+
+// first CTA of a filter: the equaliser's history [ybase, f_prev), and the debug view of the
+// call's mean and deviation
+__device__ __forceinline__ void pam_carry(DevState *dst, int slot, float *__restrict__ Y, long long ybase, long long f_prev,
+                                          const float *__restrict__ Y_prev, long long ybase_prev)
+{
+    for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
+        Y[m - ybase] = (m < 0) ? 0.f : Y_prev[m - ybase_prev];
+    if (threadIdx.x == 0) {
+        dst->pam_mu = dst->pam_nd[slot][0];
+        dst->pam_inv_sd = dst->pam_nd[slot][1];
+    }
+}
+
 __global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *__restrict__ codes, long long cbase,
-                                                  long long nb, long long n_end, long long f_prev, long long f_k,
+                                                  long long n_end, long long f_prev, long long f_k,
                                                   const float *__restrict__ rrc, int hmf, DevState *dst,
-                                                  int parity, float *__restrict__ Y, long long ybase,
+                                                  int slot, float *__restrict__ Y, long long ybase,
                                                   const float *__restrict__ Y_prev, long long ybase_prev)
 {
     extern __shared__ float xf[];
-    __shared__ float s_mu, s_inv;
     pdl_wait();
-    if (threadIdx.x == 0) {
-        double mu = (double)dst->pam_s1[parity] / (double)nb;
-        double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
-        double inv = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
-        s_mu = (float)mu;
-        s_inv = (float)inv;
-        if (blockIdx.x == 0) {
-            dst->pam_mu = mu;
-            dst->pam_inv_sd = inv;
-        }
-    }
-    __syncthreads();
+    const float s_mu = dst->pam_nf[slot][0], s_inv = dst->pam_nf[slot][1];
     long long m0 = f_prev + (long long)blockIdx.x * kMfOut;
     int L = kMfOut + 2 * hmf;
     long long n0 = m0 - hmf;
@@ -1615,14 +1632,7 @@ __global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *__restrict__ 
         if (n >= 0 && n < n_end) v = ((float)codes[n - cbase] - s_mu) * s_inv;
         xf[i] = v;
     }
-    if (blockIdx.x == 0) {
-        for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
-            Y[m - ybase] = (m < 0) ? 0.f : Y_prev[m - ybase_prev];
-        if (threadIdx.x == 0) {   // the sums of the call after next start from zero
-            dst->pam_s1[(parity + 2) % 3] = 0;
-            dst->pam_s2[(parity + 2) % 3] = 0;
-        }
-    }
+    if (blockIdx.x == 0) pam_carry(dst, slot, Y, ybase, f_prev, Y_prev, ybase_prev);
     __syncthreads();
     long long m = m0 + threadIdx.x;
     if (m >= f_k) return;
@@ -1636,26 +1646,16 @@ __global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *__restrict__ 
 // The normalised code x[n] = (code - mu) / sd of the call (complex, imaginary part 0)
 // for stream samples [cbase, n_end), the input of the resampler (which treats
 // samples before the stream as zero); the call's mean and deviation come from the
-// exact integer sums, and the sums of the next call start from zero.
-__global__ void k_pam_norm(const uint16_t *__restrict__ codes, long long cbase, long long nb, long long n_end,
-                           DevState *dst, int parity, float2 *__restrict__ X)
+// exact integer sums.
+__global__ void k_pam_norm(const uint16_t *__restrict__ codes, long long cbase, long long n_end, DevState *dst, int slot,
+                           float2 *__restrict__ X)
 {
-    __shared__ float s_mu, s_inv;
-    if (threadIdx.x == 0) {
-        double mu = (double)dst->pam_s1[parity] / (double)nb;
-        double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
-        double inv = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
-        s_mu = (float)mu;
-        s_inv = (float)inv;
-    }
-    __syncthreads();
+    const float mu = dst->pam_nf[slot][0], inv = dst->pam_nf[slot][1];
     const long long n = cbase + (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < n_end) X[n - cbase] = make_float2(((float)codes[n - cbase] - s_mu) * s_inv, 0.f);
+    if (n < n_end) X[n - cbase] = make_float2(((float)codes[n - cbase] - mu) * inv, 0.f);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        dst->pam_mu = (double)s_mu;
-        dst->pam_inv_sd = (double)s_inv;
-        dst->pam_s1[(parity + 2) % 3] = 0;   // the sums of the call after next start from zero
-        dst->pam_s2[(parity + 2) % 3] = 0;
+        dst->pam_mu = (double)mu;
+        dst->pam_inv_sd = (double)inv;
     }
 }
 
@@ -1686,11 +1686,11 @@ __global__ void __launch_bounds__(kMfOut) k_pam_mf_r(const float2 *__restrict__ 
     Y[m - ybase] = a;
 }
 
-cudaError_t launch_pam_norm(const uint16_t *codes, long long cbase, long long nb, long long n_end, DevState *dst,
-                            int parity, float2 *X, cudaStream_t st)
+cudaError_t launch_pam_norm(const uint16_t *codes, long long cbase, long long n_end, DevState *dst, int slot, float2 *X,
+                            cudaStream_t st)
 {
     const long long n = n_end - cbase;
-    k_pam_norm<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(codes, cbase, nb, n_end, dst, parity, X);
+    k_pam_norm<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(codes, cbase, n_end, dst, slot, X);
     return cudaGetLastError();
 }
 
@@ -1715,41 +1715,22 @@ cudaError_t launch_pam_mf_r(const float2 *R, long long rbase, long long f_prev, 
 // 1024}, a transpose, 32-point inverse DFTs over the former lane index; lane m_a
 // keeps m_b = 8 .. 23 (m = 256 .. 767), whose real part is y.
 __global__ void __launch_bounds__(32 * kFdWarps, 4)
-    k_pam_fd1024(const uint16_t *__restrict__ codes, long long cbase, long long nb, long long n_end,
+    k_pam_fd1024(const uint16_t *__restrict__ codes, long long cbase, long long n_end,
                  long long b_first, long long nblk, const float2 *__restrict__ H, const float2 *__restrict__ tw,
-                 DevState *dst, int parity, float *__restrict__ Y, long long ybase, long long f_prev,
+                 DevState *dst, int slot, float *__restrict__ Y, long long ybase, long long f_prev,
                  const float *__restrict__ Y_prev, long long ybase_prev, float2 *__restrict__ clk, int wbin)
 {
     __shared__ float2 s_tw[1024];
     __shared__ float2 s_t[kFdWarps][32 * kFdPitch];
-    __shared__ float s_mu, s_inv;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < 1024; i += blockDim.x) s_tw[i] = tw[i];
     pdl_wait();
-    if (threadIdx.x == 0) {
-        double mu = (double)dst->pam_s1[parity] / (double)nb;
-        double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
-        double inv = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
-        s_mu = (float)mu;
-        s_inv = (float)inv;
-    }
     __syncthreads();
-    if (blockIdx.x == 0) {
-        for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
-            Y[m - ybase] = (m < 0) ? 0.f : Y_prev[m - ybase_prev];
-        if (threadIdx.x == 0) {   // debug view; the sums of the next call start from zero
-            double mu = (double)dst->pam_s1[parity] / (double)nb;
-            double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
-            dst->pam_mu = mu;
-            dst->pam_inv_sd = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
-            dst->pam_s1[(parity + 2) % 3] = 0;
-            dst->pam_s2[(parity + 2) % 3] = 0;
-        }
-    }
+    if (blockIdx.x == 0) pam_carry(dst, slot, Y, ybase, f_prev, Y_prev, ybase_prev);
     const long long bi = (long long)blockIdx.x * kFdWarps + w;
     if (bi >= nblk) return;
     const long long blk = b_first + bi, n0 = 512 * blk - 256;
-    const float mu = s_mu, inv = s_inv;
+    const float mu = dst->pam_nf[slot][0], inv = dst->pam_nf[slot][1];
     float2 x[32];
 #pragma unroll
     for (int q = 0; q < 32; q++) {
@@ -1796,106 +1777,119 @@ __global__ void __launch_bounds__(32 * kFdWarps, 4)
     for (int mb = 8; mb < 24; mb++) Y[s0 + lane + 32 * (mb - 8)] = x[mb].x;
 }
 
-cudaError_t launch_pam_fd1024(const uint16_t *codes, long long cbase, long long nb, long long n_end,
+cudaError_t launch_pam_fd1024(const uint16_t *codes, long long cbase, long long n_end,
                               long long f_prev, long long f_k, const float2 *H, const float2 *tw, DevState *dst,
-                              int parity, float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
+                              int slot, float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
                               cudaStream_t st, float2 *clk, int wbin, bool pdl)
 {
     if (f_prev % 512 || f_k % 512 || wbin < 0 || wbin > 31) return cudaErrorInvalidValue;
     const long long nblk = (f_k - f_prev) / 512;
     if (nblk <= 0) return cudaSuccess;
-    return launch_k(k_pam_fd1024, (unsigned)((nblk + kFdWarps - 1) / kFdWarps), 32 * kFdWarps, 0, st, pdl, codes, cbase, nb,
-                    n_end, f_prev / 512, nblk, H, tw, dst, parity, Y, ybase, f_prev, Y_prev, ybase_prev, clk, wbin);
+    return launch_k(k_pam_fd1024, (unsigned)((nblk + kFdWarps - 1) / kFdWarps), 32 * kFdWarps, 0, st, pdl, codes, cbase,
+                    n_end, f_prev / 512, nblk, H, tw, dst, slot, Y, ybase, f_prev, Y_prev, ybase_prev, clk, wbin);
 }
 
-// Register-tiled PAM matched filter for a compile-time half length HMF: each thread
-// computes kPmR consecutive outputs from a sliding window held in registers (one
-// shared-memory load per tap), the taps read from shared memory as broadcasts.  Per
-// output the products are accumulated in the same order as k_pam_mf (tap index
-// ascending), so the outputs are the same bit for bit.
+// Register-tiled PAM matched filter for a compile-time half length HMF (a multiple of 4):
+// each thread computes kPmR consecutive outputs from a window of kPmR + 2 HMF inputs held in
+// registers, read from shared memory in 16-byte pieces; four spare floats per 32 keep the
+// stride-8 reads (and the staging stores) free of most bank conflicts.  The codes are loaded
+// eight at a time, the taps are kernel parameters (constant operands of the FMAs).  Per
+// output the products are accumulated in the same order as k_pam_mf (tap index ascending),
+// so the outputs are the same bit for bit.  Bound by latency (one tile per CTA, 264 FMAs a
+// thread).  2^20 samples: 6.3 us; 12.7 us with a 4-byte conflicting load per tap, 2-byte
+// code loads and the FP64 mean and deviation formed in every CTA.
 constexpr int kPmThreads = 128, kPmR = 8, kPmTile = kPmThreads * kPmR;
+__host__ __device__ __forceinline__ constexpr int pad32(int i) { return i + ((i >> 5) << 2); }
+template <int HMF>
+struct PmTaps {
+    float h[2 * HMF + 1];
+};
 
 template <int HMF>
-__global__ void __launch_bounds__(kPmThreads) k_pam_mf_t(const uint16_t *__restrict__ codes, long long cbase,
-                                                        long long nb, long long n_end, long long f_prev, long long f_k,
-                                                        const float *__restrict__ rrc, DevState *dst, int parity,
-                                                        float *__restrict__ Y, long long ybase,
-                                                        const float *__restrict__ Y_prev, long long ybase_prev)
+__global__ void __launch_bounds__(kPmThreads)
+    k_pam_mf_t(const uint16_t *__restrict__ codes, long long cbase, long long n_end, long long f_prev, long long f_k,
+               const __grid_constant__ PmTaps<HMF> taps, DevState *dst, int slot, float *__restrict__ Y, long long ybase,
+               const float *__restrict__ Y_prev, long long ybase_prev)
 {
-    __shared__ float xf[kPmTile + 2 * HMF];
-    __shared__ float s_h[2 * HMF + 1];
-    __shared__ float s_mu, s_inv;
-    for (int i = threadIdx.x; i <= 2 * HMF; i += kPmThreads) s_h[i] = __ldg(rrc + i);
+    constexpr int L = kPmTile + 2 * HMF, NW = kPmR + 2 * HMF;
+    static_assert(HMF % 4 == 0 && L % 8 == 0 && kPmR == 8, "16-byte pieces");
+    __shared__ __align__(16) float xf[pad32(L) + 4];
     pdl_wait();
-    if (threadIdx.x == 0) {
-        double mu = (double)dst->pam_s1[parity] / (double)nb;
-        double var = (double)dst->pam_s2[parity] / (double)nb - mu * mu;
-        double inv = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
-        s_mu = (float)mu;
-        s_inv = (float)inv;
-        if (blockIdx.x == 0) {
-            dst->pam_mu = mu;
-            dst->pam_inv_sd = inv;
+    const float mu = dst->pam_nf[slot][0], inv = dst->pam_nf[slot][1];
+    const long long m0 = f_prev + (long long)blockIdx.x * kPmTile, n0 = m0 - HMF;
+    const uint16_t *ct = codes + (n0 - cbase);
+    if (n0 >= 0 && n0 + L <= n_end && ((uintptr_t)ct & 15) == 0) {
+#pragma unroll
+        for (int k = 0; k < (L / 8 + kPmThreads - 1) / kPmThreads; k++) {
+            const int c = threadIdx.x + k * kPmThreads;
+            if (c >= L / 8) break;
+            const uint4 v = reinterpret_cast<const uint4 *>(ct)[c];
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            float x[8];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                x[2 * i] = ((float)(w[i] & 0xFFFFu) - mu) * inv;
+                x[2 * i + 1] = ((float)(w[i] >> 16) - mu) * inv;
+            }
+            float4 *d = reinterpret_cast<float4 *>(xf + pad32(8 * c));
+            d[0] = make_float4(x[0], x[1], x[2], x[3]);
+            d[1] = make_float4(x[4], x[5], x[6], x[7]);
+        }
+    } else {
+        for (int i = threadIdx.x; i < L; i += kPmThreads) {
+            const long long n = n0 + i;
+            xf[pad32(i)] = (n >= 0 && n < n_end) ? ((float)ct[i] - mu) * inv : 0.f;
         }
     }
+    if (blockIdx.x == 0) pam_carry(dst, slot, Y, ybase, f_prev, Y_prev, ybase_prev);
     __syncthreads();
-    const long long m0 = f_prev + (long long)blockIdx.x * kPmTile;
-    const long long n0 = m0 - HMF;
-    const float mu = s_mu, inv = s_inv;
-    for (int i = threadIdx.x; i < kPmTile + 2 * HMF; i += kPmThreads) {
-        const long long n = n0 + i;
-        xf[i] = (n >= 0 && n < n_end) ? ((float)codes[n - cbase] - mu) * inv : 0.f;
-    }
-    if (blockIdx.x == 0) {
-        for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
-            Y[m - ybase] = (m < 0) ? 0.f : Y_prev[m - ybase_prev];
-        if (threadIdx.x == 0) {   // the sums of the call after next start from zero
-            dst->pam_s1[(parity + 2) % 3] = 0;
-            dst->pam_s2[(parity + 2) % 3] = 0;
-        }
-    }
-    __syncthreads();
-    // output j = j0 + r: y = sum_{i=-HMF}^{HMF} h[i + HMF] xf[j + HMF - i]; with u = HMF - i
-    // running from 2 HMF down to 0 the window xf[j0 + u + r] slides down by one per tap
+    // output j = j0 + r: y = sum_{i=-HMF}^{HMF} h[i + HMF] xf[j + HMF - i], i ascending
     const int j0 = kPmR * threadIdx.x;
-    float win[kPmR], acc[kPmR];
+    float x[NW];
 #pragma unroll
-    for (int r = 0; r < kPmR; r++) {
-        win[r] = xf[j0 + 2 * HMF + r];
-        acc[r] = 0.f;
+    for (int q = 0; q < NW / 4; q++) {
+        const float4 v = *reinterpret_cast<const float4 *>(xf + pad32(j0 + 4 * q));
+        x[4 * q] = v.x;
+        x[4 * q + 1] = v.y;
+        x[4 * q + 2] = v.z;
+        x[4 * q + 3] = v.w;
     }
+    float acc[kPmR];
 #pragma unroll
-    for (int u = 2 * HMF; u >= 0; u--) {
-        const float hu = s_h[2 * HMF - u];
+    for (int r = 0; r < kPmR; r++) acc[r] = 0.f;
 #pragma unroll
-        for (int r = 0; r < kPmR; r++) acc[r] = fmaf(hu, win[r], acc[r]);
-        if (u > 0) {
+    for (int i = 0; i <= 2 * HMF; i++)
 #pragma unroll
-            for (int r = kPmR - 1; r > 0; r--) win[r] = win[r - 1];
-            win[0] = xf[j0 + u - 1];
-        }
-    }
+        for (int r = 0; r < kPmR; r++) acc[r] = fmaf(taps.h[i], x[2 * HMF - i + r], acc[r]);
     const long long mb = m0 + j0;
+    float *Yo = Y + (mb - ybase);
+    if (mb + kPmR <= f_k && ((uintptr_t)Yo & 15) == 0) {
+        reinterpret_cast<float4 *>(Yo)[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        reinterpret_cast<float4 *>(Yo)[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    } else {
 #pragma unroll
-    for (int r = 0; r < kPmR; r++)
-        if (mb + r < f_k) Y[mb + r - ybase] = acc[r];
+        for (int r = 0; r < kPmR; r++)
+            if (mb + r < f_k) Yo[r] = acc[r];
+    }
 }
 
-cudaError_t launch_pam_mf(const uint16_t *codes, long long cbase, long long nb, long long n_end, long long f_prev,
-                          long long f_k, const float *rrc, int hmf, DevState *dst, int parity,
+cudaError_t launch_pam_mf(const uint16_t *codes, long long cbase, long long n_end, long long f_prev,
+                          long long f_k, const float *rrc, const float *rrc_host, int hmf, DevState *dst, int slot,
                           float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
                           cudaStream_t st, bool pdl)
 {
     long long n = f_k - f_prev;
     if (hmf == 16) {   // the default span (16 symbols at 2 samples/symbol)
+        PmTaps<16> t;
+        memcpy(t.h, rrc_host, sizeof t.h);
         unsigned grid = (unsigned)((n + kPmTile - 1) / kPmTile);
-        return launch_k(k_pam_mf_t<16>, grid, kPmThreads, 0, st, pdl, codes, cbase, nb, n_end, f_prev, f_k, rrc, dst, parity,
-                        Y, ybase, Y_prev, ybase_prev);
+        return launch_k(k_pam_mf_t<16>, grid, kPmThreads, 0, st, pdl, codes, cbase, n_end, f_prev, f_k, t, dst, slot, Y, ybase,
+                        Y_prev, ybase_prev);
     }
     unsigned grid = (unsigned)((n + kMfOut - 1) / kMfOut);
     size_t smem = (size_t)(kMfOut + 2 * hmf) * sizeof(float);
-    return launch_k(k_pam_mf, grid, kMfOut, smem, st, pdl, codes, cbase, nb, n_end, f_prev, f_k, rrc, hmf, dst, parity, Y,
-                    ybase, Y_prev, ybase_prev);
+    return launch_k(k_pam_mf, grid, kMfOut, smem, st, pdl, codes, cbase, n_end, f_prev, f_k, rrc, hmf, dst, slot, Y, ybase,
+                    Y_prev, ybase_prev);
 }
 
 // bin and clear every latency slot still holding a record (rx_stats)

@@ -40,7 +40,10 @@ struct DevState {
     double cg[kSlots][4];                  // KK per slot: carrier re, carrier im, gain
     double cg_flush[4];                    // KK: carrier and gain of the last real buffer (flush)
     double pam_mu, pam_inv_sd;             // PAM: this call's normalisation (debug view)
-    long long pam_s1[3], pam_s2[3];        // PAM: integer sums of codes / codes^2, by call index mod 3
+    long long pam_s1, pam_s2;              // PAM: integer sums of codes / codes^2 of the call being unpacked
+    double pam_nd[3][2];                   // PAM: mean and 1 / deviation, by call index mod 3
+    float pam_nf[3][2];                    // the same in FP32
+    unsigned int pam_ticket;               // last-CTA ticket of the sums
     int unwrap_have[2], unwrap_b[2];       // pi/2 unwrap carry, by parity
     int diff_have[2], diff_q[2];           // differential coding: quadrant of the last symbol, by parity
     long long unwrap_m[2];
@@ -204,7 +207,7 @@ inline cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
 // (each returns cudaGetLastError() after enqueuing)
 cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *codes_prev,
                           long long nb, int nhist, long long prev_off, int first_call,
-                          int pack_order, long long *s1, long long *s2, cudaStream_t st,
+                          int pack_order, DevState *sums, int slot, cudaStream_t st,
                           LatRecord *lat, int lat_slot, bool pdl);
 
 // copy of the next call's packed history only (calls that emit no field)
@@ -247,20 +250,20 @@ cudaError_t launch_kk_fdmf(const float2 *E, long long ebase, long long f_prev, l
 
 // PAM frequency-domain form, 1024-point blocks (hop 512) at the input rate;
 // f_prev and f_k are multiples of 512
-cudaError_t launch_pam_fd1024(const uint16_t *codes, long long cbase, long long nb, long long n_end,
+cudaError_t launch_pam_fd1024(const uint16_t *codes, long long cbase, long long n_end,
                               long long f_prev, long long f_k, const float2 *H, const float2 *tw, DevState *dst,
-                              int parity, float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
+                              int slot, float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
                               cudaStream_t st, float2 *clk, int wbin, bool pdl);
 
 // PAM with the resampler: the call's normalised codes for [cbase, n_end) as a complex
 // series (imaginary 0), then the matched filter on the resampled series
-cudaError_t launch_pam_norm(const uint16_t *codes, long long cbase, long long nb, long long n_end, DevState *dst,
-                            int parity, float2 *X, cudaStream_t st);
+cudaError_t launch_pam_norm(const uint16_t *codes, long long cbase, long long n_end, DevState *dst, int slot, float2 *X,
+                            cudaStream_t st);
 cudaError_t launch_pam_mf_r(const float2 *R, long long rbase, long long f_prev, long long f_k, const float *rrc, int hmf,
                             float *Y, long long ybase, const float *Y_prev, long long ybase_prev, cudaStream_t st);
 
-cudaError_t launch_pam_mf(const uint16_t *codes, long long cbase, long long nb, long long n_end, long long f_prev,
-                          long long f_k, const float *rrc, int hmf, DevState *dst, int parity,
+cudaError_t launch_pam_mf(const uint16_t *codes, long long cbase, long long n_end, long long f_prev,
+                          long long f_k, const float *rrc, const float *rrc_host, int hmf, DevState *dst, int slot,
                           float *Y, long long ybase, const float *Y_prev, long long ybase_prev,
                           cudaStream_t st, bool pdl);
 
