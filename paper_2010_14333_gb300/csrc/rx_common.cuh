@@ -123,6 +123,16 @@ __device__ __forceinline__ f2x f2_add(f2x a, f2x b)
     return d;
 }
 
+// ticket of a CTA's contribution to sums that several CTAs add to with relaxed atomics: the
+// thread that made the adds releases them with the ticket, and the holder of the last ticket
+// has acquired all the others'
+__device__ __forceinline__ unsigned take_ticket(unsigned *ticket)
+{
+    unsigned old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(ticket) : "memory");
+    return old;
+}
+
 // padded shared-memory index: one spare element per 16 avoids bank conflicts
 // in the stride-16 radix-16 pass
 __device__ __forceinline__ int pad16(int i) { return i + (i >> 4); }

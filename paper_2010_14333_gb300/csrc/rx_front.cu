@@ -44,79 +44,91 @@ __device__ __forceinline__ void decode_pair(uint32_t b0, uint32_t b1, uint32_t b
 // them into the call's mean and 1 / deviation (slot) and clears them: the division and the
 // square root in FP64 (a few thousand cycles on this part) run once per call instead of at
 // the start of every CTA of the filter.
-constexpr int kUnpackThreads = 256;
+constexpr int kUnpackThreads = 256, kUnpackPer = 2;   // threads per CTA, groups of 8 samples per thread
 __global__ void __launch_bounds__(kUnpackThreads)
     k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ codes, const uint16_t *__restrict__ codes_prev,
              long long nb, int nhist, long long prev_off, int first_call, int order, DevState *sums, int slot,
              LatRecord *lat, int lat_slot)
 {
     pdl_wait();
-    long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (lat && g == 0) lat_start(lat, lat_slot);
-    long long ngroups = nb / 8;
-    unsigned lsum = 0, lsq = 0;   // 8 samples: below 2^28; a warp's 256: below 2^32
-    if (g < ngroups) {
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(in + 12 * g);
-        uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2);
-        uint32_t by[12];
+    if (lat && blockIdx.x == 0 && threadIdx.x == 0) lat_start(lat, lat_slot);
+    const long long ngroups = nb / 8, g0 = (long long)blockIdx.x * (kUnpackPer * kUnpackThreads) + threadIdx.x;
+    const uint32_t *in32 = reinterpret_cast<const uint32_t *>(in);
+    uint32_t w[kUnpackPer][3];
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            by[i] = (w0 >> (8 * i)) & 0xFFu;
-            by[4 + i] = (w1 >> (8 * i)) & 0xFFu;
-            by[8 + i] = (w2 >> (8 * i)) & 0xFFu;
-        }
-        uint32_t s[8];
+    for (int k = 0; k < kUnpackPer; k++) {   // every load issues first
+        const long long g = g0 + k * kUnpackThreads;
+        if (g < ngroups)
 #pragma unroll
-        for (int p = 0; p < 4; p++) decode_pair(by[3 * p], by[3 * p + 1], by[3 * p + 2], order, s[2 * p], s[2 * p + 1]);
-        uint4 o;
-        o.x = s[0] | (s[1] << 16);
-        o.y = s[2] | (s[3] << 16);
-        o.z = s[4] | (s[5] << 16);
-        o.w = s[6] | (s[7] << 16);
-        *reinterpret_cast<uint4 *>(codes + nhist + 8 * g) = o;
-#pragma unroll
-        for (int i = 0; i < 8; i++) { lsum += s[i]; lsq += s[i] * s[i]; }
-    } else if (g < ngroups + nhist) {
-        long long j = g - ngroups;   // history sample j
-        uint16_t v;
-        if (first_call) {            // before the stream: first sample replicated
-            uint32_t a, b;
-            decode_pair(in[0], in[1], in[2], order, a, b);
-            v = (uint16_t)a;
-        } else {
-            v = codes_prev[prev_off + j];
-        }
-        codes[j] = v;
+            for (int i = 0; i < 3; i++) w[k][i] = __ldg(in32 + 3 * g + i);
     }
-    if (sums) {
-        // one atomic per CTA and sum (integer: exact and order free)
-        __shared__ unsigned r1[kUnpackThreads / 32], r2[kUnpackThreads / 32];
-        lsum = __reduce_add_sync(0xffffffffu, lsum);
-        lsq = __reduce_add_sync(0xffffffffu, lsq);
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        if (lane == 0) { r1[wid] = lsum; r2[wid] = lsq; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long a = 0, b = 0;
+    unsigned lsum = 0;                // 8 samples of 12 bits per group
+    unsigned long long wsq = 0;       // lane 0: the warp's squares (256 samples: below 2^32 per group)
 #pragma unroll
-            for (int i = 0; i < kUnpackThreads / 32; i++) { a += r1[i]; b += r2[i]; }
-            unsigned long long *S1 = reinterpret_cast<unsigned long long *>(&sums->pam_s1),
-                               *S2 = reinterpret_cast<unsigned long long *>(&sums->pam_s2);
-            if (a) atomicAdd(S1, a);
-            if (b) atomicAdd(S2, b);
-            __threadfence();
-            if (atomicAdd(&sums->pam_ticket, 1u) == gridDim.x - 1) {
-                __threadfence();
-                const double mu = (double)(long long)atomicExch(S1, 0ull) / (double)nb;
-                const double var = (double)(long long)atomicExch(S2, 0ull) / (double)nb - mu * mu;
-                const double inv = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
-                sums->pam_nd[slot][0] = mu;
-                sums->pam_nd[slot][1] = inv;
-                sums->pam_nf[slot][0] = (float)mu;
-                sums->pam_nf[slot][1] = (float)inv;
-                sums->pam_ticket = 0u;
+    for (int k = 0; k < kUnpackPer; k++) {
+        const long long g = g0 + k * kUnpackThreads;
+        unsigned lsq = 0;
+        if (g < ngroups) {
+            uint32_t by[12];
+#pragma unroll
+            for (int i = 0; i < 12; i++) by[i] = (w[k][i >> 2] >> (8 * (i & 3))) & 0xFFu;
+            uint32_t s[8];
+#pragma unroll
+            for (int p = 0; p < 4; p++)
+                decode_pair(by[3 * p], by[3 * p + 1], by[3 * p + 2], order, s[2 * p], s[2 * p + 1]);
+            *reinterpret_cast<uint4 *>(codes + nhist + 8 * g) =
+                make_uint4(s[0] | (s[1] << 16), s[2] | (s[3] << 16), s[4] | (s[5] << 16), s[6] | (s[7] << 16));
+#pragma unroll
+            for (int i = 0; i < 8; i++) { lsum += s[i]; lsq += s[i] * s[i]; }
+        } else if (g < ngroups + nhist) {
+            const long long j = g - ngroups;   // history sample j
+            uint16_t v;
+            if (first_call) {            // before the stream: first sample replicated
+                uint32_t a, b;
+                decode_pair(in[0], in[1], in[2], order, a, b);
+                v = (uint16_t)a;
+            } else {
+                v = codes_prev[prev_off + j];
             }
+            codes[j] = v;
         }
+        if (sums) wsq += __reduce_add_sync(0xffffffffu, lsq);
+    }
+    if (!sums) return;
+    // one atomic per CTA and sum (integer: exact and order free)
+    __shared__ unsigned long long r[2][kUnpackThreads / 32];
+    const unsigned wsum = __reduce_add_sync(0xffffffffu, lsum);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) { r[0][wid] = wsum; r[1][wid] = wsq; }
+    __syncthreads();
+    if (wid != 0) return;
+    unsigned long long *S[2] = {reinterpret_cast<unsigned long long *>(&sums->pam_s1),
+                                reinterpret_cast<unsigned long long *>(&sums->pam_s2)};
+    unsigned last = 0;
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            unsigned long long a = 0;
+#pragma unroll
+            for (int i = 0; i < kUnpackThreads / 32; i++) a += r[q][i];
+            if (a) atomicAdd(S[q], a);
+        }
+        last = take_ticket(&sums->pam_ticket) == gridDim.x - 1;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __syncwarp();   // what lane 0's ticket acquired, for the other lanes
+    // lane 0 divides the sum, lane 1 the sum of squares
+    double q = 0.0;
+    if (lane < 2) q = (double)(long long)atomicExch(lane ? S[1] : S[0], 0ull) / (double)nb;
+    const double mu = __shfl_sync(0xffffffffu, q, 0), m2 = __shfl_sync(0xffffffffu, q, 1);
+    if (lane == 0) {
+        const double var = m2 - mu * mu;
+        const double inv = (var > 0.0) ? 1.0 / sqrt(var) : 1.0;
+        sums->pam_nd[slot][0] = mu;
+        sums->pam_nd[slot][1] = inv;
+        sums->pam_nf[slot][0] = (float)mu;
+        sums->pam_nf[slot][1] = (float)inv;
+        sums->pam_ticket = 0u;
     }
 }
 
@@ -126,7 +138,8 @@ cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *co
                           int lat_slot, bool pdl)
 {
     long long items = nb / 8 + nhist;
-    unsigned grid = (unsigned)((items + kUnpackThreads - 1) / kUnpackThreads);
+    const int per = kUnpackPer * kUnpackThreads;
+    unsigned grid = (unsigned)((items + per - 1) / per);
     return launch_k(k_unpack, grid, kUnpackThreads, 0, st, pdl, in, codes, codes_prev, nb, nhist, prev_off, first_call,
                     pack_order, sums, slot, lat, lat_slot);
 }
@@ -514,30 +527,35 @@ __device__ __forceinline__ void carrier_sums(const KkGeom &g, DevState *dst, flo
     if (lane < 2) s_q[lane][wid] = __float2ll_rn((lane ? sim : sre) * (float)kCarrierUnit);
     if (lane == 2) s_q[2][wid] = si2;
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    long long a = 0, b = 0, c = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); i++) {
-        a += s_q[0][i];
-        b += s_q[1][i];
-        c += s_q[2][i];
-    }
+    if (wid != 0) return;
+    // lane q < 3 carries total q from here on
     unsigned long long *S = dst->csum[g.slot];
-    atomicAdd(S + 0, (unsigned long long)a);
-    atomicAdd(S + 1, (unsigned long long)b);
-    atomicAdd(S + 2, (unsigned long long)c);
-    __threadfence();
-    if (atomicAdd(&dst->ticket[g.slot], 1u) != (unsigned)(ncta - 1)) return;
-    __threadfence();
-    const long long ta = (long long)atomicExch(S + 0, 0ull), tb = (long long)atomicExch(S + 1, 0ull),
-                    tc = (long long)atomicExch(S + 2, 0ull);
+    if (lane < 3) {
+        long long a = 0;
+        for (int i = 0; i < (int)(blockDim.x >> 5); i++) a += s_q[lane][i];
+        atomicAdd(S + lane, (unsigned long long)a);
+        __threadfence();   // three threads' adds before lane 0's ticket
+    }
+    __syncwarp();
+    unsigned last = 0;
+    if (lane == 0) last = take_ticket(&dst->ticket[g.slot]) == (unsigned)(ncta - 1);
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __syncwarp();   // what lane 0's ticket acquired, for the other lanes
     const double cnt = (double)(g.e_k - g.e_prev);
-    const double cr = (double)ta / kCarrierUnit / cnt, ci = (double)tb / kCarrierUnit / cnt;
-    const double ibar = (double)tc / (2.0 * cnt);
-    const double P = ibar - (cr * cr + ci * ci);
-    dst->cg[g.slot][0] = cr;
-    dst->cg[g.slot][1] = ci;
-    dst->cg[g.slot][2] = (P > 0.0) ? 1.0 / sqrt((double)g.sps * P) : 1.0;
-    dst->ticket[g.slot] = 0u;
+    double m = 0.0;
+    if (lane < 3) {
+        const double t = (double)(long long)atomicExch(S + lane, 0ull);
+        m = lane < 2 ? t * (1.0 / kCarrierUnit) / cnt : t / (2.0 * cnt);   // the scaling is exact
+    }
+    const double cr = __shfl_sync(0xffffffffu, m, 0), ci = __shfl_sync(0xffffffffu, m, 1),
+                 ibar = __shfl_sync(0xffffffffu, m, 2);
+    if (lane == 0) {
+        const double P = ibar - (cr * cr + ci * ci);
+        dst->cg[g.slot][0] = cr;
+        dst->cg[g.slot][1] = ci;
+        dst->cg[g.slot][2] = (P > 0.0) ? 1.0 / sqrt((double)g.sps * P) : 1.0;
+        dst->ticket[g.slot] = 0u;
+    }
 }
 
 // field history for the matched filter: E[n], n in [e_prev - kEHist, e_prev) (E_prev null:
