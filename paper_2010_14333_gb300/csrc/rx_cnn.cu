@@ -826,7 +826,12 @@ __global__ void k_cnn_tobf(const float *__restrict__ prm, __nv_bfloat16 *__restr
 //      M = 128 tile covers the tile's 128 symbols;
 //   MLP 32 -> 64 (M = 128, N = 64) on the symbols, bias + GELU into FP16
 //      planes, then 64 -> 2 as one more MMA (N = 16, two live columns);
-//   decisions and window records as the FIR receiver.
+//   decisions by the lanes that hold the outputs, window records as the FIR receiver.
+// Row tiles of layers 1 and 2 are committed one by one, so that a tile's epilogue runs
+// while the next one's MMAs do, and a group passes six barriers per tile.  Bound by the
+// latency of each tile's chain of MMA commits, tensor-memory loads and barriers with four
+// tiles in flight per SM (tensor pipe 21 % active): 192 us per 2^20 symbols; 196 us with one
+// commit per layer, eleven barriers and the decisions on two of eight warps.
 // Inference precision: BF16 operands by default, FP16 as the alternative
 // (activations and weights, converted from the FP32 master weights), FP32
 // accumulation in tensor memory; bias and GELU in the same packed type, GELU by its
@@ -861,17 +866,18 @@ struct RxSmem {
     static constexpr int H1 = 0;                          // fp16 planes [4][kR1][16 B] (h1, then h3)
     static constexpr int HX = H1 + 4 * kR1 * 16;          // the layer-1 input plane [kRX][16 B], then the
                                                           // even/odd h2 planes [2][4][kRE][16 B], then the
-                                                          // hidden planes [8][128][16 B], then the outputs
-                                                          // float [kTS][2]
+                                                          // hidden planes [8][128][16 B]
     static constexpr int HXB = 2 * 4 * kRE * 16;
     static constexpr int XS = HX + HXB;                   // float2 [kP0]: the next tile's input (async copy)
-    static constexpr int BAR = XS + kP0 * 8;              // mbarrier
-    static constexpr int GROUP = (BAR + 16 + 127) & ~127;
+    static constexpr int BAR = XS + kP0 * 8;              // mbarriers, one per row tile of layers 1 and 2
+    static constexpr int REC = BAR + 32;                  // uint32 [2 tiles][kWinT][4]: window records being summed
+    static constexpr int GROUP = (REC + 2 * kWinT * 16 + 127) & ~127;
     static constexpr int SLOT = GRP + kRxGroups * GROUP;  // tensor-memory base address
     static constexpr int TOTAL = SLOT + 16;
 };
 static_assert(kRX * 16 <= RxSmem::HXB && 8 * 128 * 16 <= RxSmem::HXB, "aliases of the HX region fit");
 static_assert(RxSmem::TOTAL <= 227 * 1024, "one receiver CNN CTA per SM");
+static_assert(kMT1 <= 3 && kMT2 <= 3 && kWinT == 2, "one mbarrier per row tile, two windows per tile");
 static_assert(2 * (kRE - 4) == kP2, "even / odd h2 rows cover the layer-2 positions");
 
 // barrier of one group's 256 threads (named barrier id, 1 + group); the second form
@@ -956,12 +962,13 @@ __global__ void __launch_bounds__(kRxThreads, 1)
     const int gbar = 1 + grp;   // the group's named barrier
     unsigned char *gb = sm + RxSmem::GRP + grp * RxSmem::GROUP;
     unsigned char *sH1 = gb + RxSmem::H1, *sHX = gb + RxSmem::HX;
-    float *os = reinterpret_cast<float *>(sHX);   // the outputs, after the hidden planes are consumed
+    uint32_t *rec = reinterpret_cast<uint32_t *>(gb + RxSmem::REC);
     float2 *xs = reinterpret_cast<float2 *>(gb + RxSmem::XS);
     uint64_t *bar = reinterpret_cast<uint64_t *>(gb + RxSmem::BAR);
     constexpr int PL1 = kR1 * 16, PLE = kRE * 16, EO = 4 * PLE;
 
-    if (gtid == 0) mbar_init(bar, 1);
+    if (gtid < 3) mbar_init(bar + gtid, 1);
+    if (gtid < 2 * kWinT * 4) rec[gtid] = 0;
     __syncwarp();
     if (warp == 0) tmem_alloc(tslot, kRxTmem);
     pdl_wait();
@@ -1035,49 +1042,64 @@ __global__ void __launch_bounds__(kRxThreads, 1)
     const uint64_t dH1 = umma_sdesc(aH1, PL1, 128), dW2 = umma_sdesc(aW2, 512, 128), dW3 = umma_sdesc(aW3, 512, 128);
     const uint64_t dEO = umma_sdesc(aHX, PLE, 128), dM1 = umma_sdesc(aM1, 1024, 128);
     const uint64_t dHid = umma_sdesc(aHX, 2048, 128), dM2 = umma_sdesc(aM2, 256, 128);
-    unsigned phase = 0;
+    unsigned phase = 0;   // bit b: phase of mbarrier b
     bool ok = true;
 
-    auto wait_mma = [&]() -> bool {
-        bool done = mbar_wait(bar, phase);
-        if (!done) {
+    // wait for the MMAs committed to mbarrier b; a wait that ran out is flagged and ends the
+    // group's loop at its next tile (no MMA of a later wait is waited for then)
+    auto wait_mma = [&](int b) {
+        if (ok && !mbar_wait(bar + b, (phase >> b) & 1u)) {
             atomicExch(err, (int)RX_ETIMEOUT);
-            mbar_wait(bar, phase);
+            mbar_wait(bar + b, (phase >> b) & 1u);
+            ok = false;
         }
-        phase ^= 1u;
-        return group_and(gbar, done);
+        phase ^= 1u << b;
+        __syncwarp();   // the tensor-memory loads that follow are warp-wide
+        tc_fence_after();
     };
-    // conv epilogue of MT row tiles: rows of this warp's lane quarter, channel groups
-    // 2 ch and 2 ch + 1 (8 channels each) one after the other, each with every row
-    // tile's accumulator load in flight before one wait; row -> address of its
-    // 16-byte FP16 row of channel group cq in the destination
-    auto conv_epi = [&](auto mt, int valid, const uint32_t *bias, auto dst_row) {
-        constexpr int MT = decltype(mt)::value;
+    // conv epilogue of row tile m: rows of this warp's lane quarter, channel groups 2 ch and
+    // 2 ch + 1 (8 channels each); row -> address of its 16-byte row of channel group cq in
+    // the destination
+    auto conv_epi = [&](int m, int valid, const uint32_t *bias, auto dst_row) {
+        if (128 * m + 32 * quarter >= valid) return;   // warp-uniform
+        uint32_t r[16];
+        tmem_ld16(tq + 32 * m + 16 * ch, r);
+        const int row = 128 * m + 32 * quarter + lane;
+        if (row >= valid) return;
 #pragma unroll
         for (int c = 0; c < 2; c++) {
             const int cq = 2 * ch + c;
-            uint32_t r[8 * MT];
-#pragma unroll
-            for (int m = 0; m < MT; m++)
-                tmem_ld8_nw(tq + 32 * m + 8 * cq, *reinterpret_cast<uint32_t(*)[8]>(r + 8 * m));
-            tmem_wait_ld(r);
             const uint4 b = *reinterpret_cast<const uint4 *>(bias + 4 * cq);
-#pragma unroll
-            for (int m = 0; m < MT; m++) {
-                const int row = 128 * m + 32 * quarter + lane;
-                const uint32_t *q = r + 8 * m;
-                if (row < valid)
-                    *reinterpret_cast<uint4 *>(dst_row(row, cq)) =
-                        make_uint4(gelu2<BF>(q[0], q[1], b.x), gelu2<BF>(q[2], q[3], b.y),
-                                   gelu2<BF>(q[4], q[5], b.z), gelu2<BF>(q[6], q[7], b.w));
-            }
+            const uint32_t *q = r + 8 * c;
+            *reinterpret_cast<uint4 *>(dst_row(row, cq)) =
+                make_uint4(gelu2<BF>(q[0], q[1], b.x), gelu2<BF>(q[2], q[3], b.y), gelu2<BF>(q[4], q[5], b.z),
+                           gelu2<BF>(q[6], q[7], b.w));
+        }
+    };
+    // records of tile t (buffer tp), complete once the group has passed a barrier after it
+    auto put_records = [&](int t, int tp) {
+        if (gtid < kWinT && kWinT * t + gtid < nwin) {
+            uint4 *rc = reinterpret_cast<uint4 *>(rec + 4 * (kWinT * tp + gtid));
+            const uint4 v = *rc;
+            const int s = kWinT * t + gtid;
+            winb[s] = 0;
+            winrec[s] = make_uint4(v.x, v.y, v.z, v.w << 8);
+            *rc = make_uint4(0, 0, 0, 0);
         }
     };
 
-    for (int t = t0; t < ntiles && ok; t += tstep) {
+    const int NB = mq == 2 ? 1 : 2, BPS = 2 * NB;
+    int tlast = -1, tp = 0;   // the tile whose records are being summed, and its buffer
+    // PRBS position of the tile's first bit, and how far it moves per tile of this group
+    int pos_t = (int)((long long)BPS * (k_first + (long long)kTS * t0) % 32767);
+    const int pos_step = (int)((long long)BPS * kTS * tstep % 32767);
+    for (int t = t0; t < ntiles; t += tstep) {
         // layer-1 input plane: row p = positions p .. p+3 (8 reals) in FP16, zero past kP0
         cp_async_wait_all();
-        group_sync(gbar);   // the tile's input is in xs
+        if (!group_and(gbar, ok)) break;   // the tile's input is in xs
+        if (tlast >= 0) put_records(tlast, tp);
+        tlast = t;
+        tp ^= 1;
         for (int p = gtid; p < kRX; p += kRxGroupThreads) {
             uint32_t w[4];
 #pragma unroll
@@ -1093,35 +1115,56 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         if (gtid == 0) {
             tc_fence_after();
 #pragma unroll
-            for (int m = 0; m < kMT1; m++)
+            for (int m = 0; m < kMT1; m++) {
 #pragma unroll
                 for (int ks = 0; ks < 2; ks++)
                     umma_f16(tmem + 32 * m, dX + (((128 * m + 8 * ks) * 16) >> 4), dB1 + ((2 * ks * 512) >> 4), id32,
                              ks > 0);
-            umma_commit(bar);
+                umma_commit(bar + m);
+            }
         }
-        if (!(ok = wait_mma())) break;
-        tc_fence_after();
-        conv_epi(std::integral_constant<int, kMT1>(), kP1, bh,
-                 [&](int row, int cq) { return sH1 + cq * PL1 + row * 16; });
+        // the reference bits of this lane's symbol, long before the decisions
+        const int js = 32 * quarter + lane;                       // symbol of the tile
+        const long long ksym = (long long)kTS * t + js;           // payload symbol
+        int ref = 0;
+        if (ch == 0 && ksym < 64LL * nwin) {
+            int pos = pos_t + BPS * js;
+            pos = pos >= 32767 ? pos - 32767 : pos;
+            const uint32_t w0 = __ldg(prbs_bits + (pos >> 5)), w1w = __ldg(prbs_bits + (pos >> 5) + 1);
+            ref = (int)(__funnelshift_l(w1w, w0, pos & 31) >> (32 - BPS));
+        }
+        pos_t += pos_step;
+        pos_t = pos_t >= 32767 ? pos_t - 32767 : pos_t;
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < kMT1; m++) {
+            wait_mma(m);
+            conv_epi(m, kP1, bh, [&](int row, int cq) { return sH1 + cq * PL1 + row * 16; });
+        }
+        __syncwarp();
         fence_async_smem();
         tc_fence_before();
         group_sync(gbar);
-        // layer 2 (reads h1; the input plane is free)
+        // layer 2 (reads h1; the input plane is free): the epilogue of a row tile runs while
+        // the MMAs of the next one do
         if (gtid == 0) {
             tc_fence_after();
 #pragma unroll
-            for (int m = 0; m < kMT2; m++)
+            for (int m = 0; m < kMT2; m++) {
 #pragma unroll
                 for (int ks = 0; ks < 18; ks++)
                     umma_f16(tmem + 32 * m, dH1 + (((128 * m + ks / 2) * 16 + 2 * (ks & 1) * PL1) >> 4),
                              dW2 + ((2 * ks * 512) >> 4), id32, ks > 0);
-            umma_commit(bar);
+                umma_commit(bar + m);
+            }
         }
-        if (!(ok = wait_mma())) break;
-        tc_fence_after();
-        conv_epi(std::integral_constant<int, kMT2>(), kP2, bh + 16,
-                 [&](int row, int cq) { return sHX + (row & 1) * EO + cq * PLE + (row >> 1) * 16; });
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < kMT2; m++) {
+            wait_mma(m);
+            conv_epi(m, kP2, bh + 16, [&](int row, int cq) { return sHX + (row & 1) * EO + cq * PLE + (row >> 1) * 16; });
+        }
+        __syncwarp();
         fence_async_smem();
         tc_fence_before();
         group_sync(gbar);
@@ -1136,10 +1179,10 @@ __global__ void __launch_bounds__(kRxThreads, 1)
             }
             umma_commit(bar);
         }
-        if (!(ok = wait_mma())) break;
-        tc_fence_after();
-        conv_epi(std::integral_constant<int, 1>(), kTS, bh + 32,
-                 [&](int row, int cq) { return sH1 + cq * PL1 + row * 16; });   // h3, row = symbol
+        __syncwarp();
+        wait_mma(0);
+        conv_epi(0, kTS, bh + 32, [&](int row, int cq) { return sH1 + cq * PL1 + row * 16; });   // h3, row = symbol
+        __syncwarp();
         fence_async_smem();
         tc_fence_before();
         group_sync(gbar);
@@ -1151,8 +1194,8 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                 umma_f16(tmem, dH1 + ((2 * ks * PL1) >> 4), dM1 + ((2 * ks * 1024) >> 4), id64, ks > 0);
             umma_commit(bar);
         }
-        if (!(ok = wait_mma())) break;
-        tc_fence_after();
+        __syncwarp();
+        wait_mma(0);
 #pragma unroll
         for (int c = 0; c < 2; c++) {
             // hidden units 16 hq .. + 15 of symbol row -> planes 2 hq, 2 hq + 1 (the h2 planes are free)
@@ -1180,67 +1223,50 @@ __global__ void __launch_bounds__(kRxThreads, 1)
                 umma_f16(tmem + kColOut, dHid + ((2 * ks * 2048) >> 4), dM2 + ((2 * ks * 256) >> 4), id16, ks > 0);
             umma_commit(bar);
         }
-        if (!(ok = wait_mma())) break;
-        tc_fence_after();
-        // the projection has read the hidden planes: the outputs take their place
+        __syncwarp();
+        wait_mma(0);
+        // decisions and window records: the lanes that hold the outputs decide their symbol,
+        // two warps per window; the other warps go on to the next tile's input
         if (ch == 0) {
             uint32_t r[8];
             tmem_ld8(tq + kColOut, r);
-            const int j = 32 * quarter + lane;
             const float o0 = __uint_as_float(r[0]) + c2[0], o1 = __uint_as_float(r[1]) + c2[1];
-            os[2 * j] = o0;
-            os[2 * j + 1] = o1;
-            const long long ks = (long long)kTS * t + j;
-            if (soft && ks < 64LL * nwin) soft[ks] = make_float2(o0, o1);
-        }
-        tc_fence_before();
-        group_sync(gbar);
-        // decisions and window records: warp w < kWinT of the group takes window kWinT t + w
-        if (gwarp < kWinT && kWinT * t + gwarp < nwin) {
-            const int s = kWinT * t + gwarp;
-            const float *osw = os + 2 * 64 * gwarp;
-            const int NB = mq == 2 ? 1 : 2, BPS = 2 * NB;
-            long long k0 = k_first + (long long)s * CS;
-            int pwin = (int)(((long long)BPS * k0) % 32767);
-            unsigned eA = 0, eB = 0, se = 0, nn = 0;
-            for (int h = 0; h < 2; h++) {
-                int q = lane + 32 * h;
-                float vr = scale * osw[2 * q], vi = scale * osw[2 * q + 1];
+            unsigned eA = 0, eB = 0, se = 0, nr = 0;
+            if (ksym < 64LL * nwin) {
+                if (soft) soft[ksym] = make_float2(o0, o1);
+                const float vr = scale * o0, vi = scale * o1;
                 int LI = 0, LQ = 0;
-                bool nr = false;
+                bool near = false;
                 for (int jj = 0; jj < mq - 1; jj++) {
                     float th = (float)(2 * jj - (mq - 2));
                     LI += vr >= th;
                     LQ += vi >= th;
-                    nr |= fabsf(vr - th) < 1e-4f || fabsf(vi - th) < 1e-4f;
+                    near |= fabsf(vr - th) < 1e-4f || fabsf(vi - th) < 1e-4f;
                 }
-                dec[(size_t)s * CS + q] = (uint8_t)(LI | (LQ << 3) | (nr ? 64 : 0));
-                int pos = pwin + BPS * q;
-                uint32_t w0 = __ldg(prbs_bits + (pos >> 5)), w1w = __ldg(prbs_bits + (pos >> 5) + 1);
-                int ref = (int)(__funnelshift_l(w1w, w0, pos & 31) >> (32 - BPS));
-                for (int rq = 0; rq < 4; rq++) {
-                    int a = LI, bq = LQ;
-                    if (rq & 2) { a = mq - 1 - a; bq = mq - 1 - bq; }
-                    if (rq & 1) { int tt = a; a = bq; bq = mq - 1 - tt; }
-                    unsigned ne = __popc((((a ^ (a >> 1)) << NB) | (bq ^ (bq >> 1))) ^ ref);
-                    if (rq < 2) eA += ne << (16 * rq);
-                    else eB += ne << (16 * (rq - 2));
-                    se += (ne > 0) << (8 * rq);
-                }
-                nn += nr;
+                dec[ksym] = (uint8_t)(LI | (LQ << 3) | (near ? 64 : 0));
+                // bit errors under the four rotations (qam_window's codes)
+                const int cm = mq == 2 ? 1 : 2, gI = LI ^ (LI >> 1), gQ = LQ ^ (LQ >> 1);
+                const int X = ((gI << NB) | gQ) ^ ref, Xs = ((gQ << NB) | gI) ^ ref;
+                const unsigned n0 = __popc(X), n1 = __popc(Xs ^ cm), n2 = __popc(X ^ ((cm << NB) | cm)),
+                               n3 = __popc(Xs ^ (cm << NB));
+                eA = n0 + (n1 << 16);
+                eB = n2 + (n3 << 16);
+                se = (unsigned)(n0 > 0) | ((unsigned)(n1 > 0) << 8) | ((unsigned)(n2 > 0) << 16) |
+                     ((unsigned)(n3 > 0) << 24);
+                nr = near;
             }
-            eA = warp_sum_i(eA);
-            eB = warp_sum_i(eB);
-            se = warp_sum_i(se);
-            nn = warp_sum_i(nn);
-            if (lane == 0) {
-                winb[s] = 0;
-                winrec[s] = make_uint4(eA, eB, se, nn << 8);
-            }
+            eA = __reduce_add_sync(0xffffffffu, eA);
+            eB = __reduce_add_sync(0xffffffffu, eB);
+            se = __reduce_add_sync(0xffffffffu, se);
+            nr = __reduce_add_sync(0xffffffffu, nr);
+            uint32_t *rw = rec + 4 * (kWinT * tp + (quarter >> 1));
+            if (lane < 4) atomicAdd(rw + lane, lane == 0 ? eA : lane == 1 ? eB : lane == 2 ? se : nr);
         }
-        group_sync(gbar);   // the outputs are read before the next tile's input plane
+        tc_fence_before();
     }
     cp_async_wait_all();   // a prefetch may still be in flight after an early exit
+    group_sync(gbar);
+    if (tlast >= 0) put_records(tlast, tp);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(*tslot, kRxTmem);
