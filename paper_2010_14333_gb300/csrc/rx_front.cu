@@ -961,7 +961,7 @@ cudaError_t launch_kk_hist(const KkInput &inp, cudaStream_t st, const KkSync &sy
     pk.first_call = inp.first_call;
     pk.lat = inp.lat;
     pk.lat_slot = inp.lat_slot;
-    const cudaError_t e = launch_k(k_kk_hist, 32, 256, 0, st, sync.pdl, pk);
+    const cudaError_t e = launch_k(k_kk_hist, 32, 256, 0, st, sync.pdl_first, pk);
     if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
     return e;
 }
@@ -998,10 +998,10 @@ cudaError_t launch_kk_front(const KkGeom &g, const KkInput &inp, float2 *fftws, 
         if (sync.wait_inv) cudaStreamWaitEvent(st, sync.wait_inv, 0);
         prof_stage(prof, 1, st);
         if (g.N2 == kClN2)
-            e = launch_k(k_kk_cluster, g.npairs * kClC, kClThreads, kClSmem, st, sync.pdl, g, pk, tb, E, E_prev, dst);
+            e = launch_k(k_kk_cluster, g.npairs * kClC, kClThreads, kClSmem, st, sync.pdl_first, g, pk, tb, E, E_prev, dst);
         else
             e = launch_k(pk.order ? k_kk_block<1> : k_kk_block<0>, g.npairs + (inp.hist_next ? 1 : 0), kCtaK1,
-                         BkSmem::TOTAL, st, sync.pdl, g, pk, tb, E, E_prev, dst);
+                         BkSmem::TOTAL, st, sync.pdl_first, g, pk, tb, E, E_prev, dst);
         if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
         prof_stage(prof, -2, st);
         prof_stage(prof, -3, st);
@@ -1012,7 +1012,7 @@ cudaError_t launch_kk_front(const KkGeom &g, const KkInput &inp, float2 *fftws, 
     dim3 grid(kRowN2 / kCtaK1, g.npairs);
     dim3 grid_a(kRowN2 / kCtaK1, g.npairs + (inp.hist_next ? 1 : 0));
     prof_stage(prof, 1, st);
-    e = launch_k(pk.order ? k_kk_fwd<1, kRowN2> : k_kk_fwd<0, kRowN2>, grid_a, kCtaK1, 0, st, sync.pdl, g, pk, fftws, tb,
+    e = launch_k(pk.order ? k_kk_fwd<1, kRowN2> : k_kk_fwd<0, kRowN2>, grid_a, kCtaK1, 0, st, sync.pdl_first, g, pk, fftws, tb,
                  dst);
     if (sync.rec_fwd) cudaEventRecord(sync.rec_fwd, st);
     prof_stage(prof, -2, st);

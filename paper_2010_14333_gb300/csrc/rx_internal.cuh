@@ -218,7 +218,7 @@ cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *co
 // carries as history).
 struct KkSync {
     cudaEvent_t wait_fwd, rec_fwd, wait_inv;
-    bool pdl;   // one stream: launch every kernel as a programmatic dependent
+    bool pdl_first, pdl;   // programmatic dependent launch of the first kernel and of the others
 };
 cudaError_t launch_kk_hist(const KkInput &inp, cudaStream_t st, const KkSync &sync);
 

@@ -138,7 +138,7 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
     kin.first_call = 1;
     kin.lat = nullptr;
     kin.lat_slot = 0;
-    const KkSync none = {nullptr, nullptr, nullptr, true};
+    const KkSync none = {nullptr, nullptr, nullptr, true, true};
     if (launch_kk_front(g, kin, fftws, tb, reinterpret_cast<float2 *>(field_out), nullptr, nullptr, st, nullptr, none) !=
         cudaSuccess)
         return RX_ECUDA;
