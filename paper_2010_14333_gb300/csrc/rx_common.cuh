@@ -27,20 +27,62 @@ __device__ __forceinline__ float sqrt_approx(float x)
 }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 
-// 4-point DFT in place; forward kernel e^{-2 pi i nk/4} (INV: e^{+...}, unscaled)
+// ------------------------------------------------------------ packed FP32 pairs
+// Two FP32 values in one 64-bit register, operated on by the sm_100-family paired
+// FP32 instructions (fma.rn.f32x2 and friends): each half is an IEEE round-to-
+// nearest operation, identical to the scalar one, at one instruction per pair.
+typedef unsigned long long f2x;
+__device__ __forceinline__ f2x f2_pack(float a, float b)
+{
+    f2x r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 f2_unpack(f2x v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c)
+{
+    f2x d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2x f2_mul(f2x a, f2x b)
+{
+    f2x d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2x f2_add(f2x a, f2x b)
+{
+    f2x d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2x f2_sub(f2x a, f2x b)
+{
+    f2x d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// 4-point DFT in place; forward kernel e^{-2 pi i nk/4} (INV: e^{+...}, unscaled).  Complex
+// sums and differences are one packed instruction each; the rotated difference j (b - d)
+// comes from two scalar ones that write its parts in place, so nothing is swapped: 9
+// instructions instead of 16, every part rounded as before.
 template <bool INV>
 __device__ __forceinline__ void dft4(float2 &a, float2 &b, float2 &c, float2 &d)
 {
-    float2 s0 = cadd(a, c), s1 = csub(a, c), s2 = cadd(b, d), s3 = csub(b, d);
-    a = cadd(s0, s2);
-    c = csub(s0, s2);
-    if (!INV) {   // X1 = s1 - j s3, X3 = s1 + j s3
-        b = make_float2(s1.x + s3.y, s1.y - s3.x);
-        d = make_float2(s1.x - s3.y, s1.y + s3.x);
-    } else {      // X1 = s1 + j s3, X3 = s1 - j s3
-        b = make_float2(s1.x - s3.y, s1.y + s3.x);
-        d = make_float2(s1.x + s3.y, s1.y - s3.x);
-    }
+    const f2x A = f2_pack(a.x, a.y), B = f2_pack(b.x, b.y), C = f2_pack(c.x, c.y), D = f2_pack(d.x, d.y);
+    const f2x s0 = f2_add(A, C), s1 = f2_sub(A, C), s2 = f2_add(B, D);
+    const f2x r3 = f2_pack(b.y - d.y, d.x - b.x);   // -j (b - d)
+    a = f2_unpack(f2_add(s0, s2));
+    c = f2_unpack(f2_sub(s0, s2));
+    b = f2_unpack(INV ? f2_sub(s1, r3) : f2_add(s1, r3));   // X1 = s1 -+ j s3
+    d = f2_unpack(INV ? f2_add(s1, r3) : f2_sub(s1, r3));   // X3 = s1 +- j s3
 }
 
 // W16^m = e^{-2 pi i m / 16} for m = 0..9 (the products q0*k1 of a 4x4 split)
@@ -85,42 +127,6 @@ __device__ __forceinline__ void dft16(float2 (&x)[16])
     for (int k1 = 0; k1 < 4; k1++)
 #pragma unroll
         for (int k0 = 0; k0 < 4; k0++) x[k1 + 4 * k0] = t[4 * k1 + k0];
-}
-
-// ------------------------------------------------------------ packed FP32 pairs
-// Two FP32 values in one 64-bit register, operated on by the sm_100-family paired
-// FP32 instructions (fma.rn.f32x2 and friends): each half is an IEEE round-to-
-// nearest operation, identical to the scalar one, at one instruction per pair.
-typedef unsigned long long f2x;
-__device__ __forceinline__ f2x f2_pack(float a, float b)
-{
-    f2x r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 f2_unpack(f2x v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c)
-{
-    f2x d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f2x f2_mul(f2x a, f2x b)
-{
-    f2x d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2x f2_add(f2x a, f2x b)
-{
-    f2x d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
 }
 
 // ticket of a CTA's contribution to sums that several CTAs add to with relaxed atomics: the
