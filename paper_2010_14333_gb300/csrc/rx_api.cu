@@ -964,10 +964,13 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     int ds = (int)(h->calls % kSlots);   // decision slot of this call
     // KK in the pipeline: the field of odd calls on the second front-end stream.
     // Not with the CNN receiver: its decision kernel is persistent (one CTA per SM),
-    // and a second field in flight holds SMs it waits for.
-    const bool alt = three && h->kk && h->front2 && !h->cnn;
+    // and a second field in flight holds SMs it waits for.  Nor with 4096-point blocks, whose
+    // field is one short kernel: per 2^17 / 2^20 samples 19.4 / 25.9 us on one stream against
+    // 19.7 / 28.0 on two (2^16-point blocks, three kernels: 25.3 / 32.7 against 20.9 / 29.9).
+    const bool alt = three && h->kk && h->front2 && !h->cnn && h->N == 65536;
     if (alt && par) sf = h->front2;
-    const KkSync ksync = {alt ? h->ev_hist : nullptr, alt ? h->ev_hist : nullptr, alt ? h->ev_front : nullptr, pdl_first, pdl};
+    const KkSync ksync = {alt ? h->ev_hist : nullptr, alt ? h->ev_hist : nullptr, alt ? h->ev_front : nullptr, pdl_first,
+                          pdl || (!alt && h->prof_on <= 0)};   // one front stream: its kernels follow each other
     if (host_in) {
         in = h->in_stage[isl];
         if (sc != sf) cudaStreamWaitEvent(sc, h->ev_infree[isl], 0);   // the front end kInSlots calls back is done
