@@ -952,10 +952,12 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     cudaStream_t sm = three ? smid : sf;
     // the demap (and the copy of the bits) on a fourth stream, after its equaliser
     const bool four = two && stail;
+    h->prof_cur = h->prof_on > 0 && h->calls % h->prof_on == 0;
+    if (h->prof_cur && h->prof_head - h->prof_tail >= kProfRing) prof_harvest_one(h);
     // where kernel follows kernel on a stream, each may start while the one before it drains:
     // all of them on one stream, those inside a stage when a call has two stages; not in the
     // full pipeline, whose kernels are ordered by events, nor between the profiler's events
-    const bool pdl = !three && h->prof_on <= 0, pdl_first = pdl && !two;
+    const bool pdl = !three && !h->prof_cur, pdl_first = pdl && !two;
     cudaStream_t st4 = four ? stail : sb;
     cudaError_t e = cudaSuccess;
     int par = (int)(h->calls & 1);
@@ -970,7 +972,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     const bool alt = three && h->kk && h->front2 && !h->cnn && h->N == 65536;
     if (alt && par) sf = h->front2;
     const KkSync ksync = {alt ? h->ev_hist : nullptr, alt ? h->ev_hist : nullptr, alt ? h->ev_front : nullptr, pdl_first,
-                          pdl || (!alt && h->prof_on <= 0)};   // one front stream: its kernels follow each other
+                          pdl || (!alt && !h->prof_cur)};   // one front stream: its kernels follow each other
     if (host_in) {
         in = h->in_stage[isl];
         if (sc != sf) cudaStreamWaitEvent(sc, h->ev_infree[isl], 0);   // the front end kInSlots calls back is done
@@ -985,8 +987,6 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     if (two && !three) cudaStreamWaitEvent(sf, h->ev_yfree[(h->yw + 1) % kSlots], 0);
     if (host_out) bits_out = h->bits_stage;
 
-    h->prof_cur = h->prof_on > 0 && h->calls % h->prof_on == 0;
-    if (h->prof_cur && h->prof_head - h->prof_tail >= kProfRing) prof_harvest_one(h);
     // 12-bit unpack into [history | buffer]: the PAM chain's input; the KK kernels
     // read the packed bytes themselves, so there it only feeds the debug view
     if (!h->kk || c.debug) {
@@ -1231,8 +1231,10 @@ static rx_status run_batch(rx_handle *h, const uint8_t *const *ins, uint8_t *con
     // other without events.  Per buffer of 2^17 / 2^19 / 2^21 samples: 13.2 / 13.6 / 20.8 us
     // against 15.5 / 15.9 / 24.1.
     // The KK and frequency-domain chains (longer stages) and host buffers (the copies back sit
-    // in the second stage's way) are faster with one stream per stage.
-    const bool two_stages = !one && !host && !h->kk && !h->fd;
+    // in the second stage's way) are faster with one stream per stage, and so is a handle that
+    // is being profiled (every 4th call, 2^20 samples: 18.0 us against 18.8), whose events
+    // stand between the kernels.
+    const bool two_stages = !one && !host && !h->kk && !h->fd && h->prof_on <= 0;
     cudaStream_t sf = one ? caller : h->front;
     cudaStream_t sb = one ? caller : h->back;
     cudaStream_t sc = one ? caller : h->copy;
