@@ -425,8 +425,9 @@ rx_status rx_group_destroy(rx_group *g);
  *   field_out:   DEVICE pointer, 8-byte aligned, room for 2*(nsamp - ols_v/2)
  *                floats (interleaved real, imaginary).
  *
- * The scratch (twiddle and ln tables, a packed-history region, FFT rows) is one
- * fixed device array of about 4.1 MiB in librx.so;
+ * The scratch (twiddle and ln tables, a packed-history region, FFT rows, a copy of an
+ * input that the field is written over) is one
+ * fixed device array of about 4.9 MiB in librx.so;
  * every GPU that loads the library holds it until the process exits.  Sizes
  * beyond the limits return RX_EINVAL before anything is enqueued.  The call
  * allocates nothing (no cudaMalloc, cudaFree or allocating library routine); it

@@ -26,6 +26,7 @@ constexpr size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 //            is never read for values (samples before the stream are the first sample
 //            replicated), so it only has to be a valid region of ols_n * 3 / 2 bytes
 //   fft      the two-block complex FFT rows of 2^16-point blocks, at most 2^19 complex values
+//   in       a copy of the packed input, for callers whose field lies over it
 // The field goes straight to the caller's buffer: no field history is kept and no carrier
 // sums are taken.
 constexpr int kNaSizes = 2;
@@ -35,7 +36,9 @@ constexpr size_t kOffHist = align_up(kOffTw + kNaSizes * kTabBytes);
 constexpr size_t kHistBytes = (size_t)65536 * 3 / 2;
 constexpr size_t kOffFft = align_up(kOffHist + kHistBytes);
 constexpr size_t kFftBytes = 4u << 20;                   // two-block complex FFT rows
-constexpr size_t kScratchBytes = align_up(kOffFft + kFftBytes);
+constexpr size_t kOffIn = align_up(kOffFft + kFftBytes);
+constexpr size_t kInBytes = (size_t)kNaMaxSamples * 3 / 2;
+constexpr size_t kScratchBytes = align_up(kOffIn + kInBytes);
 
 // One scratch region per GPU that loads the library (held until the process exits).
 // Every call uses it, so calls that overlap on the GPU race with each other.
@@ -128,6 +131,14 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
     tb.twN2 = tb.twN + kk_tw_entries(ols_n);
     const uint8_t *hist = base + kOffHist;
     float2 *fftws = (float2 *)(base + kOffFft);
+    // blocks read their codes while others already write the field: a field over its own
+    // input works on a copy
+    const uintptr_t in0 = (uintptr_t)packed12_in, out0 = (uintptr_t)field_out;
+    if (out0 < in0 + (uintptr_t)(nsamp * 3 / 2) && in0 < out0 + (uintptr_t)e_k * sizeof(float2)) {
+        if (cudaMemcpyAsync(base + kOffIn, packed12_in, (size_t)(nsamp * 3 / 2), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+            return RX_ECUDA;
+        packed12_in = base + kOffIn;
+    }
     KkInput kin;
     kin.hist = hist;                        // never read for values: the first call fills the pre-stream
     kin.in = packed12_in;

@@ -43,3 +43,20 @@ def test_field_of_4096_point_blocks(nsamp, v, order):
     got = out.cpu().numpy()
     assert np.all(np.isnan(got[-2:]))      # nothing is written past the field
     assert rel_rms(got[:-2].view(np.complex64), field64(codes, v)) <= FIELD_TOL
+
+
+@pytest.mark.parametrize("n, v, nsamp", [(4096, 512, 41_984), (65536, 4096, 131_072)])
+@pytest.mark.parametrize("at", [0, 4096])
+def test_field_over_its_own_input(n, v, nsamp, at):
+    """A field written over the packed samples it comes from is the field of a separate buffer,
+    bit for bit."""
+    rng = np.random.default_rng(nsamp + at)
+    packed = torch.from_numpy(synth.pack12(rng.integers(0, 4096, nsamp), 0)).cuda()
+    count, stream = nsamp - v // 2, torch.cuda.current_stream().cuda_stream
+    want = torch.empty(2 * count, dtype=torch.float32, device="cuda")
+    rx.rx_kk_field_noalloc(packed.data_ptr(), nsamp, 0, n, v, want.data_ptr(), stream)
+    both = torch.empty(2 * count, dtype=torch.float32, device="cuda")
+    src = both.view(torch.uint8)[at:at + len(packed)]
+    src.copy_(packed)
+    rx.rx_kk_field_noalloc(src.data_ptr(), nsamp, 0, n, v, both.data_ptr(), stream)
+    assert torch.equal(both, want)
