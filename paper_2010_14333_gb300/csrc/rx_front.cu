@@ -20,6 +20,7 @@
 
 #include <cooperative_groups.h>
 
+#include "rx_async.cuh"
 #include "rx_common.cuh"
 #include "rx_internal.cuh"
 
@@ -224,11 +225,16 @@ __device__ __forceinline__ void twiddle16(float2 (&x)[16], const TwSmem &tw, int
         }
     }
 }
+// Stages the factored table asynchronously: the caller waits (cp_async_wait_all) before the
+// barrier in front of its first use, so the copies are in flight beside the input's loads
+// (also asynchronous, stage_rows) instead of a round trip before them.  2^22 samples: K1a
+// 10.7 us against 13.0, K1c 16.4 against 17.6 (ncu); a batch 60.8 us per buffer against 63.1.
 __device__ __forceinline__ TwSmem stage_tw(const float2 *__restrict__ gtab, int M, float2 *sm)
 {
     int m = 31 - __clz(M);
     int s = (m + 1) / 2, lo = 1 << s, n = lo + (M >> s);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = __ldg(gtab + i);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) cp_async8(sm + i, gtab + i, true);
+    cp_async_commit();
     TwSmem t;
     t.lo = sm;
     t.hi = sm + lo;
@@ -275,8 +281,7 @@ __device__ __forceinline__ bool before_stream(const KkGeom &g, int pair, bool hb
     return ols_ws(g, 2 * pair) < 0 || (hb && ols_ws(g, 2 * pair + 1) < 0);
 }
 
-// (CTAs of kCtaK1 threads; the loop is unrolled so that every load issues before the
-// first one is used).  Samples before the stream are staged as c_first.  Byte offsets fit
+// (CTAs of kCtaK1 threads; asynchronous copies, which the caller waits for).  Samples before the stream are staged as c_first.  Byte offsets fit
 // 32 bits: a buffer is at most 2^30 samples.
 template <int N2T>
 __device__ __forceinline__ void stage_rows(const KkGeom &g, const KkPacked &pk, int pair, int c0,
@@ -297,11 +302,11 @@ __device__ __forceinline__ void stage_rows(const KkGeom &g, const KkPacked &pk, 
         const int row = i / 24, ch = i - 24 * row;
         if (row >= 16 && !hb) continue;
         const unsigned vb = (row < 16 ? v0 : v1) + (unsigned)(row & 15) * (N2T * 3 / 2) + 16 * ch;
-        uint4 w;
-        if (vb < vs) w = code_bytes(c_first, pk.order, vb);
-        else w = __ldg(reinterpret_cast<const uint4 *>((vb < hbytes ? pk.hist : in0) + vb));
-        *reinterpret_cast<uint4 *>(&raw[row][4 * ch]) = w;
+        uint32_t *dst = &raw[row][4 * ch];
+        if (vb < vs) *reinterpret_cast<uint4 *>(dst) = code_bytes(c_first, pk.order, vb);
+        else cp_async16(dst, (vb < hbytes ? pk.hist : in0) + vb);
     }
+    cp_async_commit();
 }
 
 // 12-bit code of column t of a staged row.  The row is a stream of 12-bit fields,
@@ -342,6 +347,14 @@ __device__ __forceinline__ uint32_t first_code(const KkPacked &pk, const DevStat
     return a;
 }
 
+// the ln table into shared memory, asynchronously like stage_tw: a gather over 32 random codes
+// costs a few bank conflicts there instead of one L1 wavefront per distinct cache line
+__device__ __forceinline__ void stage_ln(const float *__restrict__ lnt, float *s_ln)
+{
+    for (int i = threadIdx.x; i < kLutCodes / 4; i += blockDim.x) cp_async16(s_ln + 4 * i, lnt + 4 * i);
+    cp_async_commit();
+}
+
 // u = ln(I)/2 of both blocks of a pair at this column's 16 window positions
 template <int ORD>
 __device__ __forceinline__ void load_columns(bool hb, const uint32_t (*raw)[kRawWords], const ColPos &cp, const float *s_ln,
@@ -380,15 +393,12 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2
     __shared__ __align__(16) float s_ln[kLutCodes];
     int pair = blockIdx.y;
     const TwSmem tw = stage_tw(tb.twN, g.N, s_tw);
-    // the ln table in shared memory: a gather over 32 random codes costs a few bank
-    // conflicts there instead of one L1 wavefront per distinct cache line
-    if (pair < g.npairs)
-        for (int i = threadIdx.x; i < kLutCodes / 4; i += blockDim.x)
-            reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
+    stage_ln(tb.lnt, s_ln);
     pdl_wait();
     if (pk.lat && blockIdx.x == 0 && pair == 0 && threadIdx.x == 0) lat_start(pk.lat, pk.lat_slot);
     if (pair == g.npairs) {
         copy_hist(pk, blockIdx.x, gridDim.x);
+        cp_async_wait_all();
         return;
     }
     const int c0 = blockIdx.x * blockDim.x;
@@ -396,6 +406,7 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2
     const uint32_t c_first = before_stream(g, pair, hb) || pk.first_call ? first_code(pk, dst) : 0u;
     stage_rows<N2T>(g, pk, pair, c0, raw, hb, c_first);
     if (pk.first_call && dst && blockIdx.x == 0 && pair == 0 && threadIdx.x == 0) dst->first_code = (int)c_first;
+    cp_async_wait_all();
     __syncthreads();
     const int t = threadIdx.x, n1 = c0 + t;
     const ColPos cp = col_pos<ORD>(t);
@@ -438,13 +449,14 @@ __global__ void __launch_bounds__(256, 3) k_kk_rows(KkGeom g, float2 *__restrict
     __shared__ float2 s_tw[128];
     const TwSmem tw2 = stage_tw(twN2g, N2, s_tw);
     pdl_wait();
-    __syncthreads();
     const int t = threadIdx.x, row = blockIdx.x, k2 = row & 15;
     float2 *d = fftws + (size_t)row * N2;
     float2 x[16];
     // forward pass 0 (sub-transform size N2) straight from global memory
 #pragma unroll
     for (int r = 0; r < 16; r++) x[r] = d[t + r * TPR];
+    cp_async_wait_all();
+    __syncthreads();   // staged twiddles
     dft16<false>(x);
     twiddle16<false>(x, tw2, t);
     // a pass's 16 elements base + r stride sit at pad16(base) + r (stride + stride / 16)
@@ -634,6 +646,7 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const 
     const float2 *in = fftws + (size_t)pair * g.N + n1;
 #pragma unroll
     for (int k2 = 0; k2 < 16; k2++) x[k2] = in[k2 * N2T];
+    cp_async_wait_all();
     __syncthreads();   // staged twiddles and rows
     twiddle16<true>(x, tw, n1);
     dft16<true>(x);
@@ -674,12 +687,12 @@ __global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, c
     const int pair = blockIdx.x, t = threadIdx.x;
     const TwSmem tw = stage_tw(tb.twN, 16 * kBkN2, s_tw);
     const TwSmem tw2 = stage_tw(tb.twN2, kBkN2, s_tw + 128);
-    for (int i = t; i < kLutCodes / 4; i += kCtaK1)
-        reinterpret_cast<float4 *>(s_ln)[i] = __ldg(reinterpret_cast<const float4 *>(tb.lnt) + i);
+    stage_ln(tb.lnt, s_ln);
     pdl_wait();
     if (pk.lat && pair == 0 && t == 0) lat_start(pk.lat, pk.lat_slot);
     if (pair >= g.npairs) {
         copy_hist(pk, pair - g.npairs, gridDim.x - g.npairs);
+        cp_async_wait_all();
         return;
     }
     const bool hb = 2 * pair + 1 < g.J;
@@ -687,6 +700,7 @@ __global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, c
     stage_rows<kBkN2>(g, pk, pair, 0, raw, hb, c_first);
     if (pk.first_call && dst && pair == 0 && t == 0) dst->first_code = (int)c_first;
     if (pair == 0) carry_field(g, E, E_prev);
+    cp_async_wait_all();
     __syncthreads();
     const ColPos cp = col_pos<ORD>(t);
     float2 x[16];
@@ -799,6 +813,7 @@ __global__ void __cluster_dims__(kClC, 1, 1) __launch_bounds__(kClThreads, 3)
     // the virtual buffer), spread over the grid
     if (pk.hist_next) copy_hist(pk, blockIdx.x, gridDim.x);
     if (blockIdx.x == 0) carry_field(g, E, E_prev);
+    cp_async_wait_all();
     __syncthreads();   // staged twiddles
 
     // ---- A: forward column DFTs, scattered to the row owners
