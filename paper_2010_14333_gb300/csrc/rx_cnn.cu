@@ -176,7 +176,7 @@ __device__ __forceinline__ void conv_tile(float (&acc)[2 * NP][4], uint32_t w, i
 // sum exact), so its products with the BF16 activations are those of the FP32 weights,
 // accumulated in FP32 on the tensor cores.
 // Bound: FP32 issue of the erf GELU (472 warp-wide evaluations a segment).  4096 segments:
-// 128 us; 457 us with one 128-thread CTA per segment that staged all weights for it, layer
+// 126 us; 457 us with one 128-thread CTA per segment that staged all weights for it, layer
 // 3 at every position, 4-byte operand loads and the MLP on the CUDA cores.
 constexpr int kFwThreads = 288, kFwPerSm = 3;
 constexpr int kH1Rows = L1 + 8;              // rows L1 .. are zero (read by the last tile's taps)
@@ -351,7 +351,8 @@ __global__ void __launch_bounds__(kFwThreads, kFwPerSm)
 // pre-activation.  The transposed operands of the backward products (du and the layer
 // inputs with the positions along K, the weights with the output channels along K) are
 // read with transposing ldmatrix from the forward's own tiles, so nothing is rearranged.
-// A step of 64 segments (this kernel, the reduction and Adam): 34 us; 146 us with a forward
+// A step of 64 segments (this kernel, the reduction and Adam, each launched as the
+// dependent of the one before): 26 us; 146 us with a forward
 // and a backward kernel that passed activations through global memory and rearranged their
 // operands in shared memory.  Bound: the chain of eleven phases, each a few hundred cycles
 // of one CTA per SM.

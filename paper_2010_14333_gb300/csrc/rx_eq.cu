@@ -124,8 +124,9 @@ __device__ __forceinline__ PhaseTab phase_tab(const EqParams &p, int lane)
 // a window ahead by the caller; score: count errors against them); update: the window's
 // tap step is wanted (the last window of a block but the call's last one feeds nothing).
 // Every output is bit for bit that of one symbol per lane and
-// half a window (products and sums in the same order); 25.6 instead of 28.7 M warp
-// instructions and 33.4 instead of 35.5 us for a 2^22-sample 16QAM buffer (issue bound).
+// half a window (products and sums in the same order); with no tap step where nothing
+// uses it, 23.2 instead of 28.7 M warp instructions and 29.8 instead of 35.5 us for a
+// 2^22-sample 16QAM buffer (issue bound, 73 % of the slots).
 template <int NT, int MQ, bool FRZ = false>
 __device__ __forceinline__ WinOut qam_window(const EqParams &p, const float2 *ys, int c0, float *zs, float2 *es,
                                              float2 *ws, int mode, float mu, int lane, uint8_t *dec_out,

@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const 
 // the three-kernel form of the 2^16-point blocks, pass by pass.  CTAs from npairs on copy
 // the next call's history.
 // Bound by latency: a chain of six passes at three CTAs per SM.  41,984 samples with V = 512
-// (six CTAs): 10.2 us per call of rx_kk_field_noalloc; 28.7 us as three kernels (column DFT, rows,
+// (six CTAs): 7.0 us per call of rx_kk_field_noalloc; 28.7 us as three kernels (column DFT, rows,
 // column DFT and field, the spectrum through global memory twice), a clear and a copy.
 constexpr int kBkN2 = 256, kBkRow = kBkN2 + kBkN2 / 16;   // row length and padded row
 struct BkSmem {
