@@ -127,8 +127,10 @@ __global__ void __launch_bounds__(kT8Threads, kT8PerSm)
     const int nhalo = ns - 32;                                       // of them in the next block row (may be <= 0)
     const int ntiles = (nrows + kTileRows - 1) / kTileRows, rshift = 31 - __clz(rows_per_scale);
     float2 v[kT8Iter];
-    auto load_tile = [&](int t) {   // lane = sample of block row warp + 8 i; zero outside what the rows read
-        const int r0 = t * kTileRows, n = 32 * (min(kTileRows, nrows - r0) - 1) + ns;
+    // lane = sample of block row warp + 8 i; zero outside what the rows read (with one tap, ns
+    // is 31: no row reads sample 31, which then has no say in the scales either)
+    auto load_tile = [&](int t) {
+        const int r0 = t * kTileRows, n = lane < ns ? 32 * (min(kTileRows, nrows - r0) - 1) + ns : 0;
         const float2 *Yb = Y + (2 * (k_lo + (long long)r0 * kRowSyms) - th - ybase);
 #pragma unroll
         for (int i = 0; i < kT8Iter; i++) {
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(kT8Threads, kT8PerSm)
             unsigned char *dst = sA + (lane >> 3) * kT8Plane + (lane & 7) * 2;
             const int e0 = q < kTileRows ? s_exp[q >> rshift] : 0;
             const uint16_t h = fp8_pair(v[i], ldexpf(1.f, e0));
-            if (q < kTileRows) *reinterpret_cast<uint16_t *>(dst + q * 16) = lane < ns ? h : 0;
+            if (q < kTileRows) *reinterpret_cast<uint16_t *>(dst + q * 16) = h;
             if (q > 0) {
                 uint16_t h1 = h;
                 if ((q & (rows_per_scale - 1)) == 0) h1 = fp8_pair(v[i], ldexpf(1.f, s_exp[(q - 1) >> rshift]));
