@@ -866,7 +866,7 @@ struct RxSmem {
                                                           // hidden planes [8][128][16 B]
     static constexpr int HXB = 2 * 4 * kRE * 16;
     static constexpr int XS = HX + HXB;                   // float2 [kP0]: the next tile's input (async copy)
-    static constexpr int BAR = XS + kP0 * 8;              // mbarriers, one per row tile of layers 1 and 2
+    static constexpr int BAR = XS + kP0 * 8;              // mbarriers, one per row tile of layers 1 and 2, one of the exit
     static constexpr int REC = BAR + 32;                  // uint32 [2 tiles][kWinT][4]: window records being summed
     static constexpr int GROUP = (REC + 2 * kWinT * 16 + 127) & ~127;
     static constexpr int SLOT = GRP + kRxGroups * GROUP;  // tensor-memory base address
@@ -964,7 +964,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
     uint64_t *bar = reinterpret_cast<uint64_t *>(gb + RxSmem::BAR);
     constexpr int PL1 = kR1 * 16, PLE = kRE * 16, EO = 4 * PLE;
 
-    if (gtid < 3) mbar_init(bar + gtid, 1);
+    if (gtid < 4) mbar_init(bar + gtid, 1);
     if (gtid < 2 * kWinT * 4) rec[gtid] = 0;
     __syncwarp();
     if (warp == 0) tmem_alloc(tslot, kRxTmem);
@@ -1042,12 +1042,12 @@ __global__ void __launch_bounds__(kRxThreads, 1)
     unsigned phase = 0;   // bit b: phase of mbarrier b
     bool ok = true;
 
-    // wait for the MMAs committed to mbarrier b; a wait that ran out is flagged and ends the
-    // group's loop at its next tile (no MMA of a later wait is waited for then)
+    // wait for the MMAs committed to mbarrier b.  A wait that ran out is flagged and ends the
+    // group's loop at its next tile; until then a thread that gave up waits for nothing more,
+    // and the issuing one issues nothing more (the others' waits for it run out as well)
     auto wait_mma = [&](int b) {
         if (ok && !mbar_wait(bar + b, (phase >> b) & 1u)) {
             atomicExch(err, (int)RX_ETIMEOUT);
-            mbar_wait(bar + b, (phase >> b) & 1u);
             ok = false;
         }
         phase ^= 1u << b;
@@ -1109,7 +1109,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         fence_async_smem();
         group_sync(gbar);
         if (t + tstep < ntiles) prefetch(t + tstep);   // lands while this tile computes
-        if (gtid == 0) {
+        if (gtid == 0 && ok) {
             tc_fence_after();
 #pragma unroll
             for (int m = 0; m < kMT1; m++) {
@@ -1144,7 +1144,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         group_sync(gbar);
         // layer 2 (reads h1; the input plane is free): the epilogue of a row tile runs while
         // the MMAs of the next one do
-        if (gtid == 0) {
+        if (gtid == 0 && ok) {
             tc_fence_after();
 #pragma unroll
             for (int m = 0; m < kMT2; m++) {
@@ -1166,7 +1166,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         tc_fence_before();
         group_sync(gbar);
         // layer 3 at the symbol positions: tap d reads set d & 1 from row j + d / 2
-        if (gtid == 0) {
+        if (gtid == 0 && ok) {
             tc_fence_after();
 #pragma unroll
             for (int ks = 0; ks < 18; ks++) {
@@ -1184,7 +1184,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         tc_fence_before();
         group_sync(gbar);
         // MLP 32 -> 64 on the symbols (M = 128, N = 64, K = 32)
-        if (gtid == 0) {
+        if (gtid == 0 && ok) {
             tc_fence_after();
 #pragma unroll
             for (int ks = 0; ks < 2; ks++)
@@ -1213,7 +1213,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         tc_fence_before();
         group_sync(gbar);
         // 64 -> 2 (M = 128, N = 16 with rows 2..15 of B zero, K = 64)
-        if (gtid == 0) {
+        if (gtid == 0 && ok) {
             tc_fence_after();
 #pragma unroll
             for (int ks = 0; ks < 4; ks++)
@@ -1224,7 +1224,7 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         wait_mma(0);
         // decisions and window records: the lanes that hold the outputs decide their symbol,
         // two warps per window; the other warps go on to the next tile's input
-        if (ch == 0) {
+        if (ch == 0 && __all_sync(0xffffffffu, ok)) {
             uint32_t r[8];
             tmem_ld8(tq + kColOut, r);
             const float o0 = __uint_as_float(r[0]) + c2[0], o1 = __uint_as_float(r[1]) + c2[1];
@@ -1262,8 +1262,12 @@ __global__ void __launch_bounds__(kRxThreads, 1)
         tc_fence_before();
     }
     cp_async_wait_all();   // a prefetch may still be in flight after an early exit
-    group_sync(gbar);
-    if (tlast >= 0) put_records(tlast, tp);
+    if (group_and(gbar, ok)) {
+        if (tlast >= 0) put_records(tlast, tp);
+    } else if (gtid == 0) {   // MMAs may still be in flight: wait (bounded) for all this thread issued
+        umma_commit(bar + 3);
+        mbar_wait(bar + 3, 0);
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(*tslot, kRxTmem);
