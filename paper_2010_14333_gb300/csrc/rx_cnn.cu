@@ -103,7 +103,7 @@ struct L1Weights {
 // shared copy of the weights and biases as channel pairs: [k][pair], row 18 the biases
 constexpr int kW1Floats = 19 * CC;
 template <int NTH>
-__device__ __forceinline__ void stage_l1(float *w1, const float *__restrict__ prm, int tid)
+__device__ __forceinline__ void stage_l1(float *w1, const float *prm, int tid)
 {
     for (int i = tid; i < kW1Floats; i += NTH) {
         const int k = i / CC, o = i % CC;
@@ -199,8 +199,8 @@ static_assert(FwdSmem::H1 % 16 == 0 && FwdSmem::X % 16 == 0 && FwdSmem::XD % 16 
 static_assert(L0 * 16 <= 2 * kH2Half * CC * 2, "the doubled input fits the layer-2 rows");
 
 __global__ void __launch_bounds__(kFwThreads, kFwPerSm)
-    k_cnn_fwd(const float *__restrict__ prm, const __nv_bfloat16 *__restrict__ prm_bf, const float2 *__restrict__ y,
-              const long long *__restrict__ seg_start, int nseg, float *__restrict__ out)
+    k_cnn_fwd(const float *prm, const __nv_bfloat16 *prm_bf, const float2 *y,
+              const long long *seg_start, int nseg, float *out)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     float2 *x2 = reinterpret_cast<float2 *>(sm + FwdSmem::X);
@@ -391,9 +391,9 @@ static_assert(TrainSmem::M1 % 16 == 0 && TrainSmem::H1 % 16 == 0 && TrainSmem::D
               "16-byte rows");
 
 __global__ void __launch_bounds__(kTrThreads, 1)
-    k_cnn_train(const float *__restrict__ prm, const __nv_bfloat16 *__restrict__ prm_bf, const float2 *__restrict__ y,
-                const long long *__restrict__ seg_start, const float *__restrict__ tgt, float norm,
-                float *__restrict__ gpart, float *__restrict__ lpart)
+    k_cnn_train(const float *prm, const __nv_bfloat16 *prm_bf, const float2 *y,
+                const long long *seg_start, const float *tgt, float norm,
+                float *gpart, float *lpart)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     float4 *xd = reinterpret_cast<float4 *>(sm + TrainSmem::XD);
@@ -744,8 +744,8 @@ __global__ void __launch_bounds__(kTrThreads, 1)
 // the last CTA sums the segments' loss parts
 constexpr int kRedThreads = 128;
 __global__ void __launch_bounds__(kRedThreads)
-    k_cnn_reduce(const float *__restrict__ gpart, const float *__restrict__ lpart, int nseg, float norm,
-                 float *__restrict__ grad, float *grad_out, float *__restrict__ loss, float *loss_out)
+    k_cnn_reduce(const float *gpart, const float *lpart, int nseg, float norm,
+                 float *grad, float *grad_out, float *loss, float *loss_out)
 {
     pdl_wait();
     if (blockIdx.x == gridDim.x - 1) {
@@ -772,8 +772,8 @@ __global__ void __launch_bounds__(kRedThreads)
 }
 
 // Adam on the FP32 master weights; refreshes the BF16 copy
-__global__ void k_cnn_adam(float *__restrict__ prm, __nv_bfloat16 *__restrict__ prm_bf,
-                           float *__restrict__ m, float *__restrict__ v, const float *__restrict__ grad, float lr,
+__global__ void k_cnn_adam(float *prm, __nv_bfloat16 *prm_bf,
+                           float *m, float *v, const float *grad, float lr,
                            float b1t, float b2t)
 {
     pdl_wait();
@@ -943,10 +943,10 @@ __device__ __forceinline__ uint32_t gelu2(uint32_t a, uint32_t b, uint32_t bias)
 
 template <bool BF>
 __global__ void __launch_bounds__(kRxThreads, 1)
-    k_cnn_rx_tc(const float *__restrict__ prm, const float2 *__restrict__ y,
-                long long seg_base, long long y_end, int nwin, uint8_t *__restrict__ dec, uint8_t *__restrict__ winb,
-                uint4 *__restrict__ winrec, const uint32_t *__restrict__ prbs_bits, long long k_first, float scale,
-                int mq, float2 *__restrict__ soft, int *err)
+    k_cnn_rx_tc(const float *prm, const float2 *y,
+                long long seg_base, long long y_end, int nwin, uint8_t *dec, uint8_t *winb,
+                uint4 *winrec, const uint32_t *__restrict__ prbs_bits, long long k_first, float scale,
+                int mq, float2 *soft, int *err)
 {
     extern __shared__ __align__(16) unsigned char sm[];   // no-swizzle operands: 16-byte rows
     unsigned char *sW2 = sm + RxSmem::W2, *sW3 = sm + RxSmem::W3, *sM1 = sm + RxSmem::M1, *sM2 = sm + RxSmem::M2;

@@ -386,9 +386,9 @@ __device__ __forceinline__ WinOut pam_window(const EqParams &p, const float *ys,
 // each window's input with plain loads.
 template <bool QAM, int NT, int MQ>
 __global__ void __launch_bounds__(32 * kEqWarpsMax)
-    k_eq(EqParams p, EqGeom g, int train, const void *__restrict__ Yv, float2 *taps_in, float2 *taps_out,
-         uint8_t *__restrict__ dec, uint8_t *__restrict__ winb, uint4 *__restrict__ winrec,
-         float4 *__restrict__ dbg_win, float2 *__restrict__ dbg_z, const uint8_t *__restrict__ prbs_ext,
+    k_eq(EqParams p, EqGeom g, int train, const void *Yv, float2 *taps_in, float2 *taps_out,
+         uint8_t *dec, uint8_t *winb, uint4 *winrec,
+         float4 *dbg_win, float2 *dbg_z, const uint8_t *__restrict__ prbs_ext,
          const uint32_t *__restrict__ prbs_bits, DevState *dst)
 {
     typedef typename std::conditional<QAM, float2, float>::type T;
@@ -507,10 +507,10 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax)
 // order, so the next taps do not depend on the order the warps ran in.
 template <int NT, int MQ>
 __global__ void __launch_bounds__(32 * kEqWarpsMax)
-    k_eq_frozen(EqParams p, EqGeom g, const float2 *__restrict__ Y, const float2 *__restrict__ zin,
-                const float2 *__restrict__ taps_in, float2 *__restrict__ taps_out, uint8_t *__restrict__ dec,
-                uint8_t *__restrict__ winb, uint4 *__restrict__ winrec, float4 *__restrict__ dbg_win,
-                float2 *__restrict__ dbg_z, const uint32_t *__restrict__ prbs_bits, DevState *dst)
+    k_eq_frozen(EqParams p, EqGeom g, const float2 *Y, const float2 *zin,
+                const float2 *taps_in, float2 *taps_out, uint8_t *dec,
+                uint8_t *winb, uint4 *winrec, float4 *dbg_win,
+                float2 *dbg_z, const uint32_t *__restrict__ prbs_bits, DevState *dst)
 {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -919,7 +919,7 @@ __device__ __forceinline__ int quad_t(int LI, int LQ, int &lb)
 // 16; blast: phase index of the window before the call (have: there is one).  Indices are
 // below 32, so with bit 7 of every byte set, subtracting the other index and B/2 + 1 leaves
 // bit 7 where the difference exceeds B/2: four windows per subtraction.
-__device__ __forceinline__ int unwrap_prefix(const uint8_t *__restrict__ winb, int w0, int tid, int B, int have, int blast)
+__device__ __forceinline__ int unwrap_prefix(const uint8_t *winb, int w0, int tid, int B, int have, int blast)
 {
     const uint32_t H = (uint32_t)(B / 2 + 1) * 0x01010101u, top = 0x80808080u;
     const int nch = w0 / 16;
@@ -954,8 +954,8 @@ __device__ __forceinline__ int unwrap_prefix(const uint8_t *__restrict__ winb, i
 // stream-start pi/2 ambiguity from the first amb_syms payload symbols (windows 0.. of this,
 // the first payload call): the rotation r whose decoded symbols (rotation m_w + r) match the
 // transmitted ones best, ties to the lowest r; one warp
-__device__ __forceinline__ int find_rotation(const EqParams &p, const uint8_t *__restrict__ winb,
-                                             const uint4 *__restrict__ winrec, int lane)
+__device__ __forceinline__ int find_rotation(const EqParams &p, const uint8_t *winb,
+                                             const uint4 *winrec, int lane)
 {
     const int nw = p.amb_syms / kWin;
     int acc = 0;
@@ -988,9 +988,9 @@ __device__ __forceinline__ int find_rotation(const EqParams &p, const uint8_t *_
 
 template <bool QAM, int BPS, int MQ>
 __global__ void __launch_bounds__(kDemapThreads)
-    k_demap(EqParams p, EqGeom g, int resolve_amb, int uw_in, const uint8_t *__restrict__ dec,
-            const uint8_t *__restrict__ winb, const uint4 *__restrict__ winrec, float4 *__restrict__ dbg_win,
-            uint8_t *__restrict__ bits_out, DevState *dst)
+    k_demap(EqParams p, EqGeom g, int resolve_amb, int uw_in, const uint8_t *dec,
+            const uint8_t *winb, const uint4 *winrec, float4 *dbg_win,
+            uint8_t *bits_out, DevState *dst)
 {
     constexpr int NW = kDemapThreads / 32, WPC = kDemapWpc;
     constexpr int NB = QAM ? BPS / 2 : BPS;
@@ -1147,9 +1147,9 @@ __global__ void __launch_bounds__(kDemapThreads)
 
 template <int BPS, int MQ>
 __global__ void __launch_bounds__(kDemapThreads)
-    k_demap_diff(EqParams p, EqGeom g, int resolve_amb, int uw_in, const uint8_t *__restrict__ dec,
-            const uint8_t *__restrict__ winb, const uint4 *__restrict__ winrec, float4 *__restrict__ dbg_win,
-            uint8_t *__restrict__ bits_out, const uint32_t *__restrict__ prbs_bits, DevState *dst)
+    k_demap_diff(EqParams p, EqGeom g, int resolve_amb, int uw_in, const uint8_t *dec,
+            const uint8_t *winb, const uint4 *winrec, float4 *dbg_win,
+            uint8_t *bits_out, const uint32_t *__restrict__ prbs_bits, DevState *dst)
 {
     constexpr int NW = kDemapThreads / 32;
     constexpr int WPW = kDemapWin / NW;                            // windows per warp

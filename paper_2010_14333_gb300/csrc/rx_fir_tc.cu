@@ -112,8 +112,8 @@ __device__ __forceinline__ uint16_t fp8_pair(float2 v, float s)
 }
 
 __global__ void __launch_bounds__(kT8Threads, kT8PerSm)
-    k_fir_tc8(const float2 *__restrict__ Y, long long ybase, long long k_lo, int nrows,
-              const float2 *__restrict__ taps, int ntaps, int rows_per_scale, float2 *__restrict__ z, int *err)
+    k_fir_tc8(const float2 *Y, long long ybase, long long k_lo, int nrows,
+              const float2 *taps, int ntaps, int rows_per_scale, float2 *z, int *err)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *sA = sm, *sB = sm + kT8OffB;
@@ -135,14 +135,14 @@ __global__ void __launch_bounds__(kT8Threads, kT8PerSm)
 #pragma unroll
         for (int i = 0; i < kT8Iter; i++) {
             const int j = tid + i * kT8Threads;
-            v[i] = j < n ? __ldg(Yb + j) : make_float2(0.f, 0.f);
+            v[i] = j < n ? Yb[j] : make_float2(0.f, 0.f);
         }
     };
     int t = blockIdx.x;
     if (tid == 0) mbar_init(bar, 1);
     if (warp == 0) tmem_alloc(tslot, kTmemCols);
     pdl_wait();
-    if (tid < 32) s_w[tid] = tid < ntaps ? __ldg(taps + tid) : make_float2(0.f, 0.f);
+    if (tid < 32) s_w[tid] = tid < ntaps ? taps[tid] : make_float2(0.f, 0.f);
     if (t < ntiles) load_tile(t);
     __syncthreads();   // the taps in shared memory
     // B: Toeplitz matrix of the taps, rows n = 2 j + c (c: re / im output of symbol j), K
@@ -292,8 +292,8 @@ __device__ __forceinline__ uint32_t pack2(float a, float b)
 
 template <int PREC>
 __global__ void __launch_bounds__(kT2Threads, kT2PerSm)
-    k_fir_tc2(const float2 *__restrict__ Y, long long ybase, long long k_lo, int nrows,
-              const float2 *__restrict__ taps, int ntaps, float2 *__restrict__ z, int *err)
+    k_fir_tc2(const float2 *Y, long long ybase, long long k_lo, int nrows,
+              const float2 *taps, int ntaps, float2 *z, int *err)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *sA = sm, *sB = sm + kT2OffB;
@@ -315,14 +315,14 @@ __global__ void __launch_bounds__(kT2Threads, kT2PerSm)
 #pragma unroll
         for (int i = 0; i < kT2Iter; i++) {
             const int j = tid + i * kT2Threads;
-            v[i] = (j >= jlo && j <= jhi && j < kT2Samples) ? __ldg(Yb + j) : make_float2(0.f, 0.f);
+            v[i] = (j >= jlo && j <= jhi && j < kT2Samples) ? Yb[j] : make_float2(0.f, 0.f);
         }
     };
     int t = blockIdx.x;
     if (tid == 0) mbar_init(bar, 1);
     if (warp == 0) tmem_alloc(tslot, kTmemCols);
     pdl_wait();
-    if (tid < 32) s_w[tid] = tid < ntaps ? __ldg(taps + tid) : make_float2(0.f, 0.f);
+    if (tid < 32) s_w[tid] = tid < ntaps ? taps[tid] : make_float2(0.f, 0.f);
     if (t < ntiles) load_tile(t);
     __syncthreads();   // the taps in shared memory
     // B: rows n = 2 j + c (c: re / im output of symbol j), K index k = 64 h + 2 s + d

@@ -47,7 +47,7 @@ __device__ __forceinline__ void decode_pair(uint32_t b0, uint32_t b1, uint32_t b
 // the start of every CTA of the filter.
 constexpr int kUnpackThreads = 256, kUnpackPer = 2;   // threads per CTA, groups of 8 samples per thread
 __global__ void __launch_bounds__(kUnpackThreads)
-    k_unpack(const uint8_t *__restrict__ in, uint16_t *__restrict__ codes, const uint16_t *__restrict__ codes_prev,
+    k_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *codes_prev,
              long long nb, int nhist, long long prev_off, int first_call, int order, DevState *sums, int slot,
              LatRecord *lat, int lat_slot)
 {
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kUnpackThreads)
         const long long g = g0 + k * kUnpackThreads;
         if (g < ngroups)
 #pragma unroll
-            for (int i = 0; i < 3; i++) w[k][i] = __ldg(in32 + 3 * g + i);
+            for (int i = 0; i < 3; i++) w[k][i] = in32[3 * g + i];
     }
     unsigned lsum = 0;                // 8 samples of 12 bits per group
     unsigned long long wsq = 0;       // lane 0: the warp's squares (256 samples: below 2^32 per group)
@@ -376,7 +376,7 @@ __device__ __forceinline__ void copy_hist(const KkPacked &pk, int cta, int ncta)
     for (long long c = (long long)cta * blockDim.x + threadIdx.x; c < nch; c += (long long)ncta * blockDim.x) {
         long long vb = pk.in_bytes + 16 * c;
         const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
-        reinterpret_cast<uint4 *>(pk.hist_next)[c] = __ldg(reinterpret_cast<const uint4 *>(src));
+        reinterpret_cast<uint4 *>(pk.hist_next)[c] = *reinterpret_cast<const uint4 *>(src);
     }
 }
 
@@ -385,7 +385,7 @@ __device__ __forceinline__ void copy_hist(const KkPacked &pk, int cta, int ncta)
 // ORD: the pack order of the 12-bit input; N2T: the row length N / 16 (256 or 4096), so
 // that the stride-N2 accesses take compile-time offsets.
 template <int ORD, int N2T>
-__global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2 *__restrict__ fftws,
+__global__ void __launch_bounds__(kCtaK1) k_kk_fwd(KkGeom g, KkPacked pk, float2 *fftws,
                                                   const KkTables tb, DevState *dst)
 {
     __shared__ float2 s_tw[512];
@@ -441,7 +441,7 @@ __device__ __forceinline__ float2 hilbert_mul(float2 v, int k, int N)
 // k = k2 + 16 k1, inverse FFT (radix-16 decimation in time back to natural order).  In
 // place, one row per CTA.
 constexpr int kRowN2 = 4096, kRowPad = kRowN2 + kRowN2 / 16;   // row and padded row
-__global__ void __launch_bounds__(256, 3) k_kk_rows(KkGeom g, float2 *__restrict__ fftws,
+__global__ void __launch_bounds__(256, 3) k_kk_rows(KkGeom g, float2 *fftws,
                                                    const float2 *__restrict__ twN2g)
 {
     constexpr int P = 3, N2 = kRowN2, TPR = N2 / 16;
@@ -572,7 +572,7 @@ __device__ __forceinline__ void carrier_sums(const KkGeom &g, DevState *dst, flo
 
 // field history for the matched filter: E[n], n in [e_prev - kEHist, e_prev) (E_prev null:
 // the caller keeps none)
-__device__ __forceinline__ void carry_field(const KkGeom &g, float2 *__restrict__ E, const float2 *__restrict__ E_prev)
+__device__ __forceinline__ void carry_field(const KkGeom &g, float2 *E, const float2 *E_prev)
 {
     if (!E_prev) return;
     for (int i = threadIdx.x; i < kEHist; i += blockDim.x) {
@@ -587,7 +587,7 @@ __device__ __forceinline__ void carry_field(const KkGeom &g, float2 *__restrict_
 // integers below 2^24: exact in FP32).
 template <int ORD, int N2T>
 __device__ __forceinline__ void emit_field(const KkGeom &g, int pair, int n1, const float2 (&x)[16],
-                                           const uint32_t (*raw)[kRawWords], const ColPos &cp, float2 *__restrict__ E,
+                                           const uint32_t (*raw)[kRawWords], const ColPos &cp, float2 *E,
                                            float &sre, float &sim, float &sint)
 {
     const float invN = 1.0f / (float)g.N;
@@ -626,9 +626,9 @@ __device__ __forceinline__ void emit_field(const KkGeom &g, int pair, int n1, co
 // position, and the per-call carrier / intensity sums (exact integer totals,
 // carrier_sums).  ORD: the pack order; N2T: the row length N / 16.
 template <int ORD, int N2T>
-__global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const float2 *__restrict__ fftws,
-                                                  const KkTables tb, float2 *__restrict__ E,
-                                                  const float2 *__restrict__ E_prev, DevState *dst)
+__global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const float2 *fftws,
+                                                  const KkTables tb, float2 *E,
+                                                  const float2 *E_prev, DevState *dst)
 {
     __shared__ float2 s_tw[512];
     __shared__ __align__(16) uint32_t raw[32][kRawWords];
@@ -676,7 +676,7 @@ static_assert(kLutCodes * 4 <= BkSmem::RAW, "the ln table fits the spectrum's pl
 
 template <int ORD>
 __global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, const KkTables tb,
-                                                       float2 *__restrict__ E, const float2 *__restrict__ E_prev,
+                                                       float2 *E, const float2 *E_prev,
                                                        DevState *dst)
 {
     extern __shared__ __align__(16) unsigned char bksm[];
@@ -781,7 +781,7 @@ __device__ __forceinline__ uint32_t warp_codes(const KkPacked &pk, long long t0,
     long long vb = (3 * t0) >> 1;
     const uint32_t *src = reinterpret_cast<const uint32_t *>(vb < pk.hist_bytes ? pk.hist + vb
                                                                                 : pk.in + (vb - pk.hist_bytes));
-    uint32_t w = lane < 12 ? __ldg(src + lane) : 0u;
+    uint32_t w = lane < 12 ? src[lane] : 0u;
     int b = (3 * lane) >> 1;
     uint32_t w0 = __shfl_sync(0xffffffffu, w, b >> 2);
     uint32_t w1 = __shfl_sync(0xffffffffu, w, min((b >> 2) + 1, 31));
@@ -792,8 +792,8 @@ __device__ __forceinline__ uint32_t warp_codes(const KkPacked &pk, long long t0,
 }
 
 __global__ void __cluster_dims__(kClC, 1, 1) __launch_bounds__(kClThreads, 3)
-    k_kk_cluster(KkGeom g, KkPacked pk, const KkTables tb, float2 *__restrict__ E,
-                 const float2 *__restrict__ E_prev, DevState *dst)
+    k_kk_cluster(KkGeom g, KkPacked pk, const KkTables tb, float2 *E,
+                 const float2 *E_prev, DevState *dst)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -1048,12 +1048,12 @@ cudaError_t launch_kk_front(const KkGeom &g, const KkInput &inp, float2 *fftws, 
 // downshifted field.  CTA 0 also carries the equaliser history [ybase, f_prev).
 constexpr int kMfOut = 256;
 
-__global__ void __launch_bounds__(kMfOut) k_kk_mf(const float2 *__restrict__ E, long long ebase, long long e_k,
+__global__ void __launch_bounds__(kMfOut) k_kk_mf(const float2 *E, long long ebase, long long e_k,
                                                  long long f_prev, long long f_k, const float *__restrict__ rrc,
                                                  int hmf, const float2 *__restrict__ ds_tab, int ds_num,
-                                                 int ds_den, const double *__restrict__ cg,
-                                                 float2 *__restrict__ Y, long long ybase,
-                                                 const float2 *__restrict__ Y_prev, long long ybase_prev)
+                                                 int ds_den, const double *cg,
+                                                 float2 *Y, long long ybase,
+                                                 const float2 *Y_prev, long long ybase_prev)
 {
     extern __shared__ float2 xs[];
     pdl_wait();
@@ -1128,10 +1128,10 @@ __host__ __device__ __forceinline__ int pad8(int p) { return p + (p >> 3); }
 
 template <int HMF, int STRIDE, bool FIXED>
 __global__ void __launch_bounds__(kMfThreads)
-    k_kk_mf_t(const float2 *__restrict__ E, long long ebase, long long e_k, long long f_prev, long long f_k,
+    k_kk_mf_t(const float2 *E, long long ebase, long long e_k, long long f_prev, long long f_k,
               const __grid_constant__ MfTaps<HMF> taps, const float2 *__restrict__ ds_tab, int ds_num, int ds_den,
-              unsigned ph0, const double *__restrict__ cg, float2 *__restrict__ Y, long long ybase,
-              const float2 *__restrict__ Y_prev, long long ybase_prev)
+              unsigned ph0, const double *cg, float2 *Y, long long ybase,
+              const float2 *Y_prev, long long ybase_prev)
 {
     constexpr int NPAIR = kMfTileOut + HMF + kMfR, NIT = (NPAIR + STRIDE - 1) / STRIDE;
     static_assert(STRIDE <= kMfThreads && STRIDE % 8 == 0, "one padded slot per 8 pairs");
@@ -1415,14 +1415,14 @@ __device__ float2 *stockham(float2 *a, float2 *b, int n, int N, const float2 *__
     return a;
 }
 
-__global__ void __launch_bounds__(kFdThreads) k_kk_fdmf(const float2 *__restrict__ E, long long ebase,
+__global__ void __launch_bounds__(kFdThreads) k_kk_fdmf(const float2 *E, long long ebase,
                                                        long long b_first, int N, const float2 *__restrict__ H,
                                                        const float2 *__restrict__ tw,
                                                        const float2 *__restrict__ ds_tab, int ds_num, int ds_den,
-                                                       const double *__restrict__ cg, float2 *__restrict__ Y,
+                                                       const double *cg, float2 *Y,
                                                        long long ybase, long long f_prev,
-                                                       const float2 *__restrict__ Y_prev, long long ybase_prev,
-                                                       float2 *__restrict__ clk, int wbin)
+                                                       const float2 *Y_prev, long long ybase_prev,
+                                                       float2 *clk, int wbin)
 {
     extern __shared__ float2 fbuf[];   // [2][N]
     float2 *a = fbuf, *b = fbuf + N;
@@ -1528,11 +1528,11 @@ __device__ __forceinline__ void dft32(float2 (&x)[32])
 constexpr int kFdWarps = 4, kFdPitch = 33;
 
 __global__ void __launch_bounds__(32 * kFdWarps, 4)
-    k_kk_fd1024(const float2 *__restrict__ E, long long ebase, long long b_first, long long nblk,
+    k_kk_fd1024(const float2 *E, long long ebase, long long b_first, long long nblk,
                 const float2 *__restrict__ H, const float2 *__restrict__ tw, const float2 *__restrict__ ds_tab,
-                int ds_num, int ds_den, const double *__restrict__ cg, float2 *__restrict__ Y, long long ybase,
-                long long f_prev, const float2 *__restrict__ Y_prev, long long ybase_prev,
-                float2 *__restrict__ clk, int wbin)
+                int ds_num, int ds_den, const double *cg, float2 *Y, long long ybase,
+                long long f_prev, const float2 *Y_prev, long long ybase_prev,
+                float2 *clk, int wbin)
 {
     __shared__ float2 s_tw[1024];
     __shared__ float2 s_t[kFdWarps][32 * kFdPitch];
@@ -1636,8 +1636,8 @@ cudaError_t launch_kk_fdmf(const float2 *E, long long ebase, long long f_prev, l
 
 // first CTA of a filter: the equaliser's history [ybase, f_prev), and the debug view of the
 // call's mean and deviation
-__device__ __forceinline__ void pam_carry(DevState *dst, int slot, float *__restrict__ Y, long long ybase, long long f_prev,
-                                          const float *__restrict__ Y_prev, long long ybase_prev)
+__device__ __forceinline__ void pam_carry(DevState *dst, int slot, float *Y, long long ybase, long long f_prev,
+                                          const float *Y_prev, long long ybase_prev)
 {
     for (long long m = ybase + threadIdx.x; m < f_prev; m += blockDim.x)
         Y[m - ybase] = (m < 0) ? 0.f : Y_prev[m - ybase_prev];
@@ -1647,11 +1647,11 @@ __device__ __forceinline__ void pam_carry(DevState *dst, int slot, float *__rest
     }
 }
 
-__global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *__restrict__ codes, long long cbase,
+__global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *codes, long long cbase,
                                                   long long n_end, long long f_prev, long long f_k,
                                                   const float *__restrict__ rrc, int hmf, DevState *dst,
-                                                  int slot, float *__restrict__ Y, long long ybase,
-                                                  const float *__restrict__ Y_prev, long long ybase_prev)
+                                                  int slot, float *Y, long long ybase,
+                                                  const float *Y_prev, long long ybase_prev)
 {
     extern __shared__ float xf[];
     pdl_wait();
@@ -1748,10 +1748,10 @@ cudaError_t launch_pam_mf_r(const float2 *R, long long rbase, long long f_prev, 
 // 1024}, a transpose, 32-point inverse DFTs over the former lane index; lane m_a
 // keeps m_b = 8 .. 23 (m = 256 .. 767), whose real part is y.
 __global__ void __launch_bounds__(32 * kFdWarps, 4)
-    k_pam_fd1024(const uint16_t *__restrict__ codes, long long cbase, long long n_end,
+    k_pam_fd1024(const uint16_t *codes, long long cbase, long long n_end,
                  long long b_first, long long nblk, const float2 *__restrict__ H, const float2 *__restrict__ tw,
-                 DevState *dst, int slot, float *__restrict__ Y, long long ybase, long long f_prev,
-                 const float *__restrict__ Y_prev, long long ybase_prev, float2 *__restrict__ clk, int wbin)
+                 DevState *dst, int slot, float *Y, long long ybase, long long f_prev,
+                 const float *Y_prev, long long ybase_prev, float2 *clk, int wbin)
 {
     __shared__ float2 s_tw[1024];
     __shared__ float2 s_t[kFdWarps][32 * kFdPitch];
@@ -1840,9 +1840,9 @@ struct PmTaps {
 
 template <int HMF>
 __global__ void __launch_bounds__(kPmThreads)
-    k_pam_mf_t(const uint16_t *__restrict__ codes, long long cbase, long long n_end, long long f_prev, long long f_k,
-               const __grid_constant__ PmTaps<HMF> taps, DevState *dst, int slot, float *__restrict__ Y, long long ybase,
-               const float *__restrict__ Y_prev, long long ybase_prev)
+    k_pam_mf_t(const uint16_t *codes, long long cbase, long long n_end, long long f_prev, long long f_k,
+               const __grid_constant__ PmTaps<HMF> taps, DevState *dst, int slot, float *Y, long long ybase,
+               const float *Y_prev, long long ybase_prev)
 {
     constexpr int L = kPmTile + 2 * HMF, NW = kPmR + 2 * HMF;
     static_assert(HMF % 4 == 0 && L % 8 == 0 && kPmR == 8, "16-byte pieces");

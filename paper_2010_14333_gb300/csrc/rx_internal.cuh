@@ -182,6 +182,12 @@ struct EqParams {
 // chain), and then lets the next grid start likewise.  Every thread calls it before its
 // first access to memory another kernel of the stream reads or writes.  Without the launch
 // attribute the call does nothing.
+// Such a grid's lifetime begins before its inputs are written, so in these kernels (and the
+// device functions they use) only the constant tables are __restrict__ or read by __ldg:
+// either is a promise that nothing else writes the data while the kernel lives, which lets
+// loads move above the wait and through the read-only path.  Plain pointers cost nothing:
+// the 2^19-sample field call 12.8 us against 13.4, batches of 2^22 samples 60.4 us per buffer
+// against 61.7, the others as before.
 __device__ __forceinline__ void pdl_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
