@@ -941,8 +941,9 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     const bool lat = h->lat_dev && !h->in_group && !h->flush_mode && npay >= c.eq_block;
     const int lat_slot = (int)(h->lat_head % kLatSlots);
     LatRecord *lat_first = lat ? h->lat_dev : nullptr;
-    // the launchers detect failures with cudaGetLastError: clear an error some
-    // earlier, unrelated call left behind (a sticky one makes the launches fail)
+    // the calls below whose status is not looked at (events, waits) are checked by one
+    // cudaGetLastError at the end: clear an error some earlier, unrelated call left behind
+    // (a sticky one makes the launches fail)
     cudaError_t stale = cudaGetLastError();
     if (stale != cudaSuccess) traced(stale, "an earlier CUDA call (cleared)");
     const bool two = sf != sb;
@@ -997,8 +998,9 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
         if (three && !h->kk) cudaStreamWaitEvent(sf, h->ev_cfree[cw_new], 0);
         // a flush pad adds nothing to the PAM sums: its filter uses the last real buffer's
         const bool sums = !h->kk && !h->flush_mode;
-        e = launch_unpack(in, h->codes[cw_new], h->codes[h->cw], h->nb, h->nhist, h->nb, h->calls == 0,
-                          c.pack_order, sums ? h->st : nullptr, spar, sf, lat_first, lat_slot, pdl_first);
+        if (e == cudaSuccess)
+            e = launch_unpack(in, h->codes[cw_new], h->codes[h->cw], h->nb, h->nhist, h->nb, h->calls == 0,
+                              c.pack_order, sums ? h->st : nullptr, spar, sf, lat_first, lat_slot, pdl_first);
         lat_first = nullptr;   // stamped: the KK front end (debug view) comes after
         h->cw = cw_new;
         prof_end(h, 0, sf);
@@ -1183,6 +1185,7 @@ static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out
     }
     if (four) cudaEventRecord(h->ev_dfree[ds], st4);
     else if (two) cudaEventRecord(h->ev_yfree[h->yw], sb);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (lat && e == cudaSuccess) h->lat_head++;
     if (h->prof_cur) h->prof_head++;
     h->prof_cur = 0;

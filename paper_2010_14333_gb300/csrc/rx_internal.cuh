@@ -210,7 +210,8 @@ inline cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
 }
 
 // ------------------------------------------------------------------ launchers
-// (each returns cudaGetLastError() after enqueuing)
+// (each returns the status of its launches; calls without a status of their own are checked
+// by the caller's cudaGetLastError)
 cudaError_t launch_unpack(const uint8_t *in, uint16_t *codes, const uint16_t *codes_prev,
                           long long nb, int nhist, long long prev_off, int first_call,
                           int pack_order, DevState *sums, int slot, cudaStream_t st,
