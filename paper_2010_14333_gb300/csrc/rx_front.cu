@@ -1654,7 +1654,7 @@ __global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *codes, long l
                                                   const float *Y_prev, long long ybase_prev)
 {
     extern __shared__ float xf[];
-    pdl_wait();
+    pdl_wait_late();
     const float s_mu = dst->pam_nf[slot][0], s_inv = dst->pam_nf[slot][1];
     long long m0 = f_prev + (long long)blockIdx.x * kMfOut;
     int L = kMfOut + 2 * hmf;
@@ -1673,6 +1673,7 @@ __global__ void __launch_bounds__(kMfOut) k_pam_mf(const uint16_t *codes, long l
     float a = 0.f;
     for (int i = -hmf; i <= hmf; i++) a = fmaf(__ldg(rrc + i + hmf), xc[-i], a);
     Y[m - ybase] = a;
+    pdl_release();
 }
 
 // ========================================== PAM resampler path (ADC off the transmitter's clock)
@@ -1757,7 +1758,7 @@ __global__ void __launch_bounds__(32 * kFdWarps, 4)
     __shared__ float2 s_t[kFdWarps][32 * kFdPitch];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < 1024; i += blockDim.x) s_tw[i] = tw[i];
-    pdl_wait();
+    pdl_wait_late();
     __syncthreads();
     if (blockIdx.x == 0) pam_carry(dst, slot, Y, ybase, f_prev, Y_prev, ybase_prev);
     const long long bi = (long long)blockIdx.x * kFdWarps + w;
@@ -1808,6 +1809,7 @@ __global__ void __launch_bounds__(32 * kFdWarps, 4)
     const long long s0 = 512 * blk - ybase;
 #pragma unroll
     for (int mb = 8; mb < 24; mb++) Y[s0 + lane + 32 * (mb - 8)] = x[mb].x;
+    pdl_release();
 }
 
 cudaError_t launch_pam_fd1024(const uint16_t *codes, long long cbase, long long n_end,
@@ -1847,7 +1849,7 @@ __global__ void __launch_bounds__(kPmThreads)
     constexpr int L = kPmTile + 2 * HMF, NW = kPmR + 2 * HMF;
     static_assert(HMF % 4 == 0 && L % 8 == 0 && kPmR == 8, "16-byte pieces");
     __shared__ __align__(16) float xf[pad32(L) + 4];
-    pdl_wait();
+    pdl_wait_late();
     const float mu = dst->pam_nf[slot][0], inv = dst->pam_nf[slot][1];
     const long long m0 = f_prev + (long long)blockIdx.x * kPmTile, n0 = m0 - HMF;
     const uint16_t *ct = codes + (n0 - cbase);
@@ -1904,6 +1906,7 @@ __global__ void __launch_bounds__(kPmThreads)
         for (int r = 0; r < kPmR; r++)
             if (mb + r < f_k) Yo[r] = acc[r];
     }
+    pdl_release();
 }
 
 cudaError_t launch_pam_mf(const uint16_t *codes, long long cbase, long long n_end, long long f_prev,

@@ -188,10 +188,18 @@ struct EqParams {
 // loads move above the wait and through the read-only path.  Plain pointers cost nothing:
 // the 2^19-sample field call 12.8 us against 13.4, batches of 2^22 samples 60.4 us per buffer
 // against 61.7, the others as before.
+// The PAM filters let the next grid start only when they have stored (pdl_wait_late, then
+// pdl_release): the equaliser's few CTAs, placed while the filter still fills most SMs, pile up
+// on the first SMs that fall idle, and their serial chains then share one SM's issue slots.
+// One 2^17 / 2^20-sample PAM-2 call: 19.8 / 20.5 us against 19.8 / 23.4 with the default
+// 33-tap filter, 20.9 / 23.0 against 25.5 / 33.1 with the 17-tap one, 21.4 / 26.2 against
+// 21.5 / 36.4 in the frequency-domain form.
+__device__ __forceinline__ void pdl_wait_late() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait_late();
+    pdl_release();
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, A... args)

@@ -1,4 +1,4 @@
-"""Kernels that start while the grid before them drains (they call pdl_wait) may read data
+"""Kernels that start while the grid before them drains (they call pdl_wait or pdl_wait_late) may read data
 that is still being written when they start.  ``__restrict__`` pointers and ``__ldg`` promise
 the compiler data that nothing else writes while the kernel lives, and so allow loads above
 the wait and through the read-only path: in these kernels, and in the device functions they
@@ -29,8 +29,8 @@ def functions():
 def test_only_constant_tables_are_promised_read_only():
     every = list(functions())
     kernels = [f for f in every if f[1] == "global"]
-    dependent = [f for f in kernels if "pdl_wait()" in f[4]]
-    ordinary = [f for f in kernels if "pdl_wait()" not in f[4]]
+    dependent = [f for f in kernels if "pdl_wait" in f[4]]
+    ordinary = [f for f in kernels if "pdl_wait" not in f[4]]
     used = lambda name, fs: any(re.search(rf"\b{name}\b", f[4]) for f in fs)
     # device functions, but for those that only ordinary kernels call
     device = [f for f in every if f[1] == "device" and (used(f[2], dependent) or not used(f[2], ordinary))]
