@@ -1231,13 +1231,15 @@ static rx_status run_batch(rx_handle *h, const uint8_t *const *ins, uint8_t *con
     const bool one = h->cfg.debug != 0;             // debug views want one call at a time
     // Device buffers of the time-domain PAM chain (unpack, filter | equaliser, demap) go through
     // two streams instead of four: its kernels are short, and inside a stage they follow each
-    // other without events.  Per buffer of 2^17 / 2^19 / 2^21 samples: 13.2 / 13.6 / 20.8 us
-    // against 15.5 / 15.9 / 24.1.
-    // The KK and frequency-domain chains (longer stages) and host buffers (the copies back sit
+    // other without events.  Per buffer of 2^17 / 2^19 / 2^21 samples: 15.1 / 16.0 / 22.5 us
+    // against 17.2 / 17.0 / 24.6.
+    // With the resampler the first stage would be four kernels (2^17 / 2^20 / 2^22 samples: 25.4
+    // / 51 / 116 us against 23.4 / 39.5 / 114 with one stream per stage).  The KK and
+    // frequency-domain chains (longer stages) and host buffers (the copies back sit
     // in the second stage's way) are faster with one stream per stage, and so is a handle that
     // is being profiled (every 4th call, 2^20 samples: 18.0 us against 18.8), whose events
     // stand between the kernels.
-    const bool two_stages = !one && !host && !h->kk && !h->fd && h->prof_on <= 0;
+    const bool two_stages = !one && !host && !h->kk && !h->fd && !h->rs && h->prof_on <= 0;
     cudaStream_t sf = one ? caller : h->front;
     cudaStream_t sb = one ? caller : h->back;
     cudaStream_t sc = one ? caller : h->copy;
