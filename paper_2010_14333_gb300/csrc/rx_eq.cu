@@ -384,8 +384,11 @@ __device__ __forceinline__ WinOut pam_window(const EqParams &p, const float *ys,
 // Payload: one warp per block of eq_block symbols, input staged by one bulk copy.
 // Training (train=1): one warp runs the training windows sequentially, staging
 // each window's input with plain loads.
+// PAM: with the block size alone the compiler settles on 32 registers, for an occupancy that
+// shared memory (8 KB per warp) never allows, and exposes the latency of the serial chain's
+// loads; four CTAs per SM leave it the 53 it wants.  2^17 samples, PAM-2: 5.4 us against 7.7.
 template <bool QAM, int NT, int MQ>
-__global__ void __launch_bounds__(32 * kEqWarpsMax)
+__global__ void __launch_bounds__(32 * kEqWarpsMax, QAM ? 0 : 4)
     k_eq(EqParams p, EqGeom g, int train, const void *Yv, float2 *taps_in, float2 *taps_out,
          uint8_t *dec, uint8_t *winb, uint4 *winrec,
          float4 *dbg_win, float2 *dbg_z, const uint8_t *__restrict__ prbs_ext,
