@@ -8,7 +8,9 @@ FIR at 2 samples/symbol, blind phase search 32 phases x 64 symbols, 16QAM Gray
 demap, bit-error count.  One step runs the whole chain over a batch of
 ``--bufs-per-step`` consecutive buffers of one stream, drawn from a ring of
 ``--ring`` distinct synthetic buffers resident in HBM (the ring is larger than
-L2).  Prints one JSON line (rank 0).
+L2).  Prints one JSON line (rank 0) of at most LINE_MAX bytes: the launch
+contract's keys and a few numbers of each leg; every leg's full record goes to
+standard error, one JSON line that starts with "detail: ".
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|reference]
 
@@ -53,6 +55,40 @@ FLOPS_PER_SAMPLE = {"kk_fwd": 13.0 * OLS, "kk_rows": 60.0 * OLS, "kk_inv": 13.0 
                     "eq": 252.0, "kk_front": 86.0 * OLS}
 BYTES_PER_SAMPLE = {"unpack": 1.5 + 2.0}   # packed read + 16-bit code write
 LANES = 128                 # FP32 lanes per SM (the SM count is queried from the device)
+LINE_MAX = 3000             # bytes of the printed line: a caller may keep only the end of the output
+CONTRACT = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gpu_launches", "realtime_x", "ber", "ber_oracle", "device_error")
+# numbers of each block that the line keeps, by their path in the full record
+KEPT = {"e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+        "clocks": ("sm_mhz", "sm_max_mhz", "reasons"),
+        "roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac"),
+        "chain_hbm": ("frac",),
+        "cpu_baseline": ("value", "unit", "cores", "kind", "sample", "cores_all", "value_all_cores"),
+        "latency": ("device_p50_ms", "device_p99_ms", "host_p50_ms", "budget_ms"),
+        "cnn": ("gsa_s", "ber_cnn", "ber_lms"),
+        "precision": ("forms.frozen_f32.gsa_s", "forms.bf16.gsa_s", "forms.fp8_e4m3.gsa_s"),
+        "fd_filter": ("frequency_domain.gsa_s", "pam4.frequency_domain.gsa_s", "pam4.time_domain_33_taps.gsa_s"),
+        "batched": ("streams", "modes.serial.gsa_s", "modes.group.gsa_s", "modes.group_graph.gsa_s"),
+        "resampler": ("gsa_s", "ber"),
+        "stability": ("seconds_of_signal", "q_db_mean", "q_db_min", "q_db_max", "device_ms_max", "window_deadline_misses"),
+        "diff_coding": ("gray.raw_ber_delivered", "differential.raw_ber_delivered"),
+        "dd_symbol_equaliser": ("dd_symbol_4_taps.gsa_s", "dd_symbol_4_taps.ber")}
+
+
+def short_line(full):
+    """The printed line: CONTRACT as it is, and of each block that ran the numbers in KEPT."""
+    line = {k: full[k] for k in CONTRACT}
+    for block, paths in KEPT.items():
+        if not full.get(block):
+            continue
+        line[block] = {}
+        for path in paths:
+            v = full[block]
+            for key in path.split("."):
+                v = v.get(key) if isinstance(v, dict) else None
+            exact = block in ("e2e", "clocks", "cpu_baseline")
+            line[block][path] = float(f"{v:.5g}") if isinstance(v, float) and not exact else v
+    return line
 
 
 def workload_config(args):
@@ -556,7 +592,8 @@ def gpu_arm(args, rank, world, local):
                         "after a wrap and the timed run's own BER is not meaningful",
             "device_error": stats["device_error"], "gen_s": t_gen}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print("detail: " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
     if dist:
         dist.destroy_process_group()
 
