@@ -423,13 +423,13 @@ rx_status rx_group_destroy(rx_group *g);
  *                blocks must fit the FFT rows: ceil(J/2) * ols_n <= 2^19 complex
  *                values with J = ceil((nsamp - ols_v/2) / (ols_n - ols_v)) blocks
  *                (at ols_n = 65536 and nsamp = 2^19 that allows ols_v up to 4096).
+ *                4096-point blocks keep the limit, although they use no rows.
  *   ols_n/ols_v: as in rx_config (4096 or 65536; overlap a multiple of 64, < ols_n).
  *   field_out:   DEVICE pointer, 8-byte aligned, room for 2*(nsamp - ols_v/2)
  *                floats (interleaved real, imaginary).
  *
- * The scratch (twiddle and ln tables, a packed-history region, FFT rows, a copy of an
- * input that the field is written over) is one
- * fixed device array of about 4.9 MiB in librx.so;
+ * The scratch (twiddle and ln tables, FFT rows, a copy of an input that the field is
+ * written over) is one fixed device array of about 4.8 MiB in librx.so;
  * every GPU that loads the library holds it until the process exits.  Sizes
  * beyond the limits return RX_EINVAL before anything is enqueued.  The call
  * allocates nothing (no cudaMalloc, cudaFree or allocating library routine); it

@@ -922,7 +922,7 @@ rx_status rx_create(rx_format f, double baud, double fs, int64_t buf_len, const 
 // the back end of this call waits for its front end, and the front end of a later
 // call that reuses a matched-filter slot waits for the back end that read it.
 // With host buffers (host_in / host_out non-null) the input is copied into one of
-// two staging buffers on `sc`, overlapping the previous front end, and the bits
+// kInSlots staging buffers on `sc`, overlapping earlier front ends, and the bits
 // are copied back on `sb` after the demap.
 static rx_status enqueue_call(rx_handle *h, const uint8_t *in, uint8_t *bits_out, const uint8_t *host_in,
                               uint8_t *host_out, cudaStream_t sf, cudaStream_t sb, cudaStream_t sc,

@@ -18,8 +18,6 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <type_traits>
-
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

@@ -414,8 +414,9 @@ __global__ void __launch_bounds__(32 * kEqWarpsMax, QAM ? 0 : 4)
     if (!train && blk >= g.nblk) return;
     constexpr int BPS = QAM ? (MQ == 2 ? 2 : 4) : (MQ == 2 ? 1 : MQ == 4 ? 2 : 3);
     const int sb = blk * B;   // the block's first symbol, from pay_lo
-    // PRBS position of the block's first bit: fewer than 2^30 bits follow the call's first
-    int pwin = (int)(((unsigned)g.pos0 + (unsigned)(BPS * sb)) % 32767u), ref2 = 0;
+    // PRBS position of the block's first bit: a call has at most 3 x 2^29 bits (PAM-8, 2^30
+    // samples) and those of the symbols carried over, below 2^31
+    int pwin = (int)(((unsigned)g.pos0 + (unsigned)BPS * (unsigned)sb) % 32767u), ref2 = 0;
     if (!train) {   // the block's input, the taps and the first window's reference bits together
         if (lane == 0) {
             mbar_init(bar, 1);

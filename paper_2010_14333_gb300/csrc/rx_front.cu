@@ -281,8 +281,9 @@ __device__ __forceinline__ bool before_stream(const KkGeom &g, int pair, bool hb
     return ols_ws(g, 2 * pair) < 0 || (hb && ols_ws(g, 2 * pair + 1) < 0);
 }
 
-// (CTAs of kCtaK1 threads; asynchronous copies, which the caller waits for).  Samples before the stream are staged as c_first.  Byte offsets fit
-// 32 bits: a buffer is at most 2^30 samples.
+// The rows of a CTA's columns (kCtaK1 threads) by asynchronous copies, which the caller waits
+// for.  Samples before the stream are staged as c_first.  Byte offsets fit 32 bits: a buffer
+// is at most 2^30 samples.
 template <int N2T>
 __device__ __forceinline__ void stage_rows(const KkGeom &g, const KkPacked &pk, int pair, int c0,
                                            uint32_t (*raw)[kRawWords], bool hb, uint32_t c_first)

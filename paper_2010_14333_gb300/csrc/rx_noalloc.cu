@@ -22,19 +22,15 @@ constexpr size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
 // byte layout of the scratch array:
 //   tables   per FFT length (4096, 65536) a block [ln table | factored W_N | factored W_{N/16}]
-//   hist     the packed history the front end is handed; on a stream's first buffer it
-//            is never read for values (samples before the stream are the first sample
-//            replicated), so it only has to be a valid region of ols_n * 3 / 2 bytes
 //   fft      the two-block complex FFT rows of 2^16-point blocks, at most 2^19 complex values
 //   in       a copy of the packed input, for callers whose field lies over it
 // The field goes straight to the caller's buffer: no field history is kept and no carrier
-// sums are taken.
+// sums are taken.  The front end is handed no packed history: on a stream's first buffer all
+// samples before it are the first sample replicated, which it fills in itself.
 constexpr int kNaSizes = 2;
 constexpr size_t kTabBytes = 4096 * sizeof(float) + 1024 * sizeof(float2);   // >= one block
 constexpr size_t kOffTw = 0;
-constexpr size_t kOffHist = align_up(kOffTw + kNaSizes * kTabBytes);
-constexpr size_t kHistBytes = (size_t)65536 * 3 / 2;
-constexpr size_t kOffFft = align_up(kOffHist + kHistBytes);
+constexpr size_t kOffFft = align_up(kOffTw + kNaSizes * kTabBytes);
 constexpr size_t kFftBytes = 4u << 20;                   // two-block complex FFT rows
 constexpr size_t kOffIn = align_up(kOffFft + kFftBytes);
 constexpr size_t kInBytes = (size_t)kNaMaxSamples * 3 / 2;
@@ -112,7 +108,7 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
     g.e_prev = 0;
     g.e_k = e_k;
     g.avail = nsamp;
-    g.cbase = -(long long)ols_n;        // stream index of the packed history's first sample
+    g.cbase = -(long long)ols_n;        // stream index of the (virtual) history's first sample
     g.ebase = 0;                        // the field starts with stream sample 0
     g.sps = 4;
     g.slot = 0;
@@ -129,7 +125,6 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
     tb.lnt = (const float *)tabb;
     tb.twN = (const float2 *)(tb.lnt + 4096);
     tb.twN2 = tb.twN + kk_tw_entries(ols_n);
-    const uint8_t *hist = base + kOffHist;
     float2 *fftws = (float2 *)(base + kOffFft);
     // blocks read their codes while others already write the field: a field over its own
     // input works on a copy
@@ -140,7 +135,7 @@ extern "C" rx_status rx_kk_field_noalloc(const uint8_t *packed12_in, int64_t nsa
         packed12_in = base + kOffIn;
     }
     KkInput kin;
-    kin.hist = hist;                        // never read for values: the first call fills the pre-stream
+    kin.hist = nullptr;                     // the whole history lies before the stream: never read
     kin.in = packed12_in;
     kin.hist_next = nullptr;
     kin.hist_bytes = (long long)ols_n * 3 / 2;
