@@ -374,10 +374,18 @@ __device__ __forceinline__ void load_columns(bool hb, const uint32_t (*raw)[kRaw
 __device__ __forceinline__ void copy_hist(const KkPacked &pk, int cta, int ncta)
 {
     const long long nch = pk.hist_bytes / 16;
-    for (long long c = (long long)cta * blockDim.x + threadIdx.x; c < nch; c += (long long)ncta * blockDim.x) {
-        long long vb = pk.in_bytes + 16 * c;
-        const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
-        reinterpret_cast<uint4 *>(pk.hist_next)[c] = *reinterpret_cast<const uint4 *>(src);
+    const long long step = (long long)ncta * blockDim.x;
+    for (long long c = (long long)cta * blockDim.x + threadIdx.x; c < nch; c += 2 * step) {
+        uint4 v[2];
+#pragma unroll
+        for (int k = 0; k < 2; k++) {   // every load issues before the first one is stored
+            const long long vb = pk.in_bytes + 16 * (c + k * step);
+            const uint8_t *src = vb < pk.hist_bytes ? pk.hist + vb : pk.in + (vb - pk.hist_bytes);
+            if (c + k * step < nch) v[k] = *reinterpret_cast<const uint4 *>(src);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; k++)
+            if (c + k * step < nch) reinterpret_cast<uint4 *>(pk.hist_next)[c + k * step] = v[k];
     }
 }
 
@@ -572,13 +580,22 @@ __device__ __forceinline__ void carrier_sums(const KkGeom &g, DevState *dst, flo
 }
 
 // field history for the matched filter: E[n], n in [e_prev - kEHist, e_prev) (E_prev null:
-// the caller keeps none)
-__device__ __forceinline__ void carry_field(const KkGeom &g, float2 *E, const float2 *E_prev)
+// the caller keeps none), the samples first, first + step, .. by one thread, NB loads at a time
+template <int NB>
+__device__ __forceinline__ void carry_field(const KkGeom &g, float2 *E, const float2 *E_prev, int first, int step)
 {
     if (!E_prev) return;
-    for (int i = threadIdx.x; i < kEHist; i += blockDim.x) {
-        long long n = g.e_prev - kEHist + i;
-        E[i] = (n < 0) ? make_float2(0.f, 0.f) : E_prev[n - g.ebase_prev];
+    for (int i0 = first; i0 < kEHist; i0 += NB * step) {
+        float2 v[NB];
+#pragma unroll
+        for (int k = 0; k < NB; k++) {   // every load issues before the first one is stored
+            const int i = i0 + k * step;
+            const long long n = g.e_prev - kEHist + i;
+            v[k] = i < kEHist && n >= 0 ? E_prev[n - g.ebase_prev] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < NB; k++)
+            if (i0 + k * step < kEHist) E[i0 + k * step] = v[k];
     }
 }
 
@@ -640,7 +657,7 @@ __global__ void __launch_bounds__(kCtaK1) k_kk_inv(KkGeom g, KkPacked pk, const 
     const bool hb = 2 * pair + 1 < g.J;
     stage_rows<N2T>(g, pk, pair, c0, raw, hb, before_stream(g, pair, hb) ? first_code(pk, dst) : 0u);
     float sre = 0.f, sim = 0.f, sint = 0.f;
-    if (blockIdx.x == 0 && blockIdx.y == 0) carry_field(g, E, E_prev);
+    if (blockIdx.y == 0) carry_field<1>(g, E, E_prev, c0 + threadIdx.x, gridDim.x * blockDim.x);
     const int t = threadIdx.x, n1 = c0 + t;
     const ColPos cp = col_pos<ORD>(t);
     float2 x[16];
@@ -700,7 +717,7 @@ __global__ void __launch_bounds__(kCtaK1, 3) k_kk_block(KkGeom g, KkPacked pk, c
     const uint32_t c_first = before_stream(g, pair, hb) || pk.first_call ? first_code(pk, dst) : 0u;
     stage_rows<kBkN2>(g, pk, pair, 0, raw, hb, c_first);
     if (pk.first_call && dst && pair == 0 && t == 0) dst->first_code = (int)c_first;
-    if (pair == 0) carry_field(g, E, E_prev);
+    if (pair == 0) carry_field<kEHist / kCtaK1>(g, E, E_prev, t, kCtaK1);
     cp_async_wait_all();
     __syncthreads();
     const ColPos cp = col_pos<ORD>(t);
@@ -813,7 +830,7 @@ __global__ void __cluster_dims__(kClC, 1, 1) __launch_bounds__(kClThreads, 3)
     // history of the next call (packed bytes [in_bytes, in_bytes + hist_bytes) of
     // the virtual buffer), spread over the grid
     if (pk.hist_next) copy_hist(pk, blockIdx.x, gridDim.x);
-    if (blockIdx.x == 0) carry_field(g, E, E_prev);
+    if (blockIdx.x == 0) carry_field<kEHist / kClThreads>(g, E, E_prev, t, kClThreads);
     cp_async_wait_all();
     __syncthreads();   // staged twiddles
 
@@ -1111,6 +1128,9 @@ __global__ void __launch_bounds__(kMfOut) k_kk_mf(const float2 *E, long long eba
 // sample and 64-bit phase and range arithmetic.  Persistent CTAs that load the next tile
 // into registers during the FIR took 16.5 us alone on warm caches against 17.4 but 1 to 3 us
 // more in the receiver, where their 95 to 116 registers leave no room for other kernels.
+// A thread's loads go out in two halves (40 registers): all at once they take 50, and six
+// pipelined 2^20-sample buffers behind the cluster front end 500 us against 430, since the
+// cluster of the next buffer then finds no room beside the filter.
 template <int HMF>
 struct MfTaps {
     f2x ge[HMF + 1];   // (ge, ge)
@@ -1162,21 +1182,26 @@ __global__ void __launch_bounds__(kMfThreads)
     const float2 c = make_float2((float)cg[0], (float)cg[1]);
     const float gn = (float)cg[2];
     if (inner) {
-        float4 v[NIT];   // every load issues before the first one is used
+        constexpr int HALF = (NIT + 1) / 2;
 #pragma unroll
-        for (int k = 0; k < NIT; k++)
-            if (act && threadIdx.x + k * STRIDE < NPAIR)
-                v[k] = reinterpret_cast<const float4 *>(Et)[threadIdx.x + k * STRIDE];
+        for (int k0 = 0; k0 < NIT; k0 += HALF) {
+            float4 v[HALF];   // the loads of half the pairs issue before the first one is used
 #pragma unroll
-        for (int k = 0; k < NIT; k++) {
-            if (!FIXED && k) {
-                idx += step;
-                idx = idx >= den ? idx - den : idx;
-                w = phases(idx);
+            for (int k = k0; k < k0 + HALF && k < NIT; k++)
+                if (act && threadIdx.x + k * STRIDE < NPAIR)
+                    v[k - k0] = reinterpret_cast<const float4 *>(Et)[threadIdx.x + k * STRIDE];
+#pragma unroll
+            for (int k = k0; k < k0 + HALF && k < NIT; k++) {
+                if (!FIXED && k) {
+                    idx += step;
+                    idx = idx >= den ? idx - den : idx;
+                    w = phases(idx);
+                }
+                const float4 x = v[k - k0];
+                const float2 a = cmul(csub(make_float2(x.x, x.y), c), make_float2(w.x, w.y));
+                const float2 b = cmul(csub(make_float2(x.z, x.w), c), make_float2(w.z, w.w));
+                if (act && threadIdx.x + k * STRIDE < NPAIR) ps[k * pad8(STRIDE)] = make_float4(a.x, a.y, b.x, b.y);
             }
-            const float2 a = cmul(csub(make_float2(v[k].x, v[k].y), c), make_float2(w.x, w.y));
-            const float2 b = cmul(csub(make_float2(v[k].z, v[k].w), c), make_float2(w.z, w.w));
-            if (act && threadIdx.x + k * STRIDE < NPAIR) ps[k * pad8(STRIDE)] = make_float4(a.x, a.y, b.x, b.y);
         }
     } else if (act) {
 #pragma unroll 1

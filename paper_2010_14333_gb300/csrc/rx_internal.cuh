@@ -185,9 +185,10 @@ struct EqParams {
 // Such a grid's lifetime begins before its inputs are written, so in these kernels (and the
 // device functions they use) only the constant tables are __restrict__ or read by __ldg:
 // either is a promise that nothing else writes the data while the kernel lives, which lets
-// loads move above the wait and through the read-only path.  Plain pointers cost nothing:
-// the 2^19-sample field call 12.8 us against 13.4, batches of 2^22 samples 60.4 us per buffer
-// against 61.7, the others as before.
+// loads move above the wait and through the read-only path.  Plain pointers cost nothing once
+// the loops that copy histories load in groups by hand (a store may alias the next load): the
+// 2^19-sample field call 12.8 us against 13.4, batches of 2^22 samples 61.2 us per buffer
+// against 61.9, the others as before.
 // The PAM filters let the next grid start only when they have stored (pdl_wait_late, then
 // pdl_release): the equaliser's few CTAs, placed while the filter still fills most SMs, pile up
 // on the first SMs that fall idle, and their serial chains then share one SM's issue slots.
