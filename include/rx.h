@@ -244,9 +244,10 @@ rx_status rx_process(rx_handle *h, const uint8_t *packed12_in, uint8_t *bits_out
  * the KK field of even and odd buffers on two streams (2^16-point blocks; one
  * with 4096-point blocks), each ordered after the previous buffer's history
  * copy and field, the matched filter, the equaliser and the decisions and bits
- * each on a stream of its own.  Device buffers of the time-domain PAM chain take
- * two streams, unpack and filter on one, equaliser and bits on the other.  The
- * pipeline starts after the work already on cuda_stream, and cuda_stream waits for its last back end before anything enqueued later.
+ * each on a stream of its own.  Device buffers of the time-domain PAM chain without
+ * the resampler take two streams, unpack and filter on one, equaliser and bits on
+ * the other.  The pipeline starts after the work already on cuda_stream, and
+ * cuda_stream waits for its last back end before anything enqueued later.
  * With cfg.debug = 1 the buffers run one at a time on cuda_stream.  The stages
  * overlap only if their streams reach separate hardware queues: with several
  * handles or groups in one process, set CUDA_DEVICE_MAX_CONNECTIONS (e.g. 32)

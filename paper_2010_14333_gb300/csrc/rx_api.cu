@@ -1231,8 +1231,8 @@ static rx_status run_batch(rx_handle *h, const uint8_t *const *ins, uint8_t *con
     const bool one = h->cfg.debug != 0;             // debug views want one call at a time
     // Device buffers of the time-domain PAM chain (unpack, filter | equaliser, demap) go through
     // two streams instead of four: its kernels are short, and inside a stage they follow each
-    // other without events.  Per buffer of 2^17 / 2^19 / 2^21 samples: 15.1 / 16.0 / 22.5 us
-    // against 17.2 / 17.0 / 24.6.
+    // other without events.  Per buffer of 2^17 / 2^19 / 2^21 samples, six per call: 15.5 / 14.6 /
+    // 18.9 us against 17.1 / 16.3 / 19.7.
     // With the resampler the first stage would be four kernels (2^17 / 2^20 / 2^22 samples: 25.4
     // / 51 / 116 us against 23.4 / 39.5 / 114 with one stream per stage).  The KK and
     // frequency-domain chains (longer stages) and host buffers (the copies back sit

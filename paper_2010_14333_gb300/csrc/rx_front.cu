@@ -1124,7 +1124,7 @@ __global__ void __launch_bounds__(kMfOut) k_kk_mf(const float2 *E, long long eba
 // (the default 11/80 cycles per sample: 40) and covers a tile in as many steps as 128.
 // Bound by the shared-memory pipe and the packed FMAs (two issue cycles each: 7 us of the
 // FMA pipe for 2^21 outputs) in 1.2 waves of CTAs.  2^22-sample buffer: 17.4 us on warm caches and
-// 7.7 M warp instructions; 19.5 us and 10.1 M with taps in shared memory, phases per
+// 7.6 M warp instructions; 19.5 us and 10.1 M with taps in shared memory, phases per
 // sample and 64-bit phase and range arithmetic.  Persistent CTAs that load the next tile
 // into registers during the FIR took 16.5 us alone on warm caches against 17.4 but 1 to 3 us
 // more in the receiver, where their 95 to 116 registers leave no room for other kernels.
